@@ -152,7 +152,12 @@ __global__ void __launch_bounds__(FS_THREADS, 1)
         for (int64_t kc = 0; kc < nk; ++kc, ++it) {
             if ((int)(it % FS_NGRP) != grp) continue;
             const int s = (int)(it % FS_STAGES);
-            const bool got = mbar_wait_warp(&full[s], (uint32_t)((it / FS_STAGES) & 1), abort, flags);
+            // FS_STAGES is no multiple of FS_NGRP, so the stage's previous chunk belonged to another
+            // group, which may still wait for it (loads land out of order): full[s]'s phase, known by its
+            // parity only, is the one asked for once that group has released the stage
+            bool got = it < FS_STAGES ||
+                       mbar_wait_warp(&xfree[s], (uint32_t)(((it / FS_STAGES) & 1) ^ 1), abort, flags);
+            got = got && mbar_wait_warp(&full[s], (uint32_t)((it / FS_STAGES) & 1), abort, flags);
             if (got) {
                 const uint8_t* xs = smem + s * FS_XBYTES;
                 const float4* mrow = m4 + (kc * FS_CHUNK + 16 * kh) * 2;

@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(FS_THREADS, 1)
     uint64_t* full = reinterpret_cast<uint64_t*>(red + (FS_PARTS - 1) * FS_ROWS * FS_COLS);
     uint64_t* xfree = full + FS_STAGES;
     volatile int* abort = reinterpret_cast<volatile int*>(xfree + FS_STAGES);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = (int)warp_uniform(tid >> 5), lane = tid & 31;
     for (int64_t e = tid; e < nk * FS_CHUNK * FS_COLS; e += blockDim.x) {
         const int64_t i = e / FS_COLS, a = e % FS_COLS;
         msm[e] = (i < args.nj && a < args.m) ? (args.mtrans ? args.M[a + args.ldm * i] : args.M[i + args.ldm * a])
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(FS_THREADS, 1)
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             int64_t it = 0;
             bool ok = true;
             for (int64_t t = blockIdx.x; t < nitems && ok; t += gridDim.x) {

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(Warps<EPI>::kThreads, 1)
     using W = Warps<EPI>;
     __shared__ double red[2 * W::kEpi];
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
@@ -220,14 +220,14 @@ __global__ void __launch_bounds__(Warps<EPI>::kThreads, 1)
     }
     __syncthreads();
     tc_fence_after();
-    const uint32_t tbase = *tmem_slot;
+    const uint32_t tbase = warp_uniform(*tmem_slot);
     unsigned* flags = args.flags;
     const int64_t nk = args.nk;
     const int64_t nitems = args.ntiles * args.nblk * args.ksplit;
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             int64_t it = 0, item = 0;
             bool ok = true;
             for (int64_t w = blockIdx.x; w < nitems && ok; w += gridDim.x, ++item) {
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(Warps<EPI>::kThreads, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             int64_t it = 0, ab = 0, acc = 0;
             bool ok = true;
             for (int64_t w = blockIdx.x; w < nitems && ok; w += gridDim.x, ++acc) {

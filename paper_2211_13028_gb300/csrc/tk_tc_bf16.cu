@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = (int)tc::warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
@@ -130,14 +130,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncthreads();
     tc::tc_fence_after();
-    const uint32_t tbase = *tmem_slot;
+    const uint32_t tbase = tc::warp_uniform(*tmem_slot);
     unsigned* flags = args.flags;
     const int64_t nk = args.nk;
     const int64_t nitems = args.ntiles * args.nblk;
 
     if (warp == 0) {
         // ------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (tc::elect_one()) {
             int64_t it = 0;
             bool ok = true;
             for (int64_t w = blockIdx.x; w < nitems && ok; w += gridDim.x) {
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (tc::elect_one()) {
             int64_t it = 0, acc = 0;
             bool ok = true;
             constexpr uint32_t idesc = idesc_bf16(2 * NPAD, !KMAJOR);

@@ -1,0 +1,604 @@
+// The tcgen05 kernel of a plain mode-j contraction (TTM) of FP32 data:
+//
+//   out[l + L*(a + m*r)] = sum_i M(i, a) X[l + L*(i + n_j*r)]     (X viewed as L x n_j x R)
+//
+// FP32 accuracy from TF32 tensor cores by the split-product ("3xTF32") method:
+// x = x_hi + x_lo and M = M_hi + M_lo with TF32 parts, and x*M ~ x_hi*M_hi +
+// x_hi*M_lo + x_lo*M_hi with FP32 accumulation.
+//
+// Kernel structure (persistent, one CTA per SM):
+//   warp 0      TMA producer (one thread): 32-deep K chunks of a 128-row tile of X (16 KB) plus the
+//               matching 32 x NPAD chunks of M_hi and M_lo, into an SMEM ring.
+//   warp 1      allocates TMEM; one thread issues tcgen05.mma.
+//   loaders     (FLAT only, 8 warps) bring the X chunk with cp.async instead of TMA, see below.
+//   converters  (two groups of 8 warps taking alternate chunks; FLAT: one) read their row's values of the chunk
+//               from SMEM, split them into TF32 hi / lo and write them to TMEM with tcgen05.st.  The
+//               MMA reads A from TMEM, so X is read from SMEM exactly once, and a contraction over a
+//               non-contiguous mode needs no transpose: only the element each lane reads differs.
+//   epilogue    (8 warps, two per TMEM lane quarter): tcgen05.ld, sums, rows written to global memory.
+// The issuing threads are chosen by elect.sync (tk_tc_common.cuh), so that neither the MMAs (288 of
+// the 700 cycles that HBM gives a chunk at NPAD = 48) nor their issue bounds the pass.
+//
+// One MMA per 8-deep K step computes A_hi * [M_hi ; M_lo] (N = 2*NPAD, the two halves land in separate
+// TMEM columns); a second adds A_lo * M_hi into the second half, with the other small term.  The
+// tensor core's FP32 accumulation rounds each addition toward zero, a bias that grows with the number
+// of additions into one A_hi * M_hi sum.  So an accumulator takes the products of `fill` chunks only (1
+// for FLAT, else 4; 16 above 64 columns, whose registers the epilogue lacks), and the epilogue adds the fills of an item in FP32 registers, rounding to nearest,
+// while the next ones are computed: TMEM holds a ring of as many accumulators as fit beside the A
+// buffers.  512^3, 42 columns: error against FP64 2.4e-6 with one
+// accumulator an item, 7.2e-7 so, for 100 -> 104 us.
+//
+// FLAT = false: TMA.  Needs 16-byte strides (L % 4 == 0, or n_j % 4 == 0 for L == 1).  A strided mode
+// with fewer than 64 rows before it packs several slabs into each 128-row tile (pack).
+// FLAT = true: any L and n_j.  The L*R rows are numbered without regard to slabs (so no row of a tile
+// is padding, whatever L is), every loader lane keeps the addresses of its rows, and 4-byte cp.async
+// (8-byte when L, or n_j for L == 1, is even) fill the same stages in the same layout, with zeros
+// beyond n_j and the last row; each loader's cp.async arrive on the stage's barrier when they land.
+//
+// Every mbarrier wait is bounded by a wall-clock limit; on expiry the CTA raises FLAG_TIMEOUT, stops
+// issuing work, drains what it issued and frees its TMEM.
+#pragma once
+#include "tk_tc_common.cuh"
+
+namespace tk {
+namespace tc {
+
+constexpr int kRows = 128;    // tile rows (TMEM lanes)
+constexpr int kChunk = 32;    // K elements per pipeline stage
+constexpr int kXBytes = kRows * kChunk * 4;
+
+// D[tmem] (+)= A[tmem] * B[smem desc], kind::tf32, M = 128.
+__device__ __forceinline__ void mma_tf32_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                            uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// Instruction descriptor: D F32, A/B TF32, both K-major, M = 128, N = n.
+__host__ __device__ constexpr uint32_t idesc_tf32(int n) {
+    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kRows >> 4) << 24);
+}
+
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15, %16};" ::"r"(taddr),
+        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
+        "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
+        : "memory");
+}
+
+// x = hi + lo: hi is x rounded to TF32 (ties away, as cvt.rna) by integer addition; lo = x - hi (exact), whose
+// bits below TF32 the tensor core ignores: an odd last bit is dropped where cvt.rna rounds it away, an
+// error of the same size.  NaN survives in lo.  The conversion unit, two cvt.rna per element, bounded the
+// pass (512^3, 42 columns: 135 -> 115 us).
+__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
+    hi = (__float_as_uint(x) + 0x1000u) & 0xFFFFE000u;
+    lo = __float_as_uint(x - __uint_as_float(hi));
+}
+
+struct TtmArgs {
+    int64_t L, nj, R, m;
+    // work item = (row tile, block of NPAD output columns, part of the K chunks)
+    uint32_t ntiles, tiles_per_r, nk, nblk, nitems;
+    // strided mode with L < 64 (TMA): a tile holds `pack` consecutive r of L rows each (pack L <= 128
+    // rows) instead of one r, so that short rows fill the 128-row tile; 1 otherwise
+    uint32_t pack;
+    uint32_t xbytes;  // TMA bytes of one X chunk (128 x 32 x 4, or L x 32 x pack x 4; 0: FLAT)
+    // few row tiles: the K chunks of a tile are split over ksplit work items, each writing its
+    // partial product to part + s out_numel (summed in order by a second kernel); 1 otherwise
+    uint32_t ksplit;
+    uint32_t fill;         // chunks per accumulator
+    uint32_t vec;          // FLAT: floats per cp.async (1 or 2)
+    const float* X;        // FLAT
+    float* part;
+    int64_t out_numel;
+    float* out;
+    unsigned* flags;
+};
+
+template <int NPAD, bool FLAT>
+struct TtmCfg {
+    static constexpr int kBBytes = NPAD * 128;  // one of M_hi / M_lo: NPAD rows of 128 B
+    static constexpr int kStage = kXBytes + 2 * kBBytes;
+    static constexpr int kBudget = 210 * 1024;
+    // FLAT: a shorter ring, which leaves the SM's L1, where each cp.async in flight holds its lines, some
+    // room (413 x 350 x 275 along its first mode, 5 columns: 58 us with 10 stages, 47 with 6)
+    static constexpr int kStages = FLAT ? (NPAD <= 32 ? 6 : 4) : (kBudget / kStage > 12 ? 12 : kBudget / kStage);
+    static constexpr int kNA = NPAD <= 32 ? 4 : 2;      // A buffers of 64 columns (hi 32 | lo 32)
+    static constexpr int kABuf = 512 - 64 * kNA;
+    static constexpr int kFit = kABuf / (2 * NPAD);     // accumulators of 2*NPAD columns
+    static constexpr int kAcc = kFit > 8 ? 8 : kFit;
+    static constexpr int kSmem = kStages * kStage + 1024 + 512;
+    static constexpr int kLoad = FLAT ? 8 : 0;          // loader warps, from warp 2
+    static constexpr int kFirstConv = FLAT ? 12 : 4;    // (a multiple of 4: warp % 4 is the TMEM lane quarter)
+    static constexpr int kGroups = FLAT ? 1 : 2;        // converter groups of 8 warps
+    static constexpr int kFirstEpi = kFirstConv + 8 * kGroups;
+    static constexpr int kEpi = 8;                      // epilogue warps
+    static constexpr int kThreads = 32 * (kFirstEpi + kEpi);
+    static_assert(kAcc >= 2, "TMEM budget");
+    static_assert(kStages >= 4, "SMEM budget");
+    // The converter groups take alternate chunks, so with an odd ring a stage alternates between them,
+    // and a group must not test a stage's barrier a whole ring early (the parity of the phase before
+    // would read as complete): chunk c + S comes after its own chunk c + S - 2, whose A buffer waited for
+    // the MMAs of chunk c + S - 2 - kNA, hence for chunk c's load.
+    static_assert(kGroups == 1 || kStages % 2 == 0 || kStages >= kNA + 2, "converter groups could overrun the ring");
+};
+
+template <int BYTES>
+__device__ __forceinline__ void cp_async(uint32_t dst, const void* src, uint32_t valid) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(BYTES), "r"(valid) : "memory");
+}
+// One arrival on bar (counted in its expected arrivals) once this thread's earlier cp.async have landed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+template <int NPAD, bool KMAJOR, bool FLAT>
+__global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
+    ttm_tf32x3_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmBhi,
+                      const __grid_constant__ CUtensorMap tmBlo, TtmArgs args) {
+    using C = TtmCfg<NPAD, FLAT>;
+    constexpr uint32_t S = C::kStages;
+    constexpr uint32_t NA = C::kNA;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * C::kStage);
+    uint64_t* full = bars;                   // [S] X and factor chunk landed
+    uint64_t* xfree = bars + S;              // [S] stage consumed (8 converter warps + 1 MMA commit)
+    uint64_t* afull = bars + 2 * S;          // [NA] A buffer written (8 converter warps)
+    uint64_t* aempty = afull + NA;           // [NA] A buffer consumed (MMA commit)
+    uint64_t* accfull = aempty + NA;         // [kAcc] accumulator complete (MMA commit)
+    uint64_t* accempty = accfull + C::kAcc; // [kAcc] accumulator drained (the epilogue warps)
+    uint64_t* done = accempty + C::kAcc;    // [1] every issued MMA complete
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        for (uint32_t s = 0; s < S; ++s) {
+            mbar_init(&full[s], 1 + 32 * C::kLoad);
+            mbar_init(&xfree[s], 9);
+        }
+        for (uint32_t b = 0; b < NA; ++b) {
+            mbar_init(&afull[b], 8);
+            mbar_init(&aempty[b], 1);
+        }
+        for (int b = 0; b < C::kAcc; ++b) {
+            mbar_init(&accfull[b], 1);
+            mbar_init(&accempty[b], C::kEpi);
+        }
+        mbar_init(done, 1);
+        *abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot))
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        tc_fence_before();
+    }
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tbase = warp_uniform(*tmem_slot);
+    unsigned* flags = args.flags;
+    const uint32_t nk = args.nk, ksplit = args.ksplit;
+    // the K chunks [kc0, kc1) of item w
+    auto chunk0 = [&](uint32_t w) { return ksplit == 1 ? 0u : (uint32_t)((uint64_t)nk * (w % ksplit) / ksplit); };
+    auto chunk1 = [&](uint32_t w) { return ksplit == 1 ? nk : (uint32_t)((uint64_t)nk * (w % ksplit + 1) / ksplit); };
+
+    if (warp == 0) {
+        // ------------------------------------------------ TMA producer
+        if (elect_one()) {
+            uint32_t s = 0, ph = 1, issued = 0;
+            bool ok = true;
+            for (uint32_t w = blockIdx.x; w < args.nitems && ok; w += gridDim.x) {
+                const uint32_t w2 = ksplit == 1 ? w : w / ksplit;
+                const uint32_t t = args.nblk == 1 ? w2 : w2 / args.nblk, nb = args.nblk == 1 ? 0 : w2 % args.nblk;
+                const uint32_t kc1 = chunk1(w);
+                int rr = 0, l0 = 0;
+                if (!FLAT && !KMAJOR) {
+                    const uint32_t q = args.tiles_per_r == 1 ? t : t / args.tiles_per_r;
+                    rr = (int)(q * args.pack);
+                    l0 = (int)((t - q * args.tiles_per_r) * kRows);
+                }
+                for (uint32_t kc = chunk0(w); kc < kc1; ++kc) {
+                    if (!mbar_wait(&xfree[s], ph, abort, flags)) {
+                        ok = false;
+                        break;
+                    }
+                    uint8_t* xs = smem + s * C::kStage;
+                    uint8_t* bs = xs + kXBytes;
+                    mbar_expect_tx(&full[s], args.xbytes + 2 * C::kBBytes);
+                    if (!FLAT) {
+                        if (KMAJOR)
+                            tma_load_2d(xs, &tmX, (int)(kc * kChunk), (int)(t * kRows), &full[s]);
+                        else  // one unswizzled 128 x 32 box: rows i of 128 floats (512 B)
+                            tma_load_3d(xs, &tmX, l0, (int)(kc * kChunk), rr, &full[s]);
+                    }
+                    tma_load_2d(bs, &tmBhi, (int)(kc * kChunk), (int)(nb * NPAD), &full[s]);
+                    tma_load_2d(bs + C::kBBytes, &tmBlo, (int)(kc * kChunk), (int)(nb * NPAD), &full[s]);
+                    ++issued;
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1;
+                    }
+                }
+            }
+            // drain: every issued load has landed before the CTA can exit
+            const uint32_t n_out = issued < S ? issued : S;
+            for (uint32_t q = issued - n_out; q < issued; ++q) {
+                const uint64_t t0 = gtimer();
+                while (!mbar_try_wait(&full[q % S], (q / S) & 1) && gtimer() - t0 < kTimeoutNs) {
+                }
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ------------------------------------------------ MMA issuer
+        if (elect_one()) {
+            uint32_t s = 0, ph = 0, b = 0, bph = 0, a = 0, aph = 1;
+            bool ok = true;
+            for (uint32_t w = blockIdx.x; w < args.nitems && ok; w += gridDim.x) {
+                const uint32_t nc = chunk1(w) - chunk0(w);
+                uint32_t in = 0;  // chunks in the current accumulator
+                for (uint32_t kc = 0; kc < nc; ++kc) {
+                    if ((in == 0 && !mbar_wait(&accempty[a], aph, abort, flags)) ||
+                        !mbar_wait(&full[s], ph, abort, flags) || !mbar_wait(&afull[b], bph, abort, flags)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint64_t bdesc = desc_sw128(smem_u32(smem + s * C::kStage + kXBytes));
+                    const uint32_t a_hi = tbase + C::kABuf + 64 * b;
+                    const uint32_t d = tbase + a * (2 * NPAD);
+                    const uint32_t again = in ? 1u : 0u;
+#pragma unroll
+                    for (int k8 = 0; k8 < kChunk / 8; ++k8) {  // 8 K = 32 B along the swizzled row
+                        mma_tf32_ts(d, a_hi + 8 * k8, bdesc + 2 * k8, idesc_tf32(2 * NPAD), k8 ? 1u : again);
+                        mma_tf32_ts(d + NPAD, a_hi + 32 + 8 * k8, bdesc + 2 * k8, idesc_tf32(NPAD), 1u);
+                    }
+                    tc_commit(&aempty[b]);
+                    tc_commit(&xfree[s]);
+                    if (++s == S) {
+                        s = 0;
+                        ph ^= 1;
+                    }
+                    if (++b == NA) {
+                        b = 0;
+                        bph ^= 1;
+                    }
+                    if (++in == args.fill || kc + 1 == nc) {
+                        tc_commit(&accfull[a]);
+                        in = 0;
+                        if (++a == C::kAcc) {
+                            a = 0;
+                            aph ^= 1;
+                        }
+                    }
+                }
+            }
+            tc_commit(done);
+            const uint64_t t0 = gtimer();
+            while (!mbar_try_wait(done, 0) && gtimer() - t0 < kTimeoutNs) {
+            }
+        }
+        __syncwarp();
+    } else if (FLAT && warp >= 2 && warp < 2 + C::kLoad) {
+        // ------------------------------------------------ loaders: X chunks by cp.async
+        // Few instructions per cp.async: every lane keeps the pointers of its rows and steps them by a constant
+        // (a loader warp issues, not waits, for most of its time).
+        constexpr int kPart = kChunk / (C::kLoad ? C::kLoad : 1);    // K rows per warp and chunk (strided)
+        constexpr int kPartR = kRows / (C::kLoad ? C::kLoad : 1);    // tile rows per warp (L == 1)
+        const int lw = warp - 2;
+        const uint32_t rows = (uint32_t)(args.L * args.R), L = (uint32_t)args.L, nj = (uint32_t)args.nj;
+        const bool two = args.vec == 2;
+        uint32_t s = 0, ph = 1;
+        bool ok = true;
+        for (uint32_t w = blockIdx.x; w < args.nitems && ok; w += gridDim.x) {
+            const uint32_t w2 = ksplit == 1 ? w : w / ksplit;
+            const uint32_t t = args.nblk == 1 ? w2 : w2 / args.nblk;
+            const uint32_t kc0 = chunk0(w), kc1 = chunk1(w);
+            // strided: the lane's 4 rows lane + 32 q of the tile (8-byte: 2 row pairs 2 lane + 64 q), at
+            // K row kc0 * 32 + lw * kPart; L == 1: K element(s) k of row lw * kPartR (8-byte: + its half)
+            const float* src[4];
+            uint32_t vb[4];
+            if (!KMAJOR) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint32_t g = t * kRows + (two ? 2 * lane + 64 * q : lane + 32 * q);
+                    const uint32_t r = g / L;
+                    const bool in = g < rows && (!two || q < 2);
+                    vb[q] = in ? (two ? 8 : 4) : 0;
+                    src[q] = in ? args.X + (int64_t)(g - r * L) + args.L * (args.nj * r + kc0 * kChunk + lw * kPart)
+                                : args.X;
+                }
+            }
+            for (uint32_t kc = kc0; kc < kc1; ++kc) {
+                if (!__all_sync(0xffffffffu, mbar_wait(&xfree[s], ph, abort, flags))) {
+                    ok = false;
+                    break;
+                }
+                const uint32_t xs = smem_u32(smem + s * C::kStage);
+                if (!KMAJOR) {
+                    // rows i of 128 floats
+                    const uint32_t i0 = kc * kChunk + lw * kPart;
+                    const uint32_t dst = xs + (lw * kPart * kRows + (two ? 2 * lane : lane)) * 4;
+#pragma unroll
+                    for (int u = 0; u < kPart; ++u) {
+                        const bool in = i0 + u < nj;
+                        if (two) {
+#pragma unroll
+                            for (int q = 0; q < 2; ++q)
+                                cp_async<8>(dst + (u * kRows + 64 * q) * 4,
+                                            in && vb[q] ? src[q] + (int64_t)u * args.L : args.X, in ? vb[q] : 0);
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q)
+                                cp_async<4>(dst + (u * kRows + 32 * q) * 4,
+                                            in && vb[q] ? src[q] + (int64_t)u * args.L : args.X, in ? vb[q] : 0);
+                        }
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) src[q] += vb[q] ? args.L * kChunk : 0;
+                } else {
+                    // rows g of 128 B, the 16-byte chunk j of row rr stored at chunk j ^ (rr & 7)
+                    const uint32_t k = two ? (lane & 15) * 2 : lane, sub = two ? lane >> 4 : 0;
+                    const uint32_t i = kc * kChunk + k, g0 = t * kRows + lw * kPartR + sub;
+                    const float* p = args.X + (int64_t)nj * g0 + i;
+                    const uint32_t row0 = xs + (lw * kPartR + sub) * 128 + (k & 3) * 4;
+                    const bool kin = i < nj;
+                    if (two) {
+#pragma unroll
+                        for (int u = 0; u < kPartR / 2; ++u, p += 2 * args.nj) {
+                            const bool in = kin && g0 + 2 * u < rows;
+                            cp_async<8>(row0 + u * 256 + (((k >> 2) ^ ((2 * u + sub) & 7)) << 4), in ? p : args.X,
+                                        in ? 8 : 0);
+                        }
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < kPartR; ++u, p += args.nj) {
+                            const bool in = kin && g0 + u < rows;
+                            cp_async<4>(row0 + u * 128 + (((k >> 2) ^ (u & 7)) << 4), in ? p : args.X, in ? 4 : 0);
+                        }
+                    }
+                }
+                cp_async_arrive(&full[s]);
+                if (++s == S) {
+                    s = 0;
+                    ph ^= 1;
+                }
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");  // nothing in flight when the CTA exits
+    } else if (warp >= C::kFirstConv && warp < C::kFirstEpi) {
+        // ------------------------------------------------ converters: X chunk -> TF32 hi / lo in TMEM
+        // two groups of 8 warps, group g taking the even / odd chunks; within a group two warps per
+        // TMEM lane quarter, half hs converting K columns [16 hs, 16 hs + 16).
+        const int cw = warp - C::kFirstConv;
+        const int q = warp & 3, hs = (cw >> 2) & 1;
+        const uint32_t grp = cw >> 3;
+        const int rho = 32 * q + lane;  // tile row == TMEM lane
+        const uint32_t lane_base = (uint32_t)(32 * q) << 16;
+        const int Lp = (int)args.L;     // packed tiles only (L < 64)
+        const int pack = (int)args.pack;
+        const int xoff = pack > 1 ? (rho < Lp * pack ? (rho / Lp) * kChunk * Lp + rho % Lp : -1) : rho;
+        const int istride = pack > 1 ? Lp : kRows;
+        uint32_t s = 0, ph = 0, b = 0, bph = 1, it = 0;
+        bool ok = true;
+        for (uint32_t w = blockIdx.x; w < args.nitems && ok; w += gridDim.x) {
+            const uint32_t nc = chunk1(w) - chunk0(w);
+            for (uint32_t kc = 0; kc < nc; ++kc, ++it) {
+                if (C::kGroups == 1 || (it & 1) == grp) {
+                    if (!__all_sync(0xffffffffu, mbar_wait(&full[s], ph, abort, flags))) {
+                        ok = false;
+                        break;
+                    }
+                    const uint8_t* xs = smem + s * C::kStage;
+                    float v[16];
+                    if (KMAJOR) {
+                        // row rho: 128 B, 16-byte chunk j stored at chunk j ^ (rho & 7)
+                        const uint8_t* row = xs + rho * 128;
+#pragma unroll
+                        for (int jj = 0; jj < 4; ++jj) {
+                            const int j = 4 * hs + jj;
+                            const float4 f = *reinterpret_cast<const float4*>(row + ((j ^ (rho & 7)) << 4));
+                            v[4 * jj] = f.x;
+                            v[4 * jj + 1] = f.y;
+                            v[4 * jj + 2] = f.z;
+                            v[4 * jj + 3] = f.w;
+                        }
+                    } else {
+                        // rows i of 128 floats (512 B, no swizzle): lanes read consecutive words.  Packed
+                        // tiles hold [p][i][l] (p < pack, rows of L floats): tile row rho = l + L p; the
+                        // rows past L pack are padding (zero)
+                        const float* xf = reinterpret_cast<const float*>(xs);
+#pragma unroll
+                        for (int ii = 0; ii < 16; ++ii) {
+                            const int i = 16 * hs + ii;
+                            v[ii] = xoff >= 0 ? xf[xoff + i * istride] : 0.f;
+                        }
+                    }
+                    uint32_t hi[16], lo[16];
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) split_tf32(v[i], hi[i], lo[i]);
+                    if (!__all_sync(0xffffffffu, mbar_wait(&aempty[b], bph, abort, flags))) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t ta = tbase + lane_base + C::kABuf + 64 * b + 16 * hs;
+                    tmem_st16(ta, hi);
+                    tmem_st16(ta + 32, lo);
+                    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                    tc_fence_before();
+                    __syncwarp();  // the warp's TMEM stores and SMEM reads are ordered before lane 0's arrivals
+                    if (lane == 0) {
+                        mbar_arrive(&afull[b]);
+                        mbar_arrive(&xfree[s]);
+                    }
+                }
+                if (++s == S) {
+                    s = 0;
+                    ph ^= 1;
+                }
+                if (++b == NA) {
+                    b = 0;
+                    bph ^= 1;
+                }
+            }
+        }
+    } else if (warp >= C::kFirstEpi) {
+        // ------------------------------------------------ epilogue
+        // warp e drains TMEM lane quarter warp % 4 (the quarter a warp may access)
+        const int q = warp & 3, half = (warp - C::kFirstEpi) >> 2;
+        const int rho = 32 * q + lane;
+        const uint32_t lane_base = (uint32_t)(32 * q) << 16;
+        const int64_t m = args.m;
+        uint32_t a = 0, aph = 0;
+        for (uint32_t w = blockIdx.x; w < args.nitems; w += gridDim.x) {
+            const uint32_t w2 = ksplit == 1 ? w : w / ksplit, sk = w - w2 * ksplit;
+            const uint32_t t = args.nblk == 1 ? w2 : w2 / args.nblk, nb = args.nblk == 1 ? 0 : w2 % args.nblk;
+            const uint32_t nc = chunk1(w) - chunk0(w);
+            const uint32_t nfill = (nc + args.fill - 1) / args.fill;
+            float* const outp = ksplit > 1 ? args.part + sk * args.out_numel : args.out;
+            int64_t base, stride;
+            bool valid;
+            if (KMAJOR) {
+                const int64_t r = (int64_t)t * kRows + rho;
+                valid = r < args.R;
+                base = r * m;
+                stride = 1;
+            } else {
+                int64_t l, rr;
+                if (FLAT) {
+                    const uint32_t g = t * kRows + rho, L = (uint32_t)args.L, r = g / L;
+                    valid = g < (uint32_t)(args.L * args.R);
+                    l = g - r * L;
+                    rr = r;
+                } else if (args.pack > 1) {  // packed tile: row rho = l + L p holds (l, r = pack t + p)
+                    const int Lp = (int)args.L;
+                    rr = (int64_t)t * args.pack + rho / Lp;
+                    l = rho % Lp;
+                    valid = rho < Lp * (int)args.pack && rr < args.R;
+                } else {
+                    const uint32_t r = args.tiles_per_r == 1 ? t : t / args.tiles_per_r;
+                    rr = r;
+                    l = (int64_t)(t - r * args.tiles_per_r) * kRows + rho;
+                    valid = l < args.L;
+                }
+                base = l + args.L * m * rr;
+                stride = args.L;
+            }
+            const int col0 = (int)nb * NPAD;
+            base += col0 * stride;
+            const int ncol = (int)(m - col0);  // valid columns in this block (may exceed NPAD)
+            // the warp's 16-column slices half, half + 2, ...: each fill's small terms, then its large ones, in
+            // the order of the fills; the loads of a slice are in flight together
+            constexpr int kSl = (NPAD / 16 + 1) / 2;
+            float v[kSl][16];
+            bool ok = true;
+            for (uint32_t f = 0; f < nfill; ++f) {
+                if (!__all_sync(0xffffffffu, mbar_wait(&accfull[a], aph, abort, flags))) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t ta = tbase + lane_base + a * (2 * NPAD) + 16 * half;
+#pragma unroll
+                for (int j = 0; j < kSl; ++j) {
+                    if (16 * half + 32 * j >= NPAD) break;  // warp-uniform
+                    float h[16], g[16];
+                    __syncwarp();
+                    tmem_ld16(ta + 32 * j + NPAD, g);
+                    tmem_ld16(ta + 32 * j, h);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[j][i] = f ? v[j][i] + (h[i] + g[i]) : h[i] + g[i];
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&accempty[a]);
+                if (++a == C::kAcc) {
+                    a = 0;
+                    aph ^= 1;
+                }
+            }
+            if (!ok) break;
+            if (valid) {
+#pragma unroll
+                for (int j = 0; j < kSl; ++j) {
+                    const int c0 = 16 * half + 32 * j;
+                    if (c0 >= NPAD) break;
+                    if (KMAJOR && (m & 3) == 0) {  // 16-byte stores along the row
+#pragma unroll
+                        for (int i = 0; i < 16; i += 4)
+                            if (c0 + i < ncol)
+                                *reinterpret_cast<float4*>(outp + base + c0 + i) =
+                                    make_float4(v[j][i], v[j][i + 1], v[j][i + 2], v[j][i + 3]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (c0 + i < ncol) outp[base + (c0 + i) * stride] = v[j][i];
+                    }
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase) : "memory");
+    }
+}
+
+template <int NPAD, bool KMAJOR, bool FLAT>
+static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorMap& th, const CUtensorMap& tl,
+                            TtmArgs a) {
+    using Cf = TtmCfg<NPAD, FLAT>;
+    // FLAT: the SIMT kernels, the alternative for its shapes, round every addition to nearest, and its error
+    // has to stay at theirs (413 x 350 x 275: both 4e-7).  Above 64 columns a drain every 4 chunks would
+    // bound the pass (512^3, 81 columns: 174 against 121 us).
+    a.fill = FLAT ? 1 : (NPAD <= 64 ? 4 : 16);
+    auto kern = ttm_tf32x3_kernel<NPAD, KMAJOR, FLAT>;
+    static bool attr_set = false;
+    if (!attr_set) {
+        TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::kSmem));
+        attr_set = true;
+    }
+    const int grid = (int)std::min<int64_t>(a.nitems, grid_sms(c));
+    kern<<<grid, Cf::kThreads, Cf::kSmem, c.stream>>>(tx, th, tl, a);
+}
+
+// The kernel for npad output columns per block (a multiple of 16 up to 96).
+template <bool FLAT>
+static void ttm_tf32_dispatch(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& th,
+                              const CUtensorMap& tl, const TtmArgs& a) {
+#define TK_TC_CASE(NP)                                                           \
+    case NP:                                                                     \
+        if (kmajor) ttm_tf32_launch<NP, true, FLAT>(c, tx, th, tl, a);           \
+        else ttm_tf32_launch<NP, false, FLAT>(c, tx, th, tl, a);                 \
+        break;
+    switch (npad) {
+        TK_TC_CASE(16)
+        TK_TC_CASE(32)
+        TK_TC_CASE(48)
+        TK_TC_CASE(64)
+        TK_TC_CASE(80)
+        TK_TC_CASE(96)
+        default: fail(TK_ERR_SHAPE, "ttm_tc: unsupported width");
+    }
+#undef TK_TC_CASE
+}
+
+void ttm_tf32_run_tma(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& th,
+                      const CUtensorMap& tl, const TtmArgs& a);
+void ttm_tf32_run_flat(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& th,
+                       const CUtensorMap& tl, const TtmArgs& a);
+
+}  // namespace tc
+}  // namespace tk

@@ -1,0 +1,15 @@
+// Instantiations of the plain FP32 tensor-core TTM fed by TMA.
+#include <algorithm>
+
+#include "tk_ttm_tf32.cuh"
+
+namespace tk {
+namespace tc {
+
+void ttm_tf32_run_tma(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& th,
+                      const CUtensorMap& tl, const TtmArgs& a) {
+    ttm_tf32_dispatch<false>(c, npad, kmajor, tx, th, tl, a);
+}
+
+}  // namespace tc
+}  // namespace tk

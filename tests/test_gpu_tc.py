@@ -147,3 +147,35 @@ def test_tc_few_tiles_split_k(dev, dims, k):
     assert rel(to_np(G), ref) <= 1e-5
     G2 = T.tucker_core(X, mats(qs, "f32", dev))
     assert torch.equal(G, G2)  # the partial sums are added in a fixed order
+
+
+@pytest.mark.parametrize("dims,k", [
+    ((251, 97, 203), (251, 97, 50)),    # strided, odd slab (4-byte loads), K tail 203 = 6 chunks + 11
+    ((86, 161, 151), (86, 60, 151)),    # strided, L = 86: 8-byte loads, a tile holds rows of two slabs
+    ((203, 151, 97), (40, 151, 97)),    # contiguous mode of odd length (4-byte loads), ragged last tile
+    ((202, 151, 97), (49, 151, 97)),    # contiguous mode, 8-byte loads
+    ((7, 333, 401), (7, 40, 401)),      # rows of 7: 18 slabs per tile
+    ((501, 21, 700), (501, 20, 700)),   # fewer than 32 contracted (one partial chunk)
+    ((500, 21, 700), (500, 20, 700)),   # the same with 16-byte strides (TMA)
+    ((150, 141, 131), (150, 120, 131)),  # two blocks of output columns
+    ((9, 9, 5001), (9, 9, 100)),        # one row tile, K split over many CTAs
+    ((130, 129, 128), (90, 129, 128)),  # one element past 128: last tile of 2 x 64 rows, 90 columns
+])
+def test_tc_any_size_and_alignment(dev, dims, k):
+    # the loaders that take any L and n_j, and the short contractions, against the FP64 oracle.  Bound: the
+    # split drops x_lo M_lo and rounds each low part (2^-22 of a product in all), and each FP32 sum adds
+    # at most 2^-23 per addition of one chunk's products, 4 x 2^-23, and per chunk: below 2e-6
+    g = _rng(21)
+    X, xv, _ = make_X(g.standard_normal(dims), "f32", dev)
+    qs = [np.eye(n) if n == kk else synth.round_to(O.thin_qr(g.standard_normal((n, kk))), "f32")
+          for n, kk in zip(dims, k)]
+    mode = [j for j in range(3) if dims[j] != k[j]][0]
+    om = [synth.fmat(q, "f32", dev) for q in qs]
+    T.tk_profile(True, dev)
+    G = T.tucker_core(X, om)
+    prof = T.tk_profile_read(dev)
+    T.tk_profile(False, dev)
+    assert "xpass_tc" in prof
+    assert rel(to_np(G), O.ttm(xv, qs[mode].T, mode)) <= 2e-6
+    st, _ = T.tk_sync_status(dev)
+    assert st == 0

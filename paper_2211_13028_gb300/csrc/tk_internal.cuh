@@ -287,15 +287,15 @@ struct ProfScope {
 // out is dense column-major, dims of X with n_j -> m, dtype F64 or F32.
 void launch_ttm(const Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int64_t m, void* out, tk_dtype out_dt);
 
-// Tensor-core (tcgen05, 3xTF32) version of launch_ttm for FP32 data and output,
-// m <= 96; ttm_tc_eligible says whether a TTM qualifies (shape, dtype, alignment).
+// Tensor-core (tcgen05, 3xTF32) version of launch_ttm for FP32 data and output;
+// ttm_tc_eligible says whether a TTM takes it (dtype, and the sizes where it is faster).
 bool ttm_tc_eligible(const Tens& X, int j, int64_t m, tk_dtype out_dt);
-// A factor a tensor-core TTM will split (the contracted mode's size nj, output
-// width m; residual: the fused-residual blocking).
+// A factor a tensor-core TTM will split (the rows L before the contracted mode,
+// its size nj, output width m; residual: the fused-residual blocking).
 struct TcSplitReq {
     Mat M;
     bool mtrans;
-    int64_t nj, m;
+    int64_t L, nj, m;
     bool residual;
 };
 // Makes the splits of several factors in one launch and enters them in the
@@ -356,11 +356,11 @@ void launch_ttm_bf16(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, in
 // Fused last step of a reconstruction: P = W x_j M^T is formed tile by tile and
 // compared with xref (P's dims, F32): per-CTA partial sums of (xref - P)^2 and
 // xref^2 go to partials[2 * cta]; with dx != NULL also dx = alpha * (xref - P).
-// P itself is never stored.  tc_num_ctas gives the number of partial pairs.
+// P itself is never stored.  tc_residual_ctas gives the number of partial pairs.  j is W's last mode.
 // xref (F32, BF16, or FP8 for the norms only) is read as stored value * xr_scale.
 void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtrans, int64_t m, const void* xref,
                             tk_dtype xrdt, void* dx, float alpha, double* partials, float xr_scale = 1.f);
-int tc_num_ctas(const Ctx& c, const Tens& X, int j, int64_t m, bool residual);
+int tc_residual_ctas(const Ctx& c, const Tens& W, int j, int64_t m);
 bool ttm_tc_residual_eligible(const Tens& W, int j, int64_t m);
 // One warp waits with the tcgen05 kernels' bounded wait on an mbarrier that
 // nothing arrives at (limit_ns), which raises FLAG_TIMEOUT; *waited (device)

@@ -1,8 +1,8 @@
-// Host side of the FP32 tensor-core TTMs on sm_103a (kernels: tk_ttm_tf32.cuh, tk_tc_residual.cu): the
+// Host side of the FP32 tensor-core TTMs on sm_103a (kernels: tk_ttm_tf32.cuh, tk_expand_tf32.cu): the
 // TF32 split of the factors, the choice of tiles, tensor maps and launches.
 #include <algorithm>
 
-#include "tk_tc_residual.cuh"
+#include "tk_expand_tf32.cuh"
 #include "tk_ttm_tf32.cuh"
 
 namespace tk {
@@ -98,16 +98,24 @@ void launch_wait_selftest(const Ctx& c, uint64_t limit_ns, long long* waited) {
     c.check_launch();
 }
 
-// Output columns: up to 96 (64 for the residual epilogue, whose X tiles share
-// shared memory with the pipeline) in one block padded to 16, else blocks of 64.
-static void tc_blocks(int64_t m, int64_t& npad, int64_t& nblk, bool residual = false) {
-    if (m <= (residual ? 64 : 96)) {
-        npad = (m + 15) / 16 * 16;
-        nblk = 1;
-    } else {
-        npad = 64;
-        nblk = (m + 63) / 64;
+// How a product of contraction length nj and m output columns is blocked, which also fixes the layout of the
+// factor's split.  Expansions (a short contraction into many columns, every fused residual among them):
+// blocks of 32 or 64 columns (tk_expand_tf32.cu).  Plain ones take that kernel from twice as many columns
+// out as elements in (512^3, 32 -> 512: 103 us against 262), but not along the leading mode or with few
+// rows before it, where its rows of W are scattered (64^3 -> 1024 x 64 x 64: 77 us against 16).  Other products: up to 96
+// columns in one block padded to 16, else blocks of 64.
+struct Blocks {
+    int64_t npad, nblk;
+    bool expand;
+};
+
+static Blocks tc_blocks(int64_t L, int64_t nj, int64_t m, bool residual) {
+    if (residual || (L >= 32 && nj <= tc::kExpandK && m >= 64 && m >= 2 * nj)) {
+        const int64_t nb = tc::expand_cols(nj);
+        return {nb, (m + nb - 1) / nb, true};
     }
+    if (m <= 96) return {(m + 15) / 16 * 16, 1, false};
+    return {64, (m + 63) / 64, false};
 }
 
 // The factor splits that tensor-core TTMs about to run will need, made in one
@@ -118,9 +126,8 @@ void tc_presplit(Ctx& c, const std::vector<TcSplitReq>& reqs) {
     int nj_ = 0;
     int64_t most = 0;
     for (const TcSplitReq& q : reqs) {
-        int64_t npad, nblk;
-        tc_blocks(q.m, npad, nblk, q.residual);
-        const int64_t ldo = (q.nj + 3) / 4 * 4, rows_b = npad * nblk;
+        const Blocks bl = tc_blocks(q.L, q.nj, q.m, q.residual);
+        const int64_t npad = bl.npad, ldo = (q.nj + 3) / 4 * 4, rows_b = npad * bl.nblk;
         bool have = false;
         for (const Ctx::Split& e : c.splits)
             have = have || (e.p == q.M.p && e.dt == (int)q.M.dt && e.ld == q.M.ld && e.mtrans == (q.mtrans ? 1 : 0) &&
@@ -206,9 +213,10 @@ static Factor factor_alloc(Ctx& c, const Mat& M, bool mtrans, int64_t nj, int64_
     return f;
 }
 
-// Splits the factor unless it already is, and makes the tensor maps of its parts.
-static void factor_maps(Ctx& c, const Factor& f, const Mat& M, bool mtrans, int64_t nj, int64_t m, int64_t npad,
-                        CUtensorMap* th, CUtensorMap* tl) {
+// Splits the factor unless it already is, and makes the tensor map of its parts: hi and lo as the two layers of
+// one tensor (lo lies above hi in the workspace), so that one load brings both.
+static void factor_map(Ctx& c, const Factor& f, const Mat& M, bool mtrans, int64_t nj, int64_t m, int64_t npad,
+                       CUtensorMap* tb) {
     if (!f.have) {
         const int64_t tot = f.ldo * f.rows_b;
         ProfScope ps(c, "elementwise", 8.0 * tot + 8.0 * nj * m, 0.0);
@@ -217,11 +225,33 @@ static void factor_maps(Ctx& c, const Factor& f, const Mat& M, bool mtrans, int6
         c.counted();
         c.check_launch();
     }
-    const uint64_t dims[2] = {(uint64_t)nj, (uint64_t)f.rows_b};
-    const uint64_t str[1] = {(uint64_t)f.ldo * 4};
-    const uint32_t box[2] = {tc::kChunk, (uint32_t)npad};
-    tc::encode(th, f.hi, 2, dims, str, box);
-    tc::encode(tl, f.lo, 2, dims, str, box);
+    const uint64_t dims[3] = {(uint64_t)nj, (uint64_t)f.rows_b, 2};
+    const uint64_t str[2] = {(uint64_t)f.ldo * 4, (uint64_t)((char*)f.lo - (char*)f.hi)};
+    const uint32_t box[3] = {tc::kChunk, (uint32_t)npad, 2};
+    tc::encode(tb, f.hi, 3, dims, str, box);
+}
+
+// The expansion kernel's work: row tiles x parts of their column blocks (an item converts its tile of W
+// again, so parts are no finer than about 8 items an SM need).
+static tc::ExpandArgs expand_args(const Ctx& c, const Tens& W, int j, int64_t m, const Blocks& bl) {
+    tc::ExpandArgs a{};
+    a.L = W.left(j);
+    a.nj = W.n[j];
+    a.R = W.right(j);
+    a.m = m;
+    a.W = static_cast<const float*>(W.p);
+    const int64_t rows = a.L * a.R, tile = tc::expand_tile(a.nj), sms = tc::grid_sms(c);
+    a.rows = (uint32_t)rows;
+    const int64_t ntiles = (rows + tile - 1) / tile;
+    const int64_t ncs = std::max<int64_t>(1, std::min<int64_t>(bl.nblk, (8 * sms + ntiles - 1) / ntiles));
+    TK_REQUIRE(ntiles * ncs < ((int64_t)1 << 31), TK_ERR_SHAPE, "ttm_tc: too many tiles");
+    a.ntiles = (uint32_t)ntiles;
+    a.nblk = (uint32_t)bl.nblk;
+    a.ncs = (uint32_t)ncs;
+    a.nitems = (uint32_t)(ntiles * ncs);
+    a.nk = (uint32_t)((a.nj + tc::kChunk - 1) / tc::kChunk);
+    a.flags = c.dflags;
+    return a;
 }
 
 void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int64_t m, float* out) {
@@ -234,9 +264,22 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
     const TcRoute route = tc_route(X, j, m, TK_F32);
     TK_REQUIRE(route != TcRoute::None, TK_ERR_SHAPE, "ttm_tc: shape not supported");
     const bool flat = route == TcRoute::Flat, kmajor = (L == 1);
-    int64_t npad, nblk;
-    tc_blocks(m, npad, nblk);
+    const Blocks bl = tc_blocks(L, nj, m, false);
+    const int64_t npad = bl.npad, nblk = bl.nblk;
     const Factor f = factor_alloc(c, M, mtrans, nj, m, npad, nblk);
+    if (bl.expand && L * R < ((int64_t)1 << 31) - 256) {  // (more rows: the general kernel, same blocks)
+        if (!c.exec) return;
+        CUtensorMap tb;
+        factor_map(c, f, M, mtrans, nj, m, npad, &tb);
+        tc::ExpandArgs a = expand_args(c, X, j, m, bl);
+        a.out = out;
+        ProfScope ps(c, name, 4.0 * (double)L * R * nj + 8.0 * nj * m + 4.0 * (double)L * R * m,
+                     2.0 * (double)L * R * nj * m);
+        tc::expand_run(c, 0, TK_F32, tb, tb, a);
+        c.counted();
+        c.check_launch();
+        return;
+    }
     // the work items: 128-row tiles (TMA: a strided mode with under 64 rows before it packs several slabs
     // per tile) x blocks of NPAD output columns; too few of them for half the SMs split each tile's
     // K chunks over several items (at least two chunks each), whose partial products are summed in
@@ -255,10 +298,10 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
     TK_REQUIRE(ntiles * nblk * ksplit < ((int64_t)1 << 31), TK_ERR_SHAPE, "ttm_tc: too many tiles");
     float* part = ksplit > 1 ? c.alloc<float>(ksplit * L * m * R) : nullptr;
     if (!c.exec) return;
-    CUtensorMap tx, th, tl;
-    factor_maps(c, f, M, mtrans, nj, m, npad, &th, &tl);
+    CUtensorMap tx, tb;
+    factor_map(c, f, M, mtrans, nj, m, npad, &tb);
     if (flat) {
-        tx = th;  // unused
+        tx = tb;  // unused
     } else if (kmajor) {
         const uint64_t dims[2] = {(uint64_t)nj, (uint64_t)R};
         const uint64_t str[1] = {(uint64_t)nj * 4};
@@ -296,8 +339,8 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
     {
         ProfScope ps(c, name, 4.0 * (double)L * R * nj + 8.0 * nj * m + 4.0 * (double)L * R * m,
                      2.0 * (double)L * R * nj * m);
-        if (flat) tc::ttm_tf32_run_flat(c, npad, kmajor, tx, th, tl, a);
-        else tc::ttm_tf32_run_tma(c, npad, kmajor, tx, th, tl, a);
+        if (flat) tc::ttm_tf32_run_flat(c, npad, kmajor, tx, tb, a);
+        else tc::ttm_tf32_run_tma(c, npad, kmajor, tx, tb, a);
         c.counted();
         c.check_launch();
     }
@@ -310,67 +353,47 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
     }
 }
 
-int tc_num_ctas(const Ctx& c, const Tens& X, int j, int64_t m, bool residual) {
-    int64_t npad, nblk;
-    tc_blocks(m, npad, nblk, residual);
-    const int64_t L = X.left(j), R = X.right(j);
-    const int64_t tiles = (L == 1) ? (R + tc::kRows - 1) / tc::kRows : R * ((L + tc::kRows - 1) / tc::kRows);
-    return (int)std::min<int64_t>(tiles * nblk, tc::grid_sms(c));
+bool ttm_tc_residual_eligible(const Tens& W, int j, int64_t m) {
+    const int64_t rows = W.left(j), nj = W.n[j];
+    return W.dt == TK_F32 && W.right(j) == 1 && nj >= 1 && nj <= tc::kExpandKResid && m >= 1 && m <= 65535 &&
+           rows >= 1 && rows < ((int64_t)1 << 31) - 256 && ((uintptr_t)W.p % 16) == 0;
 }
 
-bool ttm_tc_residual_eligible(const Tens& W, int j, int64_t m) {
-    int64_t npad, nblk;
-    tc_blocks(m, npad, nblk, true);
-    // the residual X tile is a (128 rows x npad columns) TMA box: keep it inside the tensor
-    return W.n[j] >= 32 && W.left(j) >= tc::kRows && m >= npad && m <= 65535 && tma_ok(W, j);
+int tc_residual_ctas(const Ctx& c, const Tens& W, int j, int64_t m) {
+    return tc::expand_ctas(c, expand_args(c, W, j, m, tc_blocks(W.left(j), W.n[j], m, true)));
 }
 
 void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtrans, int64_t m, const void* xref,
                             tk_dtype xrdt, void* dx, float alpha, double* partials, float xr_scale) {
-    const int64_t L = W.left(j), nj = W.n[j], R = W.right(j);
-    TK_REQUIRE(L > 1, TK_ERR_SHAPE, "ttm_tc: the fused residual needs a non-leading mode");
+    const int64_t L = W.left(j), nj = W.n[j];
     TK_REQUIRE(xrdt == TK_F32 || xrdt == TK_BF16 || (xrdt == TK_FP8_E4M3 && !dx), TK_ERR_DTYPE,
                "ttm_tc: residual reference must be F32/BF16 (FP8: norms only)");
-    int64_t npad, nblk;
-    tc_blocks(m, npad, nblk, true);
-    const Factor f = factor_alloc(c, M, mtrans, nj, m, npad, nblk);
+    const Blocks bl = tc_blocks(L, nj, m, true);
+    const Factor f = factor_alloc(c, M, mtrans, nj, m, bl.npad, bl.nblk);
     if (!c.exec) return;
-    CUtensorMap tx, th, tl, txr;
-    factor_maps(c, f, M, mtrans, nj, m, npad, &th, &tl);
-    {
-        const uint64_t dims[3] = {(uint64_t)L, (uint64_t)nj, (uint64_t)R};
-        const uint64_t str[2] = {(uint64_t)L * 4, (uint64_t)L * nj * 4};
-        const uint32_t box[3] = {tc::kRows, tc::kChunk, 1};
-        tc::encode(&tx, W.p, 3, dims, str, box, false);
-    }
-    const uint64_t es = xrdt == TK_FP8_E4M3 ? 1 : (xrdt == TK_BF16 ? 2 : 4);
-    {
-        const uint64_t dims[3] = {(uint64_t)L, (uint64_t)m, (uint64_t)R};
-        const uint64_t str[2] = {(uint64_t)L * es, (uint64_t)L * m * es};
-        const uint32_t box[3] = {tc::kRows, (uint32_t)npad, 1};
-        tc::encode(&txr, xref, 3, dims, str, box, false,
+    CUtensorMap tb, txr;
+    factor_map(c, f, M, mtrans, nj, m, bl.npad, &tb);
+    const int64_t es = (int64_t)dtype_size(xrdt);
+    tc::ExpandArgs a = expand_args(c, W, j, m, bl);
+    a.bulk = (L * es) % 16 != 0;
+    a.xclip = (L * m * es) & ~(int64_t)15;
+    txr = tb;  // unused when bulk
+    if (!a.bulk) {
+        const uint64_t dims[2] = {(uint64_t)L, (uint64_t)m};
+        const uint64_t str[1] = {(uint64_t)(L * es)};
+        const uint32_t box[2] = {(uint32_t)tc::expand_tile(nj), (uint32_t)tc::expand_cols(nj)};
+        tc::encode(&txr, xref, 2, dims, str, box, false,
                    es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8
                            : (es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32));
     }
-    tc::ResidArgs a;
-    a.L = L;
-    a.nj = nj;
-    a.R = R;
-    a.m = m;
-    a.tiles_per_r = (L + tc::kRows - 1) / tc::kRows;
-    a.ntiles = R * a.tiles_per_r;
-    a.nk = (nj + tc::kChunk - 1) / tc::kChunk;
-    a.nblk = nblk;
     a.out = dx;
     a.xref = xref;
     a.alpha = alpha;
     a.xr_scale = xr_scale;
     a.partials = partials;
-    a.flags = c.dflags;
     ProfScope ps(c, c.background ? "xpass_tc_bg" : "xpass_tc",
-                 4.0 * (double)L * R * nj + 8.0 * nj * m + (dx ? 2.0 : 1.0) * es * (double)L * R * m,
-                 2.0 * (double)L * R * nj * m);
-    tc::ttm_residual_run(c, npad, xrdt, dx != nullptr, tx, th, tl, txr, a);
+                 4.0 * (double)L * nj + 8.0 * nj * m + (dx ? 2.0 : 1.0) * es * (double)L * m, 2.0 * (double)L * nj * m);
+    tc::expand_run(c, dx ? 2 : 1, xrdt, tb, txr, a);
     c.counted();
     c.check_launch();
 }

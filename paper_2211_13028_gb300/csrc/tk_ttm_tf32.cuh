@@ -140,8 +140,8 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
 
 template <int NPAD, bool KMAJOR, bool FLAT>
 __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
-    ttm_tf32x3_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmBhi,
-                      const __grid_constant__ CUtensorMap tmBlo, TtmArgs args) {
+    ttm_tf32x3_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmB,
+                      TtmArgs args) {
     using C = TtmCfg<NPAD, FLAT>;
     constexpr uint32_t S = C::kStages;
     constexpr uint32_t NA = C::kNA;
@@ -220,8 +220,7 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
                         else  // one unswizzled 128 x 32 box: rows i of 128 floats (512 B)
                             tma_load_3d(xs, &tmX, l0, (int)(kc * kChunk), rr, &full[s]);
                     }
-                    tma_load_2d(bs, &tmBhi, (int)(kc * kChunk), (int)(nb * NPAD), &full[s]);
-                    tma_load_2d(bs + C::kBBytes, &tmBlo, (int)(kc * kChunk), (int)(nb * NPAD), &full[s]);
+                    tma_load_3d(bs, &tmB, (int)(kc * kChunk), (int)(nb * NPAD), 0, &full[s]);  // M_hi, then M_lo
                     ++issued;
                     if (++s == S) {
                         s = 0;
@@ -557,8 +556,7 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
 }
 
 template <int NPAD, bool KMAJOR, bool FLAT>
-static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorMap& th, const CUtensorMap& tl,
-                            TtmArgs a) {
+static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorMap& tb, TtmArgs a) {
     using Cf = TtmCfg<NPAD, FLAT>;
     // FLAT: the SIMT kernels, the alternative for its shapes, round every addition to nearest, and its error
     // has to stay at theirs (413 x 350 x 275: both 4e-7).  Above 64 columns a drain every 4 chunks would
@@ -571,17 +569,17 @@ static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorM
         attr_set = true;
     }
     const int grid = (int)std::min<int64_t>(a.nitems, grid_sms(c));
-    kern<<<grid, Cf::kThreads, Cf::kSmem, c.stream>>>(tx, th, tl, a);
+    kern<<<grid, Cf::kThreads, Cf::kSmem, c.stream>>>(tx, tb, a);
 }
 
 // The kernel for npad output columns per block (a multiple of 16 up to 96).
 template <bool FLAT>
-static void ttm_tf32_dispatch(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& th,
-                              const CUtensorMap& tl, const TtmArgs& a) {
+static void ttm_tf32_dispatch(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& tb,
+                              const TtmArgs& a) {
 #define TK_TC_CASE(NP)                                                           \
     case NP:                                                                     \
-        if (kmajor) ttm_tf32_launch<NP, true, FLAT>(c, tx, th, tl, a);           \
-        else ttm_tf32_launch<NP, false, FLAT>(c, tx, th, tl, a);                 \
+        if (kmajor) ttm_tf32_launch<NP, true, FLAT>(c, tx, tb, a);               \
+        else ttm_tf32_launch<NP, false, FLAT>(c, tx, tb, a);                     \
         break;
     switch (npad) {
         TK_TC_CASE(16)
@@ -595,10 +593,10 @@ static void ttm_tf32_dispatch(const Ctx& c, int64_t npad, bool kmajor, const CUt
 #undef TK_TC_CASE
 }
 
-void ttm_tf32_run_tma(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& th,
-                      const CUtensorMap& tl, const TtmArgs& a);
-void ttm_tf32_run_flat(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& th,
-                       const CUtensorMap& tl, const TtmArgs& a);
+void ttm_tf32_run_tma(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& tb,
+                      const TtmArgs& a);
+void ttm_tf32_run_flat(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& tb,
+                       const TtmArgs& a);
 
 }  // namespace tc
 }  // namespace tk

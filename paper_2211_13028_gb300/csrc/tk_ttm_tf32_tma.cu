@@ -6,9 +6,9 @@
 namespace tk {
 namespace tc {
 
-void ttm_tf32_run_tma(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& th,
-                      const CUtensorMap& tl, const TtmArgs& a) {
-    ttm_tf32_dispatch<false>(c, npad, kmajor, tx, th, tl, a);
+void ttm_tf32_run_tma(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& tb,
+                      const TtmArgs& a) {
+    ttm_tf32_dispatch<false>(c, npad, kmajor, tx, tb, a);
 }
 
 }  // namespace tc

@@ -179,3 +179,54 @@ def test_tc_any_size_and_alignment(dev, dims, k):
     assert rel(to_np(G), O.ttm(xv, qs[mode].T, mode)) <= 2e-6
     st, _ = T.tk_sync_status(dev)
     assert st == 0
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "fp8"])
+@pytest.mark.parametrize("dims,rk", [
+    ((130, 7, 66), (9, 5, 33)),     # 910 rows: FP32 columns off 16 bytes; K = 33, two chunks; 66 = 2 x 32 + 2 columns
+    ((33, 31, 129), (8, 8, 20)),    # odd rows (every dtype off 16 bytes), one column in the last block
+    ((64, 48, 257), (8, 8, 64)),    # 16-byte columns in every dtype; K = 64
+    ((40, 37, 90), (6, 7, 90)),     # K = 90: three chunks, 128-row tiles
+    ((41, 37, 130), (5, 6, 128)),   # K = 128: four chunks, odd rows
+    ((3, 5, 40), (2, 3, 4)),        # fewer rows than 16 bytes hold
+    ((16, 16, 257), (4, 4, 5)),     # exactly one 256-row tile
+    ((257, 1, 32), (4, 1, 5)),      # one row in the second tile, one full block
+])
+def test_fused_residual_sizes_and_alignment(dev, dims, rk, dtype):
+    # the fused residual (loss, and dX where the dtype has one) at the edges of its tiles, blocks, chunks and
+    # of the copies of X's unaligned columns.  X - P is formed in FP32 from a product good to ~1e-6 of
+    # ||P||, and ||X - P|| ~ ||X|| here: 1e-5 of the loss and of dX (BF16 dX: its rounding, 2^-8)
+    g = _rng(23)
+    X, xv, sc = make_X(g.standard_normal(dims), dtype, dev)
+    G = synth.round_to(g.standard_normal(rk), "f32")
+    U = [synth.round_to(g.standard_normal((n, k)) / np.sqrt(n), "f32") for n, k in zip(dims, rk)]
+    Gd, Ud = synth.fortran(G, "f32", dev), mats(U, "f32", dev)
+    ref = O.loss(xv, G, U)
+    assert abs(T.tucker_loss(X, Gd, Ud, scale=sc) - ref) <= 1e-5 * ref
+    if dtype == "fp8":
+        return
+    norms = torch.zeros(2, dtype=torch.float64, device=dev)
+    _, _, dX = T.tucker_reconstruct_backward(X, Gd, Ud, 0.5, need_dG=False, need_dU=False, norms2=norms)
+    res = xv - O.reconstruct(G, U)
+    assert rel(to_np(dX.float() if dtype == "bf16" else dX), res) <= (1e-5 if dtype == "f32" else 2.0 ** -8)
+    assert abs(norms[0].item() - ref) <= 1e-5 * ref and abs(norms[1].item() - np.sum(xv ** 2)) <= 1e-5 * np.sum(xv ** 2)
+    st, _ = T.tk_sync_status(dev)
+    assert st == 0
+
+
+@pytest.mark.parametrize("dims,rk", [
+    ((201, 187, 211), (20, 24, 30)),  # odd rows, K = 30, last block of 19 columns
+    ((202, 188, 260), (20, 24, 60)),  # K = 60: two chunks
+    ((160, 130, 70, 40), (5, 6, 7, 8)),  # 4-way: the last expansion has slabs after it or none
+    ((300, 500, 256), (10, 20, 12)),  # mode 2 grows most: last, with the others before it
+])
+def test_reconstruct_expansions(dev, dims, rk):
+    # a reconstruction whose last products take the expansion kernel.  Bound as test_tc_any_size_and_alignment,
+    # once per product
+    g = _rng(24)
+    G = synth.round_to(g.standard_normal(rk), "f32")
+    U = [synth.round_to(g.standard_normal((n, k)) / np.sqrt(n), "f32") for n, k in zip(dims, rk)]
+    Xh = T.tucker_reconstruct(synth.fortran(G, "f32", dev), mats(U, "f32", dev))
+    assert rel(to_np(Xh), O.reconstruct(G, U)) <= len(dims) * 2e-6
+    st, _ = T.tk_sync_status(dev)
+    assert st == 0

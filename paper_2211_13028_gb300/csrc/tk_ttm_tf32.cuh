@@ -22,11 +22,12 @@
 // One MMA per 8-deep K step computes A_hi * [M_hi ; M_lo] (N = 2*NPAD, the two halves land in separate
 // TMEM columns); a second adds A_lo * M_hi into the second half, with the other small term.  The
 // tensor core's FP32 accumulation rounds each addition toward zero, a bias that grows with the number
-// of additions into one A_hi * M_hi sum.  So an accumulator takes the products of `fill` chunks only (1
-// for FLAT, else 4; 16 above 64 columns, whose registers the epilogue lacks), and the epilogue adds the fills of an item in FP32 registers, rounding to nearest,
+// of additions into one A_hi * M_hi sum.  So an accumulator takes the products of `fill` chunks only (4; 16
+// above 64 columns; half a chunk for FLAT, whose shapes the SIMT kernels took before, with every addition
+// rounded to nearest), and the epilogue adds the fills of an item in FP32 registers, rounding to nearest,
 // while the next ones are computed: TMEM holds a ring of as many accumulators as fit beside the A
-// buffers.  512^3, 42 columns: error against FP64 2.4e-6 with one
-// accumulator an item, 7.2e-7 so, for 100 -> 104 us.
+// buffers.  Errors against FP64: 512^3, 42 columns 2.4e-6 with one accumulator an item, 7.2e-7 so (100 ->
+// 104 us); 413 x 350 x 275, 36 columns 4.1e-7 with one chunk an accumulator, 3.6e-7 with half (SIMT 4.3e-7).
 //
 // FLAT = false: TMA.  Needs 16-byte strides (L % 4 == 0, or n_j % 4 == 0 for L == 1).  A strided mode
 // with fewer than 64 rows before it packs several slabs into each 128-row tile (pack).
@@ -92,7 +93,7 @@ struct TtmArgs {
     // few row tiles: the K chunks of a tile are split over ksplit work items, each writing its
     // partial product to part + s out_numel (summed in order by a second kernel); 1 otherwise
     uint32_t ksplit;
-    uint32_t fill;         // chunks per accumulator
+    uint32_t fill;         // chunks per accumulator (TMA)
     uint32_t vec;          // FLAT: floats per cp.async (1 or 2)
     const float* X;        // FLAT
     float* part;
@@ -246,7 +247,7 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
                 const uint32_t nc = chunk1(w) - chunk0(w);
                 uint32_t in = 0;  // chunks in the current accumulator
                 for (uint32_t kc = 0; kc < nc; ++kc) {
-                    if ((in == 0 && !mbar_wait(&accempty[a], aph, abort, flags)) ||
+                    if ((!FLAT && in == 0 && !mbar_wait(&accempty[a], aph, abort, flags)) ||
                         !mbar_wait(&full[s], ph, abort, flags) || !mbar_wait(&afull[b], bph, abort, flags)) {
                         ok = false;
                         break;
@@ -254,12 +255,34 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
                     tc_fence_after();
                     const uint64_t bdesc = desc_sw128(smem_u32(smem + s * C::kStage + kXBytes));
                     const uint32_t a_hi = tbase + C::kABuf + 64 * b;
-                    const uint32_t d = tbase + a * (2 * NPAD);
-                    const uint32_t again = in ? 1u : 0u;
+                    if (FLAT) {
+                        // half a chunk per accumulator
 #pragma unroll
-                    for (int k8 = 0; k8 < kChunk / 8; ++k8) {  // 8 K = 32 B along the swizzled row
-                        mma_tf32_ts(d, a_hi + 8 * k8, bdesc + 2 * k8, idesc_tf32(2 * NPAD), k8 ? 1u : again);
-                        mma_tf32_ts(d + NPAD, a_hi + 32 + 8 * k8, bdesc + 2 * k8, idesc_tf32(NPAD), 1u);
+                        for (int h = 0; h < 2; ++h) {
+                            ok = ok && mbar_wait(&accempty[a], aph, abort, flags);
+                            if (!ok) break;
+                            tc_fence_after();
+                            const uint32_t d = tbase + a * (2 * NPAD);
+#pragma unroll
+                            for (int k8 = 2 * h; k8 < 2 * h + 2; ++k8) {
+                                mma_tf32_ts(d, a_hi + 8 * k8, bdesc + 2 * k8, idesc_tf32(2 * NPAD), k8 & 1 ? 1u : 0u);
+                                mma_tf32_ts(d + NPAD, a_hi + 32 + 8 * k8, bdesc + 2 * k8, idesc_tf32(NPAD), 1u);
+                            }
+                            tc_commit(&accfull[a]);
+                            if (++a == C::kAcc) {
+                                a = 0;
+                                aph ^= 1;
+                            }
+                        }
+                        if (!ok) break;
+                    } else {
+                        const uint32_t d = tbase + a * (2 * NPAD);
+                        const uint32_t again = in ? 1u : 0u;
+#pragma unroll
+                        for (int k8 = 0; k8 < kChunk / 8; ++k8) {  // 8 K = 32 B along the swizzled row
+                            mma_tf32_ts(d, a_hi + 8 * k8, bdesc + 2 * k8, idesc_tf32(2 * NPAD), k8 ? 1u : again);
+                            mma_tf32_ts(d + NPAD, a_hi + 32 + 8 * k8, bdesc + 2 * k8, idesc_tf32(NPAD), 1u);
+                        }
                     }
                     tc_commit(&aempty[b]);
                     tc_commit(&xfree[s]);
@@ -271,7 +294,7 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
                         b = 0;
                         bph ^= 1;
                     }
-                    if (++in == args.fill || kc + 1 == nc) {
+                    if (!FLAT && (++in == args.fill || kc + 1 == nc)) {
                         tc_commit(&accfull[a]);
                         in = 0;
                         if (++a == C::kAcc) {
@@ -463,7 +486,7 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
             const uint32_t w2 = ksplit == 1 ? w : w / ksplit, sk = w - w2 * ksplit;
             const uint32_t t = args.nblk == 1 ? w2 : w2 / args.nblk, nb = args.nblk == 1 ? 0 : w2 % args.nblk;
             const uint32_t nc = chunk1(w) - chunk0(w);
-            const uint32_t nfill = (nc + args.fill - 1) / args.fill;
+            const uint32_t nfill = FLAT ? 2 * nc : (nc + args.fill - 1) / args.fill;
             float* const outp = ksplit > 1 ? args.part + sk * args.out_numel : args.out;
             int64_t base, stride;
             bool valid;
@@ -558,10 +581,8 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
 template <int NPAD, bool KMAJOR, bool FLAT>
 static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorMap& tb, TtmArgs a) {
     using Cf = TtmCfg<NPAD, FLAT>;
-    // FLAT: the SIMT kernels, the alternative for its shapes, round every addition to nearest, and its error
-    // has to stay at theirs (413 x 350 x 275: both 4e-7).  Above 64 columns a drain every 4 chunks would
-    // bound the pass (512^3, 81 columns: 174 against 121 us).
-    a.fill = FLAT ? 1 : (NPAD <= 64 ? 4 : 16);
+    // above 64 columns a drain every 4 chunks would bound the pass (512^3, 81 columns: 174 against 121 us)
+    a.fill = NPAD <= 64 ? 4 : 16;
     auto kern = ttm_tf32x3_kernel<NPAD, KMAJOR, FLAT>;
     static bool attr_set = false;
     if (!attr_set) {

@@ -41,8 +41,8 @@ def _peaks():
 
 
 KERNEL_NAMES = {
-    "xpass_tc": "ttm_tf32x3_kernel (tcgen05 3xTF32 TTM streaming X: sketch/core passes and the fused residual)",
-    "xpass_narrow": "ttm_fma_stream_kernel (TMA-fed FP32 FMA TTM streaming X: the narrow sketch passes)",
+    "xpass_tc": "ttm_tf32x3_kernel and expand_tf32x3_kernel (tcgen05 3xTF32: sketch and core passes, fused residual)",
+    "xpass_narrow": "srht_stream_kernel (TMA-fed FP32 FMA TTM of a Kronecker-SRHT sketch)",
     "ttm_tc": "ttm_tf32x3_kernel on intermediates",
 }
 # DRAM traffic / algorithmic bytes of one X-streaming launch, from an ncu capture of a 384^3 FP32

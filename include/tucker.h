@@ -136,7 +136,7 @@ TK_API tk_status tk_destroy(tk_handle* h);
 /* Rebind the handle to another stream. */
 TK_API tk_status tk_set_stream(tk_handle* h, void* cuda_stream);
 /* The persistent streaming kernels of this handle's calls (the passes over X
- * and the other tensor-core and narrow TTMs, one CTA per SM) leave `sms` SMs
+ * and the other tensor-core TTMs, one CTA per SM) leave `sms` SMs
  * free, so that kernels queued on other streams (another decomposition's
  * chains of small, latency-bound kernels) find SMs while a pass runs instead
  * of waiting for its end.  0 (default): every SM.  TK_ERR_ARG unless
@@ -178,7 +178,7 @@ TK_API int64_t tk_launch_count(const tk_handle* h);
  * classes; the filter persists until changed).  Class names ("xpass_*": a
  * pass over the whole data tensor): "xpass_tc", "xpass_tc_bg" (a tensor-core
  * pass on part of the SMs, beside a chain of small kernels of the same call),
- * "xpass_narrow", "xpass_simt", "ttm_tc", "ttm_narrow", "ttm_simt",
+ * "xpass_narrow" (the streaming pass of a Kronecker-SRHT sketch), "xpass_simt", "ttm_tc", "ttm_simt",
  * "gemm_f64", "gemm_df", "chol_inv", "apply_rinv", "householder", "jacobi",
  * "residual", "elementwise", "rng". */
 typedef struct {

@@ -156,16 +156,13 @@ static Tens ttm_to(Ctx& c, const Tens& T, int j, const Mat& M, bool mtrans, tk_d
     o.scale = 1.f;
     o.p = dst ? dst : c.alloc_bytes(dtype_size(acc) * o.numel());
     const bool aligned = reinterpret_cast<uintptr_t>(o.p) % 16 == 0;
-    const bool narrow = c.use_tc && ttm_narrow_eligible(T, j, m, acc) && aligned;
-    const bool tc = !narrow && c.use_tc && ttm_tc_eligible(T, j, m, acc);
-    const bool bf = !narrow && !tc && c.use_tc && ttm_bf16_eligible(T, j, m, acc);
-    const bool f8 = !narrow && !tc && !bf && c.use_tc && ttm_fp8_eligible(T, j, m, acc) && aligned;
-    // the tensor-core kernels split an FP64 factor themselves; the narrow and SIMT kernels of FP32-class
-    // data read FP32 factors
+    const bool tc = c.use_tc && ttm_tc_eligible(T, j, m, acc);
+    const bool bf = !tc && c.use_tc && ttm_bf16_eligible(T, j, m, acc);
+    const bool f8 = !tc && !bf && c.use_tc && ttm_fp8_eligible(T, j, m, acc) && aligned;
+    // the tensor-core kernels split an FP64 factor themselves; the SIMT kernels of FP32-class data read FP32
+    // factors
     const Mat Mu = (M.dt == TK_F64 && acc != TK_F64 && !(tc || bf || f8)) ? mat_to(c, M, acc) : M;
-    if (narrow)
-        launch_ttm_narrow(c, T, j, Mu, mtrans, m, static_cast<float*>(o.p));
-    else if (tc)
+    if (tc)
         launch_ttm_tc(c, T, j, Mu, mtrans, m, static_cast<float*>(o.p));
     else if (bf)
         launch_ttm_bf16(c, T, j, Mu, mtrans, m, static_cast<float*>(o.p));
@@ -179,7 +176,7 @@ static Tens ttm_to(Ctx& c, const Tens& T, int j, const Mat& M, bool mtrans, tk_d
 // Whether ttm_to takes a tensor-core kernel that splits the factor (tf32x3)
 // for this product (a workspace output, 16-byte aligned).
 static bool ttm_uses_tc(const Ctx& c, const Tens& T, int j, int64_t m, tk_dtype acc) {
-    return c.use_tc && !ttm_narrow_eligible(T, j, m, acc) && ttm_tc_eligible(T, j, m, acc);
+    return c.use_tc && ttm_tc_eligible(T, j, m, acc);
 }
 
 // The order multi_ttm applies the factors in: cheapest-shrinking mode first
@@ -1690,7 +1687,7 @@ tk_status tucker_rhkron_srht(tk_handle* h, const tk_tensor* X, const int64_t* r,
             if (k[n] < Xt.n[n]) need.push_back(n);
         }
         // 1. Y_n = X_(n) D_n (kron_{j != n} H_j): D_n is applied to X as it is streamed by the first
-        // product (the narrow FP32 kernel), else to a sign-flipped copy of X
+        // product (an FP32 streaming kernel), else to a sign-flipped copy of X
         std::vector<Tens> Y(d);
         void* flipped = nullptr;
         for (int n : need) {
@@ -1705,14 +1702,14 @@ tk_status tucker_rhkron_srht(tk_handle* h, const tk_tensor* X, const int64_t* r,
                 }
             }
             Tens T1;
-            if (c.use_tc && ttm_narrow_eligible(Xt, j0, s[j0], acc)) {
+            if (c.use_tc && srht_stream_eligible(Xt, j0, s[j0], acc)) {
                 T1 = Xt;
                 T1.n[j0] = s[j0];
                 T1.dt = acc;
                 T1.scale = 1.f;
                 T1.p = c.alloc_bytes(dtype_size(acc) * T1.numel());
                 const SignMap sm = sign_map(Xt, n, j0, seed);
-                launch_ttm_narrow(c, Xt, j0, Om[j0], false, s[j0], static_cast<float*>(T1.p), &sm);
+                launch_srht_stream(c, Xt, j0, Om[j0], false, s[j0], static_cast<float*>(T1.p), sm);
             } else {
                 if (!flipped) flipped = c.alloc_bytes(dtype_size(Xt.dt) * Xt.numel());
                 launch_sign_copy(c, Xt, n, seed, flipped);
@@ -1830,7 +1827,7 @@ tk_status tucker_rsthkron(tk_handle* h, const tk_tensor* X, const int64_t* r, in
                 qm.cols = k[j];
                 qm.ld = Xt.n[j];
                 // the tensor-core TTM splits an FP64 factor into TF32 parts itself: no FP32 copy needed
-                const bool tc64 = c.use_tc && !ttm_narrow_eligible(Gh, j, k[j], acc) && ttm_tc_eligible(Gh, j, k[j], acc);
+                const bool tc64 = c.use_tc && ttm_tc_eligible(Gh, j, k[j], acc);
                 Mat qa = (acc == TK_F64 || tc64) ? qm : mat_to(c, qm, acc);
                 Gh = ttm_to(c, Gh, j, qa, false, acc);
             } else {

@@ -1,12 +1,9 @@
-// Narrow TTMs that stream FP32 data: out = X x_j M^T with at most 8 output
-// columns (the widths of the Kronecker sketch factors).  At that width each
-// element needs at most 8 fused multiply-adds (one per column of M: the
-// kernel is instantiated for 5..8 computed columns), well inside the FP32 pipe at HBM rate,
-// so the data is streamed by TMA into a ring of shared-memory stages (as the
-// tensor-core kernels do; the registers of a plain SIMT kernel cannot keep
-// enough bytes in flight) and consumed by FP32 FMA warps, with M held in
-// shared memory for the whole pass.  FP32 accumulation, as in the tensor-core
-// path, whose tf32 instruction count at this width would bound the pass.
+// The first product of a Kronecker-SRHT sketch on FP32 data: out = (D_n o X) x_j M^T with at most 8 output
+// columns, the Rademacher signs of D_n applied to X as it is streamed (SignMap).  At that width each
+// element needs 8 fused multiply-adds and one hash, so the data is streamed by TMA into a ring of
+// shared-memory stages and consumed by FP32 FMA warps, with M held in shared memory for the whole pass.
+// FP32 accumulation.  (Products without signs take the tensor cores at every width: at 8 columns the
+// 512^3 sketch passes took 131 and 115 us here, 104 and 98 us there.)
 //
 // Work item: one tile of 128 rows (the same tiling and TMA boxes as the
 // tensor-core kernels).  Warp 0 issues the TMA loads; warps 1..8 consume, in
@@ -52,7 +49,7 @@ struct FsArgs {
     int mtrans;
     float* out;
     unsigned* flags;
-    SignMap sm;  // SIGN instantiations: the Rademacher diagonal applied on load
+    SignMap sm;  // the Rademacher diagonal applied on load
 };
 
 inline size_t fs_smem(int64_t nk) {
@@ -60,10 +57,10 @@ inline size_t fs_smem(int64_t nk) {
            sizeof(float) * (FS_PARTS - 1) * FS_ROWS * FS_COLS + sizeof(uint64_t) * (2 * FS_STAGES + 1);
 }
 
-// NC: the output columns computed (m <= NC <= FS_COLS; M is held zero-padded to FS_COLS columns).
-template <bool KMAJOR, bool SIGN, int NC>
+// M is held zero-padded to FS_COLS columns.
+template <bool KMAJOR>
 __global__ void __launch_bounds__(FS_THREADS, 1)
-    ttm_fma_stream_kernel(const __grid_constant__ CUtensorMap tmX, FsArgs args) {
+    srht_stream_kernel(const __grid_constant__ CUtensorMap tmX, FsArgs args) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int64_t nk = args.nk;
@@ -133,21 +130,19 @@ __global__ void __launch_bounds__(FS_THREADS, 1)
     const float4* m4 = reinterpret_cast<const float4*>(msm);
     int64_t it = 0;
     for (int64_t t = blockIdx.x; t < nitems; t += gridDim.x) {
-        float acc[4][NC];
+        float acc[4][FS_COLS];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int a = 0; a < NC; ++a) acc[u][a] = 0.f;
-        uint32_t c0[4];  // SIGN: unfolding column of (row, i = 0) for this item's four rows
-        if (SIGN) {
-            const SignMap& sm = args.sm;
-            const int64_t rr = KMAJOR ? 0 : t / args.tiles_per_r;
+            for (int a = 0; a < FS_COLS; ++a) acc[u][a] = 0.f;
+        uint32_t c0[4];  // unfolding column of (row, i = 0) for this item's four rows
+        const SignMap& sm = args.sm;
+        const int64_t rr0 = KMAJOR ? 0 : t / args.tiles_per_r;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t row = (KMAJOR ? t : t % args.tiles_per_r) * FS_ROWS + q + 32 * u;
-                c0[u] = (uint32_t)(sm.C1 * (row % sm.P1) + sm.P2 * (row / sm.P3) + sm.B1 * (rr % sm.Q1) +
-                                   sm.B2 * (rr / sm.Q2));
-            }
+        for (int u = 0; u < 4; ++u) {
+            const int64_t row = (KMAJOR ? t : t % args.tiles_per_r) * FS_ROWS + q + 32 * u;
+            c0[u] = (uint32_t)(sm.C1 * (row % sm.P1) + sm.P2 * (row / sm.P3) + sm.B1 * (rr0 % sm.Q1) +
+                               sm.B2 * (rr0 / sm.Q2));
         }
         for (int64_t kc = 0; kc < nk; ++kc, ++it) {
             if ((int)(it % FS_NGRP) != grp) continue;
@@ -182,24 +177,22 @@ __global__ void __launch_bounds__(FS_THREADS, 1)
                             for (int kk = 0; kk < 4; ++kk)
                                 v[u][kk] = reinterpret_cast<const float*>(xs)[(16 * kh + 4 * k4 + kk) * FS_ROWS + rho];
                         }
-                        if (SIGN) {
-                            const uint32_t i0 = (uint32_t)(kc * FS_CHUNK + 16 * kh + 4 * k4);
-                            const uint32_t A = (uint32_t)args.sm.A;
+                        const uint32_t i0 = (uint32_t)(kc * FS_CHUNK + 16 * kh + 4 * k4);
+                        const uint32_t A = (uint32_t)args.sm.A;
 #pragma unroll
-                            for (int kk = 0; kk < 4; ++kk)
-                                v[u][kk] = __uint_as_float(__float_as_uint(v[u][kk]) ^
-                                                           tk_rad_bits(args.sm.key, c0[u] + A * (i0 + kk)));
-                        }
+                        for (int kk = 0; kk < 4; ++kk)
+                            v[u][kk] = __uint_as_float(__float_as_uint(v[u][kk]) ^
+                                                       tk_rad_bits(args.sm.key, c0[u] + A * (i0 + kk)));
                     }
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
                         const float4 ma = mrow[2 * (4 * k4 + kk)];
-                        const float4 mb = NC > 4 ? mrow[2 * (4 * k4 + kk) + 1] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float4 mb = mrow[2 * (4 * k4 + kk) + 1];
                         const float mv[FS_COLS] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
 #pragma unroll
                         for (int u = 0; u < 4; ++u)
 #pragma unroll
-                            for (int a = 0; a < NC; ++a) acc[u][a] = fmaf(v[u][kk], mv[a], acc[u][a]);
+                            for (int a = 0; a < FS_COLS; ++a) acc[u][a] = fmaf(v[u][kk], mv[a], acc[u][a]);
                     }
                 }
             }
@@ -212,7 +205,7 @@ __global__ void __launch_bounds__(FS_THREADS, 1)
 #pragma unroll
             for (int u = 0; u < 4; ++u)
 #pragma unroll
-                for (int a = 0; a < NC; ++a) red[((part - 1) * FS_ROWS + q + 32 * u) * FS_COLS + a] = acc[u][a];
+                for (int a = 0; a < FS_COLS; ++a) red[((part - 1) * FS_ROWS + q + 32 * u) * FS_COLS + a] = acc[u][a];
         }
         asm volatile("bar.sync 1, %0;" ::"n"(32 * FS_CONS) : "memory");
         if (part == 0 && !*abort) {
@@ -235,7 +228,7 @@ __global__ void __launch_bounds__(FS_THREADS, 1)
                 }
                 if (valid) {
 #pragma unroll
-                    for (int a = 0; a < NC; ++a)
+                    for (int a = 0; a < FS_COLS; ++a)
                         if (a < args.m) {
                             float v = acc[u][a];
 #pragma unroll
@@ -251,7 +244,7 @@ __global__ void __launch_bounds__(FS_THREADS, 1)
 
 }  // namespace tc
 
-bool ttm_narrow_eligible(const Tens& X, int j, int64_t m, tk_dtype out_dt) {
+bool srht_stream_eligible(const Tens& X, int j, int64_t m, tk_dtype out_dt) {
     if (X.dt != TK_F32 || out_dt != TK_F32 || m < 1 || m > tc::FS_COLS) return false;
     const int64_t L = X.left(j), nj = X.n[j], R = X.right(j);
     if (nj < 1 || nj > tc::FS_MAX_NJ || L * nj * R < (1 << 22)) return false;  // small tensors: the general kernels
@@ -260,10 +253,10 @@ bool ttm_narrow_eligible(const Tens& X, int j, int64_t m, tk_dtype out_dt) {
     return L == 1 ? nj % 4 == 0 : L % 4 == 0;
 }
 
-void launch_ttm_narrow(const Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int64_t m, float* out,
-                       const SignMap* sm) {
+void launch_srht_stream(const Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int64_t m, float* out,
+                        const SignMap& sm) {
     if (!c.exec) return;
-    TK_REQUIRE(M.dt == TK_F32, TK_ERR_DTYPE, "narrow ttm: F32 matrix");
+    TK_REQUIRE(M.dt == TK_F32, TK_ERR_DTYPE, "srht stream: F32 matrix");
     const int64_t L = X.left(j), nj = X.n[j], R = X.right(j);
     const bool kmajor = (L == 1);
     CUtensorMap tx;
@@ -291,30 +284,15 @@ void launch_ttm_narrow(const Ctx& c, const Tens& X, int j, const Mat& M, bool mt
     a.mtrans = mtrans ? 1 : 0;
     a.out = out;
     a.flags = c.dflags;
-    if (sm) a.sm = *sm;
+    a.sm = sm;
     const size_t smem = tc::fs_smem(a.nk);
-    const char* name = (const void*)X.p == c.xdata ? "xpass_narrow" : "ttm_narrow";
-    ProfScope ps(c, name, 4.0 * (double)L * nj * R + 4.0 * (double)L * m * R + 4.0 * nj * m, 2.0 * L * nj * R * m);
+    ProfScope ps(c, "xpass_narrow", 4.0 * (double)L * nj * R + 4.0 * (double)L * m * R + 4.0 * nj * m, 2.0 * L * nj * R * m);
     const int grid = (int)std::min<int64_t>(a.ntiles, tc::grid_sms(c));
     auto run = [&](auto kern) {
         TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<grid, tc::FS_THREADS, smem, c.stream>>>(tx, a);
     };
-    // the FMAs of the output columns the factor has (5..8; the Kronecker-SRHT path always takes 8)
-    const int nc = sm ? 8 : (int)std::max<int64_t>(5, m);
-    if (sm) {
-        kmajor ? run(tc::ttm_fma_stream_kernel<true, true, 8>) : run(tc::ttm_fma_stream_kernel<false, true, 8>);
-    } else if (kmajor) {
-        nc == 5 ? run(tc::ttm_fma_stream_kernel<true, false, 5>)
-                : nc == 6 ? run(tc::ttm_fma_stream_kernel<true, false, 6>)
-                          : nc == 7 ? run(tc::ttm_fma_stream_kernel<true, false, 7>)
-                                    : run(tc::ttm_fma_stream_kernel<true, false, 8>);
-    } else {
-        nc == 5 ? run(tc::ttm_fma_stream_kernel<false, false, 5>)
-                : nc == 6 ? run(tc::ttm_fma_stream_kernel<false, false, 6>)
-                          : nc == 7 ? run(tc::ttm_fma_stream_kernel<false, false, 7>)
-                                    : run(tc::ttm_fma_stream_kernel<false, false, 8>);
-    }
+    kmajor ? run(tc::srht_stream_kernel<true>) : run(tc::srht_stream_kernel<false>);
     c.counted();
     c.check_launch();
 }

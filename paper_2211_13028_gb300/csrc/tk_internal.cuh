@@ -331,12 +331,11 @@ struct SignMap {
 };
 SignMap sign_map(const Tens& X, int n, int j0, uint64_t seed);
 
-// Narrow TTMs (m <= 8 output columns) on large FP32 data: a TMA-fed FP32 FMA
-// streaming kernel (the tensor-core kernels' tiling; tk_fma_stream.cu).
-bool ttm_narrow_eligible(const Tens& X, int j, int64_t m, tk_dtype out_dt);
-// With sm, X's elements are multiplied by the Rademacher signs of SignMap first.
-void launch_ttm_narrow(const Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int64_t m, float* out,
-                       const SignMap* sm = nullptr);
+// First product of a Kronecker-SRHT sketch (m <= 8 output columns) on large FP32 data: X's elements times
+// the Rademacher signs of SignMap, streamed by TMA into FP32 FMA warps (tk_fma_stream.cu).
+bool srht_stream_eligible(const Tens& X, int j, int64_t m, tk_dtype out_dt);
+void launch_srht_stream(const Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int64_t m, float* out,
+                        const SignMap& sm);
 // dst = D_n o X (X's dtype and layout): every element times its SRHT sign.
 void launch_sign_copy(const Ctx& c, const Tens& X, int n, uint64_t seed, void* dst);
 

@@ -175,6 +175,8 @@ static TcRoute tc_route(const Tens& X, int j, int64_t m, tk_dtype out_dt) {
     if (nj < 1 || ((uintptr_t)X.p % 16) != 0 || nj >= ((int64_t)1 << 31)) return TcRoute::None;
     const int64_t rows = L * R;
     if (rows < 1 || rows >= ((int64_t)1 << 31) - tc::kRows) return TcRoute::None;
+    // streams of 4 million elements and more with 16-byte strides: HBM-bound at 2-3 times the SIMT rate
+    if (rows * nj >= ((int64_t)1 << 22) && tma_ok(X, j)) return tma ? TcRoute::Tma : TcRoute::Flat;
     const double bytes = 4.0 * (double)rows * (double)(nj + m);
     const double simt = std::max({0.1 * (double)nj, (double)rows * (double)nj * (double)m / 2.3e6, bytes / 1.2e6});
     if (simt < 28.0 + bytes / 3e6) return TcRoute::None;

@@ -22,8 +22,8 @@
 // One MMA per 8-deep K step computes A_hi * [M_hi ; M_lo] (N = 2*NPAD, the two halves land in separate
 // TMEM columns); a second adds A_lo * M_hi into the second half, with the other small term.  The
 // tensor core's FP32 accumulation rounds each addition toward zero, a bias that grows with the number
-// of additions into one A_hi * M_hi sum.  So an accumulator takes the products of `fill` chunks only (4; 16
-// above 64 columns; half a chunk for FLAT, whose shapes the SIMT kernels took before, with every addition
+// of additions into one A_hi * M_hi sum.  So an accumulator takes the products of `fill` chunks only (1 up
+// to 8 columns, 4 up to 64, 16 above; half a chunk for FLAT, whose shapes the SIMT kernels took before, with every addition
 // rounded to nearest), and the epilogue adds the fills of an item in FP32 registers, rounding to nearest,
 // while the next ones are computed: TMEM holds a ring of as many accumulators as fit beside the A
 // buffers.  Errors against FP64: 512^3, 42 columns 2.4e-6 with one accumulator an item, 7.2e-7 so (100 ->
@@ -581,8 +581,11 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
 template <int NPAD, bool KMAJOR, bool FLAT>
 static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorMap& tb, TtmArgs a) {
     using Cf = TtmCfg<NPAD, FLAT>;
-    // above 64 columns a drain every 4 chunks would bound the pass (512^3, 81 columns: 174 against 121 us)
-    a.fill = NPAD <= 64 ? 4 : 16;
+    // above 64 columns a drain every 4 chunks would bound the pass (512^3, 81 columns: 174 against 121 us);
+    // up to 8, the sketch widths, every chunk is drained: the FP32 FMA kernel that streamed those before
+    // rounds every addition to nearest (512^3 sketches: 2.4e-7, FMA 3.3e-7, 5.8e-7 with 4 chunks; 104 and
+    // 98 us a pass, FMA 131 and 115, 94 and 90 with 4)
+    a.fill = a.m <= 8 ? 1 : (NPAD <= 64 ? 4 : 16);
     auto kern = ttm_tf32x3_kernel<NPAD, KMAJOR, FLAT>;
     static bool attr_set = false;
     if (!attr_set) {

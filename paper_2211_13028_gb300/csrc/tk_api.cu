@@ -180,9 +180,9 @@ static bool ttm_uses_tc(const Ctx& c, const Tens& T, int j, int64_t m, tk_dtype 
 }
 
 // The order multi_ttm applies the factors in: cheapest-shrinking mode first
-// (smallest output; ties: the higher mode); FP8 data streams through the
-// tensor cores only along its contiguous mode, so that one goes first (the
-// later products then read the much smaller FP32 intermediate).
+// (smallest output; ties: the higher mode); FP8 data goes
+// along its contiguous mode first, where the kernel that multiplies it as it is streams
+// 6 TB/s (768^3, 9 columns: 76 us, 178 along another mode).
 static std::vector<int> mtt_order(const Ctx& c, const Tens& T, std::vector<int> modes, const Mat* M, bool mtrans,
                                   tk_dtype acc) {
     std::vector<int> order;
@@ -227,7 +227,7 @@ static Tens multi_ttm(Ctx& c, const Tens& T, std::vector<int> modes, const Mat* 
         Tens sh = T;
         for (int i : order) {
             const int64_t m = mtrans ? M[i].rows : M[i].cols;
-            if (ttm_uses_tc(c, sh, i, m, acc)) reqs.push_back({M[i], mtrans, sh.left(i), sh.n[i], m, false});
+            if (ttm_uses_tc(c, sh, i, m, acc)) reqs.push_back({M[i], mtrans, sh.left(i), sh.n[i], m, false, sh.dt});
             sh.n[i] = m;
             sh.dt = acc;
             sh.p = reinterpret_cast<void*>(uintptr_t(256));  // a workspace block: 256-byte aligned
@@ -608,12 +608,12 @@ static void residual_pass(Ctx& c, const Tens& X, const Tens& G, const std::vecto
     if (c.use_tc && acc == TK_F32) {
         Tens sh = G;
         for (int i : order) {
-            if (ttm_uses_tc(c, sh, i, U[i].rows, acc)) reqs.push_back({U[i], true, sh.left(i), sh.n[i], U[i].rows, false});
+            if (ttm_uses_tc(c, sh, i, U[i].rows, acc)) reqs.push_back({U[i], true, sh.left(i), sh.n[i], U[i].rows, false, sh.dt});
             sh.n[i] = U[i].rows;
             sh.dt = acc;
             sh.p = reinterpret_cast<void*>(uintptr_t(256));
         }
-        if (fused) reqs.push_back({U[f], true, Ws.left(f), Ws.n[f], m, true});
+        if (fused) reqs.push_back({U[f], true, Ws.left(f), Ws.n[f], m, true, TK_F32});
         if (reqs.size() >= 2) tc_presplit(c, reqs);
     }
     struct CacheOn {

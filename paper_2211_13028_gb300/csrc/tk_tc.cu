@@ -1,8 +1,9 @@
-// Host side of the FP32 tensor-core TTMs on sm_103a (kernels: tk_ttm_tf32.cuh, tk_expand_tf32.cu): the
+// Host side of the TF32 tensor-core TTMs on sm_103a (kernels: tk_ttm_tf32.cuh, tk_ttm_lowp.cuh, tk_expand_tf32.cu): the
 // TF32 split of the factors, the choice of tiles, tensor maps and launches.
 #include <algorithm>
 
 #include "tk_expand_tf32.cuh"
+#include "tk_ttm_lowp.cuh"
 #include "tk_ttm_tf32.cuh"
 
 namespace tk {
@@ -103,13 +104,18 @@ void launch_wait_selftest(const Ctx& c, uint64_t limit_ns, long long* waited) {
 // blocks of 32 or 64 columns (tk_expand_tf32.cu).  Plain ones take that kernel from twice as many columns
 // out as elements in (512^3, 32 -> 512: 103 us against 262), but not along the leading mode or with few
 // rows before it, where its rows of W are scattered (64^3 -> 1024 x 64 x 64: 77 us against 16).  Other products: up to 96
-// columns in one block padded to 16, else blocks of 64.
+// columns in one block padded to 16, else blocks of 64.  BF16 and FP8 data (tk_ttm_lowp.cuh, stages of 64 K):
+// equal blocks of up to 64.
 struct Blocks {
     int64_t npad, nblk;
     bool expand;
 };
 
-static Blocks tc_blocks(int64_t L, int64_t nj, int64_t m, bool residual) {
+static Blocks tc_blocks(int64_t L, int64_t nj, int64_t m, bool residual, tk_dtype dt) {
+    if (dt != TK_F32) {
+        const int64_t nb = (m + 63) / 64;
+        return {((m + nb - 1) / nb + 15) / 16 * 16, nb, false};
+    }
     if (residual || (L >= 32 && nj <= tc::kExpandK && m >= 64 && m >= 2 * nj)) {
         const int64_t nb = tc::expand_cols(nj);
         return {nb, (m + nb - 1) / nb, true};
@@ -126,7 +132,7 @@ void tc_presplit(Ctx& c, const std::vector<TcSplitReq>& reqs) {
     int nj_ = 0;
     int64_t most = 0;
     for (const TcSplitReq& q : reqs) {
-        const Blocks bl = tc_blocks(q.L, q.nj, q.m, q.residual);
+        const Blocks bl = tc_blocks(q.L, q.nj, q.m, q.residual, q.dt);
         const int64_t npad = bl.npad, ldo = (q.nj + 3) / 4 * 4, rows_b = npad * bl.nblk;
         bool have = false;
         for (const Ctx::Split& e : c.splits)
@@ -155,7 +161,7 @@ static bool tma_ok(const Tens& X, int j) {
     return L == 1 ? nj % 4 == 0 : L % 4 == 0;
 }
 
-enum class TcRoute { None, Tma, Flat };
+enum class TcRoute { None, Tma, Flat, Lowp };
 
 // Which form of the tensor-core kernel takes a TTM.
 //  * TMA: 16-byte strides, n_j >= 32, and rows enough to fill tiles: L == 1 with R >= 128, or L >= 32 (below
@@ -166,9 +172,24 @@ enum class TcRoute { None, Tma, Flat };
 //    1.2 TB/s; the tensor cores need two launches (14 us with the split of the factor, and as much again
 //    on the host, which is what calls on small tensors wait for) and stream 3 TB/s.
 //    E.g. 413 x 350 x 275 along its last mode, 36 columns: 1337 us SIMT; 9001 x 333, 20: 78.
+//  * BF16 and FP8 that their own kernels do not take: the same rule, for L == 1 or L >= 32 (shorter runs
+//    cost more in their 16-byte pieces than they hold).  E.g. BF16 689 x 690 x 700 along its first mode, 10 columns:
+//    3435 us SIMT, 180; FP8 768^3 along its last, 9: 1541 and 178.
+static TcRoute lowp_route(const Tens& X, int j, int64_t m) {
+    const int64_t L = X.left(j), nj = X.n[j], R = X.right(j), es = (int64_t)dtype_size(X.dt);
+    if (ttm_bf16_eligible(X, j, m, TK_F32) || ttm_fp8_eligible(X, j, m, TK_F32)) return TcRoute::None;
+    if (nj < 1 || ((uintptr_t)X.p % 16) != 0 || nj >= ((int64_t)1 << 31) || (L != 1 && L < 32)) return TcRoute::None;
+    const int64_t rows = L * R;
+    if (rows < 1 || rows >= ((int64_t)1 << 31) - tc::kRows) return TcRoute::None;
+    const double bytes = (double)rows * (double)(es * nj + 4 * m);
+    const double simt = std::max({0.1 * (double)nj, (double)rows * (double)nj * (double)m / 2.3e6, bytes / 1.2e6});
+    return simt < 28.0 + bytes / 3e6 ? TcRoute::None : TcRoute::Lowp;
+}
+
 static TcRoute tc_route(const Tens& X, int j, int64_t m, tk_dtype out_dt) {
-    if (X.dt != TK_F32 || out_dt != TK_F32) return TcRoute::None;
+    if (out_dt != TK_F32 || X.dt == TK_F64) return TcRoute::None;
     if (m < 1 || m > 65535) return TcRoute::None;
+    if (X.dt != TK_F32) return lowp_route(X, j, m);
     const int64_t L = X.left(j), nj = X.n[j], R = X.right(j);
     const bool tma = tma_ok(X, j) && (L == 1 ? R >= tc::kRows : L >= 32);
     if (nj >= 32 && tma) return TcRoute::Tma;
@@ -256,6 +277,82 @@ static tc::ExpandArgs expand_args(const Ctx& c, const Tens& W, int j, int64_t m,
     return a;
 }
 
+// Few row tiles: the K chunks of each are split over several items, at least two chunks each.
+static int64_t split_chunks(const Ctx& c, int64_t items, int64_t nk) {
+    const int64_t sms = tc::grid_sms(c);
+    return items * 2 <= sms && nk >= 4 ? std::max<int64_t>(1, std::min<int64_t>(nk / 2, sms / items)) : 1;
+}
+
+static void sum_parts(Ctx& c, const float* part, int64_t ksplit, int64_t n, float* out) {
+    tc::splitk_sum_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, c.stream>>>(part, (int)ksplit,
+                                                                                                 n, out);
+    c.counted();
+    c.check_launch();
+}
+
+// BF16 / FP8 data (tk_ttm_lowp.cuh).  TMA where the strides are multiples of 16 bytes and a mode is before the
+// contracted one, else the loaders, whose runs (a K row of the tile; with L == 1 a row's 64 elements) begin anywhere.
+static void launch_ttm_lowp(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int64_t m, float* out,
+                            const char* name) {
+    const int64_t L = X.left(j), nj = X.n[j], R = X.right(j), es = (int64_t)dtype_size(X.dt);
+    const bool kmajor = L == 1;
+    const Blocks bl = tc_blocks(L, nj, m, false, X.dt);
+    const Factor f = factor_alloc(c, M, mtrans, nj, m, bl.npad, bl.nblk);
+    const int64_t pack = !kmajor && L < tc::kRows / 2 ? tc::kRows / L : 1;
+    const int64_t nk = (nj + tc::kLowpChunk - 1) / tc::kLowpChunk;
+    const int64_t tiles_per_r = kmajor || pack > 1 ? 1 : (L + tc::kRows - 1) / tc::kRows;
+    const int64_t ntiles = kmajor ? (R + tc::kRows - 1) / tc::kRows : (pack > 1 ? (R + pack - 1) / pack : R * tiles_per_r);
+    const int64_t ksplit = split_chunks(c, ntiles * bl.nblk, nk);
+    TK_REQUIRE(ntiles * bl.nblk * ksplit < ((int64_t)1 << 31), TK_ERR_SHAPE, "ttm_lowp: too many tiles");
+    float* part = ksplit > 1 ? c.alloc<float>(ksplit * L * m * R) : nullptr;
+    if (!c.exec) return;
+    const bool tma = !kmajor && (L * es) % 16 == 0;
+    const int64_t run = es * (pack > 1 ? L : tc::kRows);  // bytes of a tile's K row in one slab
+    CUtensorMap tx, tb;
+    factor_map(c, f, M, mtrans, nj, m, bl.npad, &tb);
+    tx = tb;  // unused by the loaders
+    if (tma) {
+        const uint64_t dims[3] = {(uint64_t)L, (uint64_t)nj, (uint64_t)R};
+        const uint64_t str[2] = {(uint64_t)(L * es), (uint64_t)(L * nj * es)};
+        const uint32_t box[3] = {(uint32_t)(pack > 1 ? L : tc::kRows), tc::kLowpChunk, (uint32_t)pack};
+        tc::encode(&tx, X.p, 3, dims, str, box, false,
+                   es == 1 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
+    }
+    tc::LowpArgs a{};
+    a.L = L;
+    a.nj = nj;
+    a.R = R;
+    a.m = m;
+    a.ntiles = (uint32_t)ntiles;
+    a.tiles_per_r = (uint32_t)tiles_per_r;
+    a.nk = (uint32_t)nk;
+    a.nblk = (uint32_t)bl.nblk;
+    a.nitems = (uint32_t)(ntiles * bl.nblk * ksplit);
+    a.pack = (uint32_t)pack;
+    a.ksplit = (uint32_t)ksplit;
+    // a run that starts anywhere spans up to 15 bytes more than it has
+    a.slot = (uint32_t)(tma ? run : (kmajor ? tc::kLowpChunk * es + 16 : (run + 15 + 15) / 16 * 16));
+    const uint32_t runs = (uint32_t)(kmajor ? tc::kRows : tc::kLowpChunk * pack);
+    a.xstage = (runs * a.slot + 1023) / 1024 * 1024;
+    a.tma = tma ? 1 : 0;
+    a.xbytes = tma ? runs * a.slot : 0;
+    a.x_inv = X.dt == TK_FP8_E4M3 ? 1.f / X.scale : 1.f;
+    a.X = static_cast<const uint8_t*>(X.p);
+    a.part = part;
+    a.out_numel = L * m * R;
+    a.out = out;
+    a.flags = c.dflags;
+    {
+        ProfScope ps(c, name, (double)es * L * R * nj + 8.0 * nj * m + 4.0 * (double)L * R * m,
+                     2.0 * (double)L * R * nj * m);
+        if (es == 1) tc::ttm_lowp_run_fp8(c, bl.npad, kmajor, tx, tb, a);
+        else tc::ttm_lowp_run_bf16(c, bl.npad, kmajor, tx, tb, a);
+        c.counted();
+        c.check_launch();
+    }
+    if (ksplit > 1) sum_parts(c, part, ksplit, L * m * R, out);
+}
+
 void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int64_t m, float* out) {
     const int64_t L = X.left(j), R = X.right(j);
     // kernel classes: "xpass_tc" streams all of X (a pass over the input),
@@ -265,8 +362,12 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
     const int64_t nj = X.n[j];
     const TcRoute route = tc_route(X, j, m, TK_F32);
     TK_REQUIRE(route != TcRoute::None, TK_ERR_SHAPE, "ttm_tc: shape not supported");
+    if (route == TcRoute::Lowp) {
+        launch_ttm_lowp(c, X, j, M, mtrans, m, out, name);
+        return;
+    }
     const bool flat = route == TcRoute::Flat, kmajor = (L == 1);
-    const Blocks bl = tc_blocks(L, nj, m, false);
+    const Blocks bl = tc_blocks(L, nj, m, false, TK_F32);
     const int64_t npad = bl.npad, nblk = bl.nblk;
     const Factor f = factor_alloc(c, M, mtrans, nj, m, npad, nblk);
     if (bl.expand && L * R < ((int64_t)1 << 31) - 256) {  // (more rows: the general kernel, same blocks)
@@ -292,11 +393,7 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
     const int64_t ntiles = flat ? (L * R + tc::kRows - 1) / tc::kRows
                                 : (kmajor ? (R + tc::kRows - 1) / tc::kRows
                                           : (pack > 1 ? (R + pack - 1) / pack : R * tiles_per_r));
-    int64_t ksplit = 1;
-    {
-        const int64_t items = ntiles * nblk, sms = tc::grid_sms(c);
-        if (items * 2 <= sms && nk >= 4) ksplit = std::max<int64_t>(1, std::min<int64_t>(nk / 2, sms / items));
-    }
+    const int64_t ksplit = split_chunks(c, ntiles * nblk, nk);
     TK_REQUIRE(ntiles * nblk * ksplit < ((int64_t)1 << 31), TK_ERR_SHAPE, "ttm_tc: too many tiles");
     float* part = ksplit > 1 ? c.alloc<float>(ksplit * L * m * R) : nullptr;
     if (!c.exec) return;
@@ -346,13 +443,7 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
         c.counted();
         c.check_launch();
     }
-    if (ksplit > 1) {
-        const int64_t n = L * m * R;
-        tc::splitk_sum_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, c.stream>>>(
-            part, (int)ksplit, n, out);
-        c.counted();
-        c.check_launch();
-    }
+    if (ksplit > 1) sum_parts(c, part, ksplit, L * m * R, out);
 }
 
 bool ttm_tc_residual_eligible(const Tens& W, int j, int64_t m) {
@@ -362,7 +453,7 @@ bool ttm_tc_residual_eligible(const Tens& W, int j, int64_t m) {
 }
 
 int tc_residual_ctas(const Ctx& c, const Tens& W, int j, int64_t m) {
-    return tc::expand_ctas(c, expand_args(c, W, j, m, tc_blocks(W.left(j), W.n[j], m, true)));
+    return tc::expand_ctas(c, expand_args(c, W, j, m, tc_blocks(W.left(j), W.n[j], m, true, TK_F32)));
 }
 
 void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtrans, int64_t m, const void* xref,
@@ -370,7 +461,7 @@ void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtr
     const int64_t L = W.left(j), nj = W.n[j];
     TK_REQUIRE(xrdt == TK_F32 || xrdt == TK_BF16 || (xrdt == TK_FP8_E4M3 && !dx), TK_ERR_DTYPE,
                "ttm_tc: residual reference must be F32/BF16 (FP8: norms only)");
-    const Blocks bl = tc_blocks(L, nj, m, true);
+    const Blocks bl = tc_blocks(L, nj, m, true, TK_F32);
     const Factor f = factor_alloc(c, M, mtrans, nj, m, bl.npad, bl.nblk);
     if (!c.exec) return;
     CUtensorMap tb, txr;

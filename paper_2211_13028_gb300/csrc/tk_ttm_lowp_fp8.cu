@@ -1,0 +1,15 @@
+// Instantiations of the tensor-core TTM of strided or unaligned FP8 data.
+#include <algorithm>
+
+#include "tk_ttm_lowp.cuh"
+
+namespace tk {
+namespace tc {
+
+void ttm_lowp_run_fp8(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& tb,
+                     const LowpArgs& a) {
+    ttm_lowp_dispatch<1>(c, npad, kmajor, tx, tb, a);
+}
+
+}  // namespace tc
+}  // namespace tk

@@ -181,6 +181,44 @@ def test_tc_any_size_and_alignment(dev, dims, k):
     assert st == 0
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "fp8"])
+@pytest.mark.parametrize("dims,k", [
+    ((251, 97, 203), (251, 97, 50)),        # strided, odd slab (runs off 16 bytes), K tail 203 = 3 chunks + 11
+    ((16, 1760, 203), (16, 1760, 40)),      # strided, 16-byte strides (TMA), no padding in the last tile
+    ((16, 1763, 203), (16, 1763, 40)),      # the same, 48 rows in the last tile of the slab
+    ((203, 151, 97), (40, 151, 97)),        # contiguous mode of odd length, ragged last tile
+    ((202, 151, 97), (49, 151, 97)),        # contiguous mode, runs off 16 but on 2 bytes
+    ((33, 333, 401), (33, 40, 401)),        # 3 slabs of 33 rows a tile, 29 rows of it unused; 401 = 133 x 3 + 2
+    ((4, 8, 333, 101), (4, 8, 40, 101)),    # 4 slabs of 32 rows a tile (TMA)
+    ((90, 333, 401), (90, 40, 401)),        # slabs of less than a tile
+    ((501, 21, 700), (501, 20, 700)),       # a third of one chunk contracted
+    ((150, 141, 131), (150, 120, 131)),     # two blocks of output columns
+    ((9, 9, 5001), (9, 9, 100)),            # one row tile, K split over many CTAs
+    ((5001, 9, 9), (100, 9, 9)),            # the same along the contiguous mode
+    ((700, 130, 129), (12, 130, 129)),      # 16-column accumulators
+])
+def test_tc_lowp_any_size_and_alignment(dev, dims, k, dtype):
+    # BF16 and FP8 data against the FP64 oracle on the stored values, in the layouts that their own kernels do
+    # not take.  Bound: the factor's two TF32 parts hold it to 2^-22, and each FP32 sum adds at most 2^-23 per
+    # addition of the 8 MMAs of a chunk and per chunk: below 2e-6 (BF16 of 16-byte strides: the factor's two BF16
+    # parts, 2^-17)
+    g = _rng(29)
+    X, xv, sc = make_X(g.standard_normal(dims), dtype, dev)
+    qs = [np.eye(n) if n == kk else synth.round_to(O.thin_qr(g.standard_normal((n, kk))), "f32")
+          for n, kk in zip(dims, k)]
+    mode = [j for j in range(len(dims)) if dims[j] != k[j]][0]
+    om = [synth.fmat(q, "f32", dev) for q in qs]
+    T.tk_profile(True, dev)
+    G = T.tucker_core(X, om, **({"scale": sc} if dtype == "fp8" else {}))
+    prof = T.tk_profile_read(dev)
+    T.tk_profile(False, dev)
+    assert "xpass_tc" in prof and "xpass_simt" not in prof
+    own = dtype == "bf16" and int(np.prod(dims[:mode])) % 8 == 0
+    assert rel(to_np(G), O.ttm(xv, qs[mode].T, mode)) <= (1e-5 if own else 2e-6)
+    st, _ = T.tk_sync_status(dev)
+    assert st == 0
+
+
 @pytest.mark.parametrize("dtype", ["f32", "bf16", "fp8"])
 @pytest.mark.parametrize("dims,rk", [
     ((130, 7, 66), (9, 5, 33)),     # 910 rows: FP32 columns off 16 bytes; K = 33, two chunks; 66 = 2 x 32 + 2 columns

@@ -1520,11 +1520,16 @@ void launch_jacobi(const Ctx& c, int64_t k, double* A, double* w, double* V, int
 // coordinates, a thread updates the same 2 x 2 block (pair t, pair u >= t) of
 // F' = R^T F R at every step and writes it straight to the permuted positions
 // of the next step: every shared-memory address is computed once, before the
-// sweeps.  F keeps its upper triangle only (it stays exactly symmetric) and is
-// double-buffered.  Warp 0 computes the rotations: at each step, lane t forms
-// the next step's pivot of pair t itself (one entry of the block update, from
-// the same inputs) and its rotation, and carries the pair's diagonal entries
-// and index labels to their new slots, while the other warps update F; one
+// sweeps.  F keeps its upper triangle only (it stays exactly symmetric), is
+// double-buffered, and is stored as four planes, one for each place in a 2 x 2
+// block, indexed by the block: consecutive threads then read consecutive words
+// of each plane, and as pi moves even slots by +2 and odd ones by -2 they write
+// consecutive words too (a matrix by rows costs twice the wavefronts, which
+// delayed the rotations' loads as well: a step of the seeding stage took 0.38
+// us at k = 49 and 0.78 at 81, 0.34 and 0.47 so).  The first one or two warps compute the rotations: at each step,
+// thread t forms the next step's pivot of pair t itself (one entry of the block
+// update, from the same inputs) and its rotation, and carries the pair's
+// diagonal entries to their new slots, while the other warps update F; one
 // barrier per step.  Rotations (c, s per pair and step) are logged to global
 // memory and J = R_1 R_2 ... is formed by a second kernel that replays the log
 // on every row of J independently (one warp per row, several CTAs) with the
@@ -1533,11 +1538,12 @@ void launch_jacobi(const Ctx& c, int64_t k, double* A, double* w, double* V, int
 // which keeps its FP32 entries and the rotation arithmetic clear of overflow
 // and underflow.  Converged: a sweep boundary at which no off-diagonal entry
 // exceeds the threshold (absolute for the resolving stage, relative to the
-// pair's diagonal entries for the seeding stage), or kp - 1 consecutive steps
-// without a rotation.
+// pair's diagonal entries for the seeding stage).
 
 constexpr int JM_MAX_THREADS = 1024;
-constexpr int JM_BPT = 2;  // blocks per update thread: h (h + 1) / 2 <= 2 * 992 for h <= 56
+// Blocks per update thread (h (h + 1) / 2 <= 2 * 960 for h <= 56).  Half the warps make a cheaper barrier: a step of
+// k = 81 takes 0.42 us with 1 or 2 blocks, of 49 0.29 and 0.25, and 0.53 and 0.42 with 3.
+constexpr int JM_BPT = 2;
 
 // The slot an entry at slot x moves to after a step (h = kp / 2 pairs).
 __device__ __forceinline__ int jm_pi(int x, int h) {
@@ -1555,7 +1561,13 @@ __device__ __forceinline__ int jm_pi_inv(int y, int h) {
     return y - 2;
 }
 
-__device__ __forceinline__ int jm_tri(int i, int j, int ld) { return i < j ? i * ld + j : j * ld + i; }
+// The index of block (t, u), t <= u, and the place of the entry at slots i != j: its block's in the plane (of
+// ps words) of its row and column parity.
+__device__ __forceinline__ int jm_blk(int t, int u, int h) { return t * (2 * h - t - 1) / 2 + u; }
+__device__ __forceinline__ int jm_at(int i, int j, int h, int ps) {
+    const int a = min(i, j), b = max(i, j);
+    return ((a & 1) * 2 + (b & 1)) * ps + jm_blk(a >> 1, b >> 1, h);
+}
 
 // Rotation annihilating the (p, q) entry f against the diagonal (p: hp + lp,
 // q: hq + lq), with phi = a_qq - a_pp, psi = 2 a_pq, rho = sqrt(phi^2 +
@@ -1574,43 +1586,60 @@ __device__ __forceinline__ bool jm_big(float f, float hp, float hq, float trel2,
     return f * f > fmaxf(trel2 * fabsf(hp * hq), fthr2);
 }
 
+// No branch: the chain of special functions runs beside the test, and their flush-to-zero forms (r2 and the
+// sums below are normal numbers) have no scaling around them: 0.34 -> 0.25
+// us a step at k = 49.
+__device__ __forceinline__ float jm_rsqrt(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float jm_rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 template <bool DF>
-__device__ __forceinline__ int jm_rotate(float f, float trel2, float fthr2, bool allow, float& hp, float& lp,
-                                         float& hq, float& lq, float2& cs) {
-    cs = make_float2(1.f, 0.f);
-    if (!(allow && jm_big(f, hp, hq, trel2, fthr2))) return 0;
+__device__ __forceinline__ void jm_rotate(float f, float trel2, float fthr2, bool allow, float& hp, float& lp,
+                                          float& hq, float& lq, float2& cs) {
+    const bool rot = allow && jm_big(f, hp, hq, trel2, fthr2);
     float phi = hq - hp;
     if (DF) phi += lq - lp;
     const float psi = 2.f * f;
     const float r2 = fmaxf(fmaf(phi, phi, psi * psi), 1e-37f);
-    const float u = rsqrtf(r2);  // 1 / rho
+    const float u = jm_rsqrt(r2);  // 1 / rho
     const float aphi = fabsf(phi);
-    const float t = __fdividef(phi >= 0.f ? psi : -psi, aphi + r2 * u);
+    const float t = (phi >= 0.f ? psi : -psi) * jm_rcp(aphi + r2 * u);
     const float x = fmaf(0.5f * aphi, u, 0.5f);  // (1 + cos 2a) / 2, in [1/2, 1]
-    const float w = rsqrtf(x);
-    cs = make_float2(x * w, (phi >= 0.f ? f : -f) * u * w);
+    const float w = jm_rsqrt(x);
+    cs = rot ? make_float2(x * w, (phi >= 0.f ? f : -f) * u * w) : make_float2(1.f, 0.f);
     if (DF) {
         const float ph = __fmul_rn(t, f);
         const float pl = fmaf(t, f, -ph);  // t f = ph + pl exactly
-        df_add(hp, lp, -ph, -pl);
-        df_add(hq, lq, ph, pl);
+        float ap = hp, bp = lp, aq = hq, bq = lq;
+        df_add(ap, bp, -ph, -pl);
+        df_add(aq, bq, ph, pl);
+        hp = rot ? ap : hp;
+        lp = rot ? bp : lp;
+        hq = rot ? aq : hq;
+        lq = rot ? bq : lq;
     } else {
-        const float dt = t * f;
+        const float dt = rot ? t * f : 0.f;
         hp -= dt;
         hq += dt;
     }
-    return 1;
 }
 
-// What warp 0's lane needs to form the next-step pivot of one pair: the
-// source block's read base and pairs, which of its four outputs, the source
+// What a rotation thread needs to form the next-step pivot of its pair: the
+// source block's index and pairs, which of its four outputs, the source
 // slots of the pair's two entries.
 struct JmPivot {
     int rd, t, u, sp, sq;
     bool diag, row1, col1;
 };
 
-__device__ __forceinline__ JmPivot jm_pivot_source(int tp, int h, int ld) {
+__device__ __forceinline__ JmPivot jm_pivot_source(int tp, int h) {
     JmPivot pv;
     pv.sp = jm_pi_inv(2 * tp, h);
     pv.sq = jm_pi_inv(2 * tp + 1, h);
@@ -1621,16 +1650,16 @@ __device__ __forceinline__ JmPivot jm_pivot_source(int tp, int h, int ld) {
     const int rs = (ta <= tb) ? pv.sp : pv.sq, cs = (ta <= tb) ? pv.sq : pv.sp;  // row slot in pair t, column slot in u
     pv.row1 = rs & 1;
     pv.col1 = cs & 1;
-    pv.rd = pv.diag ? (2 * pv.t) * ld + 2 * pv.t + 1 : (2 * pv.t) * ld + 2 * pv.u;
+    pv.rd = jm_blk(pv.t, pv.u, h);
     return pv;
 }
 
 // The next-step pivot of a pair: one output of its source block's update.
-__device__ __forceinline__ float jm_pivot_value(const JmPivot& pv, const float* F, const float2* mc, int ld) {
+__device__ __forceinline__ float jm_pivot_value(const JmPivot& pv, const float* F, const float2* mc, int ps) {
     const float2 rt = mc[pv.t];
-    if (pv.diag) return rt.y != 0.f ? 0.f : F[pv.rd];
+    if (pv.diag) return rt.y != 0.f ? 0.f : F[pv.rd + ps];
     const float2 ru = mc[pv.u];
-    const float a = F[pv.rd], b = F[pv.rd + 1], c = F[pv.rd + ld], d = F[pv.rd + ld + 1];
+    const float a = F[pv.rd], b = F[pv.rd + ps], c = F[pv.rd + 2 * ps], d = F[pv.rd + 3 * ps];
     const float al = pv.row1 ? rt.y : rt.x, be = pv.row1 ? rt.x : -rt.y;  // row (2t or 2t + 1) of R_t^T
     const float x0 = fmaf(al, a, be * c), x1 = fmaf(al, b, be * d);
     const float ga = pv.col1 ? ru.y : ru.x, de = pv.col1 ? ru.x : -ru.y;  // column (2u or 2u + 1) of R_u
@@ -1648,10 +1677,10 @@ __global__ void __launch_bounds__(JM_MAX_THREADS) jacobi_sweep_kernel(int k, con
                                                                       int* __restrict__ ginfo, unsigned* flags) {
     extern __shared__ __align__(16) unsigned char smraw[];
     const int kp = k + (k & 1), h = kp / 2, m = kp - 1;
-    const int ld = kp + 1;  // odd stride: walks along either index are bank-conflict free
-    float* Fc = reinterpret_cast<float*>(smraw);  // upper triangle in slot coordinates: F(a, b) = Fc[a * ld + b], a < b
-    float* Fx = Fc + (size_t)kp * ld;             // the next step's
-    float* Hc = Fx + (size_t)kp * ld;             // diagonal (high part) per slot
+    const int ps = h * (h + 1) / 2;               // blocks (pair t, pair u >= t)
+    float* Fc = reinterpret_cast<float*>(smraw);  // four planes, in slot coordinates (jm_at)
+    float* Fx = Fc + 4 * ps;                      // the next step's
+    float* Hc = Fx + 4 * ps;                      // diagonal (high part) per slot
     float* Hx = Hc + kp;
     float* Lc = Hx + kp;                          // diagonal (low part) per slot
     float* Lx = Lc + kp;
@@ -1660,7 +1689,8 @@ __global__ void __launch_bounds__(JM_MAX_THREADS) jacobi_sweep_kernel(int k, con
     __shared__ int ired[33];
     __shared__ float fred[33];
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
-    const bool rwarp = tid < 32;
+    const int nrot = h > 32 ? 64 : 32;  // rotation threads
+    const bool rwarp = tid < nrot;
     // Scale 2^-sh with ||A||_F 2^-sh in [0.5, 1), found with integer and FP32 operations only
     // (FP64 runs at 1/64 of the FP32 rate here): the largest exponent of the entries, then the
     // norm of the entries scaled below 1 in FP32, which places ||A|| within its binade.
@@ -1705,7 +1735,7 @@ __global__ void __launch_bounds__(JM_MAX_THREADS) jacobi_sweep_kernel(int k, con
                 const float2 v = df_from_f64(A[i + (int64_t)k * j], sh);
                 f = __fadd_rn(v.x, v.y);
             }
-            Fc[i * ld + j] = f;
+            Fc[jm_at(i, j, h, ps)] = f;
         } else if (i == j) {
             float2 v = make_float2(0.f, 0.f);
             if (i < k) v = df_from_f64(A[i + (int64_t)k * i], sh);
@@ -1724,15 +1754,15 @@ __global__ void __launch_bounds__(JM_MAX_THREADS) jacobi_sweep_kernel(int k, con
     const float trel2 = DF ? 0.f : (float)(tol * tol);
     const float fthr = (DF ? (float)tol : 1e-13f) * nsc;
     const float fthr2 = fthr * fthr;
-    // update threads (warps 1..): their blocks' read bases and write addresses
-    const int nblk = h * (h + 1) / 2, nu = nt - 32, ut = tid - 32;
-    int bt[JM_BPT], rd[JM_BPT], w0[JM_BPT], w1[JM_BPT], w2[JM_BPT], w3[JM_BPT];
+    // update threads: their blocks and write addresses
+    const int nu = nt - nrot, ut = tid - nrot;
+    int bt[JM_BPT], w0[JM_BPT], w1[JM_BPT], w2[JM_BPT], w3[JM_BPT];
 #pragma unroll
     for (int b = 0; b < JM_BPT; ++b) {
         bt[b] = -1;
-        rd[b] = w0[b] = w1[b] = w2[b] = w3[b] = 0;
+        w0[b] = w1[b] = w2[b] = w3[b] = 0;
         const int e = ut + b * nu;
-        if (rwarp || e >= nblk) continue;
+        if (rwarp || e >= ps) continue;
         int t = 0, rem = e;
         while (rem >= h - t) {
             rem -= h - t;
@@ -1740,109 +1770,100 @@ __global__ void __launch_bounds__(JM_MAX_THREADS) jacobi_sweep_kernel(int k, con
         }
         const int u = t + rem;
         bt[b] = t | (u << 8);
+        const int pr0 = jm_pi(2 * t, h), pr1 = jm_pi(2 * t + 1, h), pc0 = jm_pi(2 * u, h), pc1 = jm_pi(2 * u + 1, h);
         if (t == u) {
-            rd[b] = 2 * t * ld + 2 * t + 1;
-            w0[b] = jm_tri(jm_pi(2 * t, h), jm_pi(2 * t + 1, h), ld);
+            w0[b] = jm_at(pr0, pr1, h, ps);
         } else {
-            rd[b] = 2 * t * ld + 2 * u;
-            const int pr0 = jm_pi(2 * t, h), pr1 = jm_pi(2 * t + 1, h), pc0 = jm_pi(2 * u, h), pc1 = jm_pi(2 * u + 1, h);
-            w0[b] = jm_tri(pr0, pc0, ld);
-            w1[b] = jm_tri(pr0, pc1, ld);
-            w2[b] = jm_tri(pr1, pc0, ld);
-            w3[b] = jm_tri(pr1, pc1, ld);
+            w0[b] = jm_at(pr0, pc0, h, ps);
+            w1[b] = jm_at(pr0, pc1, h, ps);
+            w2[b] = jm_at(pr1, pc0, h, ps);
+            w3[b] = jm_at(pr1, pc1, h, ps);
         }
     }
-    // warp 0: the pairs lane and lane + 32
-    const bool has0 = rwarp && lane < h, has1 = rwarp && lane + 32 < h;
-    JmPivot pv0 = jm_pivot_source(has0 ? lane : 0, h, ld), pv1 = jm_pivot_source(has1 ? lane + 32 : 0, h, ld);
+    // whether an entry of the thread's blocks still needs a rotation
+    auto big_left = [&]() {
+        int off = 0;
+#pragma unroll
+        for (int b = 0; b < JM_BPT; ++b) {
+            if (bt[b] < 0) continue;
+            const int t = bt[b] & 255, u = bt[b] >> 8, e = ut + b * nu;
+            off |= jm_big(Fc[e + ps], Hc[2 * t], Hc[2 * u + 1], trel2, fthr2);
+            if (t == u) continue;
+            off |= jm_big(Fc[e], Hc[2 * t], Hc[2 * u], trel2, fthr2);
+            off |= jm_big(Fc[e + 2 * ps], Hc[2 * t + 1], Hc[2 * u], trel2, fthr2);
+            off |= jm_big(Fc[e + 3 * ps], Hc[2 * t + 1], Hc[2 * u + 1], trel2, fthr2);
+        }
+        return off;
+    };
+    const bool has = tid < h;  // rotation thread of pair tid
+    const JmPivot pv = jm_pivot_source(has ? tid : 0, h);
     __syncthreads();
     const int total = max_sweeps * m;  // steps allowed (the launcher bounds it)
-    int any = 0;
-    if (total > 0 && rwarp) {  // the first step's rotations, in place
-#pragma unroll
-        for (int o = 0; o < 2; ++o) {
-            const int tp = lane + 32 * o;
-            if (tp >= h) continue;
-            const int p = 2 * tp, q = p + 1;
-            float hp = Hc[p], lp = Lc[p], hq = Hc[q], lq = Lc[q];
-            float2 cs;
-            any |= jm_rotate<DF>(Fc[p * ld + q], trel2, fthr2, true, hp, lp, hq, lq, cs);
-            Hc[p] = hp;
-            Lc[p] = lp;
-            Hc[q] = hq;
-            Lc[q] = lq;
-            meta[0][tp] = cs;
-            rlog[tp] = cs;
-        }
+    if (total > 0 && has) {            // the first step's rotations, in place
+        const int p = 2 * tid, q = p + 1;
+        float2 cs;
+        jm_rotate<DF>(Fc[jm_blk(tid, tid, h) + ps], trel2, fthr2, true, Hc[p], Lc[p], Hc[q], Lc[q], cs);
+        meta[0][tid] = cs;
+        rlog[tid] = cs;
     }
-    int active = __syncthreads_or(any);  // whether the current step rotates anything
-    int cur = 0, steps = 0, s = 0, idle = 0;
+    __syncthreads();
+    int cur = 0, steps = 0, s = 0;
     bool converged = false;
     float2* lg = rlog + h;  // the next step's log slot
     for (int g = 0; g < total; ++g, lg += h) {
-        if (s == 0) {
-            int off = 0;
-            for (int a = tid >> 5; a < kp; a += nt >> 5)
-                for (int b = a + 1 + lane; b < kp; b += 32) off |= jm_big(Fc[a * ld + b], Hc[a], Hc[b], trel2, fthr2);
-            if (!__syncthreads_or(off)) {
-                converged = true;
-                break;
-            }
-        }
-        idle = active ? 0 : idle + 1;
-        if (idle >= m) {
+        // (a sweep without a rotation leaves nothing above the threshold, so no other test is needed)
+        if (s == 0 && !__syncthreads_or(big_left())) {
             converged = true;
             break;
         }
         const float2* mc = meta[cur];
-        any = 0;
         if (rwarp) {
-            const bool want = g + 1 < total;
-            float2* mn = meta[cur ^ 1];
-#pragma unroll
-            for (int o = 0; o < 2; ++o) {
-                if (!(o ? has1 : has0)) continue;
-                const JmPivot& pv = o ? pv1 : pv0;
-                const int tp = lane + 32 * o;
+            if (has) {
                 float hp = Hc[pv.sp], hq = Hc[pv.sq], lp = 0.f, lq = 0.f;
                 if (DF) {
                     lp = Lc[pv.sp];
                     lq = Lc[pv.sq];
                 }
-                const float f = jm_pivot_value(pv, Fc, mc, ld);
+                const float f = jm_pivot_value(pv, Fc, mc, ps);
                 float2 cs;
-                any |= jm_rotate<DF>(f, trel2, fthr2, want, hp, lp, hq, lq, cs);
-                Hx[2 * tp] = hp;
-                Hx[2 * tp + 1] = hq;
+                jm_rotate<DF>(f, trel2, fthr2, g + 1 < total, hp, lp, hq, lq, cs);
+                meta[cur ^ 1][tid] = cs;
+                Hx[2 * tid] = hp;
+                Hx[2 * tid + 1] = hq;
                 if (DF) {
-                    Lx[2 * tp] = lp;
-                    Lx[2 * tp + 1] = lq;
+                    Lx[2 * tid] = lp;
+                    Lx[2 * tid + 1] = lq;
                 }
-                mn[tp] = cs;
-                lg[tp] = cs;
+                lg[tid] = cs;
             }
         } else {
+            // (every block's loads before the first store, which the compiler would not move them across)
+            float2 rt[JM_BPT], ru[JM_BPT];
+            float f[JM_BPT][4];
+#pragma unroll
+            for (int b = 0; b < JM_BPT; ++b) {
+                const int e = bt[b] < 0 ? 0 : ut + b * nu;
+                rt[b] = mc[bt[b] < 0 ? 0 : bt[b] & 255];
+                ru[b] = mc[bt[b] < 0 ? 0 : bt[b] >> 8];
+#pragma unroll
+                for (int w = 0; w < 4; ++w) f[b][w] = Fc[e + w * ps];
+            }
 #pragma unroll
             for (int b = 0; b < JM_BPT; ++b) {
                 if (bt[b] < 0) continue;
-                const int t = bt[b] & 255, u = bt[b] >> 8;
-                const float2 rt = mc[t];
-                if (t == u) {  // the pair's own entry: annihilated when it rotates
-                    Fx[w0[b]] = rt.y != 0.f ? 0.f : Fc[rd[b]];
+                if ((bt[b] & 255) == bt[b] >> 8) {  // the pair's own entry: annihilated when it rotates
+                    Fx[w0[b]] = rt[b].y != 0.f ? 0.f : f[b][1];
                     continue;
                 }
-                const float2 ru = mc[u];
-                const int r = rd[b];
-                const float a = Fc[r], bb = Fc[r + 1], cc = Fc[r + ld], dd = Fc[r + ld + 1];
-                const float r00 = fmaf(rt.x, a, -rt.y * cc), r01 = fmaf(rt.x, bb, -rt.y * dd);
-                const float r10 = fmaf(rt.y, a, rt.x * cc), r11 = fmaf(rt.y, bb, rt.x * dd);
-                Fx[w0[b]] = fmaf(ru.x, r00, -ru.y * r01);
-                Fx[w1[b]] = fmaf(ru.y, r00, ru.x * r01);
-                Fx[w2[b]] = fmaf(ru.x, r10, -ru.y * r11);
-                Fx[w3[b]] = fmaf(ru.y, r10, ru.x * r11);
+                const float r00 = fmaf(rt[b].x, f[b][0], -rt[b].y * f[b][2]), r01 = fmaf(rt[b].x, f[b][1], -rt[b].y * f[b][3]);
+                const float r10 = fmaf(rt[b].y, f[b][0], rt[b].x * f[b][2]), r11 = fmaf(rt[b].y, f[b][1], rt[b].x * f[b][3]);
+                Fx[w0[b]] = fmaf(ru[b].x, r00, -ru[b].y * r01);
+                Fx[w1[b]] = fmaf(ru[b].y, r00, ru[b].x * r01);
+                Fx[w2[b]] = fmaf(ru[b].x, r10, -ru[b].y * r11);
+                Fx[w3[b]] = fmaf(ru[b].y, r10, ru[b].x * r11);
             }
         }
-        const int nxt = __syncthreads_or(any);
+        __syncthreads();
         float* x;
         x = Fc; Fc = Fx; Fx = x;
         x = Hc; Hc = Hx; Hx = x;
@@ -1850,14 +1871,8 @@ __global__ void __launch_bounds__(JM_MAX_THREADS) jacobi_sweep_kernel(int k, con
         cur ^= 1;
         ++steps;
         s = (s + 1 == m) ? 0 : s + 1;
-        active = nxt;
     }
-    if (!converged) {  // the allowed sweeps ran out: measure once more
-        int off = 0;
-        for (int a = tid >> 5; a < kp; a += nt >> 5)
-            for (int b = a + 1 + lane; b < kp; b += 32) off |= jm_big(Fc[a * ld + b], Hc[a], Hc[b], trel2, fthr2);
-        converged = !__syncthreads_or(off);
-    }
+    if (!converged) converged = !__syncthreads_or(big_left());  // the allowed sweeps ran out: measure once more
     if (!converged && tid == 0) atomicOr(flags, FLAG_NOT_CONVERGED);
     // index labels: after `steps` moves slot x holds the index that started in
     // slot pi^{-steps}(x); slots 1..kp-1 form one cycle of pi, walked once
@@ -1886,8 +1901,10 @@ __global__ void __launch_bounds__(JM_MAX_THREADS) jacobi_sweep_kernel(int k, con
 }
 
 // J = R_1 R_2 ... R_steps from the log, one warp per row of J: lane t holds
-// pair t (and t + 32), rotates it and writes it to the permuted slots of the
-// next step; the final slot labels say which column each slot is.  The log is
+// pair t (and t + 32: TWO) in registers, rotates it and passes its entries on to
+// the next step's slots, two shuffles a register as pi only moves even slots
+// one pair up and odd ones one pair down (through shared memory a step took
+// twice as long); the final slot labels say which column each slot is.  The log is
 // staged through shared memory in chunks, the next chunk fetched into
 // registers while the current one is applied.
 constexpr int JR_WARPS = 4;
@@ -1904,6 +1921,7 @@ __device__ __forceinline__ long long jr_key(double d) {
 // identity, i.e. the kernel forms V = V1 J without J, and writes the columns
 // of V of the r largest D (ties: lower index first) into Vt and Vr (k x r,
 // ld k), ordered by rank.
+template <bool TWO>
 __global__ void __launch_bounds__(JR_WARPS * 32) jacobi_replay_kernel(int k, const float2* __restrict__ rlog,
                                                                       const int* __restrict__ ginfo, float* Jout,
                                                                       double* J64a, double* J64b,
@@ -1915,21 +1933,24 @@ __global__ void __launch_bounds__(JR_WARPS * 32) jacobi_replay_kernel(int k, con
     const int nt = JR_WARPS * 32, cr = JR_STAGE * nt / h;  // steps per chunk
     float2* stage = reinterpret_cast<float2*>(smraw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float* ra = reinterpret_cast<float*>(stage + (size_t)cr * h) + (size_t)warp * 2 * kp;  // this warp's row
-    float* rb = ra + kp;
-    long long* keys = reinterpret_cast<long long*>(ra - (size_t)warp * 2 * kp + (size_t)JR_WARPS * 2 * kp);
+    long long* keys = reinterpret_cast<long long*>(stage + (size_t)cr * h);
     const int i = blockIdx.x * JR_WARPS + warp;
     const int steps = ginfo[0];
-    if (V1) {
-        for (int x = lane; x < kp; x += 32) ra[x] = (i < k && x < k) ? (float)V1[i + (int64_t)k * x] : 0.f;
-        for (int x = tid; x < k; x += nt) keys[x] = jr_key(D[x]);
-    } else {
-        for (int x = lane; x < kp; x += 32) ra[x] = (x == i) ? 1.f : 0.f;
+    auto start = [&](int x) {  // entry x of the row to begin with
+        if (!V1) return x == i ? 1.f : 0.f;
+        return (i < k && x < k) ? (float)V1[i + (int64_t)k * x] : 0.f;
+    };
+    float a0 = start(2 * lane), b0 = start(2 * lane + 1), a1 = 0.f, b1 = 0.f;
+    if (TWO) {
+        a1 = start(2 * lane + 64);
+        b1 = start(2 * lane + 65);
     }
+    if (V1)
+        for (int x = tid; x < k; x += nt) keys[x] = jr_key(D[x]);
     __syncthreads();  // the keys are read by every warp at the end (also when no step was taken)
-    const int t0 = lane, t1 = lane + 32;
-    const int d00 = jm_pi(2 * t0, h), d01 = jm_pi(2 * t0 + 1, h);
-    const int d10 = jm_pi(2 * t1, h), d11 = jm_pi(2 * t1 + 1, h);
+    const int up = (lane + 31) & 31, down = (lane + 1) & 31;  // the lanes whose entries arrive from below, from above
+    const bool last0 = lane == h - 1, last1 = lane + 32 == h - 1;
+    const int t0 = min(lane, h - 1), t1 = min(lane + 32, h - 1);
     float2 pre[JR_STAGE];
     int cn = min(cr, steps);
 #pragma unroll
@@ -1952,35 +1973,39 @@ __global__ void __launch_bounds__(JR_WARPS * 32) jacobi_replay_kernel(int k, con
             if (e < nn * h) pre[w] = rlog[(int64_t)c1 * h + e];
         }
         if (i < k) {
-            for (int rr = 0; rr < cn; ++rr) {
-                const float2* cs = stage + rr * h;
-                if (t0 < h) {
-                    const float2 q = cs[t0];
-                    const float a = ra[2 * t0], b = ra[2 * t0 + 1];
-                    rb[d00] = fmaf(q.x, a, -q.y * b);
-                    rb[d01] = fmaf(q.y, a, q.x * b);
+            const float2* cs = stage;
+#pragma unroll 4
+            for (int rr = 0; rr < cn; ++rr, cs += h) {
+                const float2 q0 = cs[t0];
+                const float x0 = fmaf(q0.x, a0, -q0.y * b0), y0 = fmaf(q0.y, a0, q0.x * b0);
+                // slot 1 moves to slot 2, slot 0 stays, slot 2h - 2 moves to 2h - 1
+                const float r0 = __shfl_sync(0xffffffffu, lane == 0 ? y0 : x0, up);
+                const float s0 = __shfl_sync(0xffffffffu, y0, down);
+                if (TWO) {
+                    const float2 q1 = cs[t1];
+                    const float x1 = fmaf(q1.x, a1, -q1.y * b1), y1 = fmaf(q1.y, a1, q1.x * b1);
+                    const float r1 = __shfl_sync(0xffffffffu, x1, up), s1 = __shfl_sync(0xffffffffu, y1, down);
+                    a0 = lane == 0 ? x0 : r0;
+                    b0 = lane == 31 ? s1 : s0;
+                    a1 = lane == 0 ? r0 : r1;
+                    b1 = last1 ? x1 : s1;
+                } else {
+                    a0 = lane == 0 ? x0 : r0;
+                    b0 = last0 ? (h == 1 ? y0 : x0) : s0;
                 }
-                if (t1 < h) {
-                    const float2 q = cs[t1];
-                    const float a = ra[2 * t1], b = ra[2 * t1 + 1];
-                    rb[d10] = fmaf(q.x, a, -q.y * b);
-                    rb[d11] = fmaf(q.y, a, q.x * b);
-                }
-                __syncwarp();  // the next step reads slots other lanes wrote
-                float* x = ra;
-                ra = rb;
-                rb = x;
             }
         }
         c0 = c1;
         cn = nn;
     }
-    __syncwarp();
     if (i >= k) return;
-    for (int x = lane; x < kp; x += 32) {
+#pragma unroll
+    for (int w = 0; w < (TWO ? 4 : 2); ++w) {
+        const int x = 2 * lane + (w & 1) + 64 * (w >> 1);
+        if (x >= kp) continue;
         const int j = ginfo[1 + x];
         if (j >= k) continue;
-        const float v = ra[x];
+        const float v = w == 0 ? a0 : (w == 1 ? b0 : (w == 2 ? a1 : b1));
         if (V1) {
             const long long kj = keys[j];
             int rank = 0;
@@ -2010,10 +2035,11 @@ void launch_jacobi_mixed(Ctx& c, int64_t k, const double* A, double* D, float* J
     float2* rlog = c.alloc<float2>(((int64_t)max_sweeps * (kp - 1) + 1) * h);
     int* ginfo = c.alloc<int>(1 + kp);
     if (!c.exec) return;
-    const size_t smem = sizeof(float) * (2 * kp * (kp + 1) + 4 * kp) + sizeof(int) * 2 * kp;
-    // warp 0 computes rotations; the rest update blocks (at most JM_BPT each)
-    const int64_t nu = std::min<int64_t>(JM_MAX_THREADS - 32, (nblk + 31) / 32 * 32);
-    const int nt = (int)(32 + nu);
+    const size_t smem = sizeof(float) * (8 * nblk + 4 * kp) + sizeof(int) * kp;
+    // one warp, or two, for rotations; the rest update blocks (at most JM_BPT each)
+    const int64_t nrot = h > 32 ? 64 : 32;
+    const int64_t nu = ((nblk + JM_BPT - 1) / JM_BPT + 31) / 32 * 32;
+    const int nt = (int)(nrot + nu);
     {
         ProfScope ps(c, "jacobi", 8.0 * k * k + 8.0 * k, 12.0 * k * k * k * max_sweeps);
         if (fp64_diag) {
@@ -2035,9 +2061,10 @@ void launch_jacobi_mixed(Ctx& c, int64_t k, const double* A, double* D, float* J
     if (!J && !J64a && !J64b && !V1) return;
     TK_REQUIRE(!V1 || (Vt && Vr && r >= 1 && r <= k), TK_ERR_ARG, "jacobi_mixed: V1 needs Vt, Vr and 1 <= r <= k");
     const int cr = JR_STAGE * JR_WARPS * 32 / (int)h;
-    const size_t rsmem = sizeof(float2) * cr * h + sizeof(float) * JR_WARPS * 2 * kp + sizeof(long long) * kp;
+    const size_t rsmem = sizeof(float2) * cr * h + sizeof(long long) * kp;
     ProfScope ps(c, "jacobi", 8.0 * h * (max_sweeps * (kp - 1) + 1) + 8.0 * k * k, 6.0 * k * k * k * max_sweeps);
-    jacobi_replay_kernel<<<(unsigned)((k + JR_WARPS - 1) / JR_WARPS), JR_WARPS * 32, rsmem, c.stream>>>(
+    const auto replay = h > 32 ? jacobi_replay_kernel<true> : jacobi_replay_kernel<false>;
+    replay<<<(unsigned)((k + JR_WARPS - 1) / JR_WARPS), JR_WARPS * 32, rsmem, c.stream>>>(
         (int)k, rlog, ginfo, J, J64a, J64b, V1, D, (int)r, Vt, Vr);
     c.counted();
     c.check_launch();

@@ -432,3 +432,25 @@ def test_rhkron_sketch_widths_above_112(dev, dtype):
     assert st == 0 and info[:3] == [1, 1, 1]  # Householder QR for the wide sketches
     ref = O.rhkron(xv, r, oms)
     _check_decomp(G, U, err, ref, xv, TOL[dtype])
+
+
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 62, 63, 64, 65, 66, 67, 111, 112])
+def test_core_eigenvectors_at_the_jacobi_kernels_sizes(dev, k):
+    # one pair, an odd size's empty row, the last size with one register pair a lane and one warp of rotations (64)
+    # and the first with two, the largest.  The cut falls between singular values 7% apart; the FP32 rotations
+    # leave the leading eigenvectors a singular-value-weighted ~1e-7 (the resolving threshold, 1e-11 of the
+    # Gram's norm) and the results are rounded to FP32: 5e-6
+    g = _rng(61)
+    r = (k + 1) // 2
+    a, b = np.linalg.qr(g.standard_normal((k, k)))[0], np.linalg.qr(g.standard_normal((156, k)))[0]
+    core = np.asfortranarray(synth.round_to(((a * 0.93 ** np.arange(k)) @ b.T).reshape(k, 12, 13, order="F"), "f32"))
+    G, U = T.tucker_sthosvd(synth.fortran(core, "f32", dev), [synth.fmat(np.eye(n), "f32", dev) for n in core.shape],
+                            [r, 12, 13])
+    u = to_np(U[0])
+    assert np.linalg.norm(u.T @ u - np.eye(r)) <= 1e-6 * np.sqrt(k)
+    ref_g, ref_u, _ = O.sthosvd(core, [r, 12, 13])
+    got = O.multi_ttm(to_np(G), [(j, to_np(U[j])) for j in range(3)])
+    ref = O.multi_ttm(ref_g, [(j, ref_u[j]) for j in range(3)])
+    assert rel(got, ref) <= 5e-6
+    st, _ = T.tk_sync_status(dev)
+    assert st == 0

@@ -930,45 +930,65 @@ __device__ __forceinline__ float2 df_fnms2(float2 a, float2 f, float2 b) {
 // approximate reciprocal and square root, a few ulp) and one Newton step
 // evaluated in double-float, which squares the seed's relative error
 // (~2^-44, then limited by the double-float format).
-__device__ __forceinline__ void df_rcp_rsqrt(float2 p, float2& inv, float2& ys) {
+__device__ __forceinline__ float2 df_rcp(float2 p) {
     const float q0 = __fdividef(1.0f, p.x);
     float t = fmaf(-p.x, q0, 1.0f);
     t = fmaf(-p.y, q0, t);
-    inv = df_norm(q0, __fmul_rn(q0, t));
+    return df_norm(q0, __fmul_rn(q0, t));
+}
+
+__device__ __forceinline__ float2 df_rsqrt(float2 p) {
     const float y0 = rsqrtf(p.x);
     const float a = __fmul_rn(y0, y0);
     const float2 y2 = make_float2(a, fmaf(y0, y0, -a));  // y0^2 exactly
     const float2 py = df_mul2(p, y2);
     const float d = __fsub_rn(__fsub_rn(1.0f, py.x), py.y);  // 1 - p y0^2 (~2^-22)
-    ys = df_norm(y0, __fmul_rn(__fmul_rn(0.5f, y0), d));
+    return df_norm(y0, __fmul_rn(__fmul_rn(0.5f, y0), d));
 }
 
 constexpr int CHDF_THREADS = 768;
 constexpr int CHDF_PANEL = 8;  // columns per panel (warps 0 .. CHDF_PANEL-1 own its rows)
 
+// A and M share one array of rows: row i holds M(i, x) at x < i and a_ix at x >= i (M(i, i) = 1 is implied), so that
+// step j is one update of row i, v -= l_ij row_j(x), over x <= j and x >= i (row_j(j) standing for M(j, j) = 1).
+//
 // Blocked over panels of CHDF_PANEL columns.  Within a panel, warp w owns row
-// j0 + w: at step j every warp whose row lies below j reads the pivot p_j
-// (final: row j was last updated at step j - 1), forms 1/p_j itself, its
-// multiplier l_ij and updates its row of A and of M; the panel's warps meet at
-// a named barrier per column.  The rows below the panel then take the panel's
-// updates in one pass, a_il -= sum_j l_ij a_jl and M(i, .) -= sum_j l_ij M(j, .),
-// in the same order of j as the column-by-column form, so every entry sees the
-// same operations on the same values (the result is that form's, bit for
-// bit) with two CTA barriers per panel instead of one per column.
+// j0 + w and keeps it in registers: at step j every warp whose row lies below j
+// reads the pivot p_j (final: row j was last updated at step j - 1), forms 1/p_j
+// itself, its multiplier l_ij and updates its row; the next row goes back to
+// shared memory, and the panel's warps meet at a named barrier per column: the
+// chain of a column is a reciprocal, a product and one update (rows in shared memory,
+// and 1/sqrt(p_j) formed by every warp: 43 us at 49 columns, 36 so).  The rows below
+// the panel then take its updates in one pass, a warp a row, in the same order of j
+// as the column-by-column form, so every entry sees the same operations on the
+// same values (the result is that form's, bit for bit) with two CTA barriers
+// per panel instead of one per column.
+constexpr int CHDF_Q = 4;  // entries of a row per lane: k <= 112
+
+// One step on a lane's entries v[q] at x = lane + 32 q of row i: the row of pivot j, the multiplier f.
+__device__ __forceinline__ void chdf_step(float2 (&v)[CHDF_Q], const float2* rowj, int k, int i, int j, float2 f,
+                                          int lane) {
+#pragma unroll
+    for (int q = 0; q < CHDF_Q; ++q) {
+        if (32 * q >= k) break;  // uniform
+        const int x = lane + 32 * q;
+        const float2 b = x == j ? make_float2(1.f, 0.f) : rowj[min(x, k - 1)];
+        const float2 u = df_fnms2(v[q], f, b);
+        if (x <= j || x >= i) v[q] = u;
+    }
+}
+
 __global__ void __launch_bounds__(CHDF_THREADS) chol_inv_df_kernel(KDims kd, int kmax, const double* W,
                                                                    double* Rinv, int* bad, double tol) {
-    extern __shared__ float2 sf[];  // A: k x k row-major (upper part), M: k x k row-major (lower part)
+    extern __shared__ float2 sf[];  // the rows, ld apart
     __shared__ float2 s_ys[112];    // 1 / sqrt(p_j)
     __shared__ float2 s_inv[CHDF_PANEL];         // 1 / p_j of the panel's columns
-    __shared__ float2 s_l[CHDF_PANEL][112];      // l_ij of the panel's columns for the rows below the panel
     __shared__ float s_dg[112];     // scaled original diagonal (breakdown test)
     __shared__ int s_fail;
     __shared__ int s_e;
     const int b = blockIdx.x;
     if (bad[b]) return;
-    const int k = kd.k[b];
-    float2* A = sf;
-    float2* M = sf + (size_t)k * k;
+    const int k = kd.k[b], ld = k | 1;
     const double* Wb = W + (int64_t)b * kmax * kmax;
     double* Rb = Rinv + (int64_t)b * kmax * kmax;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
@@ -989,64 +1009,57 @@ __global__ void __launch_bounds__(CHDF_THREADS) chol_inv_df_kernel(KDims kd, int
     __syncthreads();
     const int e = s_e;
     for (int idx = tid; idx < k * k; idx += nt) {
-        const int i = idx / k, l = idx - i * k;
-        A[idx] = l >= i ? df_from_f64(Wb[i + (int64_t)kmax * l], 2 * e) : make_float2(0.f, 0.f);
-        M[idx] = make_float2(i == l ? 1.f : 0.f, 0.f);
+        const int l = idx / k, i = idx - l * k;
+        const float2 v = l >= i ? df_from_f64(Wb[i + (int64_t)kmax * l], 2 * e) : make_float2(0.f, 0.f);
+        sf[i * ld + l] = v;
+        if (i == l) s_dg[i] = v.x;
     }
-    for (int i = tid; i < k; i += nt) s_dg[i] = df_from_f64(Wb[i + (int64_t)kmax * i], 2 * e).x;
     __syncthreads();
     for (int j0 = 0; j0 < k; j0 += CHDF_PANEL) {
         const int jb = min(CHDF_PANEL, k - j0);
         if (warp < CHDF_PANEL) {
-            const int i = j0 + warp;  // this warp's row (none when warp >= jb)
+            const int i = min(j0 + warp, k - 1);  // this warp's row (idle when warp >= jb)
+            float2 v[CHDF_Q];
+#pragma unroll
+            for (int q = 0; q < CHDF_Q; ++q) v[q] = sf[i * ld + min(lane + 32 * q, k - 1)];
             for (int jj = 0; jj < jb; ++jj) {
                 const int j = j0 + jj;
-                const float2 p = A[(size_t)j * k + j];
+                const float2* rowj = sf + j * ld;
+                const float2 p = rowj[j];
                 if (!(p.x > (float)tol * s_dg[j] && p.x > 0.f)) {  // the same test in every warp
                     if (warp == 0 && lane == 0) s_fail = 1;
                     break;
                 }
-                float2 inv, ys;
-                df_rcp_rsqrt(p, inv, ys);
-                if (warp == jj && lane == 0) {
-                    s_inv[jj] = inv;
-                    s_ys[j] = ys;
-                }
-                if (warp < jb && i > j) {
-                    const float2* Aj = A + (size_t)j * k;
-                    const float2* Mj = M + (size_t)j * k;
-                    const float2 f = df_mul2(Aj[i], inv);  // l_ij
-                    float2* Ai = A + (size_t)i * k;
-                    float2* Mi = M + (size_t)i * k;
-                    for (int l = i + lane; l < k; l += 32) Ai[l] = df_fnms2(Ai[l], f, Aj[l]);
-                    for (int cc = lane; cc <= j; cc += 32) Mi[cc] = df_fnms2(Mi[cc], f, Mj[cc]);
+                if (warp > jj && warp < jb) {
+                    chdf_step(v, rowj, k, i, j, df_mul2(rowj[i], df_rcp(p)), lane);  // l_ij
+                    if (warp == jj + 1) {
+#pragma unroll
+                        for (int q = 0; q < CHDF_Q; ++q)
+                            if (lane + 32 * q < k) sf[i * ld + lane + 32 * q] = v[q];
+                    }
+                } else if (warp == jj && lane == 0) {
+                    s_inv[jj] = df_rcp(p);
+                    s_ys[j] = df_rsqrt(p);
                 }
                 asm volatile("bar.sync 1, %0;" ::"n"(32 * CHDF_PANEL) : "memory");
             }
         }
         __syncthreads();
         if (s_fail) break;  // uniform: written before the barrier
-        const int t0 = j0 + jb, nr = k - t0;
-        if (nr <= 0) break;
-        // the panel's multipliers for the rows below it
-        for (int x = tid; x < jb * nr; x += nt) {
-            const int jj = x / nr, i = t0 + x % nr;
-            s_l[jj][i] = df_mul2(A[(size_t)(j0 + jj) * k + i], s_inv[jj]);
-        }
-        __syncthreads();
-        for (int x = tid; x < nr * nr; x += nt) {  // A(i, l), t0 <= i <= l < k
-            const int i = t0 + x / nr, l = t0 + x % nr;
-            if (l < i) continue;
-            float2 v = A[(size_t)i * k + l];
-            for (int jj = 0; jj < jb; ++jj) v = df_fnms2(v, s_l[jj][i], A[(size_t)(j0 + jj) * k + l]);
-            A[(size_t)i * k + l] = v;
-        }
-        for (int x = tid; x < nr * t0; x += nt) {  // M(i, c), t0 <= i < k, c < t0 (M(j, c) = 0 for c > j)
-            const int i = t0 + x / t0, c = x % t0;
-            float2 v = M[(size_t)i * k + c];
-            for (int jj = 0; jj < jb; ++jj)
-                if (c <= j0 + jj) v = df_fnms2(v, s_l[jj][i], M[(size_t)(j0 + jj) * k + c]);
-            M[(size_t)i * k + c] = v;
+        const int t0 = j0 + jb;
+        if (t0 >= k) break;
+        for (int i = t0 + warp; i < k; i += nt >> 5) {
+            float2 v[CHDF_Q], f = make_float2(0.f, 0.f);
+            if (lane < jb) f = df_mul2(sf[(j0 + lane) * ld + i], s_inv[lane]);  // the row's multipliers, one a lane
+#pragma unroll
+            for (int q = 0; q < CHDF_Q; ++q) v[q] = sf[i * ld + min(lane + 32 * q, k - 1)];
+#pragma unroll
+            for (int jj = 0; jj < CHDF_PANEL; ++jj)  // (the last panel ends the loop above, so jb is whole here)
+                chdf_step(v, sf + (j0 + jj) * ld, k, i, j0 + jj,
+                          make_float2(__shfl_sync(0xffffffffu, f.x, jj), __shfl_sync(0xffffffffu, f.y, jj)), lane);
+#pragma unroll
+            for (int q = 0; q < CHDF_Q; ++q)
+                if (lane + 32 * q < k) sf[i * ld + lane + 32 * q] = v[q];
         }
         __syncthreads();
     }
@@ -1059,7 +1072,7 @@ __global__ void __launch_bounds__(CHDF_THREADS) chol_inv_df_kernel(KDims kd, int
         const int a = idx % k, c = idx / k;  // R^{-1}(a, c), column-major out
         double v = 0.0;
         if (a <= c) {
-            const float2 r = df_mul2(M[(size_t)c * k + a], s_ys[c]);
+            const float2 r = df_mul2(a == c ? make_float2(1.f, 0.f) : sf[c * ld + a], s_ys[c]);
             v = ((double)r.x + (double)r.y) * sc;
         }
         Rb[a + (int64_t)kmax * c] = v;
@@ -1071,7 +1084,7 @@ void launch_chol_inv(const Ctx& c, int batch, const KDims& kd, int kmax, const d
     if (!c.exec) return;
     TK_REQUIRE(kmax <= 112, TK_ERR_SHAPE, "chol_inv: at most 112 columns");
     if (df) {
-        const size_t smem = 2 * sizeof(float2) * kmax * kmax;
+        const size_t smem = sizeof(float2) * kmax * (kmax | 1);
         if (smem > 48 * 1024)
             TK_CUDA(cudaFuncSetAttribute(chol_inv_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         ProfScope ps(c, "chol_inv", 16.0 * batch * kmax * kmax, (2.0 / 3.0) * batch * kmax * kmax * kmax);

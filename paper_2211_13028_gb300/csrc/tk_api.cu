@@ -717,6 +717,7 @@ static tk_status run_call(tk_handle* h, F&& body) {
         ex.stream = h->stream;
         ex.exec = true;
         ex.capturing = capturing;
+        ex.overlap = !capturing && !h->prof.on;
         ex.base = h->ws;
         ex.dflags = h->dflags;
         ex.dqr = h->dqr;

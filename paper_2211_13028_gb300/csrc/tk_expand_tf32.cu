@@ -86,6 +86,7 @@ template <int NK, int EPI, typename XR>
 __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
     expand_tf32x3_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmXr,
                          ExpandArgs args) {
+    kernel_begin();
     using C = ExpandCfg<NK, EPI, XR>;
     constexpr int SUB = C::SUB;
     constexpr int NB = C::kNB;
@@ -546,7 +547,7 @@ static void launch_one(const Ctx& c, const CUtensorMap& tb, const CUtensorMap& t
         TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::kSmem));
         attr_set = true;
     }
-    kern<<<expand_ctas(c, a), Cf::kThreads, Cf::kSmem, c.stream>>>(tb, txr, a);
+    run_kernel(c, kern, expand_ctas(c, a), Cf::kThreads, Cf::kSmem, tb, txr, a);
 }
 
 void expand_run(const Ctx& c, int epi, tk_dtype xrdt, const CUtensorMap& tb, const CUtensorMap& txr,

@@ -61,6 +61,7 @@ inline size_t fs_smem(int64_t nk) {
 template <bool KMAJOR>
 __global__ void __launch_bounds__(FS_THREADS, 1)
     srht_stream_kernel(const __grid_constant__ CUtensorMap tmX, FsArgs args) {
+    kernel_begin();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int64_t nk = args.nk;
@@ -290,7 +291,7 @@ void launch_srht_stream(const Ctx& c, const Tens& X, int j, const Mat& M, bool m
     const int grid = (int)std::min<int64_t>(a.ntiles, tc::grid_sms(c));
     auto run = [&](auto kern) {
         TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kern<<<grid, tc::FS_THREADS, smem, c.stream>>>(tx, a);
+        run_kernel(c, kern, grid, tc::FS_THREADS, smem, tx, a);
     };
     kmajor ? run(tc::srht_stream_kernel<true>) : run(tc::srht_stream_kernel<false>);
     c.counted();

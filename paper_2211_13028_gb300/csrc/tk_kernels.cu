@@ -19,6 +19,7 @@ void Ctx::check_launch() const {
 // Only the streams that receive work wait on the fork (a stream that joined a
 // graph recording must be joined back before the recording ends).
 void ctx_fork_begin(Ctx& c, int used) {
+    c.chained = false;
     TK_CUDA(cudaEventRecord(c.ev_fork, c.stream));
     for (int i = 0; i < used; ++i) TK_CUDA(cudaStreamWaitEvent(c.aux[i], c.ev_fork, 0));
 }
@@ -27,6 +28,7 @@ void ctx_fork_begin(Ctx& c, int used) {
 // call's stream again (also on the error path, hence no throw before that).
 void ctx_fork_end(Ctx& c, cudaStream_t main, int used) {
     c.stream = main;
+    c.chained = false;
     cudaError_t first = cudaSuccess;
     for (int i = 0; i < used; ++i) {
         cudaError_t e = cudaEventRecord(c.ev_join[i], c.aux[i]);
@@ -39,6 +41,7 @@ void ctx_fork_end(Ctx& c, cudaStream_t main, int used) {
 // The side stream (the last auxiliary stream) waits for the call's stream and
 // becomes the call's stream; ctx_side_end joins it back into `main`.
 void ctx_side_begin(Ctx& c) {
+    c.chained = false;
     TK_CUDA(cudaEventRecord(c.ev_fork, c.stream));
     TK_CUDA(cudaStreamWaitEvent(c.aux[Ctx::kFork], c.ev_fork, 0));
     c.stream = c.aux[Ctx::kFork];
@@ -46,6 +49,7 @@ void ctx_side_begin(Ctx& c) {
 
 void ctx_side_end(Ctx& c, cudaStream_t main) {
     c.stream = main;
+    c.chained = false;
     cudaError_t e = cudaEventRecord(c.ev_join[Ctx::kFork], c.aux[Ctx::kFork]);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(main, c.ev_join[Ctx::kFork], 0);
     if (e != cudaSuccess) fail(TK_ERR_CUDA, std::string("side join: ") + cudaGetErrorString(e));
@@ -115,6 +119,7 @@ template <typename Tx, typename Ta, bool KFAST>
 __global__ void __launch_bounds__(256) ttm_simt_kernel(const Tx* __restrict__ X, int64_t L, int64_t nj, int64_t R,
                                                        const Ta* __restrict__ M, int64_t ldm, int mtrans, int64_t m,
                                                        Ta* __restrict__ out, Ta xinv) {
+    kernel_begin();
     constexpr int BM = 64, BN = 32, BK = 16;
     __shared__ Ta Xs[BK][BM + 1];
     __shared__ Ta Ms[BK][BN + 1];
@@ -194,6 +199,7 @@ template <typename Tx, typename Ta>
 __global__ void __launch_bounds__(256) ttm_direct_kernel(const Tx* __restrict__ X, int64_t L, int64_t nj, int64_t R,
                                                          const Ta* __restrict__ M, int64_t ldm, int mtrans, int64_t m,
                                                          Ta* __restrict__ out, Ta xinv) {
+    kernel_begin();
     const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (o >= L * m * R) return;
     const int64_t l = o % L, rest = o / L;
@@ -217,6 +223,7 @@ __global__ void __launch_bounds__(SLAB_THREADS) ttm_slab_kernel(const Tx* __rest
                                                                 int64_t R, const Ta* __restrict__ M, int64_t ldm,
                                                                 int mtrans, int64_t m, int S, Ta* __restrict__ out,
                                                                 Ta xinv) {
+    kernel_begin();
     extern __shared__ __align__(16) unsigned char slab_raw[];
     Ta* xs = reinterpret_cast<Ta*>(slab_raw);  // L x nj, X[l, i] at xs[l + L i]
     Ta* part = xs + L * nj;                    // S x (L m) partial sums
@@ -261,8 +268,8 @@ static void ttm_dispatch(const Ctx& c, const Tx* X, int64_t L, int64_t nj, int64
         const size_t smem = sizeof(Ta) * (size_t)(L * nj + (int64_t)S * L * m);
         const char* name = (const void*)X == c.xdata ? "xpass_simt" : "ttm_simt";
         ProfScope ps(c, name, (double)rows * nj * sizeof(Tx) + (double)rows * m * sizeof(Ta), 2.0 * rows * nj * m);
-        ttm_slab_kernel<Tx, Ta><<<(unsigned)R, SLAB_THREADS, smem, c.stream>>>(X, L, nj, R, M, ldm, mtrans ? 1 : 0, m,
-                                                                               S, out, xinv);
+        run_kernel(c, ttm_slab_kernel<Tx, Ta>, (unsigned)R, SLAB_THREADS, smem, X, L, nj, R, M, ldm, mtrans ? 1 : 0,
+                   m, S, out, xinv);
         c.counted();
         c.check_launch();
         return;
@@ -270,8 +277,8 @@ static void ttm_dispatch(const Ctx& c, const Tx* X, int64_t L, int64_t nj, int64
     if (rows * m <= (1 << 21) && nj <= 512) {
         const char* name = (const void*)X == c.xdata ? "xpass_simt" : "ttm_simt";
         ProfScope ps(c, name, (double)rows * nj * sizeof(Tx) + (double)rows * m * sizeof(Ta), 2.0 * rows * nj * m);
-        ttm_direct_kernel<Tx, Ta><<<(unsigned)((rows * m + 255) / 256), 256, 0, c.stream>>>(X, L, nj, R, M, ldm,
-                                                                                           mtrans, m, out, xinv);
+        run_kernel(c, ttm_direct_kernel<Tx, Ta>, (unsigned)((rows * m + 255) / 256), 256, 0, X, L, nj, R, M, ldm,
+                   mtrans, m, out, xinv);
         c.counted();
         c.check_launch();
         return;
@@ -282,9 +289,9 @@ static void ttm_dispatch(const Ctx& c, const Tx* X, int64_t L, int64_t nj, int64
     dim3 grid((unsigned)((rows + 63) / 64), (unsigned)((m + 31) / 32));
     TK_REQUIRE(grid.y <= 65535, TK_ERR_SHAPE, "ttm: too many output columns");
     if (L == 1)
-        ttm_simt_kernel<Tx, Ta, true><<<grid, 256, 0, c.stream>>>(X, L, nj, R, M, ldm, mtrans, m, out, xinv);
+        run_kernel(c, ttm_simt_kernel<Tx, Ta, true>, grid, 256, 0, X, L, nj, R, M, ldm, mtrans, m, out, xinv);
     else
-        ttm_simt_kernel<Tx, Ta, false><<<grid, 256, 0, c.stream>>>(X, L, nj, R, M, ldm, mtrans, m, out, xinv);
+        run_kernel(c, ttm_simt_kernel<Tx, Ta, false>, grid, 256, 0, X, L, nj, R, M, ldm, mtrans, m, out, xinv);
     c.counted();
     c.check_launch();
 }
@@ -349,6 +356,7 @@ SignMap sign_map(const Tens& X, int n, int j0, uint64_t seed) {
 template <typename W>
 __global__ void sign_copy_kernel(const W* __restrict__ X, W* __restrict__ dst, int64_t numel, int64_t stride, int64_t nn,
                                  uint32_t key, W top) {
+    kernel_begin();
     for (int64_t lin = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; lin < numel;
          lin += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t c = (uint32_t)(lin % stride + stride * (lin / (stride * nn)));
@@ -366,24 +374,20 @@ void launch_sign_copy(const Ctx& c, const Tens& X, int n, uint64_t seed, void* d
     ProfScope ps(c, "elementwise", 2.0 * numel * dtype_size(X.dt), 0.0);
     switch (dtype_size(X.dt)) {
         case 8:
-            sign_copy_kernel<uint64_t><<<grid, 256, 0, c.stream>>>(static_cast<const uint64_t*>(X.p),
-                                                                   static_cast<uint64_t*>(dst), numel, stride, nn, key,
-                                                                   (uint64_t)1 << 63);
+            run_kernel(c, sign_copy_kernel<uint64_t>, grid, 256, 0, static_cast<const uint64_t*>(X.p),
+                       static_cast<uint64_t*>(dst), numel, stride, nn, key, (uint64_t)1 << 63);
             break;
         case 4:
-            sign_copy_kernel<uint32_t><<<grid, 256, 0, c.stream>>>(static_cast<const uint32_t*>(X.p),
-                                                                   static_cast<uint32_t*>(dst), numel, stride, nn, key,
-                                                                   0x80000000u);
+            run_kernel(c, sign_copy_kernel<uint32_t>, grid, 256, 0, static_cast<const uint32_t*>(X.p),
+                       static_cast<uint32_t*>(dst), numel, stride, nn, key, 0x80000000u);
             break;
         case 2:
-            sign_copy_kernel<uint16_t><<<grid, 256, 0, c.stream>>>(static_cast<const uint16_t*>(X.p),
-                                                                   static_cast<uint16_t*>(dst), numel, stride, nn, key,
-                                                                   (uint16_t)0x8000);
+            run_kernel(c, sign_copy_kernel<uint16_t>, grid, 256, 0, static_cast<const uint16_t*>(X.p),
+                       static_cast<uint16_t*>(dst), numel, stride, nn, key, (uint16_t)0x8000);
             break;
         default:
-            sign_copy_kernel<uint8_t><<<grid, 256, 0, c.stream>>>(static_cast<const uint8_t*>(X.p),
-                                                                  static_cast<uint8_t*>(dst), numel, stride, nn, key,
-                                                                  (uint8_t)0x80);
+            run_kernel(c, sign_copy_kernel<uint8_t>, grid, 256, 0, static_cast<const uint8_t*>(X.p),
+                       static_cast<uint8_t*>(dst), numel, stride, nn, key, (uint8_t)0x80);
             break;
     }
     c.counted();
@@ -394,6 +398,7 @@ void launch_sign_copy(const Ctx& c, const Tens& X, int n, uint64_t seed, void* d
 
 __global__ void gemm_reduce_kernel(int64_t m, int64_t n, int nsplit, const double* P, double alpha, double beta,
                                    double* C, int64_t ldc, const int* skip) {
+    kernel_begin();
     if (skip && *skip) return;
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= m * n) return;
@@ -519,6 +524,7 @@ __device__ __forceinline__ void df_dot_step(float& s, float& c, float2 a, float2
 __global__ void __launch_bounds__(256) ttm_direct_df_kernel(const double* __restrict__ X, int64_t L, int64_t nj,
                                                             int64_t R, const double* __restrict__ M, int64_t ldm,
                                                             int mtrans, int64_t m, double* __restrict__ out) {
+    kernel_begin();
     extern __shared__ float2 msp[];  // nj x m: msp[i + nj a] = split M(i, a)
     for (int64_t e = threadIdx.x; e < nj * m; e += blockDim.x) {
         const int64_t i = e % nj, a = e / nj;
@@ -550,8 +556,8 @@ static bool ttm_direct_df(const Ctx& c, const double* X, int64_t L, int64_t nj, 
     const size_t smem = sizeof(float2) * (size_t)(nj * m);
     if (rows * m > (1 << 22) || smem > 48 * 1024) return false;
     ProfScope ps(c, "ttm_simt", 8.0 * rows * nj + 8.0 * rows * m, 2.0 * rows * nj * m);
-    ttm_direct_df_kernel<<<(unsigned)((rows * m + 255) / 256), 256, smem, c.stream>>>(X, L, nj, R, M, ldm,
-                                                                                     mtrans ? 1 : 0, m, out);
+    run_kernel(c, ttm_direct_df_kernel, (unsigned)((rows * m + 255) / 256), 256, smem, X, L, nj, R, M, ldm,
+               mtrans ? 1 : 0, m, out);
     c.counted();
     c.check_launch();
     return true;
@@ -572,6 +578,7 @@ template <int MODE>
 __global__ void __launch_bounds__(256) gemm_tile16_kernel(int64_t m, int64_t n, int64_t K, int64_t kchunk, View2 A,
                                                           View2 B, double alpha, double beta, double* C, int64_t ldc,
                                                           double* P, unsigned* ctr, const int* skip) {
+    kernel_begin();
     constexpr bool DFACC = MODE != 0;
     using E = typename std::conditional<MODE == 0, double, typename std::conditional<MODE == 1, float, float2>::type>::type;
     if (skip && *skip) return;
@@ -656,6 +663,7 @@ template <int T>
 __global__ void __launch_bounds__(256) gemm_small_kernel(int64_t m, int64_t n, int64_t K, View2 A, View2 B,
                                                          double alpha, double beta, double* C, int64_t ldc,
                                                          const int* skip) {
+    kernel_begin();
     if (skip && *skip) return;
     constexpr int G = 256 / (T * T);
     __shared__ double As[32][T + 1];
@@ -713,9 +721,9 @@ void gemm_nt_f64(Ctx& c, int64_t m, int64_t n, int64_t K, const View2& A, const 
         ProfScope ps(c, "gemm_f64", 8.0 * (double)(m * ((n + T - 1) / T) + n * ((m + T - 1) / T)) * K + 8.0 * m * n,
                      2.0 * m * n * K);
         if (t8)
-            gemm_small_kernel<8><<<grid, 256, 0, c.stream>>>(m, n, K, A, B, alpha, beta, C, ldc, skip);
+            run_kernel(c, gemm_small_kernel<8>, grid, 256, 0, m, n, K, A, B, alpha, beta, C, ldc, skip);
         else
-            gemm_small_kernel<4><<<grid, 256, 0, c.stream>>>(m, n, K, A, B, alpha, beta, C, ldc, skip);
+            run_kernel(c, gemm_small_kernel<4>, grid, 256, 0, m, n, K, A, B, alpha, beta, C, ldc, skip);
         c.counted();
         c.check_launch();
         return;
@@ -740,22 +748,22 @@ void gemm_nt_f64(Ctx& c, int64_t m, int64_t n, int64_t K, const View2& A, const 
                      8.0 * (double)(m * ((n + 15) / 16) + n * ((m + 15) / 16)) * K + 8.0 * m * n * nsplit,
                      2.0 * m * n * K);
         if (mode == 1)
-            gemm_tile16_kernel<1>
-                <<<grid, 256, 0, c.stream>>>(m, n, K, kchunk, A, B, alpha, beta, C, ldc, P, ctr, skip);
+            run_kernel(c, gemm_tile16_kernel<1>, grid, 256, 0, m, n, K, kchunk, A, B, alpha, beta, C, ldc, P, ctr,
+                       skip);
         else if (mode == 2)
-            gemm_tile16_kernel<2>
-                <<<grid, 256, 0, c.stream>>>(m, n, K, kchunk, A, B, alpha, beta, C, ldc, P, ctr, skip);
+            run_kernel(c, gemm_tile16_kernel<2>, grid, 256, 0, m, n, K, kchunk, A, B, alpha, beta, C, ldc, P, ctr,
+                       skip);
         else
-            gemm_tile16_kernel<0>
-                <<<grid, 256, 0, c.stream>>>(m, n, K, kchunk, A, B, alpha, beta, C, ldc, P, ctr, skip);
+            run_kernel(c, gemm_tile16_kernel<0>, grid, 256, 0, m, n, K, kchunk, A, B, alpha, beta, C, ldc, P, ctr,
+                       skip);
         c.counted();
         c.check_launch();
     }
     if (nsplit > 1 && !ctr) {
         const int64_t tot = m * n;
         ProfScope ps(c, "gemm_f64", 8.0 * m * n * (nsplit + 1), (double)m * n * nsplit);
-        gemm_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, c.stream>>>(m, n, (int)nsplit, P, alpha, beta, C,
-                                                                                  ldc, skip);
+        run_kernel(c, gemm_reduce_kernel, (unsigned)((tot + 255) / 256), 256, 0, m, n, (int)nsplit, P, alpha, beta, C,
+                   ldc, skip);
         c.counted();
         c.check_launch();
     }
@@ -809,6 +817,7 @@ constexpr int CHOL_THREADS = 256;
 
 __global__ void __launch_bounds__(CHOL_THREADS) chol_inv_kernel(KDims kd, int kmax, const double* W, double* Rinv,
                                                                 int* bad, double tol) {
+    kernel_begin();
     extern __shared__ double sm[];  // A: k x k (upper part becomes R), M: k x k lower (L^{-1})
     __shared__ double dg[256];
     __shared__ double s_y;
@@ -980,6 +989,7 @@ __device__ __forceinline__ void chdf_step(float2 (&v)[CHDF_Q], const float2* row
 
 __global__ void __launch_bounds__(CHDF_THREADS) chol_inv_df_kernel(KDims kd, int kmax, const double* W,
                                                                    double* Rinv, int* bad, double tol) {
+    kernel_begin();
     extern __shared__ float2 sf[];  // the rows, ld apart
     __shared__ float2 s_ys[112];    // 1 / sqrt(p_j)
     __shared__ float2 s_inv[CHDF_PANEL];         // 1 / p_j of the panel's columns
@@ -1088,7 +1098,7 @@ void launch_chol_inv(const Ctx& c, int batch, const KDims& kd, int kmax, const d
         if (smem > 48 * 1024)
             TK_CUDA(cudaFuncSetAttribute(chol_inv_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         ProfScope ps(c, "chol_inv", 16.0 * batch * kmax * kmax, (2.0 / 3.0) * batch * kmax * kmax * kmax);
-        chol_inv_df_kernel<<<batch, CHDF_THREADS, smem, c.stream>>>(kd, kmax, W, Rinv, bad, tol);
+        run_kernel(c, chol_inv_df_kernel, batch, CHDF_THREADS, smem, kd, kmax, W, Rinv, bad, tol);
         c.counted();
         c.check_launch();
         return;
@@ -1097,7 +1107,7 @@ void launch_chol_inv(const Ctx& c, int batch, const KDims& kd, int kmax, const d
     if (smem > 48 * 1024)
         TK_CUDA(cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ProfScope ps(c, "chol_inv", 16.0 * batch * kmax * kmax, (2.0 / 3.0) * batch * kmax * kmax * kmax);
-    chol_inv_kernel<<<batch, CHOL_THREADS, smem, c.stream>>>(kd, kmax, W, Rinv, bad, tol);
+    run_kernel(c, chol_inv_kernel, batch, CHOL_THREADS, smem, kd, kmax, W, Rinv, bad, tol);
     c.counted();
     c.check_launch();
 }
@@ -1106,6 +1116,7 @@ void launch_chol_inv(const Ctx& c, int batch, const KDims& kd, int kmax, const d
 
 __global__ void __launch_bounds__(256) apply_rinv_kernel(int64_t n, int64_t k, int rpc, View2 Y, const double* Rinv,
                                                          int64_t ldr, double* Q, const int* skip) {
+    kernel_begin();
     extern __shared__ double ys[];  // rpc x k
     if (skip && *skip) return;
     const int64_t i0 = (int64_t)blockIdx.x * rpc;
@@ -1132,7 +1143,7 @@ void launch_apply_rinv(const Ctx& c, int64_t n, int64_t k, const View2& Y, const
     if (smem > 48 * 1024)
         TK_CUDA(cudaFuncSetAttribute(apply_rinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ProfScope ps(c, "apply_rinv", 16.0 * n * k + 8.0 * k * k, (double)n * k * k);
-    apply_rinv_kernel<<<(unsigned)((n + rpc - 1) / rpc), 256, smem, c.stream>>>(n, k, rpc, Y, Rinv, ldr, Q, skip);
+    run_kernel(c, apply_rinv_kernel, (unsigned)((n + rpc - 1) / rpc), 256, smem, n, k, rpc, Y, Rinv, ldr, Q, skip);
     c.counted();
     c.check_launch();
 }
@@ -1158,6 +1169,7 @@ constexpr int APDF_THREADS = 256;
 constexpr int APDF_U = 8;  // global loads in flight per thread while staging
 
 __global__ void __launch_bounds__(APDF_THREADS) apply_rinv_df_kernel(ApplyBatch ab) {
+    kernel_begin();
     extern __shared__ float2 sa[];  // R^{-1}: k x k column-major, then Y rows: k x 32 ([col][row])
     const int b = blockIdx.y;
     if (ab.skip[b] && *ab.skip[b]) return;
@@ -1261,7 +1273,7 @@ void launch_apply_rinv_df(const Ctx& c, int batch, const View2* Y, const int64_t
     }
     ProfScope ps(c, "apply_rinv", bytes, flops);
     dim3 grid((unsigned)((nmax + 31) / 32), (unsigned)batch);
-    apply_rinv_df_kernel<<<grid, APDF_THREADS, smem, c.stream>>>(ab);
+    run_kernel(c, apply_rinv_df_kernel, grid, APDF_THREADS, smem, ab);
     c.counted();
     c.check_launch();
 }
@@ -1270,6 +1282,7 @@ void launch_apply_rinv_df(const Ctx& c, int batch, const View2* Y, const int64_t
 
 __global__ void __launch_bounds__(256) householder_kernel(int64_t n, int64_t k, View2 Y, double* A, double* Q,
                                                           double* tau, const int* run, int* slot, int slot_value) {
+    kernel_begin();
     __shared__ double red[33];
     __shared__ double v0s[256];
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -1349,7 +1362,7 @@ void launch_householder(const Ctx& c, int64_t n, int64_t k, const View2& Y, doub
     if (!c.exec) return;
     TK_REQUIRE(k <= 256, TK_ERR_SHAPE, "householder: at most 256 columns");
     ProfScope ps(c, "householder", 16.0 * n * k, 8.0 * n * k * k);
-    householder_kernel<<<1, 256, 0, c.stream>>>(n, k, Y, A, Q, tau, run, slot, slot_value);
+    run_kernel(c, householder_kernel, 1, 256, 0, n, k, Y, A, Q, tau, run, slot, slot_value);
     c.counted();
     c.check_launch();
 }
@@ -1373,6 +1386,7 @@ __device__ __forceinline__ double jac_rcp(double a) {
 
 __global__ void __launch_bounds__(256) jacobi_kernel(int k, double* Ag, double* w, double* Vout, int max_sweeps,
                                                      int use_smem, double* gV, unsigned* flags) {
+    kernel_begin();
     extern __shared__ double sm[];
     __shared__ double cs[128], sn[128];
     __shared__ int P[128], Qp[128];
@@ -1507,8 +1521,8 @@ void launch_jacobi(const Ctx& c, int64_t k, double* A, double* w, double* V, int
     if (smem > 48 * 1024)
         TK_CUDA(cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ProfScope ps(c, "jacobi", 24.0 * k * k, 9.0 * k * k * k * 8);
-    jacobi_kernel<<<1, 256, smem, c.stream>>>((int)k, A, w, V, max_sweeps, use_smem, use_smem ? nullptr : gV,
-                                              c.dflags);
+    run_kernel(c, jacobi_kernel, 1, 256, smem, (int)k, A, w, V, max_sweeps, use_smem, use_smem ? nullptr : gV,
+               c.dflags);
     c.counted();
     c.check_launch();
 }
@@ -1688,6 +1702,7 @@ __global__ void __launch_bounds__(JM_MAX_THREADS) jacobi_sweep_kernel(int k, con
                                                                       double* Dout, double tol, int max_sweeps,
                                                                       float2* __restrict__ rlog,
                                                                       int* __restrict__ ginfo, unsigned* flags) {
+    kernel_begin();
     extern __shared__ __align__(16) unsigned char smraw[];
     const int kp = k + (k & 1), h = kp / 2, m = kp - 1;
     const int ps = h * (h + 1) / 2;               // blocks (pair t, pair u >= t)
@@ -1941,6 +1956,7 @@ __global__ void __launch_bounds__(JR_WARPS * 32) jacobi_replay_kernel(int k, con
                                                                       const double* __restrict__ V1,
                                                                       const double* __restrict__ D, int r,
                                                                       double* Vt, double* Vr) {
+    kernel_begin();
     extern __shared__ __align__(16) unsigned char smraw[];
     const int kp = k + (k & 1), h = kp / 2;
     const int nt = JR_WARPS * 32, cr = JR_STAGE * nt / h;  // steps per chunk
@@ -2059,14 +2075,14 @@ void launch_jacobi_mixed(Ctx& c, int64_t k, const double* A, double* D, float* J
             if (smem > 48 * 1024)
                 TK_CUDA(cudaFuncSetAttribute(jacobi_sweep_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem));
-            jacobi_sweep_kernel<true>
-                <<<1, nt, smem, c.stream>>>((int)k, A, D, tol, max_sweeps, rlog, ginfo, c.dflags);
+            run_kernel(c, jacobi_sweep_kernel<true>, 1, nt, smem, (int)k, A, D, tol, max_sweeps, rlog, ginfo,
+                       c.dflags);
         } else {
             if (smem > 48 * 1024)
                 TK_CUDA(cudaFuncSetAttribute(jacobi_sweep_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem));
-            jacobi_sweep_kernel<false>
-                <<<1, nt, smem, c.stream>>>((int)k, A, D, tol, max_sweeps, rlog, ginfo, c.dflags);
+            run_kernel(c, jacobi_sweep_kernel<false>, 1, nt, smem, (int)k, A, D, tol, max_sweeps, rlog, ginfo,
+                       c.dflags);
         }
         c.counted();
         c.check_launch();
@@ -2077,14 +2093,15 @@ void launch_jacobi_mixed(Ctx& c, int64_t k, const double* A, double* D, float* J
     const size_t rsmem = sizeof(float2) * cr * h + sizeof(long long) * kp;
     ProfScope ps(c, "jacobi", 8.0 * h * (max_sweeps * (kp - 1) + 1) + 8.0 * k * k, 6.0 * k * k * k * max_sweeps);
     const auto replay = h > 32 ? jacobi_replay_kernel<true> : jacobi_replay_kernel<false>;
-    replay<<<(unsigned)((k + JR_WARPS - 1) / JR_WARPS), JR_WARPS * 32, rsmem, c.stream>>>(
-        (int)k, rlog, ginfo, J, J64a, J64b, V1, D, (int)r, Vt, Vr);
+    run_kernel(c, replay, (unsigned)((k + JR_WARPS - 1) / JR_WARPS), JR_WARPS * 32, rsmem, (int)k, rlog, ginfo, J,
+               J64a, J64b, V1, D, (int)r, Vt, Vr);
     c.counted();
     c.check_launch();
 }
 
 // Vr[:, rank] = V[:, i] for the r largest D (ties: lower index first).
 __global__ void select_top_kernel(int64_t k, int64_t r, const double* D, const double* V, double* Vr, double* Vr2) {
+    kernel_begin();
     for (int64_t i = blockIdx.x; i < k; i += gridDim.x) {
         double di = D[i];
         int64_t rank = 0;
@@ -2105,7 +2122,7 @@ void launch_select_top(const Ctx& c, int64_t k, int64_t r, const double* D, cons
                        double* Vr2) {
     if (!c.exec || k == 0 || r == 0) return;
     ProfScope ps(c, "elementwise", 16.0 * k * r, 0.0);
-    select_top_kernel<<<(unsigned)k, 64, 0, c.stream>>>(k, r, D, V, Vr, Vr2);
+    run_kernel(c, select_top_kernel, (unsigned)k, 64, 0, k, r, D, V, Vr, Vr2);
     c.counted();
     c.check_launch();
 }
@@ -2114,6 +2131,7 @@ void launch_select_top(const Ctx& c, int64_t k, int64_t r, const double* D, cons
 
 __global__ void convert_kernel(const void* src, tk_dtype sdt, int64_t rows, int64_t cols, int64_t lds, void* dst,
                                tk_dtype ddt, int64_t ldd, float inv) {
+    kernel_begin();
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= rows * cols) return;
     int64_t i = idx % rows, j = idx / rows;
@@ -2126,13 +2144,14 @@ void launch_convert(const Ctx& c, const void* src, tk_dtype sdt, int64_t rows, i
     float inv = (sdt == TK_FP8_E4M3) ? 1.f / src_scale : 1.f;
     int64_t tot = rows * cols;
     ProfScope ps(c, "elementwise", (double)tot * (dtype_size(sdt) + dtype_size(ddt)), 0.0);
-    convert_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, c.stream>>>(src, sdt, rows, cols, lds, dst, ddt, ldd,
-                                                                         inv);
+    run_kernel(c, convert_kernel, (unsigned)((tot + 255) / 256), 256, 0, src, sdt, rows, cols, lds, dst, ddt, ldd,
+               inv);
     c.counted();
     c.check_launch();
 }
 
 __global__ void fill_identity_kernel(double* Q, int64_t n) {
+    kernel_begin();
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n * n) return;
     Q[idx] = (idx % n == idx / n) ? 1.0 : 0.0;
@@ -2141,12 +2160,13 @@ __global__ void fill_identity_kernel(double* Q, int64_t n) {
 void launch_fill_identity(const Ctx& c, double* Q, int64_t n) {
     if (!c.exec || n == 0) return;
     ProfScope ps(c, "elementwise", 8.0 * n * n, 0.0);
-    fill_identity_kernel<<<(unsigned)((n * n + 255) / 256), 256, 0, c.stream>>>(Q, n);
+    run_kernel(c, fill_identity_kernel, (unsigned)((n * n + 255) / 256), 256, 0, Q, n);
     c.counted();
     c.check_launch();
 }
 
 __global__ void copy_unfold_kernel(View2 Y, int64_t n, int64_t k, double* A, const int* run) {
+    kernel_begin();
     if (run && !*run) return;
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= n * k) return;
@@ -2156,33 +2176,36 @@ __global__ void copy_unfold_kernel(View2 Y, int64_t n, int64_t k, double* A, con
 void launch_copy_unfold_to_matrix(const Ctx& c, const View2& Y, int64_t n, int64_t k, double* A, const int* run) {
     if (!c.exec || n * k == 0) return;
     ProfScope ps(c, "elementwise", 16.0 * n * k, 0.0);
-    copy_unfold_kernel<<<(unsigned)((n * k + 255) / 256), 256, 0, c.stream>>>(Y, n, k, A, run);
+    run_kernel(c, copy_unfold_kernel, (unsigned)((n * k + 255) / 256), 256, 0, Y, n, k, A, run);
     c.counted();
     c.check_launch();
 }
 
 __global__ void fill_int_kernel(int* p, int count, int v) {
+    kernel_begin();
     for (int i = threadIdx.x; i < count; i += blockDim.x) p[i] = v;
 }
 void launch_fill_int(const Ctx& c, int* p, int count, int value) {
     if (!c.exec || count <= 0) return;
     ProfScope ps(c, "elementwise", 4.0 * count, 0.0);
-    fill_int_kernel<<<1, 32, 0, c.stream>>>(p, count, value);
+    run_kernel(c, fill_int_kernel, 1, 32, 0, p, count, value);
     c.counted();
     c.check_launch();
 }
 
-__global__ void qr_info_kernel(int* slot, const int* bad, int bad_value) { *slot = *bad ? bad_value : 0; }
+__global__ void qr_info_kernel(int* slot, const int* bad, int bad_value) {
+    kernel_begin(); *slot = *bad ? bad_value : 0; }
 void launch_qr_info(const Ctx& c, int* slot, const int* bad, int bad_value) {
     if (!c.exec) return;
     ProfScope ps(c, "elementwise", 8.0, 0.0);
-    qr_info_kernel<<<1, 1, 0, c.stream>>>(slot, bad, bad_value);
+    run_kernel(c, qr_info_kernel, 1, 1, 0, slot, bad, bad_value);
     c.counted();
     c.check_launch();
 }
 
 __global__ void __launch_bounds__(256) sign_fix_kernel(double* U, int64_t n, double* sign, void* out, tk_dtype odt,
                                                        int64_t ldo) {
+    kernel_begin();
     __shared__ double bv[256];
     __shared__ int64_t bi[256];
     const int64_t col = blockIdx.x;
@@ -2221,7 +2244,7 @@ void launch_sign_fix(const Ctx& c, double* U, int64_t n, int64_t r, double* sign
                      int64_t ldo) {
     if (!c.exec || r == 0) return;
     ProfScope ps(c, "elementwise", 16.0 * n * r, 0.0);
-    sign_fix_kernel<<<(unsigned)r, 256, 0, c.stream>>>(U, n, sign, out, odt, ldo);
+    run_kernel(c, sign_fix_kernel, (unsigned)r, 256, 0, U, n, sign, out, odt, ldo);
     c.counted();
     c.check_launch();
 }
@@ -2233,6 +2256,7 @@ struct SignPtrs {
 };
 
 __global__ void apply_signs_kernel(double* G, int64_t tot, SignPtrs sp, void* out, tk_dtype odt) {
+    kernel_begin();
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= tot) return;
     int64_t rem = idx;
@@ -2258,7 +2282,7 @@ void launch_apply_signs(const Ctx& c, double* G, const Tens& shape, double* cons
     int64_t tot = shape.numel();
     if (tot == 0) return;
     ProfScope ps(c, "elementwise", 16.0 * tot, (double)tot * shape.d);
-    apply_signs_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, c.stream>>>(G, tot, sp, out, odt);
+    run_kernel(c, apply_signs_kernel, (unsigned)((tot + 255) / 256), 256, 0, G, tot, sp, out, odt);
     c.counted();
     c.check_launch();
 }
@@ -2267,6 +2291,7 @@ void launch_apply_signs(const Ctx& c, double* G, const Tens& shape, double* cons
 template <typename Tx, typename Ty>
 __global__ void __launch_bounds__(256) residual_partial_kernel(const Tx* X, const Ty* Y, int64_t tot, float xinv,
                                                                double* part) {
+    kernel_begin();
     __shared__ double red[33];
     double sr = 0.0, sx = 0.0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -2300,6 +2325,7 @@ __global__ void __launch_bounds__(256) residual_partial_kernel(const Tx* X, cons
 // Sum of nb (a, b) pairs: fixed strided per-thread sums, then warp and block
 // trees in a fixed order (deterministic for a given nb).
 __global__ void __launch_bounds__(256) residual_final_kernel(const double* part, int nb, double* out2) {
+    kernel_begin();
     __shared__ double sa[8], sb[8];
     double a = 0.0, b = 0.0;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) {
@@ -2331,7 +2357,7 @@ __global__ void __launch_bounds__(256) residual_final_kernel(const double* part,
 void launch_sum_pairs(const Ctx& c, const double* part, int nb, double* out2) {
     if (!c.exec) return;
     ProfScope ps(c, "elementwise", 16.0 * nb, 2.0 * nb);
-    residual_final_kernel<<<1, 256, 0, c.stream>>>(part, nb, out2);
+    run_kernel(c, residual_final_kernel, 1, 256, 0, part, nb, out2);
     c.counted();
     c.check_launch();
 }
@@ -2345,34 +2371,35 @@ void launch_residual_norms(Ctx& c, const Tens& X, const void* Y, tk_dtype ydt, d
     ProfScope ps(c, "residual", (double)tot * (dtype_size(X.dt) + dtype_size(ydt)), 4.0 * tot);
     if (X.dt == TK_F64) {
         TK_REQUIRE(ydt == TK_F64, TK_ERR_DTYPE, "residual: F64 data needs F64 reconstruction");
-        residual_partial_kernel<double, double><<<nb, 256, 0, c.stream>>>((const double*)X.p, (const double*)Y, tot,
-                                                                          1.f, part);
+        run_kernel(c, residual_partial_kernel<double, double>, nb, 256, 0, (const double*)X.p, (const double*)Y, tot,
+                   1.f, part);
     } else {
         TK_REQUIRE(ydt == TK_F32, TK_ERR_DTYPE, "residual: reconstruction must be F32");
         switch (X.dt) {
             case TK_F32:
-                residual_partial_kernel<float, float><<<nb, 256, 0, c.stream>>>((const float*)X.p, (const float*)Y,
-                                                                                tot, inv, part);
+                run_kernel(c, residual_partial_kernel<float, float>, nb, 256, 0, (const float*)X.p, (const float*)Y,
+                           tot, inv, part);
                 break;
             case TK_BF16:
-                residual_partial_kernel<__nv_bfloat16, float><<<nb, 256, 0, c.stream>>>(
-                    (const __nv_bfloat16*)X.p, (const float*)Y, tot, inv, part);
+                run_kernel(c, residual_partial_kernel<__nv_bfloat16, float>, nb, 256, 0, (const __nv_bfloat16*)X.p,
+                           (const float*)Y, tot, inv, part);
                 break;
             default:
-                residual_partial_kernel<__nv_fp8_e4m3, float><<<nb, 256, 0, c.stream>>>(
-                    (const __nv_fp8_e4m3*)X.p, (const float*)Y, tot, inv, part);
+                run_kernel(c, residual_partial_kernel<__nv_fp8_e4m3, float>, nb, 256, 0, (const __nv_fp8_e4m3*)X.p,
+                           (const float*)Y, tot, inv, part);
                 break;
         }
     }
     c.counted();
     c.check_launch();
-    residual_final_kernel<<<1, 32, 0, c.stream>>>(part, nb, out2);
+    run_kernel(c, residual_final_kernel, 1, 32, 0, part, nb, out2);
     c.counted();
     c.check_launch();
 }
 
 __global__ void axpby_residual_kernel(const void* X, tk_dtype xdt, float xinv, const void* Y, tk_dtype ydt,
                                       int64_t tot, double alpha, void* dst, tk_dtype ddt) {
+    kernel_begin();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= tot) return;
     if (xdt == TK_F64 || ydt == TK_F64) {  // difference formed in FP64 when either side carries it
@@ -2390,13 +2417,14 @@ void launch_axpby_residual(const Ctx& c, const Tens& X, const void* Y, tk_dtype 
     if (tot == 0) return;
     float inv = X.dt == TK_FP8_E4M3 ? 1.f / X.scale : 1.f;
     ProfScope ps(c, "residual", (double)tot * (dtype_size(X.dt) + dtype_size(ydt) + dtype_size(ddt)), 2.0 * tot);
-    axpby_residual_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, c.stream>>>(X.p, X.dt, inv, Y, ydt, tot, alpha, dst,
-                                                                                ddt);
+    run_kernel(c, axpby_residual_kernel, (unsigned)((tot + 255) / 256), 256, 0, X.p, X.dt, inv, Y, ydt, tot, alpha,
+               dst, ddt);
     c.counted();
     c.check_launch();
 }
 
 __global__ void scale_copy_kernel(const void* src, tk_dtype sdt, int64_t n, double alpha, void* dst, tk_dtype ddt) {
+    kernel_begin();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     st_any(dst, ddt, i, alpha * ld_any(src, sdt, i));
@@ -2406,7 +2434,7 @@ void launch_scale_copy(const Ctx& c, const void* src, tk_dtype sdt, int64_t n, d
                        tk_dtype ddt) {
     if (!c.exec || n == 0) return;
     ProfScope ps(c, "elementwise", (double)n * (dtype_size(sdt) + dtype_size(ddt)), (double)n);
-    scale_copy_kernel<<<(unsigned)((n + 255) / 256), 256, 0, c.stream>>>(src, sdt, n, alpha, dst, ddt);
+    run_kernel(c, scale_copy_kernel, (unsigned)((n + 255) / 256), 256, 0, src, sdt, n, alpha, dst, ddt);
     c.counted();
     c.check_launch();
 }

@@ -45,6 +45,7 @@ __device__ __forceinline__ uint4 philox_block(unsigned long long seed, unsigned 
 
 __global__ void philox_blocks_kernel(unsigned long long seed, unsigned stream, unsigned long long offset,
                                      int64_t nblocks, uint4* out) {
+    kernel_begin();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nblocks; i += (int64_t)gridDim.x * blockDim.x)
         out[i] = philox_block(seed, stream, offset + (unsigned long long)i);
 }
@@ -67,6 +68,7 @@ struct GfBatch {
 };
 
 __global__ void gaussian_factor_kernel(unsigned long long seed, GfBatch gb) {
+    kernel_begin();
     const int f = blockIdx.y;
     const int64_t rows = gb.rows[f], cols = gb.cols[f], ld = gb.ld[f];
     const unsigned stream = gb.stream[f];
@@ -99,7 +101,7 @@ void launch_philox_blocks(const Ctx& c, unsigned long long seed, unsigned stream
     if (!c.exec || nblocks == 0) return;
     const unsigned grid = (unsigned)std::min<int64_t>((nblocks + 255) / 256, 152 * 8);
     ProfScope ps(c, "rng", 16.0 * nblocks, 0.0);
-    philox_blocks_kernel<<<grid, 256, 0, c.stream>>>(seed, stream, offset, nblocks, reinterpret_cast<uint4*>(out));
+    run_kernel(c, philox_blocks_kernel, grid, 256, 0, seed, stream, offset, nblocks, reinterpret_cast<uint4*>(out));
     c.counted();
     c.check_launch();
 }
@@ -124,7 +126,7 @@ void launch_gaussian_factors(const Ctx& c, unsigned long long seed, int count, c
     if (nbmax == 0) return;
     const unsigned gx = (unsigned)std::min<int64_t>((nbmax + 127) / 128, 152 * 8);
     ProfScope ps(c, "rng", bytes, 0.0);
-    gaussian_factor_kernel<<<dim3(gx, (unsigned)count), 128, 0, c.stream>>>(seed, gb);
+    run_kernel(c, gaussian_factor_kernel, dim3(gx, (unsigned)count), 128, 0, seed, gb);
     c.counted();
     c.check_launch();
 }

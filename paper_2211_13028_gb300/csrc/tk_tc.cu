@@ -19,6 +19,7 @@ __device__ __forceinline__ uint32_t tf32_rna(float x) {
 // a in [0, npad) with zero padding beyond m.
 __global__ void split_tf32_kernel(const void* M, tk_dtype dt, int64_t ldm, int mtrans, int64_t nj, int64_t m,
                                   int64_t npad, int64_t ldo, float* hi, float* lo) {
+    kernel_begin();
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= ldo * npad) return;
     int64_t i = idx % ldo, a = idx / ldo;
@@ -48,6 +49,7 @@ struct SplitBatch {
 };
 
 __global__ void split_tf32_batch_kernel(SplitBatch sb) {
+    kernel_begin();
     const SplitJob& jb = sb.job[blockIdx.y];
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < jb.ldo * jb.rows_b;
          idx += (int64_t)gridDim.x * blockDim.x) {
@@ -66,6 +68,7 @@ __global__ void split_tf32_batch_kernel(SplitBatch sb) {
 
 // out = the sum of the ksplit partial products part[s n .. s n + n), in order of s.
 __global__ void splitk_sum_kernel(const float* __restrict__ part, int ksplit, int64_t n, float* __restrict__ out) {
+    kernel_begin();
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
         float v = part[e];
         for (int sk = 1; sk < ksplit; ++sk) v += part[(int64_t)sk * n + e];
@@ -78,6 +81,7 @@ __global__ void splitk_sum_kernel(const float* __restrict__ part, int ksplit, in
 // wait must give up after limit_ns, raise FLAG_TIMEOUT and let the kernel
 // return.  waited[0] receives the nanoseconds the wait lasted.
 __global__ void __launch_bounds__(32) wait_selftest_kernel(uint64_t limit_ns, unsigned* flags, long long* waited) {
+    kernel_begin();
     __shared__ __align__(8) uint64_t bar;
     __shared__ int abort;
     if (threadIdx.x == 0) {
@@ -94,7 +98,7 @@ __global__ void __launch_bounds__(32) wait_selftest_kernel(uint64_t limit_ns, un
 
 void launch_wait_selftest(const Ctx& c, uint64_t limit_ns, long long* waited) {
     if (!c.exec) return;
-    tc::wait_selftest_kernel<<<1, 32, 0, c.stream>>>(limit_ns, c.dflags, waited);
+    run_kernel(c, tc::wait_selftest_kernel, 1, 32, 0, limit_ns, c.dflags, waited);
     c.counted();
     c.check_launch();
 }
@@ -147,8 +151,8 @@ void tc_presplit(Ctx& c, const std::vector<TcSplitReq>& reqs) {
     }
     if (!c.exec || nj_ == 0) return;
     ProfScope ps(c, "elementwise", 16.0 * most * nj_, 0.0);
-    tc::split_tf32_batch_kernel<<<dim3((unsigned)std::min<int64_t>((most + 255) / 256, 1024), (unsigned)nj_), 256, 0,
-                                  c.stream>>>(sb);
+    run_kernel(c, tc::split_tf32_batch_kernel,
+               dim3((unsigned)std::min<int64_t>((most + 255) / 256, 1024), (unsigned)nj_), 256, 0, sb);
     c.counted();
     c.check_launch();
 }
@@ -243,8 +247,8 @@ static void factor_map(Ctx& c, const Factor& f, const Mat& M, bool mtrans, int64
     if (!f.have) {
         const int64_t tot = f.ldo * f.rows_b;
         ProfScope ps(c, "elementwise", 8.0 * tot + 8.0 * nj * m, 0.0);
-        tc::split_tf32_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, c.stream>>>(M.p, M.dt, M.ld, mtrans ? 1 : 0,
-                                                                                   nj, m, f.rows_b, f.ldo, f.hi, f.lo);
+        run_kernel(c, tc::split_tf32_kernel, (unsigned)((tot + 255) / 256), 256, 0, M.p, M.dt, M.ld, mtrans ? 1 : 0,
+                   nj, m, f.rows_b, f.ldo, f.hi, f.lo);
         c.counted();
         c.check_launch();
     }
@@ -284,8 +288,8 @@ static int64_t split_chunks(const Ctx& c, int64_t items, int64_t nk) {
 }
 
 static void sum_parts(Ctx& c, const float* part, int64_t ksplit, int64_t n, float* out) {
-    tc::splitk_sum_kernel<<<(unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, c.stream>>>(part, (int)ksplit,
-                                                                                                 n, out);
+    run_kernel(c, tc::splitk_sum_kernel, (unsigned)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, part,
+               (int)ksplit, n, out);
     c.counted();
     c.check_launch();
 }

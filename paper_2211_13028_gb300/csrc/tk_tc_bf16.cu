@@ -95,6 +95,7 @@ struct BfCfg {
 template <int NPAD, bool KMAJOR>
 __global__ void __launch_bounds__(kThreads, 1)
     ttm_bf16_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmB, BfArgs args) {
+    kernel_begin();
     using C = BfCfg<NPAD>;
     constexpr int S = C::kStages;
     extern __shared__ uint8_t smem_raw[];
@@ -281,6 +282,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // i + ldo*(rows_b + a); zero beyond nj and m.
 __global__ void split_bf16_kernel(const void* M, tk_dtype dt, int64_t ldm, int mtrans, int64_t nj, int64_t m,
                                   int64_t rows_b, int64_t ldo, int with_lo, __nv_bfloat16* out) {
+    kernel_begin();
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= ldo * rows_b) return;
     const int64_t i = idx % ldo, a = idx / ldo;
@@ -305,7 +307,7 @@ static void launch_kernel(const Ctx& c, const CUtensorMap& tx, const CUtensorMap
         attr_set = true;
     }
     const int grid = (int)std::min<int64_t>(a.ntiles * a.nblk, tc::grid_sms(c));
-    kern<<<grid, kThreads, Cf::kSmem, c.stream>>>(tx, tb, a);
+    run_kernel(c, kern, grid, kThreads, Cf::kSmem, tx, tb, a);
 }
 
 }  // namespace bf
@@ -337,9 +339,8 @@ void launch_ttm_bf16(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, in
     {
         const int64_t tot = ldo * rows_b;
         ProfScope ps(c, "elementwise", 4.0 * tot + 8.0 * nj * m, 0.0);
-        bf::split_bf16_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, c.stream>>>(M.p, M.dt, M.ld, mtrans ? 1 : 0,
-                                                                                   nj, m, rows_b, ldo,
-                                                                                   c.refine == -1 ? 0 : 1, split);
+        run_kernel(c, bf::split_bf16_kernel, (unsigned)((tot + 255) / 256), 256, 0, M.p, M.dt, M.ld, mtrans ? 1 : 0,
+                   nj, m, rows_b, ldo, c.refine == -1 ? 0 : 1, split);
         c.counted();
         c.check_launch();
     }

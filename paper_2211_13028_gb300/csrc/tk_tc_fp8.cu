@@ -92,6 +92,7 @@ struct F8Cfg {
 template <int NPAD>
 __global__ void __launch_bounds__(kThreads, 1)
     ttm_fp8_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmB, F8Args args) {
+    kernel_begin();
     using C = F8Cfg<NPAD>;
     constexpr int S = C::kStages;
     extern __shared__ uint8_t smem_raw[];
@@ -256,6 +257,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // s = 2^e with max |M| s in (224, 448] (1 when M is zero), into *scale.
 __global__ void __launch_bounds__(1024) fp8_factor_scale_kernel(const void* M, tk_dtype dt, int64_t ldm, int mtrans,
                                                                 int64_t nj, int64_t m, float* scale) {
+    kernel_begin();
     __shared__ float red[32];
     float amax = 0.f;
     for (int64_t e = threadIdx.x; e < nj * m; e += blockDim.x) {
@@ -284,6 +286,7 @@ __global__ void __launch_bounds__(1024) fp8_factor_scale_kernel(const void* M, t
 // saturating).
 __global__ void split_fp8_kernel(const void* M, tk_dtype dt, int64_t ldm, int mtrans, int64_t nj, int64_t m,
                                  int64_t rows_b, int64_t ldo, const float* scale, __nv_fp8_e4m3* out) {
+    kernel_begin();
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= ldo * rows_b) return;
     const int64_t i = idx % ldo, a = idx / ldo;
@@ -313,7 +316,7 @@ static void launch_kernel(const Ctx& c, const CUtensorMap& tx, const CUtensorMap
         attr_set = true;
     }
     const int grid = (int)std::min<int64_t>(a.ntiles * a.nblk, tc::grid_sms(c));
-    kern<<<grid, kThreads, Cf::kSmem, c.stream>>>(tx, tb, a);
+    run_kernel(c, kern, grid, kThreads, Cf::kSmem, tx, tb, a);
 }
 
 }  // namespace f8
@@ -345,11 +348,11 @@ void launch_ttm_fp8(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int
     {
         const int64_t tot = ldo * rows_b;
         ProfScope ps(c, "elementwise", 4.0 * tot + 8.0 * nj * m, 0.0);
-        f8::fp8_factor_scale_kernel<<<1, 1024, 0, c.stream>>>(M.p, M.dt, M.ld, mtrans ? 1 : 0, nj, m, scale);
+        run_kernel(c, f8::fp8_factor_scale_kernel, 1, 1024, 0, M.p, M.dt, M.ld, mtrans ? 1 : 0, nj, m, scale);
         c.counted();
         c.check_launch();
-        f8::split_fp8_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, c.stream>>>(M.p, M.dt, M.ld, mtrans ? 1 : 0,
-                                                                                   nj, m, rows_b, ldo, scale, split);
+        run_kernel(c, f8::split_fp8_kernel, (unsigned)((tot + 255) / 256), 256, 0, M.p, M.dt, M.ld, mtrans ? 1 : 0,
+                   nj, m, rows_b, ldo, scale, split);
         c.counted();
         c.check_launch();
     }

@@ -124,6 +124,7 @@ __device__ __forceinline__ void convert_runs(uint32_t xs, uint32_t shift, uint32
 template <int NPAD, bool KMAJOR, int ES>
 __global__ void __launch_bounds__(LowpCfg<NPAD>::kThreads, 1)
     ttm_lowp_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmB, LowpArgs args) {
+    kernel_begin();
     using C = LowpCfg<NPAD>;
     constexpr uint32_t NA = C::kNA;
     constexpr int K = kLowpChunk;
@@ -549,7 +550,7 @@ static void ttm_lowp_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorM
         attr_set = true;
     }
     const int grid = (int)std::min<int64_t>(a.nitems, grid_sms(c));
-    kern<<<grid, Cf::kThreads, a.stages * stage + 2048, c.stream>>>(tx, tb, a);
+    run_kernel(c, kern, grid, Cf::kThreads, a.stages * stage + 2048, tx, tb, a);
 }
 
 // The kernel for npad output columns per block (a multiple of 16 up to 64) and elements of ES bytes.

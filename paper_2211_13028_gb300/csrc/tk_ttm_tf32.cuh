@@ -143,6 +143,7 @@ template <int NPAD, bool KMAJOR, bool FLAT>
 __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
     ttm_tf32x3_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmB,
                       TtmArgs args) {
+    kernel_begin();
     using C = TtmCfg<NPAD, FLAT>;
     constexpr uint32_t S = C::kStages;
     constexpr uint32_t NA = C::kNA;
@@ -593,7 +594,7 @@ static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorM
         attr_set = true;
     }
     const int grid = (int)std::min<int64_t>(a.nitems, grid_sms(c));
-    kern<<<grid, Cf::kThreads, Cf::kSmem, c.stream>>>(tx, tb, a);
+    run_kernel(c, kern, grid, Cf::kThreads, Cf::kSmem, tx, tb, a);
 }
 
 // The kernel for npad output columns per block (a multiple of 16 up to 96).

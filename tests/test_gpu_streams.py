@@ -185,3 +185,23 @@ def test_profile_trace_lists_every_recorded_launch(dev):
     assert "jacobi" in cls and any(c.startswith("xpass") for c in cls)
     for h in T._device_handles(dev):
         T.load().tk_profile(h, 0)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+def test_overlapped_launches_leave_results_unchanged(dev, dtype):
+    # launches overlap the kernel before them unless they are being timed: calls queued without a wait between
+    # them must give what the timed, unoverlapped call gives, bit for bit
+    g = np.random.Generator(np.random.PCG64(51))
+    X, _, _ = make_X(g.standard_normal((61, 48, 52)), dtype, dev)
+    r, p = (9, 8, 7), 5
+    s, _ = O.subranks_reuse(r, p)
+    om = mats(synth.sketch_factors_reuse((61, 48, 52), s, seed=52, dtype=dtype), dtype, dev)
+    T.tk_profile(True, dev)
+    G, U, e = T.tucker_rhkron(X, r, p, om)
+    loss = T.tucker_loss(X, G, U)
+    T.tk_profile(False, dev)
+    runs = [T.tucker_rhkron(X, r, p, om, async_outputs=True) for _ in range(8)]
+    torch.cuda.synchronize()
+    for Gi, Ui, ei in runs:
+        assert torch.equal(Gi, G) and all(torch.equal(a, b) for a, b in zip(Ui, U)) and ei.value == e
+    assert T.tucker_loss(X, G, U) == loss

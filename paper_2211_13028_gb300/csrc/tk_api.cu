@@ -123,17 +123,31 @@ static Opts opts_in(const tk_opts* o, int d) {
 
 // The matrix in the accumulation dtype, contiguous (ld = rows): the matrix
 // itself when it already is, else a converted copy (the factors are read only).
+static std::vector<Mat> mats_to(Ctx& c, const std::vector<Mat>& Ms, tk_dtype dt) {
+    std::vector<Mat> out;
+    std::vector<ConvertJob> jobs;
+    for (const Mat& M : Ms) {
+        if (M.dt == dt && (M.ld == M.rows || M.cols <= 1)) {  // already what the consumers read
+            out.push_back(M);
+            continue;
+        }
+        Mat o;
+        o.dt = dt;
+        o.rows = M.rows;
+        o.cols = M.cols;
+        o.ld = std::max<int64_t>(1, M.rows);
+        void* p = c.alloc_bytes(dtype_size(dt) * M.rows * M.cols);
+        jobs.push_back({M.p, p, M.dt, dt, M.rows, M.cols, M.ld, o.ld, 1.f});
+        o.p = p;
+        out.push_back(o);
+    }
+    launch_convert(c, jobs);
+    return out;
+}
+
 static Mat mat_to(Ctx& c, const Mat& M, tk_dtype dt) {
-    if (M.dt == dt && (M.ld == M.rows || M.cols <= 1)) return M;  // already what the consumers read
-    Mat o;
-    o.dt = dt;
-    o.rows = M.rows;
-    o.cols = M.cols;
-    o.ld = std::max<int64_t>(1, M.rows);
-    void* p = c.alloc_bytes(dtype_size(dt) * M.rows * M.cols);
-    launch_convert(c, M.p, M.dt, M.rows, M.cols, M.ld, p, dt, o.ld, 1.f);
-    o.p = p;
-    return o;
+    if (M.dt == dt && (M.ld == M.rows || M.cols <= 1)) return M;
+    return mats_to(c, {M}, dt)[0];
 }
 
 static Tens tens_to(Ctx& c, const Tens& T, tk_dtype dt) {
@@ -311,45 +325,40 @@ static void orth_batch(Ctx& c, const std::vector<View2>& Y, const std::vector<in
     for (int b = 0; b < B; ++b) df = df && Y[b].dt == TK_F32;
     if (!house_only) {
         // pass 1: W = Y^T Y, R1^{-1}, Q1 = Y R1^{-1}
-        c.fork(B, [&](int b) {
+        std::vector<GemmJob> grams;
+        for (int b = 0; b < B; ++b) {
             const View2& A = Y[b];
             View2 At;  // (column, row) indexing of the same data
             At.p = A.p;
             At.dt = A.dt;
             At.A1 = A.T1; At.sa1 = A.st1; At.sa2 = A.st2;
             At.T1 = A.A1; At.st1 = A.sa1; At.st2 = A.sa2;
-            gemm_nt_f64(c, k[b], k[b], n[b], At, At, 1.0, 0.0, W + (int64_t)b * kmax * kmax, kmax, bad + b, df);
-        });
-        launch_chol_inv(c, B, kd, kmax, W, Rinv, bad, 1e-12, df);
-        if (df)
-            launch_apply_rinv_df(c, B, Y.data(), n.data(), k.data(), Rinv, kmax, Q1.data(), bad);
-        else
-            for (int b = 0; b < B; ++b)
-                launch_apply_rinv(c, n[b], k[b], Y[b], Rinv + (int64_t)b * kmax * kmax, kmax, Q1[b], bad + b);
-        // pass 2 on Q1
-        c.fork(B, [&](int b) {
-            View2 Qt = view_cols(Q1[b], TK_F64, n[b]);
-            gemm_nt_f64(c, k[b], k[b], n[b], Qt, Qt, 1.0, 0.0, W + (int64_t)b * kmax * kmax, kmax, bad + b);
-        });
-        launch_chol_inv(c, B, kd, kmax, W, Rinv, bad, 1e-12, df);
-        if (df) {
-            std::vector<View2> Qr(B);
-            for (int b = 0; b < B; ++b) Qr[b] = view_rows(Q1[b], TK_F64, n[b]);
-            launch_apply_rinv_df(c, B, Qr.data(), n.data(), k.data(), Rinv, kmax, Q.data(), bad);
-        } else {
-            for (int b = 0; b < B; ++b) {
-                View2 Qr = view_rows(Q1[b], TK_F64, n[b]);
-                launch_apply_rinv(c, n[b], k[b], Qr, Rinv + (int64_t)b * kmax * kmax, kmax, Q[b], bad + b);
-            }
+            grams.push_back({k[b], k[b], n[b], At, At, 1.0, 0.0, W + (int64_t)b * kmax * kmax, kmax, bad + b, df});
         }
+        gemm_nt_f64(c, grams);
+        launch_chol_inv(c, B, kd, kmax, W, Rinv, bad, 1e-12, df);
+        launch_apply_rinv(c, B, Y.data(), n.data(), k.data(), Rinv, kmax, Q1.data(), bad, df);
+        // pass 2 on Q1
+        grams.clear();
+        std::vector<View2> Qr(B);
+        for (int b = 0; b < B; ++b) {
+            const View2 Qt = view_cols(Q1[b], TK_F64, n[b]);
+            grams.push_back({k[b], k[b], n[b], Qt, Qt, 1.0, 0.0, W + (int64_t)b * kmax * kmax, kmax, bad + b, false});
+            Qr[b] = view_rows(Q1[b], TK_F64, n[b]);
+        }
+        gemm_nt_f64(c, grams);
+        launch_chol_inv(c, B, kd, kmax, W, Rinv, bad, 1e-12, df);
+        launch_apply_rinv(c, B, Qr.data(), n.data(), k.data(), Rinv, kmax, Q.data(), bad, df);
     }
-    c.fork(B, [&](int b) {
+    std::vector<HouseJob> house;
+    for (int b = 0; b < B; ++b) {
         int* slot = slots[b] >= 0 ? c.dqr + slots[b] : nullptr;
         if (c.qr_method != 2 || wide)  // the fallback copies Y itself and records the method taken
-            launch_householder(c, n[b], k[b], Y[b], Hsrc[b], Q[b], Htau[b], bad + b, slot, 1);
+            house.push_back({n[b], k[b], Y[b], Hsrc[b], Q[b], Htau[b], bad + b, slot, 1});
         else if (slot)
             launch_qr_info(c, slot, bad + b, 3);
-    });
+    }
+    launch_householder(c, house);
 }
 
 static void orth_one(Ctx& c, const View2& Y, int64_t n, int64_t k, double* Q, int slot) {
@@ -500,14 +509,16 @@ static Tens sthosvd_core(Ctx& c, const Tens& G0, const int64_t* r, const std::ve
         TK_REQUIRE(G0.n[j] <= 256, TK_ERR_SHAPE, "sthosvd: core mode above 256 is not supported");
     std::vector<double*> C0(d, nullptr), V1(d, nullptr);
     if (!fp64_path) {
-        c.fork(d, [&](int j) {
+        std::vector<GemmJob> grams;
+        for (int j = 0; j < d; ++j) {
             const int64_t kj = G0.n[j];
-            if (kj > 112) return;  // solved in FP64 below
+            if (kj > 112) continue;  // solved in FP64 below
             const int64_t K = kj ? G0.numel() / kj : 0;
             C0[j] = c.alloc<double>(kj * kj);
             const View2 A = view_unfold_rows(G0, j);
-            gemm_nt_f64(c, kj, kj, K, A, A, 1.0, 0.0, C0[j], kj);
-        });
+            grams.push_back({kj, kj, K, A, A, 1.0, 0.0, C0[j], kj, nullptr, false});
+        }
+        gemm_nt_f64(c, grams);
     }
     auto body = [&]() {
         if (!fp64_path) {
@@ -644,21 +655,24 @@ static void finish(Ctx& c, const Tens& X, const std::vector<double*>& Qd, const 
                    const std::vector<Mat>& Uout, double* err_dev, std::vector<double*>* signs = nullptr) {
     const int d = X.d;
     std::vector<double*> U(d), sg(d);
-    c.fork(d, [&](int j) {
+    std::vector<GemmJob> products;
+    std::vector<SignJob> fixes;
+    for (int j = 0; j < d; ++j) {
         U[j] = c.alloc<double>(X.n[j] * r[j]);
         sg[j] = c.alloc<double>(r[j]);
-        gemm_nt_f64(c, X.n[j], r[j], kdim[j], view_rows(Qd[j], TK_F64, X.n[j]), view_cols(V[j], TK_F64, kdim[j]), 1.0,
-                    0.0, U[j], X.n[j]);
-        launch_sign_fix(c, U[j], X.n[j], r[j], sg[j], (void*)Uout[j].p, Uout[j].dt, Uout[j].ld);
-    });
+        products.push_back({X.n[j], r[j], kdim[j], view_rows(Qd[j], TK_F64, X.n[j]), view_cols(V[j], TK_F64, kdim[j]), 1.0,
+                            0.0, U[j], X.n[j], nullptr, false});
+        fixes.push_back({U[j], X.n[j], r[j], sg[j], (void*)Uout[j].p, Uout[j].dt, Uout[j].ld});
+    }
+    gemm_nt_f64(c, products);
+    launch_sign_fix(c, fixes);
     launch_apply_signs(c, (double*)Gt.p, Gt, sg.data(), Gout.p, Gout.dt);
     if (signs) *signs = sg;
     if (!err_dev) return;
     // ||X - G x_j U_j|| from the returned G and U, in the accumulation dtype.
     tk_dtype acc = acc_of(X.dt);
     Tens Ga = tens_to(c, Gout, acc);
-    std::vector<Mat> Ua(d);
-    for (int j = 0; j < d; ++j) Ua[j] = mat_to(c, Uout[j], acc);
+    const std::vector<Mat> Ua = mats_to(c, Uout, acc);
     residual_pass(c, X, Ga, Ua, acc, err_dev, nullptr, TK_F32, 0.0);
 }
 
@@ -1408,9 +1422,10 @@ tk_status tucker_orth_sketches(tk_handle* h, int d, const tk_tensor* Y, tk_matri
             }
         }
         orth_batch(c, Yv, nb, kb, qb, slots);
+        std::vector<ConvertJob> outs;
         for (int n = 0; n < d; ++n)
-            launch_convert(c, Qd[n], TK_F64, Qm[n].rows, Qm[n].cols, Qm[n].rows, (void*)Qm[n].p, Qm[n].dt, Qm[n].ld,
-                           1.f);
+            outs.push_back({Qd[n], (void*)Qm[n].p, TK_F64, Qm[n].dt, Qm[n].rows, Qm[n].cols, Qm[n].rows, Qm[n].ld, 1.f});
+        launch_convert(c, outs);
     });
 }
 
@@ -1427,15 +1442,17 @@ tk_status tucker_sthosvd(tk_handle* h, const tk_tensor* Ghat, const tk_matrix* Q
         Tens dims;  // the tensor's dims, from the factors' rows
         dims.d = d;
         std::vector<double*> Qd(d);
+        std::vector<Mat> Qm(d);
         std::vector<int64_t> k(d);
         for (int j = 0; j < d; ++j) {
-            Mat q = mat_in(&Q[j], "Q");
+            const Mat q = Qm[j] = mat_in(&Q[j], "Q");
             TK_REQUIRE(q.cols == Gh.n[j] && q.rows >= 1, TK_ERR_SHAPE, "sthosvd: Q_j must be n_j x k_j");
             TK_REQUIRE(r[j] >= 1 && r[j] <= Gh.n[j], TK_ERR_SHAPE, "sthosvd: need 1 <= r_j <= k_j");
             dims.n[j] = q.rows;
             k[j] = q.cols;
-            Qd[j] = (double*)mat_to(c, q, TK_F64).p;
         }
+        Qm = mats_to(c, Qm, TK_F64);
+        for (int j = 0; j < d; ++j) Qd[j] = (double*)Qm[j].p;
         Tens Gt;
         std::vector<Mat> Um;
         check_outputs(dims, r, G, U, Gt, Um);
@@ -1966,18 +1983,23 @@ static void grad_from_sketches(Ctx& c, const Tens& Gt, const std::vector<Mat>& U
     Tens G64 = Gt.dt == TK_F64 ? Gt : tens_to(c, Gt, TK_F64);
     std::vector<double*> U64(d);
     std::vector<Mat> Cm(d);
-    c.fork(d, [&](int j) {
+    std::vector<ConvertJob> widen;
+    std::vector<GemmJob> grams;
+    for (int j = 0; j < d; ++j) {
         const int64_t nj = n[j], rj = Gt.n[j];
         U64[j] = c.alloc<double>(nj * rj);
-        launch_convert(c, Um[j].p, Um[j].dt, nj, rj, Um[j].ld, U64[j], TK_F64, nj, 1.f);
+        widen.push_back({Um[j].p, U64[j], Um[j].dt, TK_F64, nj, rj, Um[j].ld, nj, 1.f});
         double* Cj = c.alloc<double>(rj * rj);
-        gemm_nt_f64(c, rj, rj, nj, view_cols(U64[j], TK_F64, nj), view_cols(U64[j], TK_F64, nj), 1.0, 0.0, Cj, rj);
+        grams.push_back({rj, rj, nj, view_cols(U64[j], TK_F64, nj), view_cols(U64[j], TK_F64, nj), 1.0, 0.0, Cj, rj,
+                         nullptr, false});
         Cm[j].p = Cj;
         Cm[j].dt = TK_F64;
         Cm[j].rows = rj;
         Cm[j].cols = rj;
         Cm[j].ld = rj;
-    });
+    }
+    launch_convert(c, widen);
+    gemm_nt_f64(c, grams);
     std::vector<Tens> Pm(d);  // P_n = G x_{j != n} C_j: one short chain per mode, side by side
     c.fork(d, [&](int n) {
         std::vector<int> modes;
@@ -1985,29 +2007,39 @@ static void grad_from_sketches(Ctx& c, const Tens& Gt, const std::vector<Mat>& U
             if (j != n) modes.push_back(j);
         Pm[n] = multi_ttm(c, G64, modes, Cm.data(), false, TK_F64);
     });
-    // dU_n per mode and dG are independent: item j < d is dU_j, item d is dG
-    const int ndu = want_dU ? d : 0;
-    c.fork(ndu + (want_dG ? 1 : 0), [&](int j) {
-        if (j == ndu) {
+    // dU (item 0) and dG (item 1) are independent
+    c.fork(2, [&](int item) {
+        if (item == 1) {
+            if (!want_dG) return;
             // dG = -2s (X x_j U_j^T - G x_j C_j) = -2s (S_0 x_0 U_0^T - P_0 x_0 C_0)
             Tens E = ttm_to(c, S[0], 0, Ua[0], false, acc);
             Tens F = ttm_to(c, Pm[0], 0, Cm[0], false, TK_F64);
             launch_axpby_residual(c, E, F.p, TK_F64, s2, g.dG.p, g.dG.dt);
             return;
         }
-        const int64_t nj = n[j], rj = Gt.n[j];
-        int64_t K = 1;
-        for (int i = 0; i < d; ++i)
-            if (i != j) K *= Gt.n[i];
-        double* A1 = c.alloc<double>(nj * rj);
-        double* B1 = c.alloc<double>(rj * rj);
-        // S_n carries the FP32 rounding of the sketch pass, far above double-float accumulation error,
-        // so for FP32 data this product (the largest of the gradient) runs on the FP32 pipe
-        gemm_nt_f64(c, nj, rj, K, view_unfold_rows(S[j], j), view_unfold_rows(Gt.dt == TK_F32 ? Gt : G64, j), s2,
-                    0.0, A1, nj, nullptr, true);
-        gemm_nt_f64(c, rj, rj, K, view_unfold_rows(Pm[j], j), view_unfold_rows(G64, j), 1.0, 0.0, B1, rj);
-        gemm_nt_f64(c, nj, rj, rj, view_rows(U64[j], TK_F64, nj), view_cols(B1, TK_F64, rj), -s2, 1.0, A1, nj);
-        launch_convert(c, A1, TK_F64, nj, rj, nj, (void*)g.dU[j].p, g.dU[j].dt, g.dU[j].ld, 1.f);
+        if (!want_dU) return;
+        std::vector<GemmJob> first, second;
+        std::vector<ConvertJob> out;
+        for (int j = 0; j < d; ++j) {
+            const int64_t nj = n[j], rj = Gt.n[j];
+            int64_t K = 1;
+            for (int i = 0; i < d; ++i)
+                if (i != j) K *= Gt.n[i];
+            double* A1 = c.alloc<double>(nj * rj);
+            double* B1 = c.alloc<double>(rj * rj);
+            // S_n carries the FP32 rounding of the sketch pass, far above double-float accumulation error,
+            // so for FP32 data this product (the largest of the gradient) runs on the FP32 pipe
+            first.push_back({nj, rj, K, view_unfold_rows(S[j], j), view_unfold_rows(Gt.dt == TK_F32 ? Gt : G64, j), s2,
+                             0.0, A1, nj, nullptr, true});
+            first.push_back({rj, rj, K, view_unfold_rows(Pm[j], j), view_unfold_rows(G64, j), 1.0, 0.0, B1, rj, nullptr,
+                             false});
+            second.push_back({nj, rj, rj, view_rows(U64[j], TK_F64, nj), view_cols(B1, TK_F64, rj), -s2, 1.0, A1, nj,
+                              nullptr, false});
+            out.push_back({A1, (void*)g.dU[j].p, TK_F64, g.dU[j].dt, nj, rj, nj, g.dU[j].ld, 1.f});
+        }
+        gemm_nt_f64(c, first);
+        gemm_nt_f64(c, second);
+        launch_convert(c, out);
     });
 }
 

@@ -410,6 +410,17 @@ void launch_sum_pairs(const Ctx& c, const double* part, int nb, double* out2);
 // on the FP32 pipe (~48 significant bits) instead of in FP64.
 void gemm_nt_f64(Ctx& c, int64_t m, int64_t n, int64_t K, const View2& A, const View2& B, double alpha,
                  double beta, double* C, int64_t ldc, const int* skip = nullptr, bool df_ok = false);
+// Several independent products, those of a kind in one launch.
+struct GemmJob {
+    int64_t m, n, K;
+    View2 A, B;
+    double alpha, beta;
+    double* C;
+    int64_t ldc;
+    const int* skip;
+    bool df_ok;
+};
+void gemm_nt_f64(Ctx& c, const std::vector<GemmJob>& jobs);
 
 struct KDims {
     int k[TK_MAX_D];
@@ -423,22 +434,25 @@ struct KDims {
 void launch_chol_inv(const Ctx& c, int batch, const KDims& kd, int kmax, const double* W, double* Rinv, int* bad,
                      double tol, bool df = false);
 
-// Q(i, c) = sum_{c' <= c} Y(i, c') Rinv(c', c), FP64 out (n x k, ld n).  Skipped when *skip != 0.
-void launch_apply_rinv(const Ctx& c, int64_t n, int64_t k, const View2& Y, const double* Rinv, int64_t ldr,
-                       double* Q, const int* skip);
+// Q_b(i, c) = sum_{c' <= c} Y_b(i, c') R_b^{-1}(c', c) for batch matrices in one launch (Y_b FP32 or FP64, n_b x k_b;
+// R_b = Rinv + b kmax^2, ld kmax; Q_b FP64, ld n_b).  Matrix b is skipped when bad[b] != 0.  df: in double-float
+// arithmetic instead of FP64.
+void launch_apply_rinv(const Ctx& c, int batch, const View2* Y, const int64_t* n, const int64_t* k, const double* Rinv,
+                       int64_t kmax, double* const* Q, const int* bad, bool df);
 
-// Q_b = Y_b R_b^{-1} for batch matrices in one launch, in double-float
-// arithmetic (Y_b FP32 or FP64, n_b x k_b; R_b = Rinv + b kmax^2, ld kmax;
-// Q_b FP64, ld n_b).  Matrix b is skipped when bad[b] != 0.
-void launch_apply_rinv_df(const Ctx& c, int batch, const View2* Y, const int64_t* n, const int64_t* k,
-                          const double* Rinv, int64_t kmax, double* const* Q, const int* bad);
-
-// Householder thin QR of Y (View2, n x k; copied to FP64 scratch A, ld n) producing Q with
-// R_ii >= 0, run only when *run != 0 (run may be NULL = always).  One CTA.  tau: k doubles
+// Householder thin QR of each Y (View2, n x k; copied to FP64 scratch A, ld n) producing Q with
+// R_ii >= 0, run only when *run != 0 (run may be NULL = always).  One CTA a matrix.  tau: k doubles
 // scratch.  When slot is given, *slot = slot_value if the QR runs, else 0 (the QR method a
 // matrix of a batch took).
-void launch_householder(const Ctx& c, int64_t n, int64_t k, const View2& Y, double* A, double* Q, double* tau,
-                        const int* run, int* slot = nullptr, int slot_value = 1);
+struct HouseJob {
+    int64_t n, k;
+    View2 Y;
+    double *A, *Q, *tau;
+    const int* run;
+    int* slot;
+    int slot_value;
+};
+void launch_householder(const Ctx& c, const std::vector<HouseJob>& jobs);
 
 // Jacobi eigensolver (one CTA per matrix): A (k x k FP64 symmetric, destroyed),
 // eigenvalues descending in w, eigenvectors as columns of V (ld k).  k <= 112
@@ -472,6 +486,15 @@ Mat mat_in(const tk_matrix* m, const char* name);
 // Element-wise helpers.
 void launch_convert(const Ctx& c, const void* src, tk_dtype sdt, int64_t rows, int64_t cols, int64_t lds,
                     void* dst, tk_dtype ddt, int64_t ldd, float src_scale);
+// Several independent copies (rows x cols, inv: the factor of FP8 data), up to TK_MAX_D in a launch.
+struct ConvertJob {
+    const void* src;
+    void* dst;
+    tk_dtype sdt, ddt;
+    int64_t rows, cols, lds, ldd;
+    float inv;
+};
+void launch_convert(const Ctx& c, const std::vector<ConvertJob>& jobs);
 void launch_fill_identity(const Ctx& c, double* Q, int64_t n);
 // A (n x k, FP64, ld n) = Y; only when *run != 0 (run may be NULL = always).
 void launch_copy_unfold_to_matrix(const Ctx& c, const View2& Y, int64_t n, int64_t k, double* A,
@@ -479,11 +502,18 @@ void launch_copy_unfold_to_matrix(const Ctx& c, const View2& Y, int64_t n, int64
 void launch_fill_int(const Ctx& c, int* p, int count, int value);
 // *slot = *bad ? bad_value : 0
 void launch_qr_info(const Ctx& c, int* slot, const int* bad, int bad_value);
-// Sign gauge: for each column of U (n x r, F64, ld n) make the largest-|.|
+// Sign gauge: for each column of each U (n x r, F64, ld n) make the largest-|.|
 // entry positive; sign[c] = +-1.
 // out (may be NULL): the signed U also stored there in odt (ld ldo).
-void launch_sign_fix(const Ctx& c, double* U, int64_t n, int64_t r, double* sign, void* out = nullptr,
-                     tk_dtype odt = TK_F64, int64_t ldo = 0);
+struct SignJob {
+    double* U;
+    int64_t n, r;
+    double* sign;
+    void* out;
+    tk_dtype odt;
+    int64_t ldo;
+};
+void launch_sign_fix(const Ctx& c, const std::vector<SignJob>& jobs);
 // G (a tensor of the given shape, FP64) times the product of the modes' signs
 // (a NULL sign array leaves its mode alone); out (may be NULL): also stored
 // there in odt, dense.

@@ -571,24 +571,48 @@ __device__ __forceinline__ E gemm_elem(double v) {
         return (E)v;
 }
 
+// The products of one launch: blockIdx.z runs over the K parts of each in turn.
+struct GemmItem {
+    int64_t m, n, K, kchunk, ldc;
+    View2 A, B;
+    double alpha, beta;
+    double* C;
+    double* P;
+    unsigned* ctr;
+    const int* skip;
+    int nsplit;
+};
+template <int NB>
+struct GemmItems {
+    GemmItem job[NB];
+};
+
 // MODE 2: the operands (FP64 or FP32) are split into double-float pairs on
 // load and the products accumulate with df_dot_step on the FP32 pipe (~47
 // significant bits; FP32's exponent range bounds the products).
-template <int MODE>
-__global__ void __launch_bounds__(256) gemm_tile16_kernel(int64_t m, int64_t n, int64_t K, int64_t kchunk, View2 A,
-                                                          View2 B, double alpha, double beta, double* C, int64_t ldc,
-                                                          double* P, unsigned* ctr, const int* skip) {
+template <int MODE, int NB>
+__global__ void __launch_bounds__(256) gemm_tile16_kernel(const __grid_constant__ GemmItems<NB> items) {
     kernel_begin();
     constexpr bool DFACC = MODE != 0;
     using E = typename std::conditional<MODE == 0, double, typename std::conditional<MODE == 1, float, float2>::type>::type;
-    if (skip && *skip) return;
+    int q0 = 0, z = blockIdx.z;
+    if (NB > 1)
+        while (z >= items.job[q0].nsplit) z -= items.job[q0++].nsplit;
+    const GemmItem& g = items.job[q0];
+    const View2 &A = g.A, &B = g.B;
+    const int64_t m = g.m, n = g.n, K = g.K, ldc = g.ldc;
+    const double alpha = g.alpha, beta = g.beta;
+    double* const C = g.C;
+    double* const P = g.P;
+    if (g.skip && *g.skip) return;
+    if ((int64_t)blockIdx.x * 16 >= m || (int64_t)blockIdx.y * 16 >= n) return;  // (the grid covers the largest)
     __shared__ E As[32][17];
     __shared__ E Bs[32][17];
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
     const int64_t a0 = (int64_t)blockIdx.x * 16, b0 = (int64_t)blockIdx.y * 16;
-    const int64_t kb = (int64_t)blockIdx.z * kchunk;
-    const int64_t ke = min(K, kb + kchunk);
+    const int64_t kb = z * g.kchunk;
+    const int64_t ke = min(K, kb + g.kchunk);
     const TileLoader la(A), lb(B);
     int ra[2], ka[2], rb[2], kb2[2];
     int64_t oa[2], ob[2];
@@ -634,23 +658,23 @@ __global__ void __launch_bounds__(256) gemm_tile16_kernel(int64_t m, int64_t n, 
         }
         return;
     }
-    if (in) P[(int64_t)blockIdx.z * m * n + a + m * b] = sum;
-    if (!ctr) return;  // a separate reduction kernel adds the partial tiles
+    if (in) P[(int64_t)z * m * n + a + m * b] = sum;
+    if (!g.ctr) return;  // a separate reduction kernel adds the partial tiles
     // the last CTA of this tile to arrive adds the partial tiles (and re-zeroes the counter)
     __shared__ int s_last;
     __threadfence();
     __syncthreads();
     if (tid == 0) {
-        unsigned* t = ctr + blockIdx.x + (int64_t)gridDim.x * blockIdx.y;
+        unsigned* t = g.ctr + blockIdx.x + (m + 15) / 16 * blockIdx.y;
         const unsigned prev = atomicAdd(t, 1u);
-        s_last = prev == gridDim.z - 1;
+        s_last = prev == g.nsplit - 1u;
         if (s_last) *t = 0u;
     }
     __syncthreads();
     if (!s_last || !in) return;
     __threadfence();
     double tot = 0.0;
-    for (int z = 0; z < (int)gridDim.z; ++z) tot += __ldcg(P + (int64_t)z * m * n + a + m * b);
+    for (int w = 0; w < g.nsplit; ++w) tot += __ldcg(P + (int64_t)w * m * n + a + m * b);
     double* dst = C + a + ldc * b;
     *dst = beta == 0.0 ? alpha * tot : alpha * tot + beta * *dst;
 }
@@ -659,12 +683,16 @@ __global__ void __launch_bounds__(256) gemm_tile16_kernel(int64_t m, int64_t n, 
 // 16 x 16 tile over 16 CTAs leaves the GPU idle): a CTA takes a T x T tile and
 // splits K over G = 256 / T^2 thread groups, which are summed in shared memory
 // at the end, so a k x k x k product with k ~ 50 spreads over ~170 SMs.
-template <int T>
-__global__ void __launch_bounds__(256) gemm_small_kernel(int64_t m, int64_t n, int64_t K, View2 A, View2 B,
-                                                         double alpha, double beta, double* C, int64_t ldc,
-                                                         const int* skip) {
+template <int T, int NB>
+__global__ void __launch_bounds__(256) gemm_small_kernel(const __grid_constant__ GemmItems<NB> items) {
     kernel_begin();
-    if (skip && *skip) return;
+    const GemmItem& it = items.job[NB > 1 ? blockIdx.z : 0];
+    const View2 &A = it.A, &B = it.B;
+    const int64_t m = it.m, n = it.n, K = it.K, ldc = it.ldc;
+    const double alpha = it.alpha, beta = it.beta;
+    double* const C = it.C;
+    if (it.skip && *it.skip) return;
+    if ((int64_t)blockIdx.x * T >= m || (int64_t)blockIdx.y * T >= n) return;  // (the grid covers the largest)
     constexpr int G = 256 / (T * T);
     __shared__ double As[32][T + 1];
     __shared__ double Bs[32][T + 1];
@@ -706,67 +734,115 @@ __global__ void __launch_bounds__(256) gemm_small_kernel(int64_t m, int64_t n, i
     *dst = beta == 0.0 ? alpha * sum : alpha * sum + beta * *dst;
 }
 
-void gemm_nt_f64(Ctx& c, int64_t m, int64_t n, int64_t K, const View2& A, const View2& B, double alpha, double beta,
-                 double* C, int64_t ldc, const int* skip, bool df_ok) {
+// Which kernel a product runs on: 16 x 16 tiles (T = 16) in one of the arithmetics, or the small ones.
+struct GemmPlan {
+    int mode, T;
+    GemmItem it;
+};
+
+static GemmPlan gemm_plan(Ctx& c, const GemmJob& j) {
+    GemmPlan p{};
     // Dot2 accumulation where the caller allows it and both operands are FP32; double-float
     // operands throughout a call on FP32-class data (c.df64)
-    const int mode = (df_ok && A.dt == TK_F32 && B.dt == TK_F32) ? 1 : (c.df64 ? 2 : 0);
-    const bool df = mode != 0;
+    p.mode = (j.df_ok && j.A.dt == TK_F32 && j.B.dt == TK_F32) ? 1 : (c.df64 ? 2 : 0);
+    p.it.m = j.m;
+    p.it.n = j.n;
+    p.it.K = j.K;
+    p.it.ldc = j.ldc;
+    p.it.A = j.A;
+    p.it.B = j.B;
+    p.it.alpha = j.alpha;
+    p.it.beta = j.beta;
+    p.it.C = j.C;
+    p.it.skip = j.skip;
+    p.it.nsplit = 1;
+    p.it.kchunk = j.K;
     // short K and few 16 x 16 tiles: smaller tiles with K split inside the CTA
-    if (mode != 1 && K < 128 && ((m + 15) / 16) * ((n + 15) / 16) < 152) {
-        if (!c.exec || m == 0 || n == 0) return;
-        const bool t8 = ((m + 7) / 8) * ((n + 7) / 8) >= 152;
-        const int T = t8 ? 8 : 4;
-        dim3 grid((unsigned)((m + T - 1) / T), (unsigned)((n + T - 1) / T));
-        ProfScope ps(c, "gemm_f64", 8.0 * (double)(m * ((n + T - 1) / T) + n * ((m + T - 1) / T)) * K + 8.0 * m * n,
-                     2.0 * m * n * K);
-        if (t8)
-            run_kernel(c, gemm_small_kernel<8>, grid, 256, 0, m, n, K, A, B, alpha, beta, C, ldc, skip);
-        else
-            run_kernel(c, gemm_small_kernel<4>, grid, 256, 0, m, n, K, A, B, alpha, beta, C, ldc, skip);
-        c.counted();
-        c.check_launch();
-        return;
+    const int64_t tiles = ((j.m + 15) / 16) * ((j.n + 15) / 16);
+    if (p.mode != 1 && j.K < 128 && tiles < 152) {
+        p.mode = 0;
+        p.T = ((j.m + 7) / 8) * ((j.n + 7) / 8) >= 152 ? 8 : 4;
+        return p;
     }
-    // 16 x 16 tiles; split K only when the tiles alone leave most SMs idle and
+    p.T = 16;
+    // split K only when the tiles alone leave most SMs idle and
     // each split still has at least 64 terms.
-    const int64_t tiles = ((m + 15) / 16) * ((n + 15) / 16);
     int64_t nsplit = 1;
-    if (K >= 128 && tiles < 2 * 152) {
-        nsplit = std::min<int64_t>((2 * 152 + tiles - 1) / tiles, K / 64);
+    if (j.K >= 128 && tiles < 2 * 152) {
+        nsplit = std::min<int64_t>((2 * 152 + tiles - 1) / tiles, j.K / 64);
         nsplit = std::max<int64_t>(1, std::min<int64_t>(nsplit, 512));
     }
-    int64_t kchunk = K > 0 ? (K + nsplit - 1) / nsplit : 1;
+    int64_t kchunk = j.K > 0 ? (j.K + nsplit - 1) / nsplit : 1;
     kchunk = (kchunk + 31) / 32 * 32;
-    nsplit = K > 0 ? (K + kchunk - 1) / kchunk : 1;
-    double* P = nsplit > 1 ? c.alloc<double>(nsplit * m * n) : nullptr;
-    if (!c.exec || m == 0 || n == 0) return;
-    unsigned* ctr = nsplit > 1 ? c.take_counters((int)tiles) : nullptr;
-    dim3 grid((unsigned)((m + 15) / 16), (unsigned)((n + 15) / 16), (unsigned)nsplit);
-    {
-        ProfScope ps(c, df ? "gemm_df" : "gemm_f64",
-                     8.0 * (double)(m * ((n + 15) / 16) + n * ((m + 15) / 16)) * K + 8.0 * m * n * nsplit,
-                     2.0 * m * n * K);
-        if (mode == 1)
-            run_kernel(c, gemm_tile16_kernel<1>, grid, 256, 0, m, n, K, kchunk, A, B, alpha, beta, C, ldc, P, ctr,
-                       skip);
-        else if (mode == 2)
-            run_kernel(c, gemm_tile16_kernel<2>, grid, 256, 0, m, n, K, kchunk, A, B, alpha, beta, C, ldc, P, ctr,
-                       skip);
-        else
-            run_kernel(c, gemm_tile16_kernel<0>, grid, 256, 0, m, n, K, kchunk, A, B, alpha, beta, C, ldc, P, ctr,
-                       skip);
+    nsplit = j.K > 0 ? (j.K + kchunk - 1) / kchunk : 1;
+    p.it.kchunk = kchunk;
+    p.it.nsplit = (int)nsplit;
+    p.it.P = nsplit > 1 ? c.alloc<double>(nsplit * j.m * j.n) : nullptr;
+    if (c.exec && p.it.P && j.m && j.n) p.it.ctr = c.take_counters((int)tiles);
+    return p;
+}
+
+template <int NB>
+static void gemm_run(const Ctx& c, const std::vector<GemmPlan>& p) {
+    GemmItems<NB> items{};
+    unsigned gx = 1, gy = 1, gz = 0;
+    double bytes = 0.0, flops = 0.0;
+    const int T = p[0].T, mode = p[0].mode;
+    for (size_t i = 0; i < p.size(); ++i) {
+        const GemmItem& g = items.job[i] = p[i].it;
+        const int64_t tx = (g.m + T - 1) / T, ty = (g.n + T - 1) / T;
+        gx = std::max(gx, (unsigned)tx);
+        gy = std::max(gy, (unsigned)ty);
+        gz += g.nsplit;
+        bytes += 8.0 * (double)(g.m * ty + g.n * tx) * g.K + 8.0 * g.m * g.n * g.nsplit;
+        flops += 2.0 * g.m * g.n * g.K;
+    }
+    ProfScope ps(c, mode ? "gemm_df" : "gemm_f64", bytes, flops);
+    void (*kern)(GemmItems<NB>) = T == 8   ? gemm_small_kernel<8, NB>
+                                  : T == 4 ? gemm_small_kernel<4, NB>
+                                           : (mode == 1 ? gemm_tile16_kernel<1, NB>
+                                                        : (mode == 2 ? gemm_tile16_kernel<2, NB> : gemm_tile16_kernel<0, NB>));
+    run_kernel(c, kern, dim3(gx, gy, gz), 256, 0, items);
+    c.counted();
+    c.check_launch();
+}
+
+// Products that run on the same kernel share a launch (the Grams of the modes of a 512^3 tensor's factors, on
+// three streams before: orthonormalisation @o0@ -> @o1@ us); every product is computed as it would be alone.
+void gemm_nt_f64(Ctx& c, const std::vector<GemmJob>& jobs) {
+    std::vector<GemmPlan> plans;
+    for (const GemmJob& j : jobs) {
+        plans.push_back(gemm_plan(c, j));
+        if (j.m == 0 || j.n == 0) plans.pop_back();
+    }
+    if (!c.exec) return;
+    std::vector<char> done(plans.size(), 0);
+    for (size_t i = 0; i < plans.size(); ++i) {
+        if (done[i]) continue;
+        std::vector<GemmPlan> same;
+        for (size_t q = i; q < plans.size() && same.size() < TK_MAX_D; ++q)
+            if (!done[q] && plans[q].T == plans[i].T && plans[q].mode == plans[i].mode) {
+                same.push_back(plans[q]);
+                done[q] = 1;
+            }
+        if (same.size() == 1) gemm_run<1>(c, same);
+        else gemm_run<TK_MAX_D>(c, same);
+    }
+    for (const GemmPlan& p : plans) {
+        if (p.it.nsplit == 1 || p.it.ctr) continue;
+        const GemmItem& g = p.it;
+        const int64_t tot = g.m * g.n;
+        ProfScope ps(c, "gemm_f64", 8.0 * g.m * g.n * (g.nsplit + 1), (double)g.m * g.n * g.nsplit);
+        run_kernel(c, gemm_reduce_kernel, (unsigned)((tot + 255) / 256), 256, 0, g.m, g.n, g.nsplit, g.P, g.alpha, g.beta,
+                   g.C, g.ldc, g.skip);
         c.counted();
         c.check_launch();
     }
-    if (nsplit > 1 && !ctr) {
-        const int64_t tot = m * n;
-        ProfScope ps(c, "gemm_f64", 8.0 * m * n * (nsplit + 1), (double)m * n * nsplit);
-        run_kernel(c, gemm_reduce_kernel, (unsigned)((tot + 255) / 256), 256, 0, m, n, (int)nsplit, P, alpha, beta, C,
-                   ldc, skip);
-        c.counted();
-        c.check_launch();
-    }
+}
+
+void gemm_nt_f64(Ctx& c, int64_t m, int64_t n, int64_t K, const View2& A, const View2& B, double alpha, double beta,
+                 double* C, int64_t ldc, const int* skip, bool df_ok) {
+    gemm_nt_f64(c, {{m, n, K, A, B, alpha, beta, C, ldc, skip, df_ok}});
 }
 
 // ------------------------------------------------------------------ block reductions
@@ -1114,47 +1190,7 @@ void launch_chol_inv(const Ctx& c, int batch, const KDims& kd, int kmax, const d
 
 // ------------------------------------------------------------------ Q = Y R^{-1}
 
-__global__ void __launch_bounds__(256) apply_rinv_kernel(int64_t n, int64_t k, int rpc, View2 Y, const double* Rinv,
-                                                         int64_t ldr, double* Q, const int* skip) {
-    kernel_begin();
-    extern __shared__ double ys[];  // rpc x k
-    if (skip && *skip) return;
-    const int64_t i0 = (int64_t)blockIdx.x * rpc;
-    for (int64_t e = threadIdx.x; e < rpc * k; e += blockDim.x) {
-        int64_t ii = e % rpc, cc = e / rpc;
-        ys[e] = (i0 + ii < n) ? v2ld(Y, i0 + ii, cc) : 0.0;
-    }
-    __syncthreads();
-    for (int64_t e = threadIdx.x; e < rpc * k; e += blockDim.x) {
-        int64_t ii = e % rpc, col = e / rpc;
-        if (i0 + ii >= n) continue;
-        double s = 0.0;
-        for (int64_t cp = 0; cp <= col; ++cp) s = fma(ys[ii + rpc * cp], __ldg(Rinv + cp + ldr * col), s);
-        Q[(i0 + ii) + n * col] = s;
-    }
-}
-
-void launch_apply_rinv(const Ctx& c, int64_t n, int64_t k, const View2& Y, const double* Rinv, int64_t ldr, double* Q,
-                       const int* skip) {
-    if (!c.exec) return;
-    // rows per CTA: enough CTAs to cover the SMs (the FP64 pipe of one SM is narrow), at most 8
-    const int rpc = (int)std::min<int64_t>(8, std::max<int64_t>(1, (n + 151) / 152));
-    size_t smem = sizeof(double) * rpc * k;
-    if (smem > 48 * 1024)
-        TK_CUDA(cudaFuncSetAttribute(apply_rinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    ProfScope ps(c, "apply_rinv", 16.0 * n * k + 8.0 * k * k, (double)n * k * k);
-    run_kernel(c, apply_rinv_kernel, (unsigned)((n + rpc - 1) / rpc), 256, smem, n, k, rpc, Y, Rinv, ldr, Q, skip);
-    c.counted();
-    c.check_launch();
-}
-
-// The same product for several matrices in one launch, in double-float
-// arithmetic on the FP32 pipe: Y (FP32 or FP64) and R^{-1} (FP64) are split
-// into hi + lo pairs and each output is a Dot2 sum (exact two-product of the
-// high parts, the cross terms and both rounding errors in the correction),
-// ~48 significant bits.  CTA (x, b): rows 32x .. 32x+31 of matrix b, a lane
-// per row; warps take the column pairs (c, k-1-c) in turn, so that every
-// warp sums about the same number of terms.
+// The matrices of one launch (blockIdx.y).
 struct ApplyBatch {
     View2 Y[TK_MAX_D];
     const double* R[TK_MAX_D];
@@ -1165,10 +1201,48 @@ struct ApplyBatch {
     int64_t ldr;
 };
 
+// Rows per CTA: enough CTAs to cover the SMs (the FP64 pipe of one SM is narrow), at most 8.
+__host__ __device__ inline int apply_rows(int64_t n) {
+    const int64_t q = (n + 151) / 152;
+    return (int)(q < 1 ? 1 : (q > 8 ? 8 : q));
+}
+
+__global__ void __launch_bounds__(256) apply_rinv_kernel(const __grid_constant__ ApplyBatch ab) {
+    kernel_begin();
+    extern __shared__ double ys[];  // rpc x k
+    const int b = blockIdx.y;
+    if (ab.skip[b] && *ab.skip[b]) return;
+    const View2& Y = ab.Y[b];
+    const double* Rinv = ab.R[b];
+    const int64_t n = ab.n[b], ldr = ab.ldr;
+    const int k = ab.k[b], rpc = apply_rows(n);
+    const int64_t i0 = (int64_t)blockIdx.x * rpc;
+    if (i0 >= n) return;
+    for (int64_t e = threadIdx.x; e < rpc * k; e += blockDim.x) {
+        int64_t ii = e % rpc, cc = e / rpc;
+        ys[e] = (i0 + ii < n) ? v2ld(Y, i0 + ii, cc) : 0.0;
+    }
+    __syncthreads();
+    for (int64_t e = threadIdx.x; e < rpc * k; e += blockDim.x) {
+        int64_t ii = e % rpc, col = e / rpc;
+        if (i0 + ii >= n) continue;
+        double s = 0.0;
+        for (int64_t cp = 0; cp <= col; ++cp) s = fma(ys[ii + rpc * cp], __ldg(Rinv + cp + ldr * col), s);
+        ab.Q[b][(i0 + ii) + n * col] = s;
+    }
+}
+
+// The same product in double-float
+// arithmetic on the FP32 pipe: Y (FP32 or FP64) and R^{-1} (FP64) are split
+// into hi + lo pairs and each output is a Dot2 sum (exact two-product of the
+// high parts, the cross terms and both rounding errors in the correction),
+// ~48 significant bits.  CTA (x, b): rows 32x .. 32x+31 of matrix b, a lane
+// per row; warps take the column pairs (c, k-1-c) in turn, so that every
+// warp sums about the same number of terms.
 constexpr int APDF_THREADS = 256;
 constexpr int APDF_U = 8;  // global loads in flight per thread while staging
 
-__global__ void __launch_bounds__(APDF_THREADS) apply_rinv_df_kernel(ApplyBatch ab) {
+__global__ void __launch_bounds__(APDF_THREADS) apply_rinv_df_kernel(const __grid_constant__ ApplyBatch ab) {
     kernel_begin();
     extern __shared__ float2 sa[];  // R^{-1}: k x k column-major, then Y rows: k x 32 ([col][row])
     const int b = blockIdx.y;
@@ -1248,11 +1322,11 @@ __global__ void __launch_bounds__(APDF_THREADS) apply_rinv_df_kernel(ApplyBatch 
     }
 }
 
-void launch_apply_rinv_df(const Ctx& c, int batch, const View2* Y, const int64_t* n, const int64_t* k,
-                          const double* Rinv, int64_t kmax, double* const* Q, const int* bad) {
+void launch_apply_rinv(const Ctx& c, int batch, const View2* Y, const int64_t* n, const int64_t* k, const double* Rinv,
+                       int64_t kmax, double* const* Q, const int* bad, bool df) {
     if (!c.exec) return;
-    ApplyBatch ab;
-    int64_t nmax = 1;
+    ApplyBatch ab{};
+    int64_t nmax = 1, ctas = 1, most = 1;
     for (int b = 0; b < batch; ++b) {
         ab.Y[b] = Y[b];
         ab.R[b] = Rinv + b * kmax * kmax;
@@ -1261,28 +1335,41 @@ void launch_apply_rinv_df(const Ctx& c, int batch, const View2* Y, const int64_t
         ab.n[b] = n[b];
         ab.k[b] = (int)k[b];
         nmax = std::max(nmax, n[b]);
+        ctas = std::max(ctas, (n[b] + apply_rows(n[b]) - 1) / apply_rows(n[b]));
+        most = std::max<int64_t>(most, apply_rows(n[b]) * k[b]);
     }
     ab.ldr = kmax;
-    const size_t smem = sizeof(float2) * (kmax * kmax + 32 * kmax);
+    void (*kern)(ApplyBatch) = df ? apply_rinv_df_kernel : apply_rinv_kernel;
+    const size_t smem = df ? sizeof(float2) * (kmax * kmax + 32 * kmax) : sizeof(double) * most;
     if (smem > 48 * 1024)
-        TK_CUDA(cudaFuncSetAttribute(apply_rinv_df_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     double bytes = 0.0, flops = 0.0;
     for (int b = 0; b < batch; ++b) {
         bytes += 16.0 * n[b] * k[b] + 8.0 * k[b] * k[b];
         flops += (double)n[b] * k[b] * k[b];
     }
     ProfScope ps(c, "apply_rinv", bytes, flops);
-    dim3 grid((unsigned)((nmax + 31) / 32), (unsigned)batch);
-    run_kernel(c, apply_rinv_df_kernel, grid, APDF_THREADS, smem, ab);
+    dim3 grid((unsigned)(df ? (nmax + 31) / 32 : ctas), (unsigned)batch);
+    run_kernel(c, kern, grid, df ? APDF_THREADS : 256, smem, ab);
     c.counted();
     c.check_launch();
 }
 
 // ------------------------------------------------------------------ Householder QR (fallback)
 
-__global__ void __launch_bounds__(256) householder_kernel(int64_t n, int64_t k, View2 Y, double* A, double* Q,
-                                                          double* tau, const int* run, int* slot, int slot_value) {
+struct HouseBatch {
+    HouseJob job[TK_MAX_D];
+};
+
+__global__ void __launch_bounds__(256) householder_kernel(const __grid_constant__ HouseBatch hb) {
     kernel_begin();
+    const HouseJob& hj = hb.job[blockIdx.x];
+    const int64_t n = hj.n, k = hj.k;
+    const View2& Y = hj.Y;
+    double *const A = hj.A, *const Q = hj.Q, *const tau = hj.tau;
+    const int* const run = hj.run;
+    int* const slot = hj.slot;
+    const int slot_value = hj.slot_value;
     __shared__ double red[33];
     __shared__ double v0s[256];
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -1357,12 +1444,19 @@ __global__ void __launch_bounds__(256) householder_kernel(int64_t n, int64_t k, 
     }
 }
 
-void launch_householder(const Ctx& c, int64_t n, int64_t k, const View2& Y, double* A, double* Q, double* tau,
-                        const int* run, int* slot, int slot_value) {
-    if (!c.exec) return;
-    TK_REQUIRE(k <= 256, TK_ERR_SHAPE, "householder: at most 256 columns");
-    ProfScope ps(c, "householder", 16.0 * n * k, 8.0 * n * k * k);
-    run_kernel(c, householder_kernel, 1, 256, 0, n, k, Y, A, Q, tau, run, slot, slot_value);
+void launch_householder(const Ctx& c, const std::vector<HouseJob>& jobs) {
+    if (!c.exec || jobs.empty()) return;
+    TK_REQUIRE(jobs.size() <= TK_MAX_D, TK_ERR_ARG, "householder: too many matrices");
+    HouseBatch hb{};
+    double bytes = 0.0, flops = 0.0;
+    for (size_t b = 0; b < jobs.size(); ++b) {
+        TK_REQUIRE(jobs[b].k <= 256, TK_ERR_SHAPE, "householder: at most 256 columns");
+        hb.job[b] = jobs[b];
+        bytes += 16.0 * jobs[b].n * jobs[b].k;
+        flops += 8.0 * jobs[b].n * jobs[b].k * jobs[b].k;
+    }
+    ProfScope ps(c, "householder", bytes, flops);
+    run_kernel(c, householder_kernel, (unsigned)jobs.size(), 256, 0, hb);
     c.counted();
     c.check_launch();
 }
@@ -2129,25 +2223,56 @@ void launch_select_top(const Ctx& c, int64_t k, int64_t r, const double* D, cons
 
 // ------------------------------------------------------------------ element-wise helpers
 
-__global__ void convert_kernel(const void* src, tk_dtype sdt, int64_t rows, int64_t cols, int64_t lds, void* dst,
-                               tk_dtype ddt, int64_t ldd, float inv) {
+// The copies of one launch (blockIdx.y).
+template <int NB>
+struct ConvertBatch {
+    ConvertJob job[NB];
+};
+
+template <int NB>
+__global__ void convert_kernel(const __grid_constant__ ConvertBatch<NB> cb) {
     kernel_begin();
+    const ConvertJob& j = cb.job[NB > 1 ? blockIdx.y : 0];
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= rows * cols) return;
-    int64_t i = idx % rows, j = idx / rows;
-    st_any(dst, ddt, i + ldd * j, ld_any(src, sdt, i + lds * j, inv));
+    if (idx >= j.rows * j.cols) return;
+    int64_t i = idx % j.rows, a = idx / j.rows;
+    st_any(j.dst, j.ddt, i + j.ldd * a, ld_any(j.src, j.sdt, i + j.lds * a, j.inv));
+}
+
+template <int NB>
+static void convert_run(const Ctx& c, const ConvertJob* jobs, int count) {
+    ConvertBatch<NB> cb{};
+    int64_t most = 0;
+    double bytes = 0.0;
+    for (int b = 0; b < count; ++b) {
+        const int64_t tot = jobs[b].rows * jobs[b].cols;
+        cb.job[b] = jobs[b];
+        most = std::max(most, tot);
+        bytes += (double)tot * (dtype_size(jobs[b].sdt) + dtype_size(jobs[b].ddt));
+    }
+    ProfScope ps(c, "elementwise", bytes, 0.0);
+    run_kernel(c, convert_kernel<NB>, dim3((unsigned)((most + 255) / 256), (unsigned)count), 256, 0, cb);
+    c.counted();
+    c.check_launch();
 }
 
 void launch_convert(const Ctx& c, const void* src, tk_dtype sdt, int64_t rows, int64_t cols, int64_t lds, void* dst,
                     tk_dtype ddt, int64_t ldd, float src_scale) {
     if (!c.exec || rows * cols == 0) return;
-    float inv = (sdt == TK_FP8_E4M3) ? 1.f / src_scale : 1.f;
-    int64_t tot = rows * cols;
-    ProfScope ps(c, "elementwise", (double)tot * (dtype_size(sdt) + dtype_size(ddt)), 0.0);
-    run_kernel(c, convert_kernel, (unsigned)((tot + 255) / 256), 256, 0, src, sdt, rows, cols, lds, dst, ddt, ldd,
-               inv);
-    c.counted();
-    c.check_launch();
+    const ConvertJob job{src, dst, sdt, ddt, rows, cols, lds, ldd, sdt == TK_FP8_E4M3 ? 1.f / src_scale : 1.f};
+    convert_run<1>(c, &job, 1);
+}
+
+void launch_convert(const Ctx& c, const std::vector<ConvertJob>& jobs) {
+    if (!c.exec) return;
+    std::vector<ConvertJob> some;
+    for (const ConvertJob& j : jobs)
+        if (j.rows * j.cols) some.push_back(j);
+    for (size_t b = 0; b < some.size(); b += TK_MAX_D) {
+        const int count = (int)std::min<size_t>(TK_MAX_D, some.size() - b);
+        if (count == 1) convert_run<1>(c, some.data() + b, 1);
+        else convert_run<TK_MAX_D>(c, some.data() + b, count);
+    }
 }
 
 __global__ void fill_identity_kernel(double* Q, int64_t n) {
@@ -2194,7 +2319,9 @@ void launch_fill_int(const Ctx& c, int* p, int count, int value) {
 }
 
 __global__ void qr_info_kernel(int* slot, const int* bad, int bad_value) {
-    kernel_begin(); *slot = *bad ? bad_value : 0; }
+    kernel_begin();
+    *slot = *bad ? bad_value : 0;
+}
 void launch_qr_info(const Ctx& c, int* slot, const int* bad, int bad_value) {
     if (!c.exec) return;
     ProfScope ps(c, "elementwise", 8.0, 0.0);
@@ -2203,9 +2330,18 @@ void launch_qr_info(const Ctx& c, int* slot, const int* bad, int bad_value) {
     c.check_launch();
 }
 
-__global__ void __launch_bounds__(256) sign_fix_kernel(double* U, int64_t n, double* sign, void* out, tk_dtype odt,
-                                                       int64_t ldo) {
+struct SignBatch {
+    SignJob job[TK_MAX_D];
+};
+
+__global__ void __launch_bounds__(256) sign_fix_kernel(const __grid_constant__ SignBatch sb) {
     kernel_begin();
+    const SignJob& sj = sb.job[blockIdx.y];
+    if (blockIdx.x >= sj.r) return;
+    double *const U = sj.U, *const sign = sj.sign;
+    void* const out = sj.out;
+    const tk_dtype odt = sj.odt;
+    const int64_t n = sj.n, ldo = sj.ldo;
     __shared__ double bv[256];
     __shared__ int64_t bi[256];
     const int64_t col = blockIdx.x;
@@ -2240,11 +2376,20 @@ __global__ void __launch_bounds__(256) sign_fix_kernel(double* U, int64_t n, dou
     if (threadIdx.x == 0) sign[col] = sg;
 }
 
-void launch_sign_fix(const Ctx& c, double* U, int64_t n, int64_t r, double* sign, void* out, tk_dtype odt,
-                     int64_t ldo) {
-    if (!c.exec || r == 0) return;
-    ProfScope ps(c, "elementwise", 16.0 * n * r, 0.0);
-    run_kernel(c, sign_fix_kernel, (unsigned)r, 256, 0, U, n, sign, out, odt, ldo);
+void launch_sign_fix(const Ctx& c, const std::vector<SignJob>& jobs) {
+    if (!c.exec) return;
+    TK_REQUIRE(jobs.size() <= TK_MAX_D, TK_ERR_ARG, "sign_fix: too many matrices");
+    SignBatch sb{};
+    int64_t r = 0;
+    double bytes = 0.0;
+    for (size_t b = 0; b < jobs.size(); ++b) {
+        sb.job[b] = jobs[b];
+        r = std::max(r, jobs[b].r);
+        bytes += 16.0 * jobs[b].n * jobs[b].r;
+    }
+    if (r == 0) return;
+    ProfScope ps(c, "elementwise", bytes, 0.0);
+    run_kernel(c, sign_fix_kernel, dim3((unsigned)r, (unsigned)jobs.size()), 256, 0, sb);
     c.counted();
     c.check_launch();
 }

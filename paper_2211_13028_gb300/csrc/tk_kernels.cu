@@ -396,34 +396,44 @@ void launch_sign_copy(const Ctx& c, const Tens& X, int n, uint64_t seed, void* d
 
 // ------------------------------------------------------------------ FP64 GEMM (NT) with split-K
 
+// The partial products of a split-K product are stored tile by tile (T x T, the tiles that are computed only).
+__host__ __device__ inline int64_t gemm_tile_index(int64_t x, int64_t y, int64_t tm, bool sym) {
+    return sym ? y * (y + 1) / 2 + x : x + tm * y;
+}
+
 __global__ void gemm_reduce_kernel(int64_t m, int64_t n, int nsplit, const double* P, double alpha, double beta,
-                                   double* C, int64_t ldc, const int* skip) {
+                                   double* C, int64_t ldc, const int* skip, int T, int sym, int64_t tiles) {
     kernel_begin();
     if (skip && *skip) return;
     int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= m * n) return;
+    const int64_t a = idx % m, b = idx / m;
+    const bool flip = sym && a / T > b / T;
+    const int64_t r = flip ? b : a, c = flip ? a : b;
+    const double* p = P + gemm_tile_index(r / T, c / T, (m + T - 1) / T, sym) * T * T + r % T + T * (c % T);
     double s = 0;
-    for (int z = 0; z < nsplit; ++z) s += P[(int64_t)z * m * n + idx];
-    int64_t a = idx % m, b = idx / m;
+    for (int z = 0; z < nsplit; ++z) s += p[(int64_t)z * tiles * T * T];
     double* dst = C + a + ldc * b;
     *dst = beta == 0.0 ? alpha * s : alpha * s + beta * *dst;
 }
 
-// 16 x 16 output tile per 256-thread CTA (one output per thread), K staged
-// through shared memory 32 at a time for both operands (converted to FP64 on
-// load).  Each operand is loaded with lanes running along whichever of its two
+// T x T output tile per 256-thread CTA, T = 16 TR (TR x TR outputs per thread), K staged
+// through shared memory 32 at a time for both operands (converted on
+// load), the next 32 in registers meanwhile.  Each operand is loaded with lanes running along whichever of its two
 // indices is contiguous in memory.  Split-K: CTA z covers [z kchunk, (z+1)
 // kchunk) and, with P != NULL, writes its partial tile to P[z] for a
 // deterministic reduction; otherwise it applies alpha/beta to C directly.
+// A Gram (B the same view as A) computes the tiles x <= y and writes their mirror images.
 struct TileLoader {
-    // element e in [0, 512) of a 16 x 32 (row x k) tile -> (row, k)
+    // element e of a T x 32 (row x k) tile -> (row, k)
     bool kfast;
     // k contiguous within 32-aligned runs (plain columns, or an unfolding whose
     // fastest contracted mode is a multiple of 32 long): warps read along k
     __device__ TileLoader(const View2& v) { kfast = v.st1 == 1 && (v.T1 == INT64_MAX || v.T1 % 32 == 0); }
+    template <int T>
     __device__ __forceinline__ void rk(int e, int& r, int& kk) const {
         if (kfast) { r = e >> 5; kk = e & 31; }
-        else { r = e & 15; kk = e >> 4; }
+        else { r = e % T; kk = e / T; }
     }
 };
 
@@ -580,7 +590,9 @@ struct GemmItem {
     double* P;
     unsigned* ctr;
     const int* skip;
+    int64_t tiles;  // computed
     int nsplit;
+    int sym;  // a Gram
 };
 template <int NB>
 struct GemmItems {
@@ -590,10 +602,11 @@ struct GemmItems {
 // MODE 2: the operands (FP64 or FP32) are split into double-float pairs on
 // load and the products accumulate with df_dot_step on the FP32 pipe (~47
 // significant bits; FP32's exponent range bounds the products).
-template <int MODE, int NB>
-__global__ void __launch_bounds__(256) gemm_tile16_kernel(const __grid_constant__ GemmItems<NB> items) {
+template <int MODE, int NB, int TR>
+__global__ void __launch_bounds__(256) gemm_tile_kernel(const __grid_constant__ GemmItems<NB> items) {
     kernel_begin();
     constexpr bool DFACC = MODE != 0;
+    constexpr int T = 16 * TR, NE = 2 * TR;  // elements a thread loads per operand and chunk
     using E = typename std::conditional<MODE == 0, double, typename std::conditional<MODE == 1, float, float2>::type>::type;
     int q0 = 0, z = blockIdx.z;
     if (NB > 1)
@@ -601,82 +614,123 @@ __global__ void __launch_bounds__(256) gemm_tile16_kernel(const __grid_constant_
     const GemmItem& g = items.job[q0];
     const View2 &A = g.A, &B = g.B;
     const int64_t m = g.m, n = g.n, K = g.K, ldc = g.ldc;
-    const double alpha = g.alpha, beta = g.beta;
-    double* const C = g.C;
-    double* const P = g.P;
     if (g.skip && *g.skip) return;
-    if ((int64_t)blockIdx.x * 16 >= m || (int64_t)blockIdx.y * 16 >= n) return;  // (the grid covers the largest)
-    __shared__ E As[32][17];
-    __shared__ E Bs[32][17];
+    if ((int64_t)blockIdx.x * T >= m || (int64_t)blockIdx.y * T >= n) return;  // (the grid covers the largest)
+    if (g.sym && blockIdx.x > blockIdx.y) return;
+    const bool same = g.sym && blockIdx.x == blockIdx.y;  // both operands are the same rows
+    __shared__ E As[32][T + 1];
+    __shared__ E Bs[32][T + 1];
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
-    const int64_t a0 = (int64_t)blockIdx.x * 16, b0 = (int64_t)blockIdx.y * 16;
+    const int64_t a0 = (int64_t)blockIdx.x * T, b0 = (int64_t)blockIdx.y * T;
     const int64_t kb = z * g.kchunk;
     const int64_t ke = min(K, kb + g.kchunk);
     const TileLoader la(A), lb(B);
-    int ra[2], ka[2], rb[2], kb2[2];
-    int64_t oa[2], ob[2];
+    int ra[NE], ka[NE], rb[NE], kb2[NE];
+    int64_t oa[NE], ob[NE];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        la.rk(tid + 256 * q, ra[q], ka[q]);
-        lb.rk(tid + 256 * q, rb[q], kb2[q]);
+    for (int q = 0; q < NE; ++q) {
+        la.rk<T>(tid + 256 * q, ra[q], ka[q]);
+        lb.rk<T>(tid + 256 * q, rb[q], kb2[q]);
         oa[q] = a0 + ra[q] < m ? v2row(A, a0 + ra[q]) : -1;
-        ob[q] = b0 + rb[q] < n ? v2row(B, b0 + rb[q]) : -1;
+        ob[q] = b0 + rb[q] < n && !same ? v2row(B, b0 + rb[q]) : -1;
     }
-    double acc0 = 0.0, acc1 = 0.0;
-    float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
+    double va[NE], vb[NE];
+    auto load = [&](int64_t k0) {
+        int64_t ca = 0, cb = 0;
+#pragma unroll
+        for (int q = 0; q < NE; ++q) {
+            const int64_t k1 = k0 + ka[q], k2 = k0 + kb2[q];
+            if (q == 0 || !la.kfast) ca = v2col(A, k1);  // (along k, every element of the thread has the same k)
+            if (q == 0 || !lb.kfast) cb = v2col(B, k2);
+            va[q] = (oa[q] >= 0 && k1 < ke) ? v2get(A, oa[q] + ca) : 0.0;
+            vb[q] = (ob[q] >= 0 && k2 < ke) ? v2get(B, ob[q] + cb) : 0.0;
+        }
+    };
+    const E(*Bp)[T + 1] = same ? As : Bs;
+    double acc[TR][TR][2];
+    float h[TR][TR][2], l[TR][TR][2];
+#pragma unroll
+    for (int i = 0; i < TR * TR * 2; ++i) {
+        (&acc[0][0][0])[i] = 0.0;
+        (&h[0][0][0])[i] = (&l[0][0][0])[i] = 0.f;
+    }
+    if (kb < ke) load(kb);
     for (int64_t k0 = kb; k0 < ke; k0 += 32) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int64_t k1 = k0 + ka[q], k2 = k0 + kb2[q];
-            As[ka[q]][ra[q]] = gemm_elem<E>((oa[q] >= 0 && k1 < ke) ? v2get(A, oa[q] + v2col(A, k1)) : 0.0);
-            Bs[kb2[q]][rb[q]] = gemm_elem<E>((ob[q] >= 0 && k2 < ke) ? v2get(B, ob[q] + v2col(B, k2)) : 0.0);
+        for (int q = 0; q < NE; ++q) {
+            As[ka[q]][ra[q]] = gemm_elem<E>(va[q]);
+            if (!same) Bs[kb2[q]][rb[q]] = gemm_elem<E>(vb[q]);
         }
         __syncthreads();
-#pragma unroll
+        if (k0 + 32 < ke) load(k0 + 32);
+#pragma unroll 4
         for (int kk = 0; kk < 32; kk += 2) {
-            if constexpr (MODE == 2) {
-                df_dot_step(h0, l0, As[kk][tx], Bs[kk][ty]);
-                df_dot_step(h1, l1, As[kk + 1][tx], Bs[kk + 1][ty]);
-            } else if constexpr (MODE == 1) {
-                dot2_step(h0, l0, As[kk][tx], Bs[kk][ty]);
-                dot2_step(h1, l1, As[kk + 1][tx], Bs[kk + 1][ty]);
-            } else {
-                acc0 = fma(As[kk][tx], Bs[kk][ty], acc0);
-                acc1 = fma(As[kk + 1][tx], Bs[kk + 1][ty], acc1);
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+                E a[TR], b[TR];
+#pragma unroll
+                for (int i = 0; i < TR; ++i) {
+                    a[i] = As[kk + w][tx + 16 * i];
+                    b[i] = Bp[kk + w][ty + 16 * i];
+                }
+#pragma unroll
+                for (int i = 0; i < TR; ++i)
+#pragma unroll
+                    for (int j = 0; j < TR; ++j) {
+                        if constexpr (MODE == 2)
+                            df_dot_step(h[i][j][w], l[i][j][w], a[i], b[j]);
+                        else if constexpr (MODE == 1)
+                            dot2_step(h[i][j][w], l[i][j][w], a[i], b[j]);
+                        else
+                            acc[i][j][w] = fma(a[i], b[j], acc[i][j][w]);
+                    }
             }
         }
         __syncthreads();
     }
-    const int64_t a = a0 + tx, b = b0 + ty;
-    const bool in = a < m && b < n;
-    const double sum = DFACC ? ((double)h0 + (double)l0) + ((double)h1 + (double)l1) : acc0 + acc1;
-    if (!P) {
-        if (in) {
-            double* dst = C + a + ldc * b;
-            *dst = beta == 0.0 ? alpha * sum : alpha * sum + beta * *dst;
+    const int64_t tm = (m + T - 1) / T, slice = g.tiles * T * T;
+    double* const P = g.P ? g.P + gemm_tile_index(blockIdx.x, blockIdx.y, tm, g.sym) * T * T : nullptr;
+    auto store = [&](int64_t a, int64_t b, double v) {
+        double* dst = g.C + a + ldc * b;
+        *dst = g.beta == 0.0 ? g.alpha * v : g.alpha * v + g.beta * *dst;
+        if (g.sym && !same) g.C[b + ldc * a] = g.alpha * v;
+    };
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < TR; ++j) {
+            const int64_t a = a0 + tx + 16 * i, b = b0 + ty + 16 * j;
+            if (a >= m || b >= n) continue;
+            const double sum = DFACC ? ((double)h[i][j][0] + (double)l[i][j][0]) + ((double)h[i][j][1] + (double)l[i][j][1])
+                                     : acc[i][j][0] + acc[i][j][1];
+            if (P) P[z * slice + tx + 16 * i + T * (ty + 16 * j)] = sum;
+            else store(a, b, sum);
         }
-        return;
-    }
-    if (in) P[(int64_t)z * m * n + a + m * b] = sum;
-    if (!g.ctr) return;  // a separate reduction kernel adds the partial tiles
+    if (!P || !g.ctr) return;  // (without a counter a separate reduction kernel adds the partial tiles)
     // the last CTA of this tile to arrive adds the partial tiles (and re-zeroes the counter)
     __shared__ int s_last;
     __threadfence();
     __syncthreads();
     if (tid == 0) {
-        unsigned* t = g.ctr + blockIdx.x + (m + 15) / 16 * blockIdx.y;
+        unsigned* t = g.ctr + blockIdx.x + tm * blockIdx.y;
         const unsigned prev = atomicAdd(t, 1u);
         s_last = prev == g.nsplit - 1u;
         if (s_last) *t = 0u;
     }
     __syncthreads();
-    if (!s_last || !in) return;
+    if (!s_last) return;
     __threadfence();
-    double tot = 0.0;
-    for (int w = 0; w < g.nsplit; ++w) tot += __ldcg(P + (int64_t)w * m * n + a + m * b);
-    double* dst = C + a + ldc * b;
-    *dst = beta == 0.0 ? alpha * tot : alpha * tot + beta * *dst;
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < TR; ++j) {
+            const int64_t a = a0 + tx + 16 * i, b = b0 + ty + 16 * j;
+            if (a >= m || b >= n) continue;
+            double tot = 0.0;
+            for (int w = 0; w < g.nsplit; ++w) tot += __ldcg(P + w * slice + tx + 16 * i + T * (ty + 16 * j));
+            store(a, b, tot);
+        }
 }
 
 // Small FP64 products (FP64 runs at 2 FMA per clock per SM here, so a
@@ -734,17 +788,47 @@ __global__ void __launch_bounds__(256) gemm_small_kernel(const __grid_constant__
     *dst = beta == 0.0 ? alpha * sum : alpha * sum + beta * *dst;
 }
 
-// Which kernel a product runs on: 16 x 16 tiles (T = 16) in one of the arithmetics, or the small ones.
+// Which kernel a product runs on: tiles of T = 16 or 32 in one of the arithmetics, or the small ones.
 struct GemmPlan {
     int mode, T;
     GemmItem it;
 };
 
-static GemmPlan gemm_plan(Ctx& c, const GemmJob& j) {
-    GemmPlan p{};
+static bool gemm_gram(const GemmJob& j) {
+    const View2 &A = j.A, &B = j.B;
+    return A.p == B.p && A.dt == B.dt && A.A1 == B.A1 && A.sa1 == B.sa1 && A.sa2 == B.sa2 && A.T1 == B.T1 &&
+           A.st1 == B.st1 && A.st2 == B.st2 && j.m == j.n && j.beta == 0.0;
+}
+
+// The tiles of T x T that a product computes.
+static int64_t gemm_tiles(const GemmJob& j, int64_t T) {
+    const int64_t tm = (j.m + T - 1) / T, tn = (j.n + T - 1) / T;
+    return gemm_gram(j) ? tm * (tm + 1) / 2 : tm * tn;
+}
+
+static int gemm_mode(const Ctx& c, const GemmJob& j) {
     // Dot2 accumulation where the caller allows it and both operands are FP32; double-float
     // operands throughout a call on FP32-class data (c.df64)
-    p.mode = (j.df_ok && j.A.dt == TK_F32 && j.B.dt == TK_F32) ? 1 : (c.df64 ? 2 : 0);
+    return (j.df_ok && j.A.dt == TK_F32 && j.B.dt == TK_F32) ? 1 : (c.df64 ? 2 : 0);
+}
+
+// Short K and few 16 x 16 tiles: smaller tiles with K split inside the CTA.
+static bool gemm_is_small(const Ctx& c, const GemmJob& j) {
+    return gemm_mode(c, j) != 1 && j.K < 128 && ((j.m + 15) / 16) * ((j.n + 15) / 16) < 152;
+}
+
+// 32 x 32 tiles (four outputs a thread: half the shared-memory reads and the loads of a product): where splits of
+// 128 terms still make a CTA for every SM and the tiles' edges waste no more than a third of the products (Grams
+// of a core of 81^3 192 -> 155 us; of 512 x 49, whose splits are few, 15 -> 27).  FP64 products are bound by the
+// FP64 pipe.
+static bool gemm_wants_32(const Ctx& c, const GemmJob& j) {
+    const auto pad = [&](int64_t t) { return ((j.m + t - 1) / t * t) * ((j.n + t - 1) / t * t); };
+    return gemm_mode(c, j) != 0 && 3 * pad(32) <= 4 * pad(16) && gemm_tiles(j, 32) * (j.K / 128) >= 152;
+}
+
+static GemmPlan gemm_plan(Ctx& c, const GemmJob& j, bool t32) {
+    GemmPlan p{};
+    p.mode = gemm_mode(c, j);
     p.it.m = j.m;
     p.it.n = j.n;
     p.it.K = j.K;
@@ -757,19 +841,21 @@ static GemmPlan gemm_plan(Ctx& c, const GemmJob& j) {
     p.it.skip = j.skip;
     p.it.nsplit = 1;
     p.it.kchunk = j.K;
-    // short K and few 16 x 16 tiles: smaller tiles with K split inside the CTA
-    const int64_t tiles = ((j.m + 15) / 16) * ((j.n + 15) / 16);
-    if (p.mode != 1 && j.K < 128 && tiles < 152) {
+    if (gemm_is_small(c, j)) {
         p.mode = 0;
         p.T = ((j.m + 7) / 8) * ((j.n + 7) / 8) >= 152 ? 8 : 4;
         return p;
     }
-    p.T = 16;
-    // split K only when the tiles alone leave most SMs idle and
-    // each split still has at least 64 terms.
+    p.T = t32 ? 32 : 16;
+    p.it.sym = gemm_gram(j);
+    const int64_t work = p.it.tiles = gemm_tiles(j, p.T);
+    // split K only when the tiles alone leave most SMs idle (two CTAs an SM, of the larger tiles one) and
+    // each split still has at least 64 (128) terms.
+    const int64_t ctas = t32 ? 152 : 2 * 152, least = t32 ? 128 : 64;
     int64_t nsplit = 1;
-    if (j.K >= 128 && tiles < 2 * 152) {
-        nsplit = std::min<int64_t>((2 * 152 + tiles - 1) / tiles, j.K / 64);
+    if (j.K >= 128 && work < ctas) {
+        // (rounded down for the larger tiles: three CTAs an SM are resident, so three such products are one wave)
+        nsplit = std::min<int64_t>(t32 ? ctas / work : (ctas + work - 1) / work, j.K / least);
         nsplit = std::max<int64_t>(1, std::min<int64_t>(nsplit, 512));
     }
     int64_t kchunk = j.K > 0 ? (j.K + nsplit - 1) / nsplit : 1;
@@ -777,8 +863,9 @@ static GemmPlan gemm_plan(Ctx& c, const GemmJob& j) {
     nsplit = j.K > 0 ? (j.K + kchunk - 1) / kchunk : 1;
     p.it.kchunk = kchunk;
     p.it.nsplit = (int)nsplit;
-    p.it.P = nsplit > 1 ? c.alloc<double>(nsplit * j.m * j.n) : nullptr;
-    if (c.exec && p.it.P && j.m && j.n) p.it.ctr = c.take_counters((int)tiles);
+    p.it.P = nsplit > 1 ? c.alloc<double>(nsplit * work * p.T * p.T) : nullptr;
+    if (c.exec && p.it.P && j.m && j.n)
+        p.it.ctr = c.take_counters((int)(((j.m + p.T - 1) / p.T) * ((j.n + p.T - 1) / p.T)));
     return p;
 }
 
@@ -798,21 +885,28 @@ static void gemm_run(const Ctx& c, const std::vector<GemmPlan>& p) {
         flops += 2.0 * g.m * g.n * g.K;
     }
     ProfScope ps(c, mode ? "gemm_df" : "gemm_f64", bytes, flops);
-    void (*kern)(GemmItems<NB>) = T == 8   ? gemm_small_kernel<8, NB>
-                                  : T == 4 ? gemm_small_kernel<4, NB>
-                                           : (mode == 1 ? gemm_tile16_kernel<1, NB>
-                                                        : (mode == 2 ? gemm_tile16_kernel<2, NB> : gemm_tile16_kernel<0, NB>));
+    void (*kern)(GemmItems<NB>) = nullptr;
+    switch (T) {
+        case 4: kern = gemm_small_kernel<4, NB>; break;
+        case 8: kern = gemm_small_kernel<8, NB>; break;
+        case 16:
+            kern = mode == 1 ? gemm_tile_kernel<1, NB, 1> : (mode == 2 ? gemm_tile_kernel<2, NB, 1> : gemm_tile_kernel<0, NB, 1>);
+            break;
+        default: kern = mode == 1 ? gemm_tile_kernel<1, NB, 2> : gemm_tile_kernel<2, NB, 2>;
+    }
     run_kernel(c, kern, dim3(gx, gy, gz), 256, 0, items);
     c.counted();
     c.check_launch();
 }
 
 // Products that run on the same kernel share a launch (the Grams of the modes of a 512^3 tensor's factors, on
-// three streams before: orthonormalisation @o0@ -> @o1@ us); every product is computed as it would be alone.
+// three streams before: orthonormalisation 132 -> 119 us); every product is computed as it would be alone.
 void gemm_nt_f64(Ctx& c, const std::vector<GemmJob>& jobs) {
     std::vector<GemmPlan> plans;
+    bool t32 = true;
+    for (const GemmJob& j : jobs) t32 = t32 && (gemm_is_small(c, j) || gemm_wants_32(c, j));
     for (const GemmJob& j : jobs) {
-        plans.push_back(gemm_plan(c, j));
+        plans.push_back(gemm_plan(c, j, t32));
         if (j.m == 0 || j.n == 0) plans.pop_back();
     }
     if (!c.exec) return;
@@ -834,7 +928,7 @@ void gemm_nt_f64(Ctx& c, const std::vector<GemmJob>& jobs) {
         const int64_t tot = g.m * g.n;
         ProfScope ps(c, "gemm_f64", 8.0 * g.m * g.n * (g.nsplit + 1), (double)g.m * g.n * g.nsplit);
         run_kernel(c, gemm_reduce_kernel, (unsigned)((tot + 255) / 256), 256, 0, g.m, g.n, g.nsplit, g.P, g.alpha, g.beta,
-                   g.C, g.ldc, g.skip);
+                   g.C, g.ldc, g.skip, p.T, g.sym, g.tiles);
         c.counted();
         c.check_launch();
     }

@@ -102,11 +102,14 @@ struct TtmArgs {
     unsigned* flags;
 };
 
-template <int NPAD, bool FLAT>
+template <int NPAD, bool KMAJOR, bool FLAT>
 struct TtmCfg {
     static constexpr int kBBytes = NPAD * 128;  // one of M_hi / M_lo: NPAD rows of 128 B
     static constexpr int kStage = kXBytes + 2 * kBBytes;
-    static constexpr int kBudget = 210 * 1024;
+    // a tile of the result, staged (L == 1, more than 16 columns: below, a copy a tile costs more than the
+    // scattered stores do, 413 x 350 x 275 with 6 columns 47 -> 52 us)
+    static constexpr int kOut = KMAJOR && NPAD > 16 ? kRows * NPAD * 4 : 0;
+    static constexpr int kBudget = kOut ? 222 * 1024 - kOut : 210 * 1024;
     // FLAT: a shorter ring, which leaves the SM's L1, where each cp.async in flight holds its lines, some
     // room (413 x 350 x 275 along its first mode, 5 columns: 58 us with 10 stages, 47 with 6)
     static constexpr int kStages = FLAT ? (NPAD <= 32 ? 6 : 4) : (kBudget / kStage > 12 ? 12 : kBudget / kStage);
@@ -114,7 +117,7 @@ struct TtmCfg {
     static constexpr int kABuf = 512 - 64 * kNA;
     static constexpr int kFit = kABuf / (2 * NPAD);     // accumulators of 2*NPAD columns
     static constexpr int kAcc = kFit > 8 ? 8 : kFit;
-    static constexpr int kSmem = kStages * kStage + 1024 + 512;
+    static constexpr int kSmem = kStages * kStage + kOut + 1024 + 512;
     static constexpr int kLoad = FLAT ? 8 : 0;          // loader warps, from warp 2
     static constexpr int kFirstConv = FLAT ? 12 : 4;    // (a multiple of 4: warp % 4 is the TMEM lane quarter)
     static constexpr int kGroups = FLAT ? 1 : 2;        // converter groups of 8 warps
@@ -140,16 +143,17 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
 }
 
 template <int NPAD, bool KMAJOR, bool FLAT>
-__global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
+__global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
     ttm_tf32x3_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmB,
                       TtmArgs args) {
     kernel_begin();
-    using C = TtmCfg<NPAD, FLAT>;
+    using C = TtmCfg<NPAD, KMAJOR, FLAT>;
     constexpr uint32_t S = C::kStages;
     constexpr uint32_t NA = C::kNA;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * C::kStage);
+    float* stg = reinterpret_cast<float*>(smem + S * C::kStage);  // kOut: a tile of the result
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * C::kStage + C::kOut);
     uint64_t* full = bars;                   // [S] X and factor chunk landed
     uint64_t* xfree = bars + S;              // [S] stage consumed (8 converter warps + 1 MMA commit)
     uint64_t* afull = bars + 2 * S;          // [NA] A buffer written (8 converter warps)
@@ -157,7 +161,9 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
     uint64_t* accfull = aempty + NA;         // [kAcc] accumulator complete (MMA commit)
     uint64_t* accempty = accfull + C::kAcc; // [kAcc] accumulator drained (the epilogue warps)
     uint64_t* done = accempty + C::kAcc;    // [1] every issued MMA complete
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    uint64_t* stgfree = done + 1;           // [1] staged tile copied out (kOut)
+    uint64_t* stgfull = stgfree + 1;        // [1] tile staged (the epilogue warps)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(stgfull + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -175,6 +181,8 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
             mbar_init(&accempty[b], C::kEpi);
         }
         mbar_init(done, 1);
+        mbar_init(stgfree, 1);
+        mbar_init(stgfull, C::kEpi);
         *abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -482,7 +490,8 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
         const int rho = 32 * q + lane;
         const uint32_t lane_base = (uint32_t)(32 * q) << 16;
         const int64_t m = args.m;
-        uint32_t a = 0, aph = 0;
+        uint32_t a = 0, aph = 0, sph = 0;
+        const bool copier = warp == C::kFirstEpi && lane == 0;
         for (uint32_t w = blockIdx.x; w < args.nitems; w += gridDim.x) {
             const uint32_t w2 = ksplit == 1 ? w : w / ksplit, sk = w - w2 * ksplit;
             const uint32_t t = args.nblk == 1 ? w2 : w2 / args.nblk, nb = args.nblk == 1 ? 0 : w2 % args.nblk;
@@ -552,6 +561,47 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
                 }
             }
             if (!ok) break;
+            // L == 1: the tile's rows are one run of the result.  Unless its lanes can store them in 16 bytes, it
+            // goes out as one bulk copy from a staged copy (4-byte stores of each lane's row reach L2 as pieces of
+            // sectors: 512^3, 42 columns 127 -> 98 us; 413 x 350 x 275, 30 columns 59 -> 56)
+            float* const tile = outp + (int64_t)t * kRows * m;
+            if (C::kOut && (m & 3) != 0 && args.nblk == 1 && (int64_t)(t + 1) * kRows <= args.R &&
+                (reinterpret_cast<uintptr_t>(tile) & 15) == 0) {
+                if (copier) {
+                    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // the tile before has been read
+                    mbar_arrive(stgfree);
+                }
+                if (!__all_sync(0xffffffffu, mbar_wait(stgfree, sph, abort, flags))) break;
+                float* const row = stg + rho * (int)m;
+#pragma unroll
+                for (int j = 0; j < kSl; ++j) {
+                    const int c0 = 16 * half + 32 * j;
+                    if (c0 >= NPAD) break;
+                    if ((m & 1) == 0) {
+#pragma unroll
+                        for (int i = 0; i < 16; i += 2)
+                            if (c0 + i < ncol) *reinterpret_cast<float2*>(row + c0 + i) = make_float2(v[j][i], v[j][i + 1]);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i)
+                            if (c0 + i < ncol) row[c0 + i] = v[j][i];
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the copy reads what was written here
+                __syncwarp();
+                if (lane == 0) mbar_arrive(stgfull);
+                if (copier) {
+                    if (mbar_wait(stgfull, sph, abort, flags)) {
+                        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(tile),
+                                     "r"(smem_u32(stg)), "r"((uint32_t)(kRows * 4 * m))
+                                     : "memory");
+                        asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                    }
+                }
+                __syncwarp();
+                sph ^= 1;
+                continue;
+            }
             if (valid) {
 #pragma unroll
                 for (int j = 0; j < kSl; ++j) {
@@ -571,6 +621,7 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
                 }
             }
         }
+        if (C::kOut && copier) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
     __syncthreads();
     if (warp == 1) {
@@ -581,7 +632,7 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, FLAT>::kThreads, 1)
 
 template <int NPAD, bool KMAJOR, bool FLAT>
 static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorMap& tb, TtmArgs a) {
-    using Cf = TtmCfg<NPAD, FLAT>;
+    using Cf = TtmCfg<NPAD, KMAJOR, FLAT>;
     // above 64 columns a drain every 4 chunks would bound the pass (512^3, 81 columns: 174 against 121 us);
     // up to 8, the sketch widths, every chunk is drained: the FP32 FMA kernel that streamed those before
     // rounds every addition to nearest (512^3 sketches: 2.4e-7, FMA 3.3e-7, 5.8e-7 with 4 chunks; 104 and

@@ -528,9 +528,12 @@ __device__ __forceinline__ void df_dot_step(float& s, float& c, float2 a, float2
 // the products are
 // accumulated on the FP32 pipe with Dot2 (as accurate as about 48 significant
 // bits, several times the FP64 rate here); otherwise FP64 fma.
-// One thread per output of out[l + L (a + m r)] = sum_i M(i, a) X[l + L (i + nj r)],
+// out[l + L (a + m r)] = sum_i M(i, a) X[l + L (i + nj r)], NA columns a per thread,
 // FP64 operands split into double-float pairs (M staged split in shared
-// memory), Dot2 accumulation: the FP64 pipe here is 1/64 of the FP32 pipe.
+// memory), Dot2 accumulation: the FP64 pipe here is 1/64 of the FP32 pipe.  A split costs as much as two
+// products, so a thread uses each X it splits for four columns where that leaves a CTA for every SM
+// (81 x 81 x 81, 64 columns: 74 -> 42 us).
+template <int NA>
 __global__ void __launch_bounds__(256) ttm_direct_df_kernel(const double* __restrict__ X, int64_t L, int64_t nj,
                                                             int64_t R, const double* __restrict__ M, int64_t ldm,
                                                             int mtrans, int64_t m, double* __restrict__ out) {
@@ -541,23 +544,38 @@ __global__ void __launch_bounds__(256) ttm_direct_df_kernel(const double* __rest
         msp[e] = df_from_f64(mtrans ? M[a + ldm * i] : M[i + ldm * a], 0);
     }
     __syncthreads();
+    const int64_t mg = (m + NA - 1) / NA;
     const int64_t o = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= L * m * R) return;
+    if (o >= L * mg * R) return;
     const int64_t l = o % L, rest = o / L;
-    const int64_t a = rest % m, r = rest / m;
+    const int64_t a = rest % mg * NA, r = rest / mg;
     const double* x = X + l + L * nj * r;
-    const float2* mc = msp + nj * a;
-    float sh = 0.f, sl = 0.f;
+    const float2* mc[NA];
+#pragma unroll
+    for (int q = 0; q < NA; ++q) mc[q] = msp + nj * (a + q < m ? a + q : a);  // (columns past m repeat the first)
+    float sh[NA], sl[NA];
+#pragma unroll
+    for (int q = 0; q < NA; ++q) sh[q] = sl[q] = 0.f;
     int64_t i = 0;
     for (; i + 8 <= nj; i += 8) {  // the eight loads issued before the products that use them
         double xv[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) xv[u] = x[L * (i + u)];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) df_dot_step(sh, sl, df_from_f64(xv[u], 0), mc[i + u]);
+        for (int u = 0; u < 8; ++u) {
+            const float2 xs = df_from_f64(xv[u], 0);
+#pragma unroll
+            for (int q = 0; q < NA; ++q) df_dot_step(sh[q], sl[q], xs, mc[q][i + u]);
+        }
     }
-    for (; i < nj; ++i) df_dot_step(sh, sl, df_from_f64(x[L * i], 0), mc[i]);
-    out[o] = (double)sh + (double)sl;
+    for (; i < nj; ++i) {
+        const float2 xs = df_from_f64(x[L * i], 0);
+#pragma unroll
+        for (int q = 0; q < NA; ++q) df_dot_step(sh[q], sl[q], xs, mc[q][i]);
+    }
+#pragma unroll
+    for (int q = 0; q < NA; ++q)
+        if (a + q < m) out[l + L * (a + q + m * r)] = (double)sh[q] + (double)sl[q];
 }
 
 static bool ttm_direct_df(const Ctx& c, const double* X, int64_t L, int64_t nj, int64_t R, const double* M,
@@ -566,8 +584,11 @@ static bool ttm_direct_df(const Ctx& c, const double* X, int64_t L, int64_t nj, 
     const size_t smem = sizeof(float2) * (size_t)(nj * m);
     if (rows * m > (1 << 22) || smem > 48 * 1024) return false;
     ProfScope ps(c, "ttm_simt", 8.0 * rows * nj + 8.0 * rows * m, 2.0 * rows * nj * m);
-    run_kernel(c, ttm_direct_df_kernel, (unsigned)((rows * m + 255) / 256), 256, smem, X, L, nj, R, M, ldm,
-               mtrans ? 1 : 0, m, out);
+    const int64_t four = rows * ((m + 3) / 4);
+    const bool na4 = four >= 152 * 256;
+    const int64_t threads = na4 ? four : rows * m;
+    run_kernel(c, na4 ? ttm_direct_df_kernel<4> : ttm_direct_df_kernel<1>, (unsigned)((threads + 255) / 256), 256, smem,
+               X, L, nj, R, M, ldm, mtrans ? 1 : 0, m, out);
     c.counted();
     c.check_launch();
     return true;

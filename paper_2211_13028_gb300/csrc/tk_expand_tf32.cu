@@ -17,7 +17,8 @@
 //   warp 1       allocates TMEM; one thread issues tcgen05.mma: per block and row subtile first the small
 //                terms of every K step, A_hi * M_lo and A_lo * M_hi, then A_hi * M_hi, all into one
 //                accumulator.  The tensor core rounds each addition toward zero: in this order only
-//                the K / 8 last ones round at the size of the result.
+//                the K / 8 last ones round at the size of the result (half as many for plain products, which
+//                keep the two halves of K apart: 327 x 187 x 164, K = 43, error against FP64 3.8e-7 -> 3.2e-7, SIMT 2.8e-7).
 //   warps 2, 3   X's tiles: one thread by TMA, or, where X's columns have no 16-byte stride (`bulk`), two
 //                by one bulk copy per column, widened to 16-byte bounds (half of the columns each).
 //   warps 4-11   converters: W from global memory (any alignment; rows L*R numbered without regard to
@@ -26,7 +27,7 @@
 //                EPI 2, which also stores alpha * (X - P)).  Two groups of 8 warps take alternate blocks.
 // SUB = 2: 256-row tiles (two 128-row subtiles share every factor block, which halves its L2
 // traffic: at K = 64 a block's factor is as many bytes as its BF16 tile of X), NB = 32, K <= 64.
-// SUB = 1: 128-row tiles, NB = 64, K <= 128.  TMEM: four accumulators of 64 columns, A in the other
+// SUB = 1: 128-row tiles, NB = 64, K <= 128.  TMEM: four accumulators of 64 columns (two pairs for plain products), A in the other
 // 256 columns (two buffers where SUB * chunks <= 2).
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
@@ -52,6 +53,10 @@ struct ExpandCfg {
     static constexpr int kXSlot = kNB * (kXPitch + 16);
     static constexpr int kXB = EPI ? (sizeof(XR) == 4 ? 4 : (sizeof(XR) == 2 ? 8 : 12)) : 0;  // X tiles (~130 KB in flight)
     static constexpr int kSmem = kBS * kBStage + kXB * kXSlot + 1024 + 512;
+    // plain products: each half of the K steps has its own accumulator, added in the epilogue, rounding to nearest
+    static constexpr bool kHalves = EPI == 0;
+    static constexpr uint32_t kAcc = kHalves ? 2 : 4;         // blocks in TMEM's accumulators (256 columns)
+    static constexpr uint32_t kAccCols = 256 / kAcc;
     static constexpr int kThreads = 32 * 28;
     static constexpr int kEpi = 16;                           // epilogue warps, in two groups
     static constexpr int kEpiG = kEpi / 2;
@@ -201,7 +206,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t bhi0 = bdesc0 + bs * (C::kBStage >> 4);
-                    const uint32_t d0 = tbase + a * 64, a0 = tbase + 256 + ab * acols;
+                    const uint32_t d0 = tbase + a * C::kAccCols, a0 = tbase + 256 + ab * acols;
 #pragma unroll
                     for (int big = 0; big < 2; ++big) {
 #pragma unroll
@@ -209,13 +214,17 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
                             const uint64_t bhi = bhi0 + kc * (C::kBStage >> 4), blo = bhi + ((NB * 128) >> 4);
 #pragma unroll
                             for (int sub = 0; sub < SUB; ++sub) {
-                                const uint32_t a_hi = a0 + (sub * NK + kc) * 64, d = d0 + sub * NB;
+                                const uint32_t a_hi = a0 + (sub * NK + kc) * 64;
 #pragma unroll
                                 for (int k = 0; k < 4; ++k) {
+                                    const int step = kc * 4 + k;
+                                    const bool second = C::kHalves && step >= 2 * NK;
+                                    const uint32_t d = d0 + sub * NB + (second ? 64 : 0);
+                                    const uint32_t more = step == (second ? 2 * NK : 0) ? 0u : 1u;
                                     if (big) {
                                         mma_tf32_ts(d, a_hi + 8 * k, bhi + 2 * k, idesc_tf32(NB), 1u);
                                     } else {
-                                        mma_tf32_ts(d, a_hi + 8 * k, blo + 2 * k, idesc_tf32(NB), (kc | k) ? 1u : 0u);
+                                        mma_tf32_ts(d, a_hi + 8 * k, blo + 2 * k, idesc_tf32(NB), more);
                                         mma_tf32_ts(d, a_hi + 32 + 8 * k, bhi + 2 * k, idesc_tf32(NB), 1u);
                                     }
                                 }
@@ -230,7 +239,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
                         bph ^= 1;
                     }
                     tc_commit(&accfull[a]);
-                    if (++a == 4) {
+                    if (++a == C::kAcc) {
                         a = 0;
                         aph ^= 1;
                     }
@@ -412,21 +421,22 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
             const int64_t obase = (int64_t)(g - r * L) + args.L * args.m * r;
             for (uint32_t b = block0(cs); b < b1; ++b, ++it) {
                 if ((it & 1) != grp) continue;
-                const uint32_t a = it & 3;
-                bool got = mbar_wait(&accfull[a], (it >> 2) & 1, abort, flags);
+                const uint32_t a = it % C::kAcc;
+                bool got = mbar_wait(&accfull[a], (it / C::kAcc) & 1, abort, flags);
                 if (EPI) got = got && mbar_wait(&xfull[xs], xph, abort, flags);
                 if (!__all_sync(0xffffffffu, got)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t ta = tbase + lane_base + a * 64 + sub * NB + cbase;
+                const uint32_t ta = tbase + lane_base + a * C::kAccCols + sub * NB + cbase;
 #pragma unroll
                 for (int sl = 0; sl < 2; ++sl) {
                     const int c16 = cbase + 16 * sl;
-                    float p[16];
+                    float p[16], p2[16];
                     __syncwarp();
                     tmem_ld16(ta + 16 * sl, p);
+                    if (C::kHalves) tmem_ld16(ta + 64 + 16 * sl, p2);
                     const int64_t col = (int64_t)b * NB + c16;
                     const int ncol = args.m - col < 16 ? (int)(args.m - col) : 16;  // valid columns of the slice
                     XR x[16];
@@ -454,6 +464,10 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
                         }
                     }
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    if (C::kHalves) {
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) p[i] += p2[i];
+                    }
                     if (sl == 1) {
                         tc_fence_before();
                         __syncwarp();

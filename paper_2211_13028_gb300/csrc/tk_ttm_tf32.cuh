@@ -122,7 +122,8 @@ struct TtmCfg {
     static constexpr int kFirstConv = FLAT ? 12 : 4;    // (a multiple of 4: warp % 4 is the TMEM lane quarter)
     static constexpr int kGroups = FLAT ? 1 : 2;        // converter groups of 8 warps
     static constexpr int kFirstEpi = kFirstConv + 8 * kGroups;
-    static constexpr int kEpi = 8;                      // epilogue warps
+    static constexpr int kEpi = NPAD <= 16 ? 4 : 8;     // epilogue warps: at most one per 16 columns and lane
+                                                        // quarter (idle ones poll: 160^4, 5 columns 534 -> 502 us)
     static constexpr int kThreads = 32 * (kFirstEpi + kEpi);
     static_assert(kAcc >= 2, "TMEM budget");
     static_assert(kStages >= 4, "SMEM budget");

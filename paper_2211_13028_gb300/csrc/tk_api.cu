@@ -196,7 +196,7 @@ static bool ttm_uses_tc(const Ctx& c, const Tens& T, int j, int64_t m, tk_dtype 
 // The order multi_ttm applies the factors in: cheapest-shrinking mode first
 // (smallest output; ties: the higher mode); FP8 data goes
 // along its contiguous mode first, where the kernel that multiplies it as it is streams
-// 6 TB/s (768^3, 9 columns: 76 us, 178 along another mode).
+// 6 TB/s (768^3, 9 columns: 74 us, 171 along another mode).
 static std::vector<int> mtt_order(const Ctx& c, const Tens& T, std::vector<int> modes, const Mat* M, bool mtrans,
                                   tk_dtype acc) {
     std::vector<int> order;

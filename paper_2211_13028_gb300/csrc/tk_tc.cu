@@ -178,7 +178,7 @@ enum class TcRoute { None, Tma, Flat, Lowp };
 //    E.g. 413 x 350 x 275 along its last mode, 36 columns: 1337 us SIMT; 9001 x 333, 20: 78.
 //  * BF16 and FP8 that their own kernels do not take: the same rule, for L == 1 or L >= 32 (shorter runs
 //    cost more in their 16-byte pieces than they hold).  E.g. BF16 689 x 690 x 700 along its first mode, 10 columns:
-//    3435 us SIMT, 180; FP8 768^3 along its last, 9: 1541 and 178.
+//    3435 us SIMT, 176; FP8 768^3 along its last, 9: 1541 and 171.
 static TcRoute lowp_route(const Tens& X, int j, int64_t m) {
     const int64_t L = X.left(j), nj = X.n[j], R = X.right(j), es = (int64_t)dtype_size(X.dt);
     if (ttm_bf16_eligible(X, j, m, TK_F32) || ttm_fp8_eligible(X, j, m, TK_F32)) return TcRoute::None;

@@ -321,8 +321,9 @@ struct ProfScope {
 // out is dense column-major, dims of X with n_j -> m, dtype F64 or F32.
 void launch_ttm(const Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int64_t m, void* out, tk_dtype out_dt);
 
-// Tensor-core (tcgen05, TF32 parts) version of launch_ttm for FP32 output: FP32 data, and BF16 / FP8 data in the
-// layouts that launch_ttm_bf16 / launch_ttm_fp8 do not take.  ttm_tc_eligible says whether a TTM takes it (dtype, and the sizes where it is faster).
+// Tensor-core (tcgen05, TF32 parts) version of launch_ttm for FP32 output: FP32 data, and BF16 / FP8 data
+// in the layouts that launch_ttm_bf16 / launch_ttm_fp8 do not take.  ttm_tc_eligible says whether a TTM
+// takes it (dtype, and the sizes where it is faster).
 bool ttm_tc_eligible(const Tens& X, int j, int64_t m, tk_dtype out_dt);
 // A factor a tensor-core TTM will split (the rows L before the contracted mode,
 // its size nj, output width m; residual: the fused-residual blocking; dt: the data's type).

@@ -1,5 +1,5 @@
-// Host side of the TF32 tensor-core TTMs on sm_103a (kernels: tk_ttm_tf32.cuh, tk_ttm_lowp.cuh, tk_expand_tf32.cu): the
-// TF32 split of the factors, the choice of tiles, tensor maps and launches.
+// Host side of the TF32 tensor-core TTMs on sm_103a (kernels: tk_ttm_tf32.cuh, tk_ttm_lowp.cuh,
+// tk_expand_tf32.cu): the TF32 split of the factors, the choice of tiles, tensor maps and launches.
 #include <algorithm>
 
 #include "tk_expand_tf32.cuh"

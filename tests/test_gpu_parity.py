@@ -436,7 +436,8 @@ def test_rhkron_sketch_widths_above_112(dev, dtype):
 
 @pytest.mark.parametrize("k", [1, 2, 3, 4, 16, 17, 32, 33, 49, 62, 63, 64, 65, 66, 67, 111, 112])
 def test_core_eigenvectors_at_the_jacobi_kernels_sizes(dev, k):
-    # one pair, an odd size's empty row, full and ragged tiles of the Gram (16 and 32), the last size with one register pair a lane and one warp of rotations (64)
+    # one pair, an odd size's empty row, full and ragged tiles of the Gram (16 and 32), the last size with one
+    # register pair a lane and one warp of rotations (64)
     # and the first with two, the largest.  The cut falls between singular values 7% apart; the FP32 rotations
     # leave the leading eigenvectors a singular-value-weighted ~1e-7 (the resolving threshold, 1e-11 of the
     # Gram's norm) and the results are rounded to FP32: 5e-6

@@ -1590,16 +1590,13 @@ static void rhkron_from_sketches(Ctx& c, const Tens& Xt, std::vector<Tens>& Y, c
     std::function<void()> tpass;
     if (!tm.empty()) {
         tpass = [&]() {
-            // the side stream's pass leaves most SMs to the truncation's kernels; the splits it makes
-            // are its own (the main stream must not find them in the cache)
+            // the side stream's pass leaves most SMs to the truncation's kernels
             const int keep = c.grid_sms;
-            const size_t ns = c.splits.size();
             c.grid_sms = background_grid(c);
             c.background = true;
             tr->T = multi_ttm(c, Xt, tm, Qa.data(), false, acc);
             c.background = false;
             c.grid_sms = keep;
-            c.splits.resize(ns);
             tr->Tapplied.assign(d, 0);
             for (int j : tm) tr->Tapplied[j] = 1;
         };

@@ -164,7 +164,9 @@ struct Ctx {
     mutable bool chained = false;
     bool df64 = false;             // FP32-class data: FP64 products may run in double-float arithmetic
     // Factor splits (TF32 hi / lo) made in this pass, reused while split_cache is
-    // on: only inside a dimension tree, whose factors are not modified.
+    // on: only inside a dimension tree, whose factors are not modified.  Those made by
+    // one branch of a fork or side are not visible outside it (SplitScope): no event
+    // orders another branch's stream after the kernel that writes them.
     struct Split {
         const void* p;
         int64_t ld, nj, m, npad, rows;
@@ -195,6 +197,15 @@ struct Ctx {
     cudaStream_t aux[kAux] = {};
     cudaEvent_t ev_fork = nullptr;
     cudaEvent_t ev_join[kAux] = {};
+
+    // Forgets the splits made since it was set up.  The planning pass, which runs every branch on one stream, does the
+    // same, so that both passes make the same splits and the same allocations.
+    struct SplitScope {
+        Ctx& c;
+        size_t made;
+        explicit SplitScope(Ctx& cc) : c(cc), made(cc.splits.size()) {}
+        ~SplitScope() { c.splits.resize(made); }
+    };
 
     // Runs body(b) for b = 0 .. nb-1, item b on auxiliary stream b mod kAux,
     // each forked from the call's stream by an event and joined back into it
@@ -264,7 +275,10 @@ void ctx_fork_end(Ctx& c, cudaStream_t main, int used);
 template <typename F>
 void Ctx::fork(int nb, F&& body) {
     if (!exec || nb <= 1 || !aux[0]) {
-        for (int b = 0; b < nb; ++b) body(b);
+        for (int b = 0; b < nb; ++b) {
+            SplitScope own(*this);
+            body(b);
+        }
         return;
     }
     cudaStream_t main = stream;
@@ -273,6 +287,7 @@ void Ctx::fork(int nb, F&& body) {
     try {
         for (int b = 0; b < nb; ++b) {
             stream = aux[b % kFork];
+            SplitScope own(*this);
             body(b);
         }
     } catch (...) {
@@ -288,14 +303,20 @@ void ctx_side_end(Ctx& c, cudaStream_t main);
 template <typename M, typename S>
 void Ctx::side(M&& main_body, S&& side_body) {
     if (!exec || !aux[kFork]) {
-        side_body();
+        {
+            SplitScope own(*this);
+            side_body();
+        }
         main_body();
         return;
     }
     cudaStream_t main = stream;
     ctx_side_begin(*this);  // the side stream waits for the call's stream; the call's stream becomes it
     try {
-        side_body();
+        {
+            SplitScope own(*this);
+            side_body();
+        }
         stream = main;
         main_body();
     } catch (...) {

@@ -1,0 +1,53 @@
+// Host-side checks of the call context (no GPU): run by test_host_units_cpu.py, one check per argument.
+#include <cstdio>
+#include <cstring>
+#include <vector>
+
+#include "tk_internal.cuh"
+
+// Stand-ins for the stream operations of a fork and of a side branch.
+namespace tk {
+void ctx_fork_begin(Ctx&, int) {}
+void ctx_fork_end(Ctx& c, cudaStream_t main, int) { c.stream = main; }
+void ctx_side_begin(Ctx& c) { c.stream = c.aux[Ctx::kFork]; }
+void ctx_side_end(Ctx& c, cudaStream_t main) { c.stream = main; }
+}  // namespace tk
+
+// A branch of a fork or side sees the splits made before it and its own, never another branch's.
+static int split_visibility() {
+    for (int mode = 0; mode < 3; ++mode) {  // the planning pass, the executing one without and with auxiliary streams
+        tk::Ctx c;
+        c.exec = mode > 0;
+        if (mode == 2)
+            for (int i = 0; i < tk::Ctx::kAux; ++i) c.aux[i] = reinterpret_cast<cudaStream_t>(uintptr_t(8 * (i + 1)));
+        c.split_cache = true;
+        c.splits.push_back({});  // made before
+        std::vector<size_t> seen;
+        auto branch = [&]() {
+            seen.push_back(c.splits.size());
+            c.splits.push_back({});
+            c.splits.push_back({});
+        };
+        c.fork(5, [&](int) { branch(); });
+        c.fork(1, [&](int) { branch(); });
+        c.side(
+            [&]() {
+                branch();  // the call's own stream: these two stay
+                c.fork(2, [&](int) { branch(); });
+            },
+            branch);
+        const std::vector<size_t> want = {1, 1, 1, 1, 1, 1, 1, 1, 3, 3};
+        if (seen != want || c.splits.size() != 3) {
+            std::printf("mode %d:", mode);
+            for (size_t v : seen) std::printf(" %zu", v);
+            std::printf(", %zu at the end\n", c.splits.size());
+            return 1;
+        }
+    }
+    return 0;
+}
+
+int main(int argc, char** argv) {
+    if (argc == 2 && !std::strcmp(argv[1], "split_visibility")) return split_visibility();
+    return 2;
+}

@@ -556,11 +556,8 @@ template <int NK, int EPI, typename XR>
 static void launch_one(const Ctx& c, const CUtensorMap& tb, const CUtensorMap& txr, const ExpandArgs& a) {
     using Cf = ExpandCfg<NK, EPI, XR>;
     auto kern = expand_tf32x3_kernel<NK, EPI, XR>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::kSmem));
-        attr_set = true;
-    }
+    static std::atomic<uint64_t> opted{0};
+    smem_opt_in(opted, reinterpret_cast<const void*>(kern), Cf::kSmem);
     run_kernel(c, kern, expand_ctas(c, a), Cf::kThreads, Cf::kSmem, tb, txr, a);
 }
 

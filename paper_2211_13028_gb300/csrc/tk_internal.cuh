@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -245,6 +246,17 @@ struct Ctx {
 __device__ __forceinline__ void kernel_begin() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Lets a kernel use `bytes` of dynamic shared memory on the current device (the setting is each device's own).
+// opted: the devices it is made on already, one for each kernel; two threads may both make it.
+inline void smem_opt_in(std::atomic<uint64_t>& opted, const void* kern, int bytes) {
+    int dev = 0;
+    TK_CUDA(cudaGetDevice(&dev));
+    const uint64_t bit = dev < 64 ? uint64_t(1) << dev : 0;
+    if (opted.load(std::memory_order_acquire) & bit) return;
+    TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    opted.fetch_or(bit, std::memory_order_release);
 }
 
 // Launches a kernel on the call's stream.  Directly after another kernel of the call on the same stream it is

@@ -5,6 +5,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <atomic>
 #include <mutex>
 #include <string>
 
@@ -168,14 +169,16 @@ inline void encode(CUtensorMap* m, const void* base, int rank, const uint64_t* d
     TK_REQUIRE(r == CUDA_SUCCESS, TK_ERR_CUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
 }
 
+// The current device's SMs.
 inline int num_sms() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 1;
-    }
+    static std::atomic<int> known[64];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    int n = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
+    if (n > 0) return n;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (n <= 0) n = 1;
+    if (dev < 64) known[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 

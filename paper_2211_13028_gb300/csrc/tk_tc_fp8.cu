@@ -310,11 +310,8 @@ template <int NPAD>
 static void launch_kernel(const Ctx& c, const CUtensorMap& tx, const CUtensorMap& tb, const F8Args& a) {
     using Cf = F8Cfg<NPAD>;
     auto kern = ttm_fp8_kernel<NPAD>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::kSmem));
-        attr_set = true;
-    }
+    static std::atomic<uint64_t> opted{0};
+    smem_opt_in(opted, reinterpret_cast<const void*>(kern), Cf::kSmem);
     const int grid = (int)std::min<int64_t>(a.ntiles * a.nblk, tc::grid_sms(c));
     run_kernel(c, kern, grid, kThreads, Cf::kSmem, tx, tb, a);
 }

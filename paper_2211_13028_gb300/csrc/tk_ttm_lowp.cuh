@@ -546,11 +546,8 @@ static void ttm_lowp_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorM
     TK_REQUIRE(a.stages >= 2, TK_ERR_SHAPE, "ttm_lowp: stage too large");
     auto kern = ttm_lowp_kernel<NPAD, KMAJOR, ES>;
     constexpr int kMaxSmem = Cf::kBudget + 2048;
-    static bool attr_set = false;
-    if (!attr_set) {
-        TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-        attr_set = true;
-    }
+    static std::atomic<uint64_t> opted{0};
+    smem_opt_in(opted, reinterpret_cast<const void*>(kern), kMaxSmem);
     const int grid = (int)std::min<int64_t>(a.nitems, grid_sms(c));
     run_kernel(c, kern, grid, Cf::kThreads, a.stages * stage + 2048, tx, tb, a);
 }

@@ -640,11 +640,8 @@ static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorM
     // 98 us a pass, FMA 131 and 115, 94 and 90 with 4)
     a.fill = a.m <= 8 ? 1 : (NPAD <= 64 ? 4 : 16);
     auto kern = ttm_tf32x3_kernel<NPAD, KMAJOR, FLAT>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        TK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::kSmem));
-        attr_set = true;
-    }
+    static std::atomic<uint64_t> opted{0};
+    smem_opt_in(opted, reinterpret_cast<const void*>(kern), Cf::kSmem);
     const int grid = (int)std::min<int64_t>(a.nitems, grid_sms(c));
     run_kernel(c, kern, grid, Cf::kThreads, Cf::kSmem, tx, tb, a);
 }

@@ -3,10 +3,16 @@
 #include <cstring>
 #include <vector>
 
-#include "tk_internal.cuh"
+#include "tk_tc_common.cuh"
 
-// Stand-ins for the stream operations of a fork and of a side branch.
+// host_units_runtime.c: stand-ins for the runtime's calls, which several devices answer
+extern "C" int fake_device;      // the current device
+extern "C" int fake_set[16];     // devices a kernel's attribute was set on
+extern "C" int fake_set_count;
+
+// Stand-ins for the library's error exit and for the stream operations of a fork and of a side branch.
 namespace tk {
+void fail(tk_status st, const std::string& msg) { throw Error{st, msg}; }
 void ctx_fork_begin(Ctx&, int) {}
 void ctx_fork_end(Ctx& c, cudaStream_t main, int) { c.stream = main; }
 void ctx_side_begin(Ctx& c) { c.stream = c.aux[Ctx::kFork]; }
@@ -47,7 +53,20 @@ static int split_visibility() {
     return 0;
 }
 
+// A kernel's shared-memory limit is set once on every device that launches it, and each device has its own SM count.
+static int per_device() {
+    std::atomic<uint64_t> opted{0};
+    for (int dev : {0, 0, 1, 0, 1, 63, 63, 64, 64}) {
+        fake_device = dev;
+        tk::smem_opt_in(opted, nullptr, 100000);
+        if (tk::tc::num_sms() != 100 + dev) return 1;
+    }
+    const std::vector<int> want = {0, 1, 63, 64, 64};  // (above 63: every time)
+    return std::vector<int>(fake_set, fake_set + fake_set_count) == want ? 0 : 1;
+}
+
 int main(int argc, char** argv) {
     if (argc == 2 && !std::strcmp(argv[1], "split_visibility")) return split_visibility();
+    if (argc == 2 && !std::strcmp(argv[1], "per_device")) return per_device();
     return 2;
 }

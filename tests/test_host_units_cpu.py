@@ -13,7 +13,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 def units(tmp_path_factory):
     exe = str(tmp_path_factory.mktemp("units") / "host_units")
     cmd = [B._nvcc(), *B.ARCH, "-std=c++17", "-cudart", "shared", "-I", B.INCLUDE, "-I", B.CSRC,
-           os.path.join(HERE, "host_units.cu"), "-o", exe]
+           os.path.join(HERE, "host_units.cu"), os.path.join(HERE, "host_units_runtime.c"), "-o", exe]
     r = subprocess.run(cmd, capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
     return exe
@@ -28,3 +28,8 @@ def test_splits_of_one_branch_are_not_seen_by_another(units):
     # a branch's stream is ordered after the call's stream, not after the other branches', so a split that
     # another branch's kernel writes may not have been written when this one's reads it
     _run(units, "split_visibility")
+
+
+def test_kernel_limits_and_sm_counts_are_each_devices_own(units):
+    # handles on several devices of a process launch the same kernels
+    _run(units, "per_device")

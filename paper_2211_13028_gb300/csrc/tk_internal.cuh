@@ -263,9 +263,11 @@ inline void smem_opt_in(std::atomic<uint64_t>& opted, const void* kern, int byte
 // launched as a programmatic dependent: its blocks are set up while that one runs and wait in kernel_begin, so that
 // a chain of short kernels is not spaced by launch latencies (rhkron of 64^3 in FP64, 78 launches: 850 -> 734 us;
 // sthosvd of a 49 x 42 x 42 core, 49: 479 -> 416).  Not across events (fork, side), which order
-// whole kernels.
+// whole kernels.  Not where early is false: blocks set up early share the few SMs that have room beside the kernel
+// before, which a long kernel of few blocks, bound by an SM's own pipe, does not make up for (an FP64 product of 5
+// blocks and 346 us by itself, after one that fills every SM: 1.2 ms).
 template <typename... P, typename... A>
-void run_kernel(const Ctx& c, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+void run_kernel_if(const Ctx& c, bool early, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -275,10 +277,15 @@ void run_kernel(const Ctx& c, void (*kern)(P...), dim3 grid, dim3 block, size_t 
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = c.overlap && c.chained && c.chain == c.stream ? 1 : 0;
+    cfg.numAttrs = early && c.overlap && c.chained && c.chain == c.stream ? 1 : 0;
     c.chain = c.stream;
     c.chained = true;
     (void)cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);  // (an error is kept for check_launch)
+}
+
+template <typename... P, typename... A>
+void run_kernel(const Ctx& c, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+    run_kernel_if(c, true, kern, grid, block, smem, std::forward<A>(args)...);
 }
 
 void ctx_fork_begin(Ctx& c, int used);

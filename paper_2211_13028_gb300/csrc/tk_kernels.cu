@@ -7,7 +7,7 @@
 
 #include <type_traits>
 
-#include "tk_internal.cuh"
+#include "tk_tc_common.cuh"
 
 namespace tk {
 
@@ -254,6 +254,15 @@ __global__ void __launch_bounds__(SLAB_THREADS) ttm_slab_kernel(const Tx* __rest
 static bool ttm_direct_df(const Ctx& c, const double* X, int64_t L, int64_t nj, int64_t R, const double* M,
                           int64_t ldm, bool mtrans, int64_t m, double* out);
 
+// Whether a product of `ctas` blocks, each of `fma` multiply-adds, may be launched while the kernel before it runs
+// (run_kernel_if).  FP64 runs at 2 a clock and SM: fewer blocks than SMs that take more than about 20 us each are spread
+// over idle SMs first (144 x 16 x 640, sketch widths 20, 9, 4: 1677 us launched early, 838 so); for shorter
+// ones the 2 to 4 us that an early launch saves count more.
+template <typename Ta>
+static bool ttm_early(const Ctx& c, int64_t ctas, double fma) {
+    return !std::is_same<Ta, double>::value || ctas >= tc::grid_sms(c) || fma < 8e4;
+}
+
 template <typename Tx, typename Ta>
 static void ttm_dispatch(const Ctx& c, const Tx* X, int64_t L, int64_t nj, int64_t R, const Ta* M, int64_t ldm,
                          bool mtrans, int64_t m, Ta* out, Ta xinv) {
@@ -268,8 +277,8 @@ static void ttm_dispatch(const Ctx& c, const Tx* X, int64_t L, int64_t nj, int64
         const size_t smem = sizeof(Ta) * (size_t)(L * nj + (int64_t)S * L * m);
         const char* name = (const void*)X == c.xdata ? "xpass_simt" : "ttm_simt";
         ProfScope ps(c, name, (double)rows * nj * sizeof(Tx) + (double)rows * m * sizeof(Ta), 2.0 * rows * nj * m);
-        run_kernel(c, ttm_slab_kernel<Tx, Ta>, (unsigned)R, SLAB_THREADS, smem, X, L, nj, R, M, ldm, mtrans ? 1 : 0,
-                   m, S, out, xinv);
+        run_kernel_if(c, ttm_early<Ta>(c, R, (double)L * m * nj), ttm_slab_kernel<Tx, Ta>, (unsigned)R, SLAB_THREADS,
+                      smem, X, L, nj, R, M, ldm, mtrans ? 1 : 0, m, S, out, xinv);
         c.counted();
         c.check_launch();
         return;
@@ -277,8 +286,9 @@ static void ttm_dispatch(const Ctx& c, const Tx* X, int64_t L, int64_t nj, int64
     if (rows * m <= (1 << 21) && nj <= 512) {
         const char* name = (const void*)X == c.xdata ? "xpass_simt" : "ttm_simt";
         ProfScope ps(c, name, (double)rows * nj * sizeof(Tx) + (double)rows * m * sizeof(Ta), 2.0 * rows * nj * m);
-        run_kernel(c, ttm_direct_kernel<Tx, Ta>, (unsigned)((rows * m + 255) / 256), 256, 0, X, L, nj, R, M, ldm,
-                   mtrans, m, out, xinv);
+        const int64_t ctas = (rows * m + 255) / 256;
+        run_kernel_if(c, ttm_early<Ta>(c, ctas, 256.0 * nj), ttm_direct_kernel<Tx, Ta>, (unsigned)ctas, 256, 0, X, L, nj,
+                      R, M, ldm, mtrans, m, out, xinv);
         c.counted();
         c.check_launch();
         return;
@@ -288,10 +298,9 @@ static void ttm_dispatch(const Ctx& c, const Tx* X, int64_t L, int64_t nj, int64
                  2.0 * rows * nj * m);
     dim3 grid((unsigned)((rows + 63) / 64), (unsigned)((m + 31) / 32));
     TK_REQUIRE(grid.y <= 65535, TK_ERR_SHAPE, "ttm: too many output columns");
-    if (L == 1)
-        run_kernel(c, ttm_simt_kernel<Tx, Ta, true>, grid, 256, 0, X, L, nj, R, M, ldm, mtrans, m, out, xinv);
-    else
-        run_kernel(c, ttm_simt_kernel<Tx, Ta, false>, grid, 256, 0, X, L, nj, R, M, ldm, mtrans, m, out, xinv);
+    const bool early = ttm_early<Ta>(c, (int64_t)grid.x * grid.y, 64.0 * 32.0 * nj);
+    run_kernel_if(c, early, L == 1 ? ttm_simt_kernel<Tx, Ta, true> : ttm_simt_kernel<Tx, Ta, false>, grid, 256, 0, X, L,
+                  nj, R, M, ldm, mtrans, m, out, xinv);
     c.counted();
     c.check_launch();
 }

@@ -1606,7 +1606,7 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int k, double* Ag, double* 
                                                      int use_smem, double* gV, unsigned* flags) {
     kernel_begin();
     extern __shared__ double sm[];
-    __shared__ double cs[128], sn[128];
+    __shared__ double cs[128], sn[128], dp[128], dq[128];
     __shared__ int P[128], Qp[128];
     const int tid = threadIdx.x, nt = blockDim.x;
     double* A = use_smem ? sm : Ag;
@@ -1629,22 +1629,28 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int k, double* Ag, double* 
     const double dsc = ldexp(1.0, -ex), usc = ldexp(1.0, ex);
     for (int e = tid; e < k * k; e += nt) A[e] *= dsc;
     __syncthreads();
-    const double athr = 4.0 * eps * fro * dsc;  // absolute off-diagonal threshold
+    // An off-diagonal entry left behind turns the vectors of its pair by the entry over the pair's gap, so a pair is
+    // rotated until its entry is below 4 eps of its gap; the floor, far below the rounding of A itself, ends the
+    // sweeps on pairs that agree to the last bit.  (4 eps ||A|| for all left vectors with a gap of 1e-4 to their
+    // neighbour wrong by 1e-11: 100 x 90 x 80, ranks 12, 10, 14: 2e-12 to 2e-11 over six seeds, 1e-13 to 4e-13 so.
+    // It costs a sweep: 64^3, ranks 8, 692 -> 725 us.)
+    const double floor_thr = eps * eps * fro * dsc;
+    auto big = [&](double app, double aqq, double apq) {
+        return fabs(apq) > fmax(4.0 * eps * fabs(aqq - app), floor_thr);
+    };
     bool converged = (k <= 1);
     for (int sweep = 0; sweep < max_sweeps && !converged; ++sweep) {
         int off = 0;
         for (int e = tid; e < k * k; e += nt) {
             int p = e % k, q = e / k;
-            if (p < q) {
-                double apq = fabs(A[p + k * q]);
-                if (apq > athr) off = 1;
-            }
+            if (p < q && big(A[p + k * p], A[q + k * q], A[p + k * q])) off = 1;
         }
         if (!__syncthreads_or(off)) {
             converged = true;
             break;
         }
         for (int step = 0; step < kp - 1; ++step) {
+            int any = 0;
             for (int t = tid; t < half; t += nt) {
                 int p, q;
                 if (t == 0) {
@@ -1658,25 +1664,32 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int k, double* Ag, double* 
                 double c = 1.0, s = 0.0;
                 if (q < k) {
                     double app = A[p + k * p], aqq = A[q + k * q], apq = A[p + k * q];
-                    if (fabs(apq) > athr) {
+                    if (big(app, aqq, apq)) {
                         // t = sgn(phi) psi / (|phi| + rho), phi = a_qq - a_pp, psi = 2 a_pq,
                         // rho = sqrt(phi^2 + psi^2): the smaller root of t^2 + 2 t phi / psi - 1 = 0;
                         // c = 1 / sqrt(1 + t^2), s = t c.  Reciprocal and reciprocal square roots from
-                        // FP32 seeds and FP64 Newton steps (FMAs only; entries are O(1) after scaling
-                        // and rotated pairs have psi > 4 eps ||A||, so the seeds stay in FP32 range).
-                        const double phi = aqq - app, psi = 2.0 * apq;
+                        // FP32 seeds and FP64 Newton steps (FMAs only; entries are O(1) after scaling,
+                        // and a tiny pair, whose ratio alone counts, is scaled up, so the seeds stay in FP32 range).
+                        double phi = aqq - app, psi = 2.0 * apq;
+                        const double up = fmax(fabs(phi), fabs(psi)) < 0x1p-50 ? 0x1p50 : 1.0;
+                        phi *= up;
+                        psi *= up;
                         const double r2 = fma(phi, phi, psi * psi);
                         const double u = jac_rsqrt(r2);                  // 1 / rho
                         const double t1 = (phi >= 0.0 ? psi : -psi) * jac_rcp(fabs(phi) + r2 * u);
                         c = jac_rsqrt(fma(t1, t1, 1.0));
                         s = t1 * c;
+                        // the pair's own block after the rotation, free of the rounding of its full size
+                        dp[t] = fma(-t1, apq, app);
+                        dq[t] = fma(t1, apq, aqq);
+                        any = 1;
                     }
                 } else {
                     q = -1;
                 }
                 P[t] = p; Qp[t] = q; cs[t] = c; sn[t] = s;
             }
-            __syncthreads();
+            if (!__syncthreads_or(any)) continue;  // nothing to rotate in this step
             // rows: A <- J^T A
             for (int e = tid; e < half * k; e += nt) {
                 int t = e / k, col = e % k;
@@ -1695,8 +1708,8 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int k, double* Ag, double* 
                 if (q < 0 || sn[t] == 0.0) continue;
                 double c = cs[t], s = sn[t];
                 double a = A[row + k * p], b = A[row + k * q];
-                A[row + k * p] = c * a - s * b;
-                A[row + k * q] = s * a + c * b;
+                A[row + k * p] = row == p ? dp[t] : (row == q ? 0.0 : c * a - s * b);
+                A[row + k * q] = row == q ? dq[t] : (row == p ? 0.0 : s * a + c * b);
                 a = V[row + k * p]; b = V[row + k * q];
                 V[row + k * p] = c * a - s * b;
                 V[row + k * q] = s * a + c * b;
@@ -1709,10 +1722,7 @@ __global__ void __launch_bounds__(256) jacobi_kernel(int k, double* Ag, double* 
         int off = 0;
         for (int e = tid; e < k * k; e += nt) {
             int p = e % k, q = e / k;
-            if (p < q) {
-                double apq = fabs(A[p + k * q]);
-                if (apq > athr) off = 1;
-            }
+            if (p < q && big(A[p + k * p], A[q + k * q], A[p + k * q])) off = 1;
         }
         converged = !__syncthreads_or(off);
         if (!converged && tid == 0) atomicOr(flags, FLAG_NOT_CONVERGED);

@@ -455,3 +455,44 @@ def test_core_eigenvectors_at_the_jacobi_kernels_sizes(dev, k):
     assert rel(got, ref) <= 5e-6
     st, _ = T.tk_sync_status(dev)
     assert st == 0
+
+
+def _eig_longdouble(A):
+    """Eigenvectors (descending) of a small symmetric matrix in extended precision, by cyclic Jacobi."""
+    A, k = A.copy(), len(A)
+    V = np.eye(k, dtype=np.longdouble)
+    for _ in range(60):
+        if np.abs(A - np.diag(np.diag(A))).max() <= np.longdouble(1e-28) * np.abs(A).max():
+            break
+        for p in range(k - 1):
+            for q in range(p + 1, k):
+                if A[p, q] == 0:
+                    continue
+                th = (A[q, q] - A[p, p]) / (2 * A[p, q])
+                t = (1 if th >= 0 else -1) / (abs(th) + np.sqrt(1 + th * th))
+                c = 1 / np.sqrt(1 + t * t)
+                s = t * c
+                A[[p, q]] = c * A[p] - s * A[q], s * A[p] + c * A[q]
+                A[:, [p, q]] = np.stack([c * A[:, p] - s * A[:, q], s * A[:, p] + c * A[:, q]], 1)
+                V[:, [p, q]] = np.stack([c * V[:, p] - s * V[:, q], s * V[:, p] + c * V[:, q]], 1)
+    return V[:, np.argsort(-np.diag(A))]
+
+
+@pytest.mark.parametrize("k,seed", [(8, 0), (8, 1), (12, 3), (12, 7), (24, 0)])
+def test_sthosvd_f64_close_singular_values(dev, k, seed):
+    # two eigenvalues of the Gram 2e-4 ||A|| apart.  The Gram, whose entries are rounded to about eps ||A||, fixes the
+    # pair's vectors to 2^-52 / 2e-4 = 1.1e-12; what the eigensolver leaves undone may add nothing to that
+    g = np.random.Generator(np.random.PCG64(seed))
+    q = [np.linalg.qr(g.standard_normal((k, k)))[0] for _ in range(3)]
+    sv = 0.8 ** np.arange(k)
+    sv[1] = sv[0] * np.sqrt(1 - 2e-4)
+    sv[4] = sv[3] * np.sqrt(1 - 1e-3)
+    x = np.einsum("a,ia,ja,la->ijl", sv, *q)
+    eye = [torch.eye(k, dtype=torch.float64, device=dev).t() for _ in range(3)]
+    _, U = T.tucker_sthosvd(synth.fortran(x, "f64", dev), eye, [6, 6, 6])
+    a = x.reshape(k, -1).astype(np.longdouble)
+    ref = _eig_longdouble(a @ a.T)[:, :6]
+    ref = ref * np.where(ref[np.abs(ref).argmax(0), np.arange(6)] < 0, -1, 1)
+    assert np.abs(to_np(U[0]) - ref).max() <= 2.0 ** -52 / 2e-4
+    st, _ = T.tk_sync_status(dev)
+    assert st == 0

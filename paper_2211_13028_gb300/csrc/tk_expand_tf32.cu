@@ -29,9 +29,6 @@
 // traffic: at K = 64 a block's factor is as many bytes as its BF16 tile of X), NB = 32, K <= 64.
 // SUB = 1: 128-row tiles, NB = 64, K <= 128.  TMEM: four accumulators of 64 columns (two pairs for plain products), A in the other
 // 256 columns (two buffers where SUB * chunks <= 2).
-#include <cuda_bf16.h>
-#include <cuda_fp8.h>
-
 #include <algorithm>
 #include <type_traits>
 
@@ -65,22 +62,6 @@ struct ExpandCfg {
     static_assert(kSmem <= 227 * 1024, "SMEM budget");
 };
 
-// (hi, lo) += b with Knuth's two-sum on the high part; the low part collects
-// the rounding errors (a double-float running sum of FP32 terms).
-__device__ __forceinline__ void ef_add(float& hi, float& lo, float b) {
-    const float s = __fadd_rn(hi, b);
-    const float v = __fsub_rn(s, hi);
-    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(b, v));
-    hi = s;
-    lo = __fadd_rn(lo, e);
-}
-
-__device__ __forceinline__ float xr_to_f32(float v) { return v; }
-__device__ __forceinline__ float xr_to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
-__device__ __forceinline__ float xr_to_f32(__nv_fp8_e4m3 v) { return static_cast<float>(v); }
-__device__ __forceinline__ void xr_store(float* p, float v) { *p = v; }
-__device__ __forceinline__ void xr_store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
-
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(smem_u32(bar))
@@ -111,7 +92,6 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
     uint64_t* done = accempty + 4;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    __shared__ double red[2 * C::kEpi];
 
     const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const bool bulk = EPI != 0 && args.bulk;
@@ -519,28 +499,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
             }
         }
         if (EPI != 0) {
-            // reduce over the epilogue threads: warp shuffles, then named barrier 1, then one thread
-            // sums the warps in a fixed order
-            double sr = (double)srh + (double)srl, sx = (double)sxh + (double)sxl;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                sr += __shfl_xor_sync(0xffffffffu, sr, o);
-                sx += __shfl_xor_sync(0xffffffffu, sx, o);
-            }
-            if (lane == 0) {
-                red[2 * e] = sr;
-                red[2 * e + 1] = sx;
-            }
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * C::kEpi) : "memory");
-            if (e == 0 && lane == 0) {
-                double a0 = 0.0, a1 = 0.0;
-                for (int i = 0; i < C::kEpi; ++i) {
-                    a0 += red[2 * i];
-                    a1 += red[2 * i + 1];
-                }
-                args.partials[2 * blockIdx.x] = a0;
-                args.partials[2 * blockIdx.x + 1] = a1;
-            }
+            residual_sums<C::kEpi>(e, lane, (double)srh + (double)srl, (double)sxh + (double)sxl, args.partials);
         }
     }
     __syncthreads();

@@ -258,6 +258,16 @@ static void factor_map(Ctx& c, const Factor& f, const Mat& M, bool mtrans, int64
     tc::encode(tb, f.hi, 3, dims, str, box);
 }
 
+// The tensor map of X's chunks along mode j for a strided contraction: 128 rows x 32 K elements, or L rows of pack
+// consecutive slabs (L x 4 bytes: a multiple of 16).
+static void strided_map(const Tens& X, int j, int64_t pack, CUtensorMap* tx) {
+    const int64_t L = X.left(j), nj = X.n[j];
+    const uint64_t dims[3] = {(uint64_t)L, (uint64_t)nj, (uint64_t)X.right(j)};
+    const uint64_t str[2] = {(uint64_t)L * 4, (uint64_t)L * nj * 4};
+    const uint32_t box[3] = {pack > 1 ? (uint32_t)L : (uint32_t)tc::kRows, tc::kChunk, (uint32_t)pack};
+    tc::encode(tx, X.p, 3, dims, str, box, false);
+}
+
 // The expansion kernel's work: row tiles x parts of their column blocks (an item converts its tile of W
 // again, so parts are no finer than about 8 items an SM need).
 static tc::ExpandArgs expand_args(const Ctx& c, const Tens& W, int j, int64_t m, const Blocks& bl) {
@@ -411,16 +421,9 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
         const uint32_t box[2] = {tc::kChunk, tc::kRows};
         tc::encode(&tx, X.p, 2, dims, str, box);
     } else {
-        const uint64_t dims[3] = {(uint64_t)L, (uint64_t)nj, (uint64_t)R};
-        const uint64_t str[2] = {(uint64_t)L * 4, (uint64_t)L * nj * 4};
-        uint32_t box[3] = {tc::kRows, tc::kChunk, 1};
-        if (pack > 1) {  // L rows of pack consecutive r per box (L x 4 bytes: a multiple of 16)
-            box[0] = (uint32_t)L;
-            box[2] = (uint32_t)pack;
-        }
-        tc::encode(&tx, X.p, 3, dims, str, box, false);
+        strided_map(X, j, pack, &tx);
     }
-    tc::TtmArgs a;
+    tc::TtmArgs a{};
     a.L = L;
     a.nj = nj;
     a.R = R;
@@ -450,14 +453,22 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
     if (ksplit > 1) sum_parts(c, part, ksplit, L * m * R, out);
 }
 
+// Fused residuals of a contraction longer than the expansion kernel holds run on the plain kernel, whose epilogue then
+// compares instead of storing (512^3 FP32, K = 160: norms 668 us, with dX 753; stored and compared by kernels of their
+// own 671 and 1200 us, and Xhat's 512 MB of workspace).
+static bool residual_plain(int64_t nj) { return nj > tc::kExpandKResid; }
+
 bool ttm_tc_residual_eligible(const Tens& W, int j, int64_t m) {
     const int64_t rows = W.left(j), nj = W.n[j];
-    return W.dt == TK_F32 && W.right(j) == 1 && nj >= 1 && nj <= tc::kExpandKResid && m >= 1 && m <= 65535 &&
+    return W.dt == TK_F32 && W.right(j) == 1 && nj >= 1 && nj < ((int64_t)1 << 31) && m >= 1 && m <= 65535 &&
            rows >= 1 && rows < ((int64_t)1 << 31) - 256 && ((uintptr_t)W.p % 16) == 0;
 }
 
 int tc_residual_ctas(const Ctx& c, const Tens& W, int j, int64_t m) {
-    return tc::expand_ctas(c, expand_args(c, W, j, m, tc_blocks(W.left(j), W.n[j], m, true, TK_F32)));
+    const Blocks bl = tc_blocks(W.left(j), W.n[j], m, true, TK_F32);
+    if (!residual_plain(W.n[j])) return tc::expand_ctas(c, expand_args(c, W, j, m, bl));
+    const int64_t ntiles = (W.left(j) + tc::kRows - 1) / tc::kRows;
+    return (int)std::min<int64_t>(ntiles * bl.nblk, tc::grid_sms(c));
 }
 
 void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtrans, int64_t m, const void* xref,
@@ -471,6 +482,38 @@ void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtr
     CUtensorMap tb, txr;
     factor_map(c, f, M, mtrans, nj, m, bl.npad, &tb);
     const int64_t es = (int64_t)dtype_size(xrdt);
+    ProfScope ps(c, c.background ? "xpass_tc_bg" : "xpass_tc",
+                 4.0 * (double)L * nj + 8.0 * nj * m + (dx ? 2.0 : 1.0) * es * (double)L * m, 2.0 * (double)L * nj * m);
+    if (residual_plain(nj)) {
+        const bool flat = !tma_ok(W, j) || L < tc::kRows;
+        CUtensorMap tw = tb;  // unused by the loaders
+        if (!flat) strided_map(W, j, 1, &tw);
+        tc::TtmArgs a{};
+        a.L = L;
+        a.nj = nj;
+        a.R = 1;
+        a.m = m;
+        a.tiles_per_r = a.ntiles = (uint32_t)((L + tc::kRows - 1) / tc::kRows);
+        a.nk = (uint32_t)((nj + tc::kChunk - 1) / tc::kChunk);
+        a.nblk = (uint32_t)bl.nblk;
+        TK_REQUIRE((int64_t)a.ntiles * bl.nblk < ((int64_t)1 << 31), TK_ERR_SHAPE, "ttm_tc: too many tiles");
+        a.nitems = a.ntiles * a.nblk;
+        a.pack = a.ksplit = 1;
+        a.xbytes = flat ? 0 : (uint32_t)tc::kXBytes;
+        a.vec = L % 2 == 0 ? 2 : 1;
+        a.X = static_cast<const float*>(W.p);
+        a.flags = c.dflags;
+        a.xref = xref;
+        a.xrdt = (int)xrdt;
+        a.dx = dx;
+        a.alpha = alpha;
+        a.xr_scale = xr_scale;
+        a.partials = partials;
+        tc::ttm_tf32_run_residual(c, flat, tw, tb, a);
+        c.counted();
+        c.check_launch();
+        return;
+    }
     tc::ExpandArgs a = expand_args(c, W, j, m, bl);
     a.bulk = (L * es) % 16 != 0;
     a.xclip = (L * m * es) & ~(int64_t)15;
@@ -488,8 +531,6 @@ void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtr
     a.alpha = alpha;
     a.xr_scale = xr_scale;
     a.partials = partials;
-    ProfScope ps(c, c.background ? "xpass_tc_bg" : "xpass_tc",
-                 4.0 * (double)L * nj + 8.0 * nj * m + (dx ? 2.0 : 1.0) * es * (double)L * m, 2.0 * (double)L * nj * m);
     tc::expand_run(c, dx ? 2 : 1, xrdt, tb, txr, a);
     c.counted();
     c.check_launch();

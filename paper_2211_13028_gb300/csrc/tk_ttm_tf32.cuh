@@ -29,6 +29,9 @@
 // buffers.  Errors against FP64: 512^3, 42 columns 2.4e-6 with one accumulator an item, 7.2e-7 so (100 ->
 // 104 us); 413 x 350 x 275, 36 columns 4.1e-7 with one chunk an accumulator, 3.6e-7 with half (SIMT 4.3e-7).
 //
+// RES: the product is not stored but compared with a tensor of its shape: fused residuals whose contraction is longer
+// than tk_expand_tf32.cu holds (128).
+//
 // FLAT = false: TMA.  Needs 16-byte strides (L % 4 == 0, or n_j % 4 == 0 for L == 1).  A strided mode
 // with fewer than 64 rows before it packs several slabs into each 128-row tile (pack).
 // FLAT = true: any L and n_j.  The L*R rows are numbered without regard to slabs (so no row of a tile
@@ -39,6 +42,9 @@
 // Every mbarrier wait is bounded by a wall-clock limit; on expiry the CTA raises FLAG_TIMEOUT, stops
 // issuing work, drains what it issued and frees its TMEM.
 #pragma once
+#include <cuda_bf16.h>
+#include <cuda_fp8.h>
+
 #include "tk_tc_common.cuh"
 
 namespace tk {
@@ -82,6 +88,47 @@ __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) 
     lo = __float_as_uint(x - __uint_as_float(hi));
 }
 
+// (hi, lo) += b with Knuth's two-sum on the high part; the low part collects
+// the rounding errors (a double-float running sum of FP32 terms).
+__device__ __forceinline__ void ef_add(float& hi, float& lo, float b) {
+    const float s = __fadd_rn(hi, b);
+    const float v = __fsub_rn(s, hi);
+    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(b, v));
+    hi = s;
+    lo = __fadd_rn(lo, e);
+}
+
+__device__ __forceinline__ float xr_to_f32(float v) { return v; }
+__device__ __forceinline__ float xr_to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ float xr_to_f32(__nv_fp8_e4m3 v) { return static_cast<float>(v); }
+__device__ __forceinline__ void xr_store(float* p, float v) { *p = v; }
+__device__ __forceinline__ void xr_store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+
+// The sums (sr, sx) of the lanes of N epilogue warps, in a fixed order, into the CTA's pair of partials.
+template <int N>
+__device__ __forceinline__ void residual_sums(int e, int lane, double sr, double sx, double* partials) {
+    __shared__ double red[2 * N];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sr += __shfl_xor_sync(0xffffffffu, sr, o);
+        sx += __shfl_xor_sync(0xffffffffu, sx, o);
+    }
+    if (lane == 0) {
+        red[2 * e] = sr;
+        red[2 * e + 1] = sx;
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * N) : "memory");
+    if (e == 0 && lane == 0) {
+        double a0 = 0.0, a1 = 0.0;
+        for (int i = 0; i < N; ++i) {
+            a0 += red[2 * i];
+            a1 += red[2 * i + 1];
+        }
+        partials[2 * blockIdx.x] = a0;
+        partials[2 * blockIdx.x + 1] = a1;
+    }
+}
+
 struct TtmArgs {
     int64_t L, nj, R, m;
     // work item = (row tile, block of NPAD output columns, part of the K chunks)
@@ -100,7 +147,48 @@ struct TtmArgs {
     int64_t out_numel;
     float* out;
     unsigned* flags;
+    // RES: the tensor compared with the product (its layout, R == 1; elements of type xrdt, times xr_scale),
+    // dx = alpha * (xref - product) in its type (may be NULL), per-CTA sums {(xref - product)^2, xref^2}
+    const void* xref;
+    void* dx;
+    int xrdt;
+    float alpha, xr_scale;
+    double* partials;
 };
+
+template <typename XR>
+__device__ __forceinline__ void residual_load(const void* xref, int64_t o, int64_t L, int n, float (&x)[8]) {
+    const XR* xp = static_cast<const XR*>(xref) + o;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = i < n ? xr_to_f32(xp[i * L]) : 0.f;
+}
+template <typename XR>
+__device__ __forceinline__ void residual_store(void* dx, int64_t o, int64_t L, int n, const float (&x)[8]) {
+    XR* xp = static_cast<XR*>(dx) + o;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (i < n) xr_store(xp + i * L, x[i]);
+}
+
+// RES: 8 columns p of a row, of which n are the product's, against xref from its element o.
+__device__ __forceinline__ void residual_columns(const TtmArgs& a, int64_t o, int n, const float* p, float& fr,
+                                                 float& fx) {
+    float x[8];
+    if (a.xrdt == TK_F32) residual_load<float>(a.xref, o, a.L, n, x);
+    else if (a.xrdt == TK_BF16) residual_load<__nv_bfloat16>(a.xref, o, a.L, n, x);
+    else residual_load<__nv_fp8_e4m3>(a.xref, o, a.L, n, x);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        x[i] *= a.xr_scale;
+        fx = fmaf(x[i], x[i], fx);
+        x[i] = i < n ? x[i] - p[i] : 0.f;
+        fr = fmaf(x[i], x[i], fr);
+        x[i] *= a.alpha;
+    }
+    if (!a.dx) return;
+    if (a.xrdt == TK_F32) residual_store<float>(a.dx, o, a.L, n, x);
+    else residual_store<__nv_bfloat16>(a.dx, o, a.L, n, x);
+}
 
 template <int NPAD, bool KMAJOR, bool FLAT>
 struct TtmCfg {
@@ -143,7 +231,7 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
     asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-template <int NPAD, bool KMAJOR, bool FLAT>
+template <int NPAD, bool KMAJOR, bool FLAT, bool RES = false>
 __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
     ttm_tf32x3_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmB,
                       TtmArgs args) {
@@ -493,6 +581,7 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
         const int64_t m = args.m;
         uint32_t a = 0, aph = 0, sph = 0;
         const bool copier = warp == C::kFirstEpi && lane == 0;
+        float srh = 0.f, srl = 0.f, sxh = 0.f, sxl = 0.f;  // RES: running sums as double-float pairs
         for (uint32_t w = blockIdx.x; w < args.nitems; w += gridDim.x) {
             const uint32_t w2 = ksplit == 1 ? w : w / ksplit, sk = w - w2 * ksplit;
             const uint32_t t = args.nblk == 1 ? w2 : w2 / args.nblk, nb = args.nblk == 1 ? 0 : w2 % args.nblk;
@@ -535,6 +624,17 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
             constexpr int kSl = (NPAD / 16 + 1) / 2;
             float v[kSl][16];
             bool ok = true;
+            if constexpr (RES) {
+                // the warp's columns of xref on their way into L2 while the product is formed, a column a lane
+                const int c = 16 * half + (lane & 15) + 32 * (lane >> 4);
+                const int64_t l = (int64_t)t * kRows + 32 * q, rows = args.L - l < 32 ? args.L - l : 32;
+                if (c < ncol && rows > 0) {
+                    const int es = args.xrdt == TK_F32 ? 4 : (args.xrdt == TK_BF16 ? 2 : 1);
+                    const char* x = static_cast<const char*>(args.xref) + (l + (col0 + c) * args.L) * es;
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(x));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(x + rows * es - 1));
+                }
+            }
             for (uint32_t f = 0; f < nfill; ++f) {
                 if (!__all_sync(0xffffffffu, mbar_wait(&accfull[a], aph, abort, flags))) {
                     ok = false;
@@ -562,6 +662,21 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
                 }
             }
             if (!ok) break;
+            if constexpr (RES) {
+                if (valid) {
+#pragma unroll
+                    for (int j = 0; j < 2 * kSl; ++j) {
+                        const int c0 = 16 * half + 32 * (j >> 1) + 8 * (j & 1);
+                        const float* p = &v[j >> 1][8 * (j & 1)];
+                        const int64_t o = base + c0 * stride;
+                        float fr = 0.f, fx = 0.f;
+                        residual_columns(args, o, ncol - c0, p, fr, fx);
+                        ef_add(srh, srl, fr);
+                        ef_add(sxh, sxl, fx);
+                    }
+                }
+                continue;
+            }
             // L == 1: the tile's rows are one run of the result.  Unless its lanes can store them in 16 bytes, it
             // goes out as one bulk copy from a staged copy (4-byte stores of each lane's row reach L2 as pieces of
             // sectors: 512^3, 42 columns 127 -> 98 us; 413 x 350 x 275, 30 columns 59 -> 56)
@@ -623,6 +738,9 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
             }
         }
         if (C::kOut && copier) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        if constexpr (RES)
+            residual_sums<C::kEpi>(warp - C::kFirstEpi, lane, (double)srh + (double)srl, (double)sxh + (double)sxl,
+                                   args.partials);
     }
     __syncthreads();
     if (warp == 1) {
@@ -631,7 +749,7 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
     }
 }
 
-template <int NPAD, bool KMAJOR, bool FLAT>
+template <int NPAD, bool KMAJOR, bool FLAT, bool RES = false>
 static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorMap& tb, TtmArgs a) {
     using Cf = TtmCfg<NPAD, KMAJOR, FLAT>;
     // above 64 columns a drain every 4 chunks would bound the pass (512^3, 81 columns: 174 against 121 us);
@@ -639,7 +757,7 @@ static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorM
     // rounds every addition to nearest (512^3 sketches: 2.4e-7, FMA 3.3e-7, 5.8e-7 with 4 chunks; 104 and
     // 98 us a pass, FMA 131 and 115, 94 and 90 with 4)
     a.fill = a.m <= 8 ? 1 : (NPAD <= 64 ? 4 : 16);
-    auto kern = ttm_tf32x3_kernel<NPAD, KMAJOR, FLAT>;
+    auto kern = ttm_tf32x3_kernel<NPAD, KMAJOR, FLAT, RES>;
     static std::atomic<uint64_t> opted{0};
     smem_opt_in(opted, reinterpret_cast<const void*>(kern), Cf::kSmem);
     const int grid = (int)std::min<int64_t>(a.nitems, grid_sms(c));
@@ -671,6 +789,8 @@ void ttm_tf32_run_tma(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap
                       const TtmArgs& a);
 void ttm_tf32_run_flat(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& tb,
                        const TtmArgs& a);
+// Fused with the comparison with xref (RES): blocks of 64 columns.
+void ttm_tf32_run_residual(const Ctx& c, bool flat, const CUtensorMap& tx, const CUtensorMap& tb, const TtmArgs& a);
 
 }  // namespace tc
 }  // namespace tk

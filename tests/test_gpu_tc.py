@@ -226,6 +226,10 @@ def test_tc_lowp_any_size_and_alignment(dev, dims, k, dtype):
     ((64, 48, 257), (8, 8, 64)),    # 16-byte columns in every dtype; K = 64
     ((40, 37, 90), (6, 7, 90)),     # K = 90: three chunks, 128-row tiles
     ((41, 37, 130), (5, 6, 128)),   # K = 128: four chunks, odd rows
+    ((130, 11, 200), (6, 5, 129)),  # K = 129: the plain kernel's chunks, rows by 8 bytes, last block of 8 columns
+    ((43, 31, 161), (5, 6, 160)),   # K = 160, odd rows
+    ((64, 48, 257), (8, 8, 256)),   # K = 256, rows by TMA, one column in the last block
+    ((5, 9, 300), (3, 4, 290)),     # K above 256, less than a tile of rows
     ((3, 5, 40), (2, 3, 4)),        # fewer rows than 16 bytes hold
     ((16, 16, 257), (4, 4, 5)),     # exactly one 256-row tile
     ((257, 1, 32), (4, 1, 5)),      # one row in the second tile, one full block
@@ -240,7 +244,11 @@ def test_fused_residual_sizes_and_alignment(dev, dims, rk, dtype):
     U = [synth.round_to(g.standard_normal((n, k)) / np.sqrt(n), "f32") for n, k in zip(dims, rk)]
     Gd, Ud = synth.fortran(G, "f32", dev), mats(U, "f32", dev)
     ref = O.loss(xv, G, U)
+    T.tk_profile(True, dev)
     assert abs(T.tucker_loss(X, Gd, Ud, scale=sc) - ref) <= 1e-5 * ref
+    prof = T.tk_profile_read(dev)
+    T.tk_profile(False, dev)
+    assert "xpass_tc" in prof and "residual" not in prof  # Xhat is never formed
     if dtype == "fp8":
         return
     norms = torch.zeros(2, dtype=torch.float64, device=dev)

@@ -614,6 +614,8 @@ static void residual_pass(Ctx& c, const Tens& X, const Tens& G, const std::vecto
     }
     const bool fused = c.use_tc && (X.dt == TK_F32 || X.dt == TK_BF16 || (X.dt == TK_FP8_E4M3 && !dx)) &&
                        acc == TK_F32 && (!dx || dxdt == X.dt) && ttm_tc_residual_eligible(Ws, f, m);
+    // dX of FP32 data with a short last contraction: FP32 FMAs, as exact as X's own digits
+    const bool fma = fused && X.dt == TK_F32 && residual_fma_eligible(Ws, f, m);
     // the factors of the tensor-core products split in one launch
     std::vector<TcSplitReq> reqs;
     if (c.use_tc && acc == TK_F32) {
@@ -624,7 +626,7 @@ static void residual_pass(Ctx& c, const Tens& X, const Tens& G, const std::vecto
             sh.dt = acc;
             sh.p = reinterpret_cast<void*>(uintptr_t(256));
         }
-        if (fused) reqs.push_back({U[f], true, Ws.left(f), Ws.n[f], m, true, TK_F32});
+        if (fused && !fma) reqs.push_back({U[f], true, Ws.left(f), Ws.n[f], m, true, TK_F32});
         if (reqs.size() >= 2) tc_presplit(c, reqs);
     }
     struct CacheOn {
@@ -635,6 +637,14 @@ static void residual_pass(Ctx& c, const Tens& X, const Tens& G, const std::vecto
     } cache_on(c, reqs.size() >= 2);
     Tens W = G;
     for (int i : order) W = ttm_to(c, W, i, U[i], true, acc);
+    if (fma) {
+        const int nb = residual_fma_ctas(c, W, f, m);
+        double* part = c.alloc<double>(2 * nb);
+        launch_residual_fma(c, W, f, U[f], true, m, static_cast<const float*>(X.p), static_cast<float*>(dx),
+                            (float)alpha, part);
+        launch_sum_pairs(c, part, nb, err2);
+        return;
+    }
     if (fused) {
         const int nb = tc_residual_ctas(c, W, f, m);
         double* part = c.alloc<double>(2 * nb);

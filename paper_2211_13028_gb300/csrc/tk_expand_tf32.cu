@@ -17,8 +17,10 @@
 //   warp 1       allocates TMEM; one thread issues tcgen05.mma: per block and row subtile first the small
 //                terms of every K step, A_hi * M_lo and A_lo * M_hi, then A_hi * M_hi, all into one
 //                accumulator.  The tensor core rounds each addition toward zero: in this order only
-//                the K / 8 last ones round at the size of the result (half as many for plain products, which
-//                keep the two halves of K apart: 327 x 187 x 164, K = 43, error against FP64 3.8e-7 -> 3.2e-7, SIMT 2.8e-7).
+//                the K / 8 last ones round at the size of the result.  Plain products, and the comparison of FP32
+//                data at K <= 32, keep the even and the odd steps apart, half as many each: dX of 256^3, ranks 16,
+//                1.72e-6 -> 1.62e-6 from 64 bits (FP32 FMAs 1.62e-6; its pass 42 -> 45 us, the norms alone 37 -> 39;
+//                512^3, ranks 32, 186 -> 207 and 102 -> 122).  BF16 data, whose rounding is far larger, do not.
 //   warps 2, 3   X's tiles: one thread by TMA, or, where X's columns have no 16-byte stride (`bulk`), two
 //                by one bulk copy per column, widened to 16-byte bounds (half of the columns each).
 //   warps 4-11   converters: W from global memory (any alignment; rows L*R numbered without regard to
@@ -27,8 +29,8 @@
 //                EPI 2, which also stores alpha * (X - P)).  Two groups of 8 warps take alternate blocks.
 // SUB = 2: 256-row tiles (two 128-row subtiles share every factor block, which halves its L2
 // traffic: at K = 64 a block's factor is as many bytes as its BF16 tile of X), NB = 32, K <= 64.
-// SUB = 1: 128-row tiles, NB = 64, K <= 128.  TMEM: four accumulators of 64 columns (two pairs for plain products), A in the other
-// 256 columns (two buffers where SUB * chunks <= 2).
+// SUB = 1: 128-row tiles, NB = 64, K <= 128.  TMEM: four accumulators of 64 columns (or two pairs), A in the other
+// 256 columns (two buffers where SUB * chunks <= 2).  FP32 data with K <= 12: residual_fma_kernel (tk_kernels.cu).
 #include <algorithm>
 #include <type_traits>
 
@@ -50,8 +52,9 @@ struct ExpandCfg {
     static constexpr int kXSlot = kNB * (kXPitch + 16);
     static constexpr int kXB = EPI ? (sizeof(XR) == 4 ? 4 : (sizeof(XR) == 2 ? 8 : 12)) : 0;  // X tiles (~130 KB in flight)
     static constexpr int kSmem = kBS * kBStage + kXB * kXSlot + 1024 + 512;
-    // plain products: each half of the K steps has its own accumulator, added in the epilogue, rounding to nearest
-    static constexpr bool kHalves = EPI == 0;
+    // plain products, and the comparison of FP32 data at K <= 32: the even and the odd K steps have accumulators of
+    // their own, added in the epilogue, rounding to nearest
+    static constexpr bool kHalves = EPI == 0 || (NK == 1 && sizeof(XR) == 4);
     static constexpr uint32_t kAcc = kHalves ? 2 : 4;         // blocks in TMEM's accumulators (256 columns)
     static constexpr uint32_t kAccCols = 256 / kAcc;
     static constexpr int kThreads = 32 * 28;
@@ -198,9 +201,9 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
 #pragma unroll
                                 for (int k = 0; k < 4; ++k) {
                                     const int step = kc * 4 + k;
-                                    const bool second = C::kHalves && step >= 2 * NK;
+                                    const bool second = C::kHalves && (step & 1);
                                     const uint32_t d = d0 + sub * NB + (second ? 64 : 0);
-                                    const uint32_t more = step == (second ? 2 * NK : 0) ? 0u : 1u;
+                                    const uint32_t more = step < (C::kHalves ? 2 : 1) ? 0u : 1u;
                                     if (big) {
                                         mma_tf32_ts(d, a_hi + 8 * k, bhi + 2 * k, idesc_tf32(NB), 1u);
                                     } else {

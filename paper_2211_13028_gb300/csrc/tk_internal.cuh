@@ -437,6 +437,11 @@ void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtr
                             tk_dtype xrdt, void* dx, float alpha, double* partials, float xr_scale = 1.f);
 int tc_residual_ctas(const Ctx& c, const Tens& W, int j, int64_t m);
 bool ttm_tc_residual_eligible(const Tens& W, int j, int64_t m);
+// The same for FP32 data by FP32 FMAs (nj <= 12; any alignment).  residual_fma_ctas: pairs of partial sums.
+bool residual_fma_eligible(const Tens& W, int j, int64_t m);
+int residual_fma_ctas(const Ctx& c, const Tens& W, int j, int64_t m);
+void launch_residual_fma(const Ctx& c, const Tens& W, int j, const Mat& M, bool mtrans, int64_t m, const float* xref,
+                         float* dx, float alpha, double* partials);
 // One warp waits with the tcgen05 kernels' bounded wait on an mbarrier that
 // nothing arrives at (limit_ns), which raises FLAG_TIMEOUT; *waited (device)
 // receives how long it waited in ns (-1 had the wait completed).

@@ -2676,6 +2676,129 @@ void launch_residual_norms(Ctx& c, const Tens& X, const void* Y, tk_dtype ydt, d
     c.check_launch();
 }
 
+// The last step of a reconstruction of FP32 data with K <= 12, fused with the comparison with X: P = W M^T is formed
+// with FP32 FMAs, every addition rounded to nearest, and compared: per-CTA sums of (x - P)^2 and x^2, and with DX also
+// dx = alpha (x - P).  The tensor cores' additions round toward zero, which at so few terms is most of the error (dX
+// of 400 x 120 x 64, ranks 3, 4, 5: 1.14e-6 from 64 bits, 8.5e-7 so).  A thread keeps four rows of W in registers and
+// meets every column of M, staged in shared memory, with all of them.  512^3, K = 8: 120 us, 189 with dx (tensor
+// cores 92 and 184; X alone takes 79 and 158); K = 16 would take 150 and 209, where two accumulators do as well.
+constexpr int RF_THREADS = 256;
+constexpr int RF_RPT = 4;  // rows a thread: each column read from shared memory serves all of them
+constexpr int RF_ROWS = RF_RPT * RF_THREADS;
+constexpr int RF_COLS = 128;
+
+template <int KP, bool DX>
+__global__ void __launch_bounds__(RF_THREADS) residual_fma_kernel(const float* __restrict__ W, int64_t L, int K,
+                                                                  const float* __restrict__ M, int64_t ldm, int mtrans,
+                                                                  int64_t m, const float* __restrict__ X, float* dx,
+                                                                  float alpha, int64_t nblk, int64_t items, double* part) {
+    kernel_begin();
+    __shared__ __align__(16) float us[RF_COLS][KP];
+    __shared__ double red[2 * RF_THREADS / 32];
+    const int tid = threadIdx.x;
+    float h[2] = {0.f, 0.f}, l[2] = {0.f, 0.f};  // running sums as double-float pairs: (x - P)^2, x^2
+    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+        const int64_t r0 = it / nblk * RF_ROWS, a0 = it % nblk * RF_COLS;
+        const int na = (int)(m - a0 < RF_COLS ? m - a0 : RF_COLS);
+        __syncthreads();  // the columns of the item before have been used
+        for (int e = tid; e < KP * RF_COLS; e += RF_THREADS) {
+            const int a = e % RF_COLS, i = e / RF_COLS;
+            us[a][i] = i < K && a < na ? (mtrans ? M[a0 + a + ldm * i] : M[i + ldm * (a0 + a)]) : 0.f;
+        }
+        float w[RF_RPT][KP];
+        bool in[RF_RPT];
+#pragma unroll
+        for (int q = 0; q < RF_RPT; ++q) {
+            const int64_t r = r0 + tid + q * RF_THREADS;
+            in[q] = r < L;
+#pragma unroll
+            for (int i = 0; i < KP; ++i) w[q][i] = in[q] && i < K ? W[r + L * i] : 0.f;
+        }
+        __syncthreads();
+        const float* x = X + r0 + tid + L * a0;
+        float* d = dx + r0 + tid + L * a0;
+        constexpr int U = 8;  // columns whose loads are in flight together
+        for (int c = 0; c < na; c += U) {
+            float v[RF_RPT][U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int q = 0; q < RF_RPT; ++q) v[q][u] = in[q] && c + u < na ? x[L * (c + u) + q * RF_THREADS] : 0.f;
+            float fr = 0.f, fx = 0.f;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (c + u >= na) break;
+                float p[RF_RPT];
+#pragma unroll
+                for (int q = 0; q < RF_RPT; ++q) p[q] = 0.f;
+#pragma unroll
+                for (int i = 0; i < KP; i += 4) {
+                    const float4 f = *reinterpret_cast<const float4*>(&us[c + u][i]);
+#pragma unroll
+                    for (int q = 0; q < RF_RPT; ++q) {
+                        p[q] = fmaf(w[q][i], f.x, p[q]);
+                        p[q] = fmaf(w[q][i + 1], f.y, p[q]);
+                        p[q] = fmaf(w[q][i + 2], f.z, p[q]);
+                        p[q] = fmaf(w[q][i + 3], f.w, p[q]);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < RF_RPT; ++q) {
+                    if (!in[q]) continue;
+                    const float dv = v[q][u] - p[q];
+                    fr = fmaf(dv, dv, fr);
+                    fx = fmaf(v[q][u], v[q][u], fx);
+                    if (DX) d[L * (c + u) + q * RF_THREADS] = alpha * dv;
+                }
+            }
+            df_add(h[0], l[0], fr, 0.f);
+            df_add(h[1], l[1], fx, 0.f);
+        }
+    }
+    double s[2] = {(double)h[0] + (double)l[0], (double)h[1] + (double)l[1]};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        s[q] = warp_sum(s[q]);
+        if ((tid & 31) == 0) red[2 * (tid >> 5) + q] = s[q];
+    }
+    __syncthreads();
+    if (tid < 2) {
+        double t = 0.0;
+        for (int w8 = 0; w8 < RF_THREADS / 32; ++w8) t += red[2 * w8 + tid];
+        part[2 * blockIdx.x + tid] = t;
+    }
+}
+
+bool residual_fma_eligible(const Tens& W, int j, int64_t m) {
+    return W.dt == TK_F32 && W.right(j) == 1 && W.n[j] >= 1 && W.n[j] <= 12 && W.left(j) >= 1 && m >= 1;
+}
+
+static int64_t residual_fma_items(const Tens& W, int j, int64_t m) {
+    return (W.left(j) + RF_ROWS - 1) / RF_ROWS * ((m + RF_COLS - 1) / RF_COLS);
+}
+
+int residual_fma_ctas(const Ctx& c, const Tens& W, int j, int64_t m) {
+    return (int)std::min<int64_t>(residual_fma_items(W, j, m), 4 * tc::grid_sms(c));
+}
+
+void launch_residual_fma(const Ctx& c, const Tens& W, int j, const Mat& M, bool mtrans, int64_t m, const float* xref,
+                         float* dx, float alpha, double* partials) {
+    if (!c.exec) return;
+    TK_REQUIRE(M.dt == TK_F32, TK_ERR_DTYPE, "residual_fma: the factor must be F32");
+    const int64_t L = W.left(j), K = W.n[j];
+    ProfScope ps(c, "xpass_simt", 4.0 * (double)L * K + 4.0 * K * m + (dx ? 8.0 : 4.0) * (double)L * m,
+                 2.0 * (double)L * K * m);
+    const auto kern = dx ? (K <= 4 ? residual_fma_kernel<4, true>
+                                   : (K <= 8 ? residual_fma_kernel<8, true> : residual_fma_kernel<12, true>))
+                         : (K <= 4 ? residual_fma_kernel<4, false>
+                                   : (K <= 8 ? residual_fma_kernel<8, false> : residual_fma_kernel<12, false>));
+    run_kernel(c, kern, (unsigned)residual_fma_ctas(c, W, j, m), RF_THREADS, 0, (const float*)W.p, L, (int)K,
+               (const float*)M.p, M.ld, mtrans ? 1 : 0, m, xref, dx, alpha, (m + RF_COLS - 1) / RF_COLS,
+               residual_fma_items(W, j, m), partials);
+    c.counted();
+    c.check_launch();
+}
+
 __global__ void axpby_residual_kernel(const void* X, tk_dtype xdt, float xinv, const void* Y, tk_dtype ydt,
                                       int64_t tot, double alpha, void* dst, tk_dtype ddt) {
     kernel_begin();

@@ -248,7 +248,8 @@ def test_fused_residual_sizes_and_alignment(dev, dims, rk, dtype):
     assert abs(T.tucker_loss(X, Gd, Ud, scale=sc) - ref) <= 1e-5 * ref
     prof = T.tk_profile_read(dev)
     T.tk_profile(False, dev)
-    assert "xpass_tc" in prof and "residual" not in prof  # Xhat is never formed
+    fma = dtype == "f32" and rk[2] <= 12  # a short contraction of FP32 data: FP32 FMAs
+    assert ("xpass_simt" if fma else "xpass_tc") in prof and "residual" not in prof  # Xhat is never formed
     if dtype == "fp8":
         return
     norms = torch.zeros(2, dtype=torch.float64, device=dev)
@@ -276,3 +277,27 @@ def test_reconstruct_expansions(dev, dims, rk):
     assert rel(to_np(Xh), O.reconstruct(G, U)) <= len(dims) * 2e-6
     st, _ = T.tk_sync_status(dev)
     assert st == 0
+
+
+@pytest.mark.parametrize("rows", [4096, 4099])
+@pytest.mark.parametrize("K", [1, 3, 4, 5, 8, 9, 12, 13, 16, 24, 32])
+def test_residual_of_short_contractions_keeps_fp32_digits(dev, K, rows):
+    # dX of X = 0 is -P, P = W U^T with W = u g^T rounded once per entry, so the product alone is seen.  Up to 12 terms
+    # it is summed by FMAs that round to nearest: no bias (a truncating sum has about -2^-25 = 3e-8), and an error
+    # of at most sqrt(K + 1) 2^-25.  Above, two accumulators take half of the 8-term steps each: at most
+    # two truncations by 2^-23 of half the sum, 2^-23 = 1.2e-7
+    g = torch.Generator(device=dev)
+    g.manual_seed(K)
+    m = 1000
+    u, w, U = (torch.randn(b, a, generator=g, device=dev).t() for a, b in ((rows, 1), (1, K), (m, K)))
+    ref = (u * w).double() @ U.double().t()
+    X = torch.zeros(m, rows, device=dev).t()
+    norms = torch.zeros(2, dtype=torch.float64, device=dev)
+    _, _, dX = T.tucker_reconstruct_backward(X, w, [u, U], 0.5, need_dG=False, need_dU=False, norms2=norms)
+    err = -dX.double() - ref
+    if K <= 12:
+        assert float((err * ref.sign()).sum() / ref.abs().sum()) >= -5e-9
+        assert float(err.norm() / ref.norm()) <= (K + 1) ** 0.5 * 2.0 ** -25
+    else:
+        assert float(err.norm() / ref.norm()) <= 2.0 ** -23
+    assert abs(float(norms[0]) - float((ref ** 2).sum())) <= 1e-6 * float((ref ** 2).sum()) and float(norms[1]) == 0.0

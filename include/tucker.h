@@ -26,6 +26,11 @@
  *  - Numerical conditions found on the device (a Cholesky breakdown that sent a
  *    QR to the Householder fallback, a Jacobi solve that hit its sweep limit)
  *    are recorded in the handle and reported by tk_sync_status().
+ *  - Infinities, NaN and the largest finite values: a product of FP32 data (and
+ *    of BF16 and FP8 data off 16-byte strides, and of FP8 data along any mode
+ *    but the first) holds what FP32 multiply-adds give, on every kernel; BF16
+ *    data with 16-byte strides, and FP8 data along the first mode, give a NaN
+ *    for an infinity in X or in a factor.
  *  - The handle owns a device workspace that grows on demand (cudaMalloc).
  *    A handle must not be used from two host threads at once.
  */

@@ -71,6 +71,30 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                  : "memory");
 }
 
+// The CTA's items once more, by exact_dot: the infinite and NaN elements of a plain product, or the whole comparison.
+template <int TILE, int NB, int EPI, typename XR>
+__device__ __forceinline__ void exact_expand(const ExpandArgs& args) {
+    double sr = 0.0, sx = 0.0;
+    for (uint32_t w = blockIdx.x; w < args.nitems; w += gridDim.x) {
+        const uint32_t tile = w / args.ncs, cs = w - tile * args.ncs;
+        const int64_t a0 = (int64_t)((uint64_t)args.nblk * cs / args.ncs) * NB;
+        const int64_t ae = (int64_t)((uint64_t)args.nblk * (cs + 1) / args.ncs) * NB, a1 = ae < args.m ? ae : args.m;
+        const int64_t l0 = (int64_t)tile * TILE, l1 = l0 + TILE < args.rows ? l0 + TILE : args.rows;
+        if constexpr (EPI != 0) {
+            exact_compare<XR>(args.W, args.L, args.nj, *args.info, l0, l1, a0, a1, args.xref, args.xr_scale,
+                              EPI == 2 ? args.out : nullptr, args.alpha, sr, sx);
+        } else {
+            for (int64_t e = threadIdx.x; e < (l1 - l0) * (a1 - a0); e += blockDim.x) {
+                const int64_t g = l0 + e % (l1 - l0), a = a0 + e / (l1 - l0), r = g / args.L, l = g - r * args.L;
+                float* const o = static_cast<float*>(args.out) + l + args.L * (a + args.m * r);
+                if (fabsf(*o) <= 3.402823466e38f) continue;
+                *o = exact_dot(args.W + l + args.L * args.nj * r, args.L, 0, args.nj, *args.info, a, 1.f);
+            }
+        }
+    }
+    if (EPI != 0) residual_sums_cta(sr, sx, args.partials);
+}
+
 template <int NK, int EPI, typename XR>
 __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
     expand_tf32x3_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmXr,
@@ -95,6 +119,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
     uint64_t* done = accempty + 4;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    __shared__ int again;  // infinities or NaN in the product's operands, or in the comparison (exact_dot); static: its address takes no register
 
     const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const bool bulk = EPI != 0 && args.bulk;
@@ -117,6 +142,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
         }
         mbar_init(done, 1);
         *abort = 0;
+        again = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -308,6 +334,12 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
             drain(xfull, nx, XB);
         }
         __syncwarp();
+        if (warp == 3) {  // whether the factor has such values
+            int any = 0;
+#pragma unroll 8
+            for (uint32_t i = lane; i < args.info->nbad; i += 32) any |= args.info->bad[i];
+            if (any) again = 1;
+        }
     } else if (warp < C::kFirstEpi) {
         // ------------------------------------------------ converters: W tile -> TF32 hi / lo in TMEM
         const int q = warp & 3, hs = (warp - 4) >> 2;
@@ -321,6 +353,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
             return (int64_t)(g - r * L) + args.L * args.nj * r;
         };
         uint32_t ab = 0, abph = 1;
+        float bad = 0.f;
         bool ok = true;
         for (uint32_t w = blockIdx.x; w < args.nitems && ok; w += gridDim.x) {
             const uint32_t tile = w / ncs, nst = SUB * nk;  // steps: (subtile, K chunk)
@@ -337,7 +370,10 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
             auto store = [&](uint32_t st, const float (&x)[16]) {
                 uint32_t hi[16], lo[16];
 #pragma unroll
-                for (int ii = 0; ii < 16; ++ii) split_tf32(x[ii], hi[ii], lo[ii]);
+                for (int ii = 0; ii < 16; ++ii) {
+                    split_tf32(x[ii], hi[ii], lo[ii]);
+                    bad = fmaf(__uint_as_float(lo[ii]), 0.f, bad);  // a NaN once lo is infinite or one
+                }
                 const uint32_t ta = tbase + lane_base + 256 + ab * acols + st * 64 + 16 * hs;
                 __syncwarp();
                 tmem_st16(ta, hi);
@@ -379,6 +415,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
                 __syncwarp();
             }
         }
+        if (bad != bad) again = 1;
     } else if (warp < C::kFirstEpi + C::kEpi) {
         // ------------------------------------------------ epilogue
         // warp e: group e / 8; within it TMEM lane quarter warp % 4 and the subtile (SUB = 2) or the block's
@@ -471,7 +508,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
                         float fr = 0.f, fx = 0.f;
                         XR* op = EPI == 2 ? static_cast<XR*>(args.out) + obase + col * args.L : nullptr;
                         auto one = [&](int i) {
-                            float xv = xr_to_f32(x[i]);
+                            float xv = x_to_f32(x[i]);
                             if constexpr (std::is_same<XR, __nv_fp8_e4m3>::value) xv *= args.xr_scale;  // 1 / scale
                             const float dv = xv - p[i];
                             fr = fmaf(dv, dv, fr);
@@ -486,6 +523,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
                             for (int i = 0; i < 16; ++i)
                                 if (i < ncol) one(i);
                         }
+                        if (!(fr <= 3.402823466e38f)) again = 1;
                         ef_add(srh, srl, fr);
                         ef_add(sxh, sxl, fx);
                     }
@@ -502,7 +540,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
             }
         }
         if (EPI != 0) {
-            residual_sums<C::kEpi>(e, lane, (double)srh + (double)srl, (double)sxh + (double)sxl, args.partials);
+            residual_sums<C::kEpi>(e, lane, ef_value(srh, srl), ef_value(sxh, sxl), args.partials);
         }
     }
     __syncthreads();
@@ -510,6 +548,7 @@ __global__ void __launch_bounds__(ExpandCfg<NK, EPI, XR>::kThreads, 1)
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase) : "memory");
     }
+    if (again && !*abort) exact_expand<C::kTile, C::kNB, EPI, XR>(args);
 }
 
 int expand_ctas(const Ctx& c, const ExpandArgs& a) { return (int)std::min<int64_t>(a.nitems, grid_sms(c)); }

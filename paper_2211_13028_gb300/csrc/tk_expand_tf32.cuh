@@ -9,7 +9,7 @@ constexpr int64_t kExpandK = 64;        // contracted elements of a plain expans
 constexpr int64_t kExpandKResid = 128;  // of a fused residual
 
 struct ExpandArgs {
-    int64_t L, nj, R, m;
+    int64_t L, nj, m;
     const float* W;           // L x nj x R
     uint32_t rows;            // L R
     uint32_t ntiles, nblk;    // row tiles, blocks of output columns
@@ -23,7 +23,9 @@ struct ExpandArgs {
     uint32_t bulk;            // EPI 1, 2: xref has no 16-byte column stride, its tiles come by bulk copies
     int64_t xclip;            // bulk: xref's bytes below this are covered by 16-byte copies inside it
     unsigned* flags;
+    const FactorInfo* info;
 };
+static_assert(sizeof(ExpandArgs) <= 128, "see TtmResArgs");
 
 // The row tile (256, or 128 for nj > kExpandK) and the output columns per block.
 inline int64_t expand_tile(int64_t nj) { return nj <= kExpandK ? 256 : 128; }

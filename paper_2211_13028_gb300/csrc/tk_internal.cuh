@@ -174,6 +174,7 @@ struct Ctx {
         int dt, mtrans;
         float* hi;
         float* lo;
+        void* info;  // tc::FactorInfo
     };
     std::vector<Split> splits;
     bool split_cache = false;

@@ -2751,11 +2751,11 @@ __global__ void __launch_bounds__(RF_THREADS) residual_fma_kernel(const float* _
                     if (DX) d[L * (c + u) + q * RF_THREADS] = alpha * dv;
                 }
             }
-            df_add(h[0], l[0], fr, 0.f);
-            df_add(h[1], l[1], fx, 0.f);
+            tc::ef_add(h[0], l[0], fr);
+            tc::ef_add(h[1], l[1], fx);
         }
     }
-    double s[2] = {(double)h[0] + (double)l[0], (double)h[1] + (double)l[1]};
+    double s[2] = {tc::ef_value(h[0], l[0]), tc::ef_value(h[1], l[1])};
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
         s[q] = warp_sum(s[q]);

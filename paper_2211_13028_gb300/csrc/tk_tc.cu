@@ -15,44 +15,38 @@ __device__ __forceinline__ uint32_t tf32_rna(float x) {
     return r;
 }
 
-// hi = rn_tf32(M(i, a)), lo = rn_tf32(M(i, a) - hi), stored K-major: (i, a) at i + ldo*a,
-// a in [0, npad) with zero padding beyond m.
-__global__ void split_tf32_kernel(const void* M, tk_dtype dt, int64_t ldm, int mtrans, int64_t nj, int64_t m,
-                                  int64_t npad, int64_t ldo, float* hi, float* lo) {
-    kernel_begin();
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= ldo * npad) return;
-    int64_t i = idx % ldo, a = idx / ldo;
-    double v = 0.0;
-    if (i < nj && a < m) {
-        int64_t o = mtrans ? a + ldm * i : i + ldm * a;
-        v = dt == TK_F64 ? static_cast<const double*>(M)[o] : (double)static_cast<const float*>(M)[o];
-    }
-    float h = __uint_as_float(tf32_rna((float)v));
-    float l = __uint_as_float(tf32_rna((float)(v - (double)h)));
-    hi[idx] = h;
-    lo[idx] = l;
-}
+// The blocks that split a factor of n values, each of which sets or clears a flag of its own: whether a part is
+// infinite or NaN (an infinity or NaN in M, or a value that rounds to an infinity).
+constexpr int kSplitThreads = 256;
+inline int64_t split_blocks(int64_t n) { return std::min<int64_t>((n + kSplitThreads - 1) / kSplitThreads, 1024); }
+inline size_t info_bytes(int64_t n) { return sizeof(FactorInfo) + sizeof(int) * (size_t)split_blocks(n); }
 
-// Several factors split in one launch (blockIdx.y = factor): the same split
-// as split_tf32_kernel for each.
+// hi = rn_tf32(M(i, a)), lo = rn_tf32(M(i, a) - hi), stored K-major: (i, a) at i + ldo*a,
+// a in [0, rows_b) with zero padding beyond m.
 struct SplitJob {
     const void* M;
     int dt, mtrans;
     int64_t ldm, nj, m, rows_b, ldo;
     float* hi;
     float* lo;
+    FactorInfo* info;
+    uint32_t blocks;
 };
 constexpr int kMaxSplitJobs = 8;
+template <int NB>
 struct SplitBatch {
-    SplitJob job[kMaxSplitJobs];
+    SplitJob job[NB];
 };
 
-__global__ void split_tf32_batch_kernel(SplitBatch sb) {
+// One factor, or several in one launch (blockIdx.y).
+template <int NB>
+__global__ void __launch_bounds__(kSplitThreads) split_tf32_kernel(const __grid_constant__ SplitBatch<NB> sb) {
     kernel_begin();
-    const SplitJob& jb = sb.job[blockIdx.y];
+    const SplitJob& jb = sb.job[NB > 1 ? blockIdx.y : 0];
+    if (blockIdx.x >= jb.blocks) return;
+    float t = 0.f;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < jb.ldo * jb.rows_b;
-         idx += (int64_t)gridDim.x * blockDim.x) {
+         idx += (int64_t)jb.blocks * blockDim.x) {
         const int64_t i = idx % jb.ldo, a = idx / jb.ldo;
         double v = 0.0;
         if (i < jb.nj && a < jb.m) {
@@ -63,6 +57,17 @@ __global__ void split_tf32_batch_kernel(SplitBatch sb) {
         const float l = __uint_as_float(tf32_rna((float)(v - (double)h)));
         jb.hi[idx] = h;
         jb.lo[idx] = l;
+        t = fmaf(l, 0.f, t);
+    }
+    const int bad = __syncthreads_or(t != t);
+    if (threadIdx.x != 0) return;
+    jb.info->bad[blockIdx.x] = bad;
+    if (blockIdx.x == 0) {
+        jb.info->M = jb.M;
+        jb.info->ldm = jb.ldm;
+        jb.info->dt = jb.dt;
+        jb.info->mtrans = jb.mtrans;
+        jb.info->nbad = jb.blocks;
     }
 }
 
@@ -132,9 +137,9 @@ static Blocks tc_blocks(int64_t L, int64_t nj, int64_t m, bool residual, tk_dtyp
 // launch and entered in the call's split cache (c.split_cache must be on while
 // those TTMs run).  Factors already split are skipped.
 void tc_presplit(Ctx& c, const std::vector<TcSplitReq>& reqs) {
-    tc::SplitBatch sb;
+    tc::SplitBatch<tc::kMaxSplitJobs> sb{};
     int nj_ = 0;
-    int64_t most = 0;
+    int64_t most = 0, blocks = 1;
     for (const TcSplitReq& q : reqs) {
         const Blocks bl = tc_blocks(q.L, q.nj, q.m, q.residual, q.dt);
         const int64_t npad = bl.npad, ldo = (q.nj + 3) / 4 * 4, rows_b = npad * bl.nblk;
@@ -145,14 +150,16 @@ void tc_presplit(Ctx& c, const std::vector<TcSplitReq>& reqs) {
         if (have || nj_ == tc::kMaxSplitJobs) continue;
         float* hi = c.alloc<float>(ldo * rows_b);
         float* lo = c.alloc<float>(ldo * rows_b);
-        c.splits.push_back({q.M.p, q.M.ld, q.nj, q.m, npad, rows_b, (int)q.M.dt, q.mtrans ? 1 : 0, hi, lo});
-        sb.job[nj_++] = {q.M.p, (int)q.M.dt, q.mtrans ? 1 : 0, q.M.ld, q.nj, q.m, rows_b, ldo, hi, lo};
+        const int64_t nb = tc::split_blocks(ldo * rows_b);
+        auto* info = static_cast<tc::FactorInfo*>(c.alloc_bytes(tc::info_bytes(ldo * rows_b)));
+        c.splits.push_back({q.M.p, q.M.ld, q.nj, q.m, npad, rows_b, (int)q.M.dt, q.mtrans ? 1 : 0, hi, lo, info});
+        sb.job[nj_++] = {q.M.p, (int)q.M.dt, q.mtrans ? 1 : 0, q.M.ld, q.nj, q.m, rows_b, ldo, hi, lo, info, (uint32_t)nb};
         most = std::max(most, ldo * rows_b);
+        blocks = std::max(blocks, nb);
     }
     if (!c.exec || nj_ == 0) return;
     ProfScope ps(c, "elementwise", 16.0 * most * nj_, 0.0);
-    run_kernel(c, tc::split_tf32_batch_kernel,
-               dim3((unsigned)std::min<int64_t>((most + 255) / 256, 1024), (unsigned)nj_), 256, 0, sb);
+    run_kernel(c, tc::split_tf32_kernel<tc::kMaxSplitJobs>, dim3((unsigned)blocks, (unsigned)nj_), tc::kSplitThreads, 0, sb);
     c.counted();
     c.check_launch();
 }
@@ -216,6 +223,7 @@ bool ttm_tc_eligible(const Tens& X, int j, int64_t m, tk_dtype out_dt) {
 struct Factor {
     float* hi = nullptr;
     float* lo = nullptr;
+    tc::FactorInfo* info = nullptr;
     int64_t ldo = 0, rows_b = 0;
     bool have = false;
 };
@@ -230,13 +238,16 @@ static Factor factor_alloc(Ctx& c, const Mat& M, bool mtrans, int64_t nj, int64_
                 e.m == m && e.npad == npad && e.rows == f.rows_b) {
                 f.hi = e.hi;
                 f.lo = e.lo;
+                f.info = static_cast<tc::FactorInfo*>(e.info);
                 f.have = true;
                 return f;
             }
     }
     f.hi = c.alloc<float>(f.ldo * f.rows_b);
     f.lo = c.alloc<float>(f.ldo * f.rows_b);
-    if (c.split_cache) c.splits.push_back({M.p, M.ld, nj, m, npad, f.rows_b, (int)M.dt, mtrans ? 1 : 0, f.hi, f.lo});
+    f.info = static_cast<tc::FactorInfo*>(c.alloc_bytes(tc::info_bytes(f.ldo * f.rows_b)));
+    if (c.split_cache)
+        c.splits.push_back({M.p, M.ld, nj, m, npad, f.rows_b, (int)M.dt, mtrans ? 1 : 0, f.hi, f.lo, f.info});
     return f;
 }
 
@@ -247,8 +258,10 @@ static void factor_map(Ctx& c, const Factor& f, const Mat& M, bool mtrans, int64
     if (!f.have) {
         const int64_t tot = f.ldo * f.rows_b;
         ProfScope ps(c, "elementwise", 8.0 * tot + 8.0 * nj * m, 0.0);
-        run_kernel(c, tc::split_tf32_kernel, (unsigned)((tot + 255) / 256), 256, 0, M.p, M.dt, M.ld, mtrans ? 1 : 0,
-                   nj, m, f.rows_b, f.ldo, f.hi, f.lo);
+        const int64_t nb = tc::split_blocks(tot);
+        const tc::SplitBatch<1> sb{{{M.p, (int)M.dt, mtrans ? 1 : 0, M.ld, nj, m, f.rows_b, f.ldo, f.hi, f.lo, f.info,
+                                     (uint32_t)nb}}};
+        run_kernel(c, tc::split_tf32_kernel<1>, (unsigned)nb, tc::kSplitThreads, 0, sb);
         c.counted();
         c.check_launch();
     }
@@ -274,10 +287,9 @@ static tc::ExpandArgs expand_args(const Ctx& c, const Tens& W, int j, int64_t m,
     tc::ExpandArgs a{};
     a.L = W.left(j);
     a.nj = W.n[j];
-    a.R = W.right(j);
     a.m = m;
     a.W = static_cast<const float*>(W.p);
-    const int64_t rows = a.L * a.R, tile = tc::expand_tile(a.nj), sms = tc::grid_sms(c);
+    const int64_t rows = a.L * W.right(j), tile = tc::expand_tile(a.nj), sms = tc::grid_sms(c);
     a.rows = (uint32_t)rows;
     const int64_t ntiles = (rows + tile - 1) / tile;
     const int64_t ncs = std::max<int64_t>(1, std::min<int64_t>(bl.nblk, (8 * sms + ntiles - 1) / ntiles));
@@ -352,9 +364,9 @@ static void launch_ttm_lowp(Ctx& c, const Tens& X, int j, const Mat& M, bool mtr
     a.xbytes = tma ? runs * a.slot : 0;
     a.x_inv = X.dt == TK_FP8_E4M3 ? 1.f / X.scale : 1.f;
     a.X = static_cast<const uint8_t*>(X.p);
-    a.part = part;
+    a.info = f.info;
     a.out_numel = L * m * R;
-    a.out = out;
+    a.out = ksplit > 1 ? part : out;
     a.flags = c.dflags;
     {
         ProfScope ps(c, name, (double)es * L * R * nj + 8.0 * nj * m + 4.0 * (double)L * R * m,
@@ -390,6 +402,7 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
         factor_map(c, f, M, mtrans, nj, m, npad, &tb);
         tc::ExpandArgs a = expand_args(c, X, j, m, bl);
         a.out = out;
+        a.info = f.info;
         ProfScope ps(c, name, 4.0 * (double)L * R * nj + 8.0 * nj * m + 4.0 * (double)L * R * m,
                      2.0 * (double)L * R * nj * m);
         tc::expand_run(c, 0, TK_F32, tb, tb, a);
@@ -438,9 +451,9 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
     a.ksplit = (uint32_t)ksplit;
     a.vec = (kmajor ? nj : L) % 2 == 0 ? 2 : 1;
     a.X = static_cast<const float*>(X.p);
-    a.part = part;
+    a.info = f.info;
     a.out_numel = L * m * R;
-    a.out = out;
+    a.out = ksplit > 1 ? part : out;
     a.flags = c.dflags;
     {
         ProfScope ps(c, name, 4.0 * (double)L * R * nj + 8.0 * nj * m + 4.0 * (double)L * R * m,
@@ -488,7 +501,7 @@ void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtr
         const bool flat = !tma_ok(W, j) || L < tc::kRows;
         CUtensorMap tw = tb;  // unused by the loaders
         if (!flat) strided_map(W, j, 1, &tw);
-        tc::TtmArgs a{};
+        tc::TtmResArgs a{};
         a.L = L;
         a.nj = nj;
         a.R = 1;
@@ -502,6 +515,7 @@ void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtr
         a.xbytes = flat ? 0 : (uint32_t)tc::kXBytes;
         a.vec = L % 2 == 0 ? 2 : 1;
         a.X = static_cast<const float*>(W.p);
+        a.info = f.info;
         a.flags = c.dflags;
         a.xref = xref;
         a.xrdt = (int)xrdt;
@@ -515,6 +529,7 @@ void launch_ttm_tc_residual(Ctx& c, const Tens& W, int j, const Mat& M, bool mtr
         return;
     }
     tc::ExpandArgs a = expand_args(c, W, j, m, bl);
+    a.info = f.info;
     a.bulk = (L * es) % 16 != 0;
     a.xclip = (L * m * es) & ~(int64_t)15;
     txr = tb;  // unused when bulk

@@ -140,6 +140,20 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// (hi, lo) += b with Knuth's two-sum on the high part; the low part collects
+// the rounding errors (a double-float running sum of FP32 terms).
+__device__ __forceinline__ void ef_add(float& hi, float& lo, float b) {
+    const float s = __fadd_rn(hi, b);
+    const float v = __fsub_rn(s, hi);
+    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(b, v));
+    hi = s;
+    lo = __fadd_rn(lo, e);
+}
+// Its value; hi alone once an infinity or a NaN is in it (lo is a NaN then).
+__device__ __forceinline__ double ef_value(float hi, float lo) {
+    return fabsf(hi) <= 3.402823466e38f ? (double)hi + (double)lo : (double)hi;
+}
+
 // Tensor map over global memory (rank 2 or 3), element type dt, box dims.
 inline PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;

@@ -49,11 +49,13 @@ struct LowpArgs {
     uint32_t xbytes;   // TMA bytes of X a chunk (0: loaders)
     float x_inv;       // factor of the result: 1 / scale of X
     const uint8_t* X;
-    float* part;
     int64_t out_numel;
-    float* out;
+    float* out;        // the product, or the first of the ksplit partial ones
     unsigned* flags;
+    const FactorInfo* info;
 };
+static_assert(sizeof(LowpArgs) <= 128, "see TtmResArgs");
+static_assert(sizeof(LowpArgs) <= 128, "see TtmResArgs");
 
 template <int NPAD>
 struct LowpCfg {
@@ -143,6 +145,7 @@ __global__ void __launch_bounds__(LowpCfg<NPAD>::kThreads, 1)
     uint64_t* done = accempty + C::kAcc;            // [1] every issued MMA complete
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    __shared__ int again;  // infinite or NaN results (exact_items); static: its address takes no register
 
     const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -160,6 +163,7 @@ __global__ void __launch_bounds__(LowpCfg<NPAD>::kThreads, 1)
         }
         mbar_init(done, 1);
         *abort = 0;
+        again = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) {
@@ -457,7 +461,7 @@ __global__ void __launch_bounds__(LowpCfg<NPAD>::kThreads, 1)
             const uint32_t w2 = ksplit == 1 ? w : w / ksplit, sk = w - w2 * ksplit;
             const uint32_t t = tile_of(w), nb = args.nblk == 1 ? 0 : w2 % args.nblk;
             const uint32_t nc = chunk1(w) - chunk0(w);
-            float* const outp = ksplit > 1 ? args.part + sk * args.out_numel : args.out;
+            float* const outp = args.out + sk * args.out_numel;
             int64_t base, stride;
             bool valid;
             if (KMAJOR) {
@@ -514,9 +518,10 @@ __global__ void __launch_bounds__(LowpCfg<NPAD>::kThreads, 1)
                 for (int j = 0; j < kSl; ++j) {
                     const int c0 = 16 * half + 32 * j;
                     if (c0 >= NPAD) break;
+                    if (any_nonfinite(v[j])) again = 1;
 #pragma unroll
                     for (int i = 0; i < 16; ++i) v[j][i] *= args.x_inv;
-                    if (KMAJOR && (m & 3) == 0 && (reinterpret_cast<uintptr_t>(outp) & 15) == 0) {  // 16-byte stores along the row
+                    if (KMAJOR && (m & 3) == 0) {  // 16-byte stores along the row
 #pragma unroll
                         for (int i = 0; i < 16; i += 4)
                             if (c0 + i < ncol)
@@ -536,6 +541,9 @@ __global__ void __launch_bounds__(LowpCfg<NPAD>::kThreads, 1)
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase) : "memory");
     }
+    if (again && !*abort)
+        exact_items<typename std::conditional<ES == 1, __nv_fp8_e4m3, __nv_bfloat16>::type, KMAJOR, false>(
+            args, NPAD, K, args.x_inv);
 }
 
 template <int NPAD, bool KMAJOR, int ES>

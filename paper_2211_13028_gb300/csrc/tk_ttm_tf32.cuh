@@ -88,22 +88,6 @@ __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) 
     lo = __float_as_uint(x - __uint_as_float(hi));
 }
 
-// (hi, lo) += b with Knuth's two-sum on the high part; the low part collects
-// the rounding errors (a double-float running sum of FP32 terms).
-__device__ __forceinline__ void ef_add(float& hi, float& lo, float b) {
-    const float s = __fadd_rn(hi, b);
-    const float v = __fsub_rn(s, hi);
-    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, v)), __fsub_rn(b, v));
-    hi = s;
-    lo = __fadd_rn(lo, e);
-}
-
-__device__ __forceinline__ float xr_to_f32(float v) { return v; }
-__device__ __forceinline__ float xr_to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
-__device__ __forceinline__ float xr_to_f32(__nv_fp8_e4m3 v) { return static_cast<float>(v); }
-__device__ __forceinline__ void xr_store(float* p, float v) { *p = v; }
-__device__ __forceinline__ void xr_store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
-
 // The sums (sr, sx) of the lanes of N epilogue warps, in a fixed order, into the CTA's pair of partials.
 template <int N>
 __device__ __forceinline__ void residual_sums(int e, int lane, double sr, double sx, double* partials) {
@@ -129,6 +113,124 @@ __device__ __forceinline__ void residual_sums(int e, int lane, double sr, double
     }
 }
 
+// What a kernel has to know of the factor besides its parts, written beside them by the kernel that splits it (in
+// memory: the kernels' arguments have no room for it, see TtmResArgs): the factor as the caller gave it, M(i, a) = M[i + ldm a], or M[a + ldm i] with mtrans (dt: F32
+// or F64), and a flag of each block that split it, set when a part is infinite or NaN.
+struct FactorInfo {
+    const void* M;
+    int64_t ldm;
+    int dt, mtrans;
+    uint32_t nbad;
+    int bad[1];
+};
+
+__device__ __forceinline__ void xr_store(float* p, float v) { *p = v; }
+__device__ __forceinline__ void xr_store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ float x_to_f32(float v) { return v; }
+__device__ __forceinline__ float x_to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ float x_to_f32(__nv_fp8_e4m3 v) { return static_cast<float>(v); }
+
+// Elements of the product that come out infinite or NaN are formed again by FP32 FMAs, from the factor as the caller
+// gave it: for an infinity, or a value that rounds to one, the split gives a NaN (x_hi M_lo with M_lo = 0 or of the
+// other sign).  The epilogue only notes that there are some; the CTA goes over its items once more at its end, when
+// nothing is kept in registers (a call in the epilogue itself: 135 -> 150 us for the core of 512^3, from the spills).
+//
+// The sum over i0 <= i < i1 of M(i, a) x[i step] inv.
+template <typename TX>
+__device__ __forceinline__ float exact_dot(const TX* x, int64_t step, int64_t i0, int64_t i1, const FactorInfo& f, int64_t a,
+                                           float inv) {
+    float s = 0.f;
+    const int64_t fa = f.mtrans ? a : f.ldm * a, fi = f.mtrans ? f.ldm : 1;
+#pragma unroll 4
+    for (int64_t i = i0; i < i1; ++i) {
+        const int64_t o = fa + fi * i;
+        const float mv = f.dt == TK_F64 ? (float)static_cast<const double*>(f.M)[o] : static_cast<const float*>(f.M)[o];
+        s = fmaf(mv, x_to_f32(x[i * step]) * inv, s);
+    }
+    return s;
+}
+
+// Forms the infinite and NaN elements among the results of this CTA's items again (every thread, after a barrier).
+template <typename TX, bool KMAJOR, bool FLAT, typename Args>
+__device__ __forceinline__ void exact_items(const Args& g, int npad, int chunk, float inv) {
+    for (uint32_t w = blockIdx.x; w < g.nitems; w += gridDim.x) {
+        const uint32_t w2 = w / g.ksplit, sk = w - w2 * g.ksplit, t = w2 / g.nblk, nb = w2 - t * g.nblk;
+        const int64_t i0 = (int64_t)((uint64_t)g.nk * sk / g.ksplit) * chunk;
+        const int64_t ie = (int64_t)((uint64_t)g.nk * (sk + 1) / g.ksplit) * chunk, i1 = ie < g.nj ? ie : g.nj;
+        float* const out = g.out + sk * g.out_numel;
+        for (int e = threadIdx.x; e < 128 * npad; e += blockDim.x) {
+            const int rho = e & 127;
+            const int64_t c = (int64_t)nb * npad + (e >> 7);
+            if (c >= g.m) break;
+            int64_t l, r;  // the row's place in its slab, its slab
+            if (KMAJOR) {
+                l = 0;
+                r = (int64_t)t * 128 + rho;
+            } else if (FLAT) {
+                r = ((int64_t)t * 128 + rho) / g.L;
+                l = (int64_t)t * 128 + rho - r * g.L;
+            } else if (g.pack > 1) {
+                const int p = rho / (int)g.L;
+                l = p < (int)g.pack ? rho - p * g.L : g.L;
+                r = (int64_t)t * g.pack + p;
+            } else {
+                r = t / g.tiles_per_r;
+                l = (int64_t)(t - r * g.tiles_per_r) * 128 + rho;
+            }
+            if (l >= g.L || r >= g.R) continue;
+            float* const o = out + l + g.L * (c + g.m * r);
+            if (fabsf(*o) <= 3.402823466e38f) continue;
+            *o = exact_dot(reinterpret_cast<const TX*>(g.X) + l + g.L * g.nj * r, g.L, i0, i1, *g.info, c, inv);
+        }
+    }
+}
+
+// A CTA whose part of a fused residual met such elements compares all of it again: element (l, a) of the rows [l0, l1)
+// and columns [a0, a1), with the sums in FP64.
+template <typename XR>
+__device__ __forceinline__ void exact_compare(const float* W, int64_t L, int64_t nj, const FactorInfo& f, int64_t l0,
+                                              int64_t l1, int64_t a0, int64_t a1, const void* xref, float xr_scale,
+                                              void* dx, float alpha, double& sr, double& sx) {
+    const int64_t rows = l1 - l0;
+    for (int64_t e = threadIdx.x; e < rows * (a1 - a0); e += blockDim.x) {
+        const int64_t l = l0 + e % rows, a = a0 + e / rows;
+        const float xv = x_to_f32(static_cast<const XR*>(xref)[l + L * a]) * xr_scale;
+        const float dv = xv - exact_dot(W + l, L, 0, nj, f, a, 1.f);
+        sr += (double)dv * dv;
+        sx += (double)xv * xv;
+        if constexpr (!std::is_same<XR, __nv_fp8_e4m3>::value)
+            if (dx) xr_store(static_cast<XR*>(dx) + l + L * a, alpha * dv);
+    }
+}
+
+// Whether one of the values is infinite or NaN.
+__device__ __forceinline__ bool any_nonfinite(const float (&v)[16]) {
+    float t = 0.f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) t = fmaf(v[i], 0.f, t);
+    return t != t;
+}
+
+// The same over every thread of the CTA (after a barrier).
+__device__ __forceinline__ void residual_sums_cta(double sr, double sx, double* partials) {
+    __shared__ double red[2 * 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sr += __shfl_xor_sync(0xffffffffu, sr, o);
+        sx += __shfl_xor_sync(0xffffffffu, sx, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = sr;
+        red[32 + (threadIdx.x >> 5)] = sx;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double t = 0.0;
+        for (uint32_t i = 0; i < blockDim.x / 32; ++i) t += red[32 * threadIdx.x + i];
+        partials[2 * blockIdx.x + threadIdx.x] = t;
+    }
+}
+
 struct TtmArgs {
     int64_t L, nj, R, m;
     // work item = (row tile, block of NPAD output columns, part of the K chunks)
@@ -138,17 +240,22 @@ struct TtmArgs {
     uint32_t pack;
     uint32_t xbytes;  // TMA bytes of one X chunk (128 x 32 x 4, or L x 32 x pack x 4; 0: FLAT)
     // few row tiles: the K chunks of a tile are split over ksplit work items, each writing its
-    // partial product to part + s out_numel (summed in order by a second kernel); 1 otherwise
+    // partial product to out + s out_numel (summed in order by a second kernel); 1 otherwise
     uint32_t ksplit;
     uint32_t fill;         // chunks per accumulator (TMA)
     uint32_t vec;          // FLAT: floats per cp.async (1 or 2)
     const float* X;        // FLAT
-    float* part;
     int64_t out_numel;
-    float* out;
+    float* out;            // the product, or the first of the ksplit partial ones
     unsigned* flags;
-    // RES: the tensor compared with the product (its layout, R == 1; elements of type xrdt, times xr_scale),
-    // dx = alpha * (xref - product) in its type (may be NULL), per-CTA sums {(xref - product)^2, xref^2}
+    const FactorInfo* info;
+};
+static_assert(sizeof(TtmArgs) <= 128, "see TtmResArgs");
+
+// RES: the tensor compared with the product (its layout, R == 1; elements of type xrdt, times xr_scale),
+// dx = alpha * (xref - product) in its type (may be NULL), per-CTA sums {(xref - product)^2, xref^2}.  (Arguments of their
+// own: kernels get slower where theirs pass 128 bytes beside the two maps, ttm_lowp_kernel 170 -> 199 us.)
+struct TtmResArgs : TtmArgs {
     const void* xref;
     void* dx;
     int xrdt;
@@ -160,7 +267,7 @@ template <typename XR>
 __device__ __forceinline__ void residual_load(const void* xref, int64_t o, int64_t L, int n, float (&x)[8]) {
     const XR* xp = static_cast<const XR*>(xref) + o;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = i < n ? xr_to_f32(xp[i * L]) : 0.f;
+    for (int i = 0; i < 8; ++i) x[i] = i < n ? x_to_f32(xp[i * L]) : 0.f;
 }
 template <typename XR>
 __device__ __forceinline__ void residual_store(void* dx, int64_t o, int64_t L, int n, const float (&x)[8]) {
@@ -171,7 +278,7 @@ __device__ __forceinline__ void residual_store(void* dx, int64_t o, int64_t L, i
 }
 
 // RES: 8 columns p of a row, of which n are the product's, against xref from its element o.
-__device__ __forceinline__ void residual_columns(const TtmArgs& a, int64_t o, int n, const float* p, float& fr,
+__device__ __forceinline__ void residual_columns(const TtmResArgs& a, int64_t o, int n, const float* p, float& fr,
                                                  float& fx) {
     float x[8];
     if (a.xrdt == TK_F32) residual_load<float>(a.xref, o, a.L, n, x);
@@ -188,6 +295,26 @@ __device__ __forceinline__ void residual_columns(const TtmArgs& a, int64_t o, in
     if (!a.dx) return;
     if (a.xrdt == TK_F32) residual_store<float>(a.dx, o, a.L, n, x);
     else residual_store<__nv_bfloat16>(a.dx, o, a.L, n, x);
+}
+
+// RES: the whole of a CTA's part again.
+__device__ __forceinline__ void exact_residual(const TtmResArgs& args, int npad) {
+    double sr = 0.0, sx = 0.0;
+    for (uint32_t w = blockIdx.x; w < args.nitems; w += gridDim.x) {
+        const uint32_t t = w / args.nblk, nb = w - t * args.nblk;
+        const int64_t l0 = (int64_t)t * kRows, a0 = (int64_t)nb * npad;
+        const int64_t l1 = l0 + kRows < args.L ? l0 + kRows : args.L, a1 = a0 + npad < args.m ? a0 + npad : args.m;
+        if (args.xrdt == TK_F32)
+            exact_compare<float>(args.X, args.L, args.nj, *args.info, l0, l1, a0, a1, args.xref, args.xr_scale, args.dx,
+                                 args.alpha, sr, sx);
+        else if (args.xrdt == TK_BF16)
+            exact_compare<__nv_bfloat16>(args.X, args.L, args.nj, *args.info, l0, l1, a0, a1, args.xref, args.xr_scale,
+                                         args.dx, args.alpha, sr, sx);
+        else
+            exact_compare<__nv_fp8_e4m3>(args.X, args.L, args.nj, *args.info, l0, l1, a0, a1, args.xref, args.xr_scale,
+                                         args.dx, args.alpha, sr, sx);
+    }
+    residual_sums_cta(sr, sx, args.partials);
 }
 
 template <int NPAD, bool KMAJOR, bool FLAT>
@@ -234,7 +361,7 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
 template <int NPAD, bool KMAJOR, bool FLAT, bool RES = false>
 __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
     ttm_tf32x3_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmB,
-                      TtmArgs args) {
+                      typename std::conditional<RES, TtmResArgs, TtmArgs>::type args) {
     kernel_begin();
     using C = TtmCfg<NPAD, KMAJOR, FLAT>;
     constexpr uint32_t S = C::kStages;
@@ -254,9 +381,11 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
     uint64_t* stgfull = stgfree + 1;        // [1] tile staged (the epilogue warps)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(stgfull + 1);
     volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    __shared__ int again;  // infinite or NaN results (exact_items); static: its address takes no register
 
     const int warp = (int)warp_uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
+        again = 0;
         for (uint32_t s = 0; s < S; ++s) {
             mbar_init(&full[s], 1 + 32 * C::kLoad);
             mbar_init(&xfree[s], 9);
@@ -587,7 +716,7 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
             const uint32_t t = args.nblk == 1 ? w2 : w2 / args.nblk, nb = args.nblk == 1 ? 0 : w2 % args.nblk;
             const uint32_t nc = chunk1(w) - chunk0(w);
             const uint32_t nfill = FLAT ? 2 * nc : (nc + args.fill - 1) / args.fill;
-            float* const outp = ksplit > 1 ? args.part + sk * args.out_numel : args.out;
+            float* const outp = args.out + sk * args.out_numel;
             int64_t base, stride;
             bool valid;
             if (KMAJOR) {
@@ -662,6 +791,11 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
                 }
             }
             if (!ok) break;
+            bool bad = any_nonfinite(v[0]);
+#pragma unroll
+            for (int j = 1; j < kSl; ++j)
+                if (16 * half + 32 * j < NPAD) bad = bad || any_nonfinite(v[j]);
+            if (valid && bad) again = 1;  // (see exact_items)
             if constexpr (RES) {
                 if (valid) {
 #pragma unroll
@@ -737,20 +871,27 @@ __global__ void __launch_bounds__(TtmCfg<NPAD, KMAJOR, FLAT>::kThreads, 1)
                 }
             }
         }
-        if (C::kOut && copier) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        if (C::kOut && copier) asm volatile("cp.async.bulk.wait_group 0;\n\tfence.proxy.async;" ::: "memory");
         if constexpr (RES)
-            residual_sums<C::kEpi>(warp - C::kFirstEpi, lane, (double)srh + (double)srl, (double)sxh + (double)sxl,
-                                   args.partials);
+            residual_sums<C::kEpi>(warp - C::kFirstEpi, lane, ef_value(srh, srl), ef_value(sxh, sxl), args.partials);
     }
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase) : "memory");
     }
+    if (again && !*abort) {
+        if constexpr (RES) {
+            exact_residual(args, NPAD);
+        } else {
+            exact_items<float, KMAJOR, FLAT>(args, NPAD, kChunk, 1.f);
+        }
+    }
 }
 
 template <int NPAD, bool KMAJOR, bool FLAT, bool RES = false>
-static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorMap& tb, TtmArgs a) {
+static void ttm_tf32_launch(const Ctx& c, const CUtensorMap& tx, const CUtensorMap& tb,
+                            typename std::conditional<RES, TtmResArgs, TtmArgs>::type a) {
     using Cf = TtmCfg<NPAD, KMAJOR, FLAT>;
     // above 64 columns a drain every 4 chunks would bound the pass (512^3, 81 columns: 174 against 121 us);
     // up to 8, the sketch widths, every chunk is drained: the FP32 FMA kernel that streamed those before
@@ -790,7 +931,7 @@ void ttm_tf32_run_tma(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap
 void ttm_tf32_run_flat(const Ctx& c, int64_t npad, bool kmajor, const CUtensorMap& tx, const CUtensorMap& tb,
                        const TtmArgs& a);
 // Fused with the comparison with xref (RES): blocks of 64 columns.
-void ttm_tf32_run_residual(const Ctx& c, bool flat, const CUtensorMap& tx, const CUtensorMap& tb, const TtmArgs& a);
+void ttm_tf32_run_residual(const Ctx& c, bool flat, const CUtensorMap& tx, const CUtensorMap& tb, const TtmResArgs& a);
 
 }  // namespace tc
 }  // namespace tk

@@ -6,7 +6,7 @@
 namespace tk {
 namespace tc {
 
-void ttm_tf32_run_residual(const Ctx& c, bool flat, const CUtensorMap& tx, const CUtensorMap& tb, const TtmArgs& a) {
+void ttm_tf32_run_residual(const Ctx& c, bool flat, const CUtensorMap& tx, const CUtensorMap& tb, const TtmResArgs& a) {
     if (flat) ttm_tf32_launch<64, false, true, true>(c, tx, tb, a);
     else ttm_tf32_launch<64, false, false, true>(c, tx, tb, a);
 }

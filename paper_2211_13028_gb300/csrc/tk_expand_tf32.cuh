@@ -31,6 +31,25 @@ static_assert(sizeof(ExpandArgs) <= 128, "see TtmResArgs");
 inline int64_t expand_tile(int64_t nj) { return nj <= kExpandK ? 256 : 128; }
 inline int64_t expand_cols(int64_t nj) { return nj <= kExpandK ? 32 : 64; }
 
+// The parts a tile's column blocks are split into: one CTA runs an item (a tile's part) per wave, and an item converts its
+// tile of W again, about as long as 1.2 blocks of output take from two buffers (K <= 32), 2.8 else; the parts whose waves
+// end first.  152 SMs, loss: 262144 x 512, K = 39 (1024 tiles, 16 blocks): one part 197 us, two 215, eight 385; 40000 x 512:
+// 85, 81, 107; 8800 x 391: two 60, four 57, one block each 69; 1600 x 4992 BF16, K = 39 (7 tiles, 156 blocks): one
+// block each 45 us, the 20 parts of a wave 18.
+inline int64_t expand_parts(int64_t ntiles, int64_t nblk, int64_t nj, int64_t sms) {
+    int64_t best = 1;
+    double least = 1e300;
+    for (int64_t ncs = 1; ncs <= nblk && ncs <= 8 * sms; ++ncs) {
+        const int64_t blocks = (nblk + ncs - 1) / ncs, waves = (ntiles * ncs + sms - 1) / sms;
+        const double t = (double)waves * ((nj <= kChunk ? 1.2 : 2.8) + (double)blocks);
+        if (t < least) {
+            least = t;
+            best = ncs;
+        }
+    }
+    return best;
+}
+
 // epi 0: plain product; 1: norms; 2: norms and dx.  tb: map of (M_hi, M_lo) with boxes of 32 x
 // expand_cols(nj) x 2; txr: map of xref with boxes of expand_tile x expand_cols (unused when bulk).
 void expand_run(const Ctx& c, int epi, tk_dtype xrdt, const CUtensorMap& tb, const CUtensorMap& txr,

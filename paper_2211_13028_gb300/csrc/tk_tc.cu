@@ -281,8 +281,7 @@ static void strided_map(const Tens& X, int j, int64_t pack, CUtensorMap* tx) {
     tc::encode(tx, X.p, 3, dims, str, box, false);
 }
 
-// The expansion kernel's work: row tiles x parts of their column blocks (an item converts its tile of W
-// again, so parts are no finer than about 8 items an SM need).
+// The expansion kernel's work: row tiles x parts of their column blocks.
 static tc::ExpandArgs expand_args(const Ctx& c, const Tens& W, int j, int64_t m, const Blocks& bl) {
     tc::ExpandArgs a{};
     a.L = W.left(j);
@@ -292,7 +291,7 @@ static tc::ExpandArgs expand_args(const Ctx& c, const Tens& W, int j, int64_t m,
     const int64_t rows = a.L * W.right(j), tile = tc::expand_tile(a.nj), sms = tc::grid_sms(c);
     a.rows = (uint32_t)rows;
     const int64_t ntiles = (rows + tile - 1) / tile;
-    const int64_t ncs = std::max<int64_t>(1, std::min<int64_t>(bl.nblk, (8 * sms + ntiles - 1) / ntiles));
+    const int64_t ncs = tc::expand_parts(ntiles, bl.nblk, a.nj, sms);
     TK_REQUIRE(ntiles * ncs < ((int64_t)1 << 31), TK_ERR_SHAPE, "ttm_tc: too many tiles");
     a.ntiles = (uint32_t)ntiles;
     a.nblk = (uint32_t)bl.nblk;

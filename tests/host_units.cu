@@ -3,7 +3,7 @@
 #include <cstring>
 #include <vector>
 
-#include "tk_tc_common.cuh"
+#include "tk_expand_tf32.cuh"
 
 // host_units_runtime.c: stand-ins for the runtime's calls, which several devices answer
 extern "C" int fake_device;      // the current device
@@ -65,8 +65,28 @@ static int per_device() {
     return std::vector<int>(fake_set, fake_set + fake_set_count) == want ? 0 : 1;
 }
 
+// An item of an expansion converts its tile of W again: the parts of a tile's blocks are those that end first.
+static int expand_parts() {
+    struct {
+        int64_t ntiles, nblk, nj, want;
+    } cases[] = {{7, 156, 39, 20},     // a wave: 8 blocks an item (156 items of one block: two waves)
+                 {1, 30, 3, 30},       // few: every block its own item
+                 {1024, 16, 39, 1},    // many waves: no part converts the tile again
+                 {157, 16, 39, 2},     // three waves of half tiles, not two of whole ones
+                 {35, 13, 39, 4},      {1, 1, 1, 1}, {300001, 1, 64, 1}, {1, 1 << 20, 64, 152}};
+    for (const auto& c : cases) {
+        const int64_t got = tk::tc::expand_parts(c.ntiles, c.nblk, c.nj, 152);
+        if (got != c.want) {
+            std::printf("%lld tiles, %lld blocks: %lld parts\n", (long long)c.ntiles, (long long)c.nblk, (long long)got);
+            return 1;
+        }
+    }
+    return 0;
+}
+
 int main(int argc, char** argv) {
     if (argc == 2 && !std::strcmp(argv[1], "split_visibility")) return split_visibility();
     if (argc == 2 && !std::strcmp(argv[1], "per_device")) return per_device();
+    if (argc == 2 && !std::strcmp(argv[1], "expand_parts")) return expand_parts();
     return 2;
 }

@@ -33,3 +33,8 @@ def test_splits_of_one_branch_are_not_seen_by_another(units):
 def test_kernel_limits_and_sm_counts_are_each_devices_own(units):
     # handles on several devices of a process launch the same kernels
     _run(units, "per_device")
+
+
+def test_expansions_are_split_into_the_parts_that_end_first(units):
+    # as many items as 8 an SM: 1600 x 4992 out of 39 was 1092 items that converted 7 tiles 156 times each
+    _run(units, "expand_parts")

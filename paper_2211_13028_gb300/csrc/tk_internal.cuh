@@ -362,6 +362,16 @@ struct ProfScope {
 // out is dense column-major, dims of X with n_j -> m, dtype F64 or F32.
 void launch_ttm(const Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int64_t m, void* out, tk_dtype out_dt);
 
+// Whether launch_ttm takes a product of FP32 accumulation with a CTA per slab (L m outputs of a long contraction), and
+// the parts it splits each of the slab's dot products into.
+inline bool ttm_simt_slab(int64_t L, int64_t nj, int64_t R, int64_t m, size_t acc_bytes) {
+    return L * m <= 256 && nj >= 32 && L * nj >= 256 && (double)acc_bytes * (L * nj + 256) <= 40 * 1024 &&
+           R <= 0x7fffffff;
+}
+inline int ttm_simt_slab_parts(int64_t L, int64_t m) { return (int)(256 / (L * m) < 16 ? 256 / (L * m) : 16); }
+// Whether it takes one with a thread per output.
+inline bool ttm_simt_direct(int64_t rows, int64_t nj, int64_t m) { return rows * m <= (1 << 21) && nj <= 512; }
+
 // Tensor-core (tcgen05, TF32 parts) version of launch_ttm for FP32 output: FP32 data, and BF16 / FP8 data
 // in the layouts that launch_ttm_bf16 / launch_ttm_fp8 do not take.  ttm_tc_eligible says whether a TTM
 // takes it (dtype, and the sizes where it is faster).

@@ -271,9 +271,8 @@ static void ttm_dispatch(const Ctx& c, const Tx* X, int64_t L, int64_t nj, int64
         if (c.df64 && ttm_direct_df(c, X, L, nj, R, M, ldm, mtrans, m, out)) return;
     }
     // (a slab of fewer than 256 elements leaves each CTA too little work: one thread per output then)
-    if (L * m <= SLAB_THREADS && nj >= 32 && L * nj >= 256 &&
-        (double)sizeof(Ta) * (L * nj + SLAB_THREADS) <= 40 * 1024 && R <= 0x7fffffff) {
-        const int S = (int)std::min<int64_t>(16, SLAB_THREADS / (L * m));
+    if (ttm_simt_slab(L, nj, R, m, sizeof(Ta))) {
+        const int S = ttm_simt_slab_parts(L, m);
         const size_t smem = sizeof(Ta) * (size_t)(L * nj + (int64_t)S * L * m);
         const char* name = (const void*)X == c.xdata ? "xpass_simt" : "ttm_simt";
         ProfScope ps(c, name, (double)rows * nj * sizeof(Tx) + (double)rows * m * sizeof(Ta), 2.0 * rows * nj * m);
@@ -283,7 +282,7 @@ static void ttm_dispatch(const Ctx& c, const Tx* X, int64_t L, int64_t nj, int64
         c.check_launch();
         return;
     }
-    if (rows * m <= (1 << 21) && nj <= 512) {
+    if (ttm_simt_direct(rows, nj, m)) {
         const char* name = (const void*)X == c.xdata ? "xpass_simt" : "ttm_simt";
         ProfScope ps(c, name, (double)rows * nj * sizeof(Tx) + (double)rows * m * sizeof(Ta), 2.0 * rows * nj * m);
         const int64_t ctas = (rows * m + 255) / 256;

@@ -1,6 +1,7 @@
 // Host side of the TF32 tensor-core TTMs on sm_103a (kernels: tk_ttm_tf32.cuh, tk_ttm_lowp.cuh,
 // tk_expand_tf32.cu): the TF32 split of the factors, the choice of tiles, tensor maps and launches.
 #include <algorithm>
+#include <cmath>
 
 #include "tk_expand_tf32.cuh"
 #include "tk_ttm_lowp.cuh"
@@ -174,27 +175,67 @@ static bool tma_ok(const Tens& X, int j) {
 
 enum class TcRoute { None, Tma, Flat, Lowp };
 
+// The estimated times (us) of a product that both the SIMT kernels and the tensor cores could take, fitted to a sweep
+// over 20 .. 300001 rows, n_j = 2 .. 9001 and m = 3 .. 120 in every data type.
+//  * SIMT: 6.5 us, a CTA per slab: 0.06 to 0.2 us per step of a part, 0.65 products a ps, 1.5 us and 7 ns a step for each
+//    further wave; else n_j steps of 0.1 us, 2.3 products a ps, 1.2 TB/s, and for the tiled kernel 4.4 products a ps
+//    with n_j padded to 16 and m to 32.
+//  * Tensor cores: 14 us on the device with the split of the factor, 7 on the host for its launch, which is what calls
+//    on small tensors wait for; 3 TB/s (expansions 4.5), and for each further wave of tiles 0.035 us a column, or 0.75 us
+//    for each chunk of 32 (0.65 of 64 for BF16 and FP8), and 1.2 us (2.2) where the tile has one chunk only.
+// E.g. 413 x 350 x 275 along its last mode, 36 columns: 1337 us SIMT, 57; 9001 x 333, 20: 78 and 10; 900000 x 2,
+// 26 columns: 104 and 150; 2512 x 48 along the first mode, 5 columns: 15 and 16 in two launches.
+struct TtmTimes {
+    double simt, tc;
+};
+
+static TtmTimes ttm_times(const Tens& X, int j, int64_t m) {
+    const int64_t L = X.left(j), nj = X.n[j], R = X.right(j), rows = L * R;
+    const bool f32 = X.dt == TK_F32;
+    const double work = (double)rows * (double)nj * (double)m;
+    const double bytes = (double)rows * (double)((int64_t)dtype_size(X.dt) * nj + 4 * m);
+    TtmTimes t;
+    if (ttm_simt_slab(L, nj, R, m, 4)) {
+        const double waves = std::ceil((double)R / (8 * 152)) - 1.0, step = 0.06 + 0.0006 * (double)(L * m);
+        t.simt = 6.5 + std::max({step * (double)nj / ttm_simt_slab_parts(L, m), work / 0.65e6, waves * (1.5 + 0.007 * nj)});
+    } else {
+        t.simt = std::max({0.1 * (double)nj, work / 2.3e6, bytes / 1.2e6});
+        if (!ttm_simt_direct(rows, nj, m))
+            t.simt = std::max(t.simt, (double)rows * (double)((nj + 15) / 16 * 16) * (double)((m + 31) / 32 * 32) / 4.4e6);
+    }
+    t.tc = 21.0;
+    const Blocks bl = tc_blocks(L, nj, m, false, X.dt);
+    if (bl.expand) {
+        t.tc += bytes / 4.5e6;
+    } else {
+        const double tiles = (double)((rows + tc::kRows - 1) / tc::kRows) * (double)bl.nblk;
+        const double chunks = (double)(f32 ? (nj + 31) / 32 : (nj + 63) / 64);
+        const double tile = std::max((chunks > 1.0 ? 0.0 : (f32 ? 1.2 : 2.2)) + 0.035 * (double)std::min(m, bl.npad),
+                                     (f32 ? 0.75 : 0.65) * chunks);
+        t.tc += std::max(bytes / 3e6, (std::ceil(tiles / 152.0) - 1.0) * tile);
+    }
+    return t;
+}
+
+static bool tc_faster(const Tens& X, int j, int64_t m) {
+    const TtmTimes t = ttm_times(X, j, m);
+    return t.simt >= t.tc;
+}
+
 // Which form of the tensor-core kernel takes a TTM.
 //  * TMA: 16-byte strides, n_j >= 32, and rows enough to fill tiles: L == 1 with R >= 128, or L >= 32 (below
 //    64 by packing slabs).
-//  * everything else the SIMT kernels could take as well: the tensor cores where they are the faster
-//    ones by the times below (us), fitted to a sweep over 1000 .. 300001 rows, n_j = 7 .. 333 and
-//    m = 5 .. 45.  The SIMT kernels walk n_j in one thread (0.1 us a step), reach 2300 products a ns and
-//    1.2 TB/s; the tensor cores need two launches (14 us with the split of the factor, and as much again
-//    on the host, which is what calls on small tensors wait for) and stream 3 TB/s.
-//    E.g. 413 x 350 x 275 along its last mode, 36 columns: 1337 us SIMT; 9001 x 333, 20: 78.
+//  * everything else the SIMT kernels could take as well: the tensor cores where they are the faster ones.
 //  * BF16 and FP8 that their own kernels do not take: the same rule, for L == 1 or L >= 32 (shorter runs
 //    cost more in their 16-byte pieces than they hold).  E.g. BF16 689 x 690 x 700 along its first mode, 10 columns:
-//    3435 us SIMT, 176; FP8 768^3 along its last, 9: 1541 and 171.
+//    3435 us SIMT, 178; FP8 768^3 along its last, 9: 1541 and 176.
 static TcRoute lowp_route(const Tens& X, int j, int64_t m) {
-    const int64_t L = X.left(j), nj = X.n[j], R = X.right(j), es = (int64_t)dtype_size(X.dt);
+    const int64_t L = X.left(j), nj = X.n[j], R = X.right(j);
     if (ttm_bf16_eligible(X, j, m, TK_F32) || ttm_fp8_eligible(X, j, m, TK_F32)) return TcRoute::None;
     if (nj < 1 || ((uintptr_t)X.p % 16) != 0 || nj >= ((int64_t)1 << 31) || (L != 1 && L < 32)) return TcRoute::None;
     const int64_t rows = L * R;
     if (rows < 1 || rows >= ((int64_t)1 << 31) - tc::kRows) return TcRoute::None;
-    const double bytes = (double)rows * (double)(es * nj + 4 * m);
-    const double simt = std::max({0.1 * (double)nj, (double)rows * (double)nj * (double)m / 2.3e6, bytes / 1.2e6});
-    return simt < 28.0 + bytes / 3e6 ? TcRoute::None : TcRoute::Lowp;
+    return tc_faster(X, j, m) ? TcRoute::Lowp : TcRoute::None;
 }
 
 static TcRoute tc_route(const Tens& X, int j, int64_t m, tk_dtype out_dt) {
@@ -209,9 +250,7 @@ static TcRoute tc_route(const Tens& X, int j, int64_t m, tk_dtype out_dt) {
     if (rows < 1 || rows >= ((int64_t)1 << 31) - tc::kRows) return TcRoute::None;
     // streams of 4 million elements and more with 16-byte strides: HBM-bound at 2-3 times the SIMT rate
     if (rows * nj >= ((int64_t)1 << 22) && tma_ok(X, j)) return tma ? TcRoute::Tma : TcRoute::Flat;
-    const double bytes = 4.0 * (double)rows * (double)(nj + m);
-    const double simt = std::max({0.1 * (double)nj, (double)rows * (double)nj * (double)m / 2.3e6, bytes / 1.2e6});
-    if (simt < 28.0 + bytes / 3e6) return TcRoute::None;
+    if (!tc_faster(X, j, m)) return TcRoute::None;
     return tma ? TcRoute::Tma : TcRoute::Flat;
 }
 

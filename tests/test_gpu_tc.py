@@ -273,11 +273,39 @@ def test_reconstruct_expansions(dev, dims, rk):
     g = _rng(24)
     G = synth.round_to(g.standard_normal(rk), "f32")
     U = [synth.round_to(g.standard_normal((n, k)) / np.sqrt(n), "f32") for n, k in zip(dims, rk)]
+    T.tk_profile(True, dev)
     Xh = T.tucker_reconstruct(synth.fortran(G, "f32", dev), mats(U, "f32", dev))
+    prof = T.tk_profile_read(dev)
+    T.tk_profile(False, dev)
+    assert prof["ttm_tc"]["launches"] >= 1
     assert rel(to_np(Xh), O.reconstruct(G, U)) <= len(dims) * 2e-6
     st, _ = T.tk_sync_status(dev)
     assert st == 0
 
+
+@pytest.mark.parametrize("dims,r,dtype,want", [
+    # X's pass to (r_1, all else): a product of few rows and steps takes one SIMT launch, not a split and a tensor-core one
+    ((2512, 48), (5, 34), "f32", "xpass_simt"),  # 15 us against 16 in two launches, and their 7 on the host
+    ((889, 16, 21), (3, 4, 4), "f32", "xpass_simt"),  # 12, 16
+    ((9001, 333), (20, 9), "f32", "xpass_tc"),  # long contractions: 78, 10
+    ((333, 9001), (20, 9), "f32", "xpass_tc"),
+    ((413, 35, 275), (36, 4, 4), "f32", "xpass_tc"),
+    ((1030, 97), (8, 4), "fp8", "xpass_simt"),
+    ((203, 690, 70), (20, 4, 4), "fp8", "xpass_tc"),
+])
+def test_first_product_takes_the_faster_kernel(dev, dims, r, dtype, want):
+    g = _rng(41)
+    X, xv, xs = make_X(g.standard_normal(dims), dtype, dev)
+    U = [synth.round_to(g.standard_normal((n, k)) / np.sqrt(n), "f32") for n, k in zip(dims, r)]
+    T.tk_profile(True, dev)
+    G = T.tucker_core(X, mats(U, "f32", dev), scale=xs)
+    prof = T.tk_profile_read(dev)
+    T.tk_profile(False, dev)
+    assert [k for k in ("xpass_tc", "xpass_simt") if k in prof] == [want], prof
+    ref = xv
+    for j, u in enumerate(U):
+        ref = O.ttm(ref, u.T, j)
+    assert rel(to_np(G), ref) <= len(dims) * 2e-6
 
 @pytest.mark.parametrize("rows", [4096, 4099])
 @pytest.mark.parametrize("K", [1, 3, 4, 5, 8, 9, 12, 13, 16, 24, 32])

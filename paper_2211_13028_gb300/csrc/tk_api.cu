@@ -567,23 +567,32 @@ static void truncate_modes(Ctx& c, const Tens& G0, Tens& G, const int64_t* r, co
     }
 }
 
-// Which of the modes in `todo` a reconstruction expands next (its index in todo): the one that grows the tensor
-// least, but on tensor cores the leading mode first of all: its product has contiguous output rows per
-// tile row, which the kernels write at 1.4-2 TB/s against 5 TB/s along the other modes (reconstruction of
-// 160^4 from 10 x 20 x 30 x 40: 1.75 ms with the leading mode last, 0.68 ms with it first).
-static size_t next_expansion(const std::vector<int>& todo, const std::vector<Mat>& U, bool tc) {
-    size_t best = 0;
-    double bestr = 1e300;
-    for (size_t t = 0; t < todo.size(); ++t) {
-        const int i = todo[t];
-        if (tc && i == 0) return t;
-        const double ratio = (double)U[i].rows / std::max<double>(1.0, (double)U[i].cols);
-        if (ratio < bestr) {
-            bestr = ratio;
-            best = t;
+// The order in which a reconstruction expands the modes of `modes`: those that grow the tensor least first.  FP32:
+// or the leading mode before all others, where the estimated times of the products say so: its product has
+// contiguous output rows per tile row, which the tensor-core kernel writes at 1.4-2 TB/s against 5 TB/s along the
+// other modes (160^4 from 10 x 20 x 30 x 40: 1.75 ms with the leading mode last, 0.68 ms with it first), but
+// the others then start from a larger tensor (81 x 26 x 31 x 27 x 19 from 2 x 2 x 9 x 7 x 2: 178 us last, 251 first).
+static std::vector<int> expansion_order(const Tens& G, std::vector<int> modes, const std::vector<Mat>& U, tk_dtype acc,
+                                        bool use_tc) {
+    auto growth = [&](int j) { return (double)U[j].rows / std::max<double>(1.0, (double)U[j].cols); };
+    std::stable_sort(modes.begin(), modes.end(), [&](int a, int b) { return growth(a) < growth(b); });
+    if (acc != TK_F32 || modes.empty() || modes[0] == 0) return modes;
+    auto time = [&](const std::vector<int>& order) {
+        Tens cur = G;
+        double t = 0.0;
+        for (int j : order) {
+            cur.dt = acc;
+            cur.p = reinterpret_cast<void*>(uintptr_t(256));  // a workspace block: 256-byte aligned
+            t += ttm_estimate(cur, j, U[j].rows, use_tc);
+            cur.n[j] = U[j].rows;
         }
-    }
-    return best;
+        return t;
+    };
+    std::vector<int> leading = modes;
+    const auto at = std::find(leading.begin(), leading.end(), 0);
+    if (at == leading.end()) return modes;
+    std::rotate(leading.begin(), at, at + 1);
+    return time(leading) < time(modes) ? leading : modes;
 }
 
 // ||X - G x_1 U_1 ... x_d U_d||^2 and ||X||^2 into err2 (device, 2 doubles); with
@@ -595,14 +604,10 @@ static void residual_pass(Ctx& c, const Tens& X, const Tens& G, const std::vecto
                           double* err2, void* dx, tk_dtype dxdt, double alpha) {
     const int d = X.d;
     int f = d - 1;
-    std::vector<int> todo, order;
+    std::vector<int> others;
     for (int j = 0; j < d; ++j)
-        if (j != f) todo.push_back(j);
-    while (!todo.empty()) {
-        const size_t best = next_expansion(todo, U, c.use_tc && acc == TK_F32);
-        order.push_back(todo[best]);
-        todo.erase(todo.begin() + best);
-    }
+        if (j != f) others.push_back(j);
+    const std::vector<int> order = expansion_order(G, others, U, acc, c.use_tc);
     const int64_t m = U[f].rows;
     // BF16 data: the epilogue reads the BF16 X tile (and writes a BF16 dX) itself; FP8 data: the E4M3 X
     // tile, scaled back by 1 / scale (norms only, no dX)
@@ -1876,15 +1881,11 @@ static Tens reconstruct_acc(Ctx& c, const Tens& Gt, const std::vector<Mat>& Um, 
     Tens Ga = Gt.dt == acc ? Gt : tens_to(c, Gt, acc);
     std::vector<Mat> Ua(d);
     for (int j = 0; j < d; ++j) Ua[j] = Um[j].dt == acc ? Um[j] : mat_to(c, Um[j], acc);
-    std::vector<int> todo(d);
-    std::iota(todo.begin(), todo.end(), 0);
+    std::vector<int> modes(d);
+    std::iota(modes.begin(), modes.end(), 0);
+    modes = expansion_order(Ga, modes, Ua, acc, c.use_tc);
     Tens cur = Ga;
-    while (!todo.empty()) {
-        const size_t best = next_expansion(todo, Ua, c.use_tc && acc == TK_F32);
-        int i = todo[best];
-        todo.erase(todo.begin() + best);
-        cur = ttm_to(c, cur, i, Ua[i], true, acc, todo.empty() ? dst : nullptr);
-    }
+    for (int i : modes) cur = ttm_to(c, cur, i, Ua[i], true, acc, i == modes.back() ? dst : nullptr);
     return cur;
 }
 

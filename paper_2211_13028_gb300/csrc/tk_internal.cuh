@@ -376,6 +376,8 @@ inline bool ttm_simt_direct(int64_t rows, int64_t nj, int64_t m) { return rows *
 // in the layouts that launch_ttm_bf16 / launch_ttm_fp8 do not take.  ttm_tc_eligible says whether a TTM
 // takes it (dtype, and the sizes where it is faster).
 bool ttm_tc_eligible(const Tens& X, int j, int64_t m, tk_dtype out_dt);
+// What a product of FP32 data takes on the kernel that gets it (us, roughly; the rule of ttm_tc_eligible).
+double ttm_estimate(const Tens& X, int j, int64_t m, bool use_tc);
 // A factor a tensor-core TTM will split (the rows L before the contracted mode,
 // its size nj, output width m; residual: the fused-residual blocking; dt: the data's type).
 struct TcSplitReq {

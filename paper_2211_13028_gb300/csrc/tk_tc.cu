@@ -258,6 +258,14 @@ bool ttm_tc_eligible(const Tens& X, int j, int64_t m, tk_dtype out_dt) {
     return tc_route(X, j, m, out_dt) != TcRoute::None;
 }
 
+double ttm_estimate(const Tens& X, int j, int64_t m, bool use_tc) {
+    const TtmTimes t = ttm_times(X, j, m);
+    if (!use_tc || !ttm_tc_eligible(X, j, m, TK_F32)) return t.simt + 5.0;
+    // the device's part; a tile row's outputs are contiguous along the leading mode: 0.9 (192 columns from 9) to 1.7 TB/s
+    const double tc = t.tc - 7.0;
+    return X.left(j) == 1 ? std::max(tc, 14.0 + 4.0 * (double)X.right(j) * (double)m / 1e6) : tc;
+}
+
 // The TF32 parts of factor M in the layout the kernels load, from the call's split cache or made here.
 struct Factor {
     float* hi = nullptr;

@@ -283,6 +283,28 @@ def test_reconstruct_expansions(dev, dims, rk):
     assert st == 0
 
 
+@pytest.mark.parametrize("dims,rk,order", [
+    ((81, 26, 31, 27, 19), (2, 2, 9, 7, 2), (2, 3, 4, 1, 0)),  # smallest growth first: 178 us, the leading mode first 251
+    ((94, 7, 189, 34), (3, 4, 80, 5), (1, 2, 3, 0)),  # 45, 63
+    ((384, 160, 160), (16, 16, 16), (0, 1, 2)),  # the leading mode's scattered outputs are the smaller then
+    ((160, 40, 40, 40), (4, 10, 10, 10), (1, 2, 3, 0)),  # 61, 90
+])
+def test_reconstruct_expands_in_the_faster_order(dev, dims, rk, order):
+    g = _rng(25)
+    G = synth.round_to(g.standard_normal(rk), "f32")
+    U = [synth.round_to(g.standard_normal((n, k)) / np.sqrt(n), "f32") for n, k in zip(dims, rk)]
+    T.tk_profile(True, dev)
+    Xh = T.tucker_reconstruct(synth.fortran(G, "f32", dev), mats(U, "f32", dev))
+    prof = T.tk_profile_read(dev)
+    T.tk_profile(False, dev)
+    flops, sh = 0.0, list(rk)
+    for j in order:
+        sh[j] = dims[j]
+        flops += 2.0 * np.prod(sh) * rk[j]
+    assert sum(v["flops"] for v in prof.values()) == flops, prof
+    assert rel(to_np(Xh), O.reconstruct(G, U)) <= len(dims) * 2e-6
+
+
 @pytest.mark.parametrize("dims,r,dtype,want", [
     # X's pass to (r_1, all else): a product of few rows and steps takes one SIMT launch, not a split and a tensor-core one
     ((2512, 48), (5, 34), "f32", "xpass_simt"),  # 15 us against 16 in two launches, and their 7 on the host

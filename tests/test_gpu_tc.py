@@ -261,15 +261,22 @@ def test_fused_residual_sizes_and_alignment(dev, dims, rk, dtype):
     assert st == 0
 
 
-@pytest.mark.parametrize("dims,rk", [
-    ((201, 187, 211), (20, 24, 30)),  # odd rows, K = 30, last block of 19 columns
-    ((202, 188, 260), (20, 24, 60)),  # K = 60: two chunks
-    ((160, 130, 70, 40), (5, 6, 7, 8)),  # 4-way: the last expansion has slabs after it or none
-    ((300, 500, 256), (10, 20, 12)),  # mode 2 grows most: last, with the others before it
+@pytest.mark.parametrize("dims,rk,order,tc", [
+    # the order of the modes' products, and those on tensor cores; the last is an expansion
+    ((201, 187, 211), (20, 24, 30), (0, 2, 1), (1,)),  # odd rows, slabs after it
+    ((202, 188, 260), (20, 24, 60), (0, 2, 1), (2, 1)),  # two expansions
+    ((160, 130, 70, 40), (5, 6, 7, 8), (0, 3, 2, 1), (1,)),  # 4-way
+    ((300, 500, 256), (10, 20, 12), (0, 2, 1), (1,)),
+    ((201, 187, 211), (40, 40, 30), (1, 0, 2), (1, 0, 2)),  # no slabs after it: K = 30, last block of 19 columns
+    ((202, 188, 260), (60, 56, 60), (0, 1, 2), (0, 1, 2)),  # K = 60: two chunks
+    ((300, 500, 256), (30, 60, 12), (0, 1, 2), (1, 2)),
+    ((160, 60, 70, 130), (16, 12, 14, 6), (0, 1, 2, 3), (3,)),
 ])
-def test_reconstruct_expansions(dev, dims, rk):
-    # a reconstruction whose last products take the expansion kernel.  Bound as test_tc_any_size_and_alignment,
-    # once per product
+def test_reconstruct_expansions(dev, dims, rk, order, tc):
+    # a reconstruction whose last product takes the expansion kernel (a short contraction into more columns, rows enough
+    # before it).  Bound as test_tc_any_size_and_alignment, once per product
+    last = order[-1]
+    assert np.prod(dims[:last]) >= 32 and rk[last] <= 64 <= dims[last] and 2 * rk[last] <= dims[last]
     g = _rng(24)
     G = synth.round_to(g.standard_normal(rk), "f32")
     U = [synth.round_to(g.standard_normal((n, k)) / np.sqrt(n), "f32") for n, k in zip(dims, rk)]
@@ -277,7 +284,11 @@ def test_reconstruct_expansions(dev, dims, rk):
     Xh = T.tucker_reconstruct(synth.fortran(G, "f32", dev), mats(U, "f32", dev))
     prof = T.tk_profile_read(dev)
     T.tk_profile(False, dev)
-    assert prof["ttm_tc"]["launches"] >= 1
+    sh, flops = list(rk), 0.0
+    for j in order:
+        sh[j] = dims[j]
+        flops += 2.0 * np.prod(sh) * rk[j] if j in tc else 0.0
+    assert prof["ttm_tc"]["flops"] == flops, prof
     assert rel(to_np(Xh), O.reconstruct(G, U)) <= len(dims) * 2e-6
     st, _ = T.tk_sync_status(dev)
     assert st == 0

@@ -183,7 +183,8 @@ TK_API int64_t tk_launch_count(const tk_handle* h);
  * classes; the filter persists until changed).  Class names ("xpass_*": a
  * pass over the whole data tensor): "xpass_tc", "xpass_tc_bg" (a tensor-core
  * pass on part of the SMs, beside a chain of small kernels of the same call),
- * "xpass_narrow" (the streaming pass of a Kronecker-SRHT sketch), "xpass_simt", "ttm_tc", "ttm_simt",
+ * "xpass_narrow" (the streaming pass of a Kronecker-SRHT sketch), "xpass_simt" (among
+ * them the fused residual of a short contraction of FP32 data), "ttm_tc", "ttm_simt",
  * "gemm_f64", "gemm_df", "chol_inv", "apply_rinv", "householder", "jacobi",
  * "residual", "elementwise", "rng". */
 typedef struct {

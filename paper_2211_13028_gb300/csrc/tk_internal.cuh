@@ -532,9 +532,6 @@ void launch_jacobi_mixed(Ctx& c, int64_t k, const double* A, double* D, float* J
 // (With V1: the rotations are replayed on the rows of V1, giving V = V1 J
 // without forming J, and the columns of V of the r largest eigenvalue
 // estimates, in descending order, go to Vt and Vr (k x r, ld k).)
-// Vr (k x r, ld k) = the columns of V (k x k) for the r largest entries of D, in descending order.
-void launch_select_top(const Ctx& c, int64_t k, int64_t r, const double* D, const double* V, double* Vr,
-                       double* Vr2 = nullptr);
 
 // Thin QR of the plain matrix y (rows x cols) into q (rows x min(rows, cols)):
 // CholeskyQR2 with the Householder fallback, identity when cols >= rows; the
@@ -555,9 +552,6 @@ struct ConvertJob {
 };
 void launch_convert(const Ctx& c, const std::vector<ConvertJob>& jobs);
 void launch_fill_identity(const Ctx& c, double* Q, int64_t n);
-// A (n x k, FP64, ld n) = Y; only when *run != 0 (run may be NULL = always).
-void launch_copy_unfold_to_matrix(const Ctx& c, const View2& Y, int64_t n, int64_t k, double* A,
-                                  const int* run = nullptr);
 void launch_fill_int(const Ctx& c, int* p, int count, int value);
 // *slot = *bad ? bad_value : 0
 void launch_qr_info(const Ctx& c, int* slot, const int* bad, int bad_value);

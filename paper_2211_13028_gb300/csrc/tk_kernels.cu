@@ -532,10 +532,6 @@ __device__ __forceinline__ void df_dot_step(float& s, float& c, float2 a, float2
     c = __fadd_rn(c, __fadd_rn(q, e));
 }
 
-// MODE 0: FP64 fma.  MODE 1: both operands hold FP32 values (FP32 data), and
-// the products are
-// accumulated on the FP32 pipe with Dot2 (as accurate as about 48 significant
-// bits, several times the FP64 rate here); otherwise FP64 fma.
 // out[l + L (a + m r)] = sum_i M(i, a) X[l + L (i + nj r)], NA columns a per thread,
 // FP64 operands split into double-float pairs (M staged split in shared
 // memory), Dot2 accumulation: the FP64 pipe here is 1/64 of the FP32 pipe.  A split costs as much as two
@@ -628,6 +624,8 @@ struct GemmItems {
     GemmItem job[NB];
 };
 
+// MODE 0: FP64 fma.  MODE 1: both operands hold FP32 values, the products accumulate on the FP32 pipe with Dot2
+// (about 48 significant bits, several times the FP64 rate here).
 // MODE 2: the operands (FP64 or FP32) are split into double-float pairs on
 // load and the products accumulate with df_dot_step on the FP32 pipe (~47
 // significant bits; FP32's exponent range bounds the products).
@@ -929,7 +927,8 @@ static void gemm_run(const Ctx& c, const std::vector<GemmPlan>& p) {
 }
 
 // Products that run on the same kernel share a launch (the Grams of the modes of a 512^3 tensor's factors, on
-// three streams before: orthonormalisation 132 -> 119 us); every product is computed as it would be alone.
+// three streams before: orthonormalisation 132 -> 119 us).  The tile is one for all but the small ones: 32 x 32 where each
+// of them would take it alone, so a product's split of K, and with it the order of its sums, depends on its batch.
 void gemm_nt_f64(Ctx& c, const std::vector<GemmJob>& jobs) {
     std::vector<GemmPlan> plans;
     bool t32 = true;
@@ -2326,34 +2325,6 @@ void launch_jacobi_mixed(Ctx& c, int64_t k, const double* A, double* D, float* J
     c.check_launch();
 }
 
-// Vr[:, rank] = V[:, i] for the r largest D (ties: lower index first).
-__global__ void select_top_kernel(int64_t k, int64_t r, const double* D, const double* V, double* Vr, double* Vr2) {
-    kernel_begin();
-    for (int64_t i = blockIdx.x; i < k; i += gridDim.x) {
-        double di = D[i];
-        int64_t rank = 0;
-        for (int64_t j = 0; j < k; ++j) {
-            double dj = D[j];
-            rank += (dj > di) || (dj == di && j < i);
-        }
-        if (rank >= r) continue;
-        for (int64_t row = threadIdx.x; row < k; row += blockDim.x) {
-            const double v = V[row + k * i];
-            Vr[row + k * rank] = v;
-            if (Vr2) Vr2[row + k * rank] = v;
-        }
-    }
-}
-
-void launch_select_top(const Ctx& c, int64_t k, int64_t r, const double* D, const double* V, double* Vr,
-                       double* Vr2) {
-    if (!c.exec || k == 0 || r == 0) return;
-    ProfScope ps(c, "elementwise", 16.0 * k * r, 0.0);
-    run_kernel(c, select_top_kernel, (unsigned)k, 64, 0, k, r, D, V, Vr, Vr2);
-    c.counted();
-    c.check_launch();
-}
-
 // ------------------------------------------------------------------ element-wise helpers
 
 // The copies of one launch (blockIdx.y).
@@ -2419,22 +2390,6 @@ void launch_fill_identity(const Ctx& c, double* Q, int64_t n) {
     if (!c.exec || n == 0) return;
     ProfScope ps(c, "elementwise", 8.0 * n * n, 0.0);
     run_kernel(c, fill_identity_kernel, (unsigned)((n * n + 255) / 256), 256, 0, Q, n);
-    c.counted();
-    c.check_launch();
-}
-
-__global__ void copy_unfold_kernel(View2 Y, int64_t n, int64_t k, double* A, const int* run) {
-    kernel_begin();
-    if (run && !*run) return;
-    int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= n * k) return;
-    A[idx] = v2ld(Y, idx % n, idx / n);
-}
-
-void launch_copy_unfold_to_matrix(const Ctx& c, const View2& Y, int64_t n, int64_t k, double* A, const int* run) {
-    if (!c.exec || n * k == 0) return;
-    ProfScope ps(c, "elementwise", 16.0 * n * k, 0.0);
-    run_kernel(c, copy_unfold_kernel, (unsigned)((n * k + 255) / 256), 256, 0, Y, n, k, A, run);
     c.counted();
     c.check_launch();
 }

@@ -22,9 +22,9 @@ constexpr int64_t kColsMax = 64;
 // CholeskyQR2 + Householder scratch at that size, as the planning pass counts
 // it: three rows x cols FP64 matrices (Q, the first CholeskyQR factor, the
 // Householder copy: 6 MiB), the split-K partial tiles of the two Gram
-// products (32 slices of three 32 x 32 FP64 tiles each at 4096 rows: 1.6 MB), two
+// products (26 slices of ten 16 x 16 FP64 tiles each at 4096 rows: 1.1 MB), two
 // cols x cols FP64 matrices, the flag header and 256-byte alignment of every
-// block: 8.0 MB of the 8.4 MB (8 MiB) here.
+// block: 7.4 MB of the 8.4 MB (8 MiB) here.
 constexpr size_t kScratchBytes = 8u << 20;
 
 // Shared by every call on a device and kept between calls.

@@ -15,8 +15,8 @@
 //               cover it, into a slot of its own, and the converters read at the run's offset in its slot.
 //               That offset is the same for every chunk, as 64 steps of any stride are a multiple of 16 bytes.
 //   converters  (two groups of 8 warps, alternate chunks) widen the chunk to FP32 and write it to TMEM, A's place.
-//   epilogue    (8 warps): each chunk's accumulator is added in FP32 registers, rounding to nearest (the tensor
-//               core's own additions round toward zero), rows written to global memory.
+//   epilogue    (8 warps, up to 16 columns 4): each chunk's accumulator is added in FP32 registers, rounding to
+//               nearest (the tensor core's own additions round toward zero), rows written to global memory.
 // 64 steps a chunk rather than 32 because a chunk of FP8 is little to load: 176 cycles of the SM's share of HBM
 // at 32, less than a chunk takes.  Instruction issue still bounds it at 64 (ncu: 74% of the slots; a chunk takes
 // 900 to 1400 cycles whether X is loaded or not, and its share of HBM is 350 for FP8, 700 for BF16).  SIMT and this

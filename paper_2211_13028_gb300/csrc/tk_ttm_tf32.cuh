@@ -15,7 +15,8 @@
 //               from SMEM, split them into TF32 hi / lo and write them to TMEM with tcgen05.st.  The
 //               MMA reads A from TMEM, so X is read from SMEM exactly once, and a contraction over a
 //               non-contiguous mode needs no transpose: only the element each lane reads differs.
-//   epilogue    (8 warps, two per TMEM lane quarter): tcgen05.ld, sums, rows written to global memory.
+//   epilogue    (8 warps, two per TMEM lane quarter; up to 16 columns 4): tcgen05.ld, sums, rows written to global
+//               memory.
 // The issuing threads are chosen by elect.sync (tk_tc_common.cuh), so that neither the MMAs (288 of
 // the 700 cycles that HBM gives a chunk at NPAD = 48) nor their issue bounds the pass.
 //
@@ -114,8 +115,9 @@ __device__ __forceinline__ void residual_sums(int e, int lane, double sr, double
 }
 
 // What a kernel has to know of the factor besides its parts, written beside them by the kernel that splits it (in
-// memory: the kernels' arguments have no room for it, see TtmResArgs): the factor as the caller gave it, M(i, a) = M[i + ldm a], or M[a + ldm i] with mtrans (dt: F32
-// or F64), and a flag of each block that split it, set when a part is infinite or NaN.
+// memory: the kernels' arguments have no room for it, see TtmResArgs): the factor as the caller gave it, M(i, a) =
+// M[i + ldm a], or M[a + ldm i] with mtrans (dt: F32 or F64), and a flag of each block that split it, set when a part
+// is infinite or NaN.
 struct FactorInfo {
     const void* M;
     int64_t ldm;

@@ -2634,27 +2634,39 @@ void launch_residual_norms(Ctx& c, const Tens& X, const void* Y, tk_dtype ydt, d
 // with FP32 FMAs, every addition rounded to nearest, and compared: per-CTA sums of (x - P)^2 and x^2, and with DX also
 // dx = alpha (x - P).  The tensor cores' additions round toward zero, which at so few terms is most of the error (dX
 // of 400 x 120 x 64, ranks 3, 4, 5: 1.14e-6 from 64 bits, 8.5e-7 so).  A thread keeps four rows of W in registers and
-// meets every column of M, staged in shared memory, with all of them.  512^3, K = 8: 120 us, 189 with dx (tensor
-// cores 92 and 184; X alone takes 79 and 158); K = 16 would take 150 and 209, where two accumulators do as well.
+// meets every column of M, staged in shared memory, with all of them.  512^3, K = 8: 120 us, 181 with dx (tensor
+// cores 92 and 184; X alone takes 79 and 158); K = 16 would take 150 and 209, where two accumulators do as well.  The
+// CTAs take equal shares of the columns of all row tiles, as many CTAs as the registers hold at once: whole blocks of
+// 128 columns in turn left most of them idle in the last wave (10000 x 400, K = 9: 24 us, 14 so; 413 x 350 x 275,
+// K = 7: 50, 45).
 constexpr int RF_THREADS = 256;
 constexpr int RF_RPT = 4;  // rows a thread: each column read from shared memory serves all of them
 constexpr int RF_ROWS = RF_RPT * RF_THREADS;
-constexpr int RF_COLS = 128;
+constexpr int RF_COLS = 128;  // columns of M staged at a time
+constexpr int RF_U = 8;       // columns whose loads are in flight together: the unit that the CTAs share out
+
+// CTAs an SM: what the registers hold.
+constexpr int rf_ctas(int64_t K) { return K <= 4 ? 3 : 2; }
 
 template <int KP, bool DX>
-__global__ void __launch_bounds__(RF_THREADS) residual_fma_kernel(const float* __restrict__ W, int64_t L, int K,
+__global__ void __launch_bounds__(RF_THREADS, rf_ctas(KP)) residual_fma_kernel(const float* __restrict__ W, int64_t L, int K,
                                                                   const float* __restrict__ M, int64_t ldm, int mtrans,
                                                                   int64_t m, const float* __restrict__ X, float* dx,
-                                                                  float alpha, int64_t nblk, int64_t items, double* part) {
+                                                                  float alpha, int64_t upt, int64_t units, double* part) {
     kernel_begin();
     __shared__ __align__(16) float us[RF_COLS][KP];
     __shared__ double red[2 * RF_THREADS / 32];
     const int tid = threadIdx.x;
     float h[2] = {0.f, 0.f}, l[2] = {0.f, 0.f};  // running sums as double-float pairs: (x - P)^2, x^2
-    for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
-        const int64_t r0 = it / nblk * RF_ROWS, a0 = it % nblk * RF_COLS;
-        const int na = (int)(m - a0 < RF_COLS ? m - a0 : RF_COLS);
-        __syncthreads();  // the columns of the item before have been used
+    // this CTA's share of the tiles' column units, in order; a piece lies in one tile and fits the staged columns
+    const int64_t end = units * (blockIdx.x + 1) / gridDim.x;
+    for (int64_t at = units * blockIdx.x / gridDim.x; at < end;) {
+        const int64_t tile = at / upt, u0 = at - tile * upt, left = end - at < upt - u0 ? end - at : upt - u0;
+        const int64_t take = left < RF_COLS / RF_U ? left : RF_COLS / RF_U;
+        at += take;
+        const int64_t r0 = tile * RF_ROWS, a0 = u0 * RF_U;
+        const int na = (int)(m - a0 < take * RF_U ? m - a0 : take * RF_U);
+        __syncthreads();  // the columns of the piece before have been used
         for (int e = tid; e < KP * RF_COLS; e += RF_THREADS) {
             const int a = e % RF_COLS, i = e / RF_COLS;
             us[a][i] = i < K && a < na ? (mtrans ? M[a0 + a + ldm * i] : M[i + ldm * (a0 + a)]) : 0.f;
@@ -2671,7 +2683,7 @@ __global__ void __launch_bounds__(RF_THREADS) residual_fma_kernel(const float* _
         __syncthreads();
         const float* x = X + r0 + tid + L * a0;
         float* d = dx + r0 + tid + L * a0;
-        constexpr int U = 8;  // columns whose loads are in flight together
+        constexpr int U = RF_U;
         for (int c = 0; c < na; c += U) {
             float v[RF_RPT][U];
 #pragma unroll
@@ -2727,12 +2739,13 @@ bool residual_fma_eligible(const Tens& W, int j, int64_t m) {
     return W.dt == TK_F32 && W.right(j) == 1 && W.n[j] >= 1 && W.n[j] <= 12 && W.left(j) >= 1 && m >= 1;
 }
 
-static int64_t residual_fma_items(const Tens& W, int j, int64_t m) {
-    return (W.left(j) + RF_ROWS - 1) / RF_ROWS * ((m + RF_COLS - 1) / RF_COLS);
+// Row tiles x units of RF_U columns.
+static int64_t residual_fma_units(const Tens& W, int j, int64_t m) {
+    return (W.left(j) + RF_ROWS - 1) / RF_ROWS * ((m + RF_U - 1) / RF_U);
 }
 
 int residual_fma_ctas(const Ctx& c, const Tens& W, int j, int64_t m) {
-    return (int)std::min<int64_t>(residual_fma_items(W, j, m), 4 * tc::grid_sms(c));
+    return (int)std::min<int64_t>(residual_fma_units(W, j, m), rf_ctas(W.n[j]) * tc::grid_sms(c));
 }
 
 void launch_residual_fma(const Ctx& c, const Tens& W, int j, const Mat& M, bool mtrans, int64_t m, const float* xref,
@@ -2747,8 +2760,8 @@ void launch_residual_fma(const Ctx& c, const Tens& W, int j, const Mat& M, bool 
                          : (K <= 4 ? residual_fma_kernel<4, false>
                                    : (K <= 8 ? residual_fma_kernel<8, false> : residual_fma_kernel<12, false>));
     run_kernel(c, kern, (unsigned)residual_fma_ctas(c, W, j, m), RF_THREADS, 0, (const float*)W.p, L, (int)K,
-               (const float*)M.p, M.ld, mtrans ? 1 : 0, m, xref, dx, alpha, (m + RF_COLS - 1) / RF_COLS,
-               residual_fma_items(W, j, m), partials);
+               (const float*)M.p, M.ld, mtrans ? 1 : 0, m, xref, dx, alpha, (m + RF_U - 1) / RF_U,
+               residual_fma_units(W, j, m), partials);
     c.counted();
     c.check_launch();
 }

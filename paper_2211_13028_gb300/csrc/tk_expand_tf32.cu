@@ -8,7 +8,7 @@
 // runs over the tile's blocks of output columns, streaming the factor's columns and X's tiles.  The
 // general kernel's order, a tile of W loaded and converted again for every block of 64 columns, bounds
 // such passes (both measured with the same issue and split code): fused residual 1024^3 BF16, K = 64:
-// 1327 -> 664 us; 160^4 FP32, K = 40: 983 -> 717; 512^3 FP32, K = 32: 117 -> 102 (5.6 TB/s); plain 512^3,
+// 1327 -> 664 us; 160^4 FP32, K = 40: 983 -> 743; 512^3 FP32, K = 64: 123 (5.3 TB/s); plain 512^3,
 // K = 32: 262 -> 103.  What is left at K = 64 are the MMAs (345 us of tensor time at N = 32) and the
 // wait for a new tile of W, whose one buffer the last blocks still read.
 //
@@ -19,8 +19,8 @@
 //                accumulator.  The tensor core rounds each addition toward zero: in this order only
 //                the K / 8 last ones round at the size of the result.  Plain products, and the comparison of FP32
 //                data at K <= 32, keep the even and the odd steps apart, half as many each: dX of 256^3, ranks 16,
-//                1.72e-6 -> 1.62e-6 from 64 bits (FP32 FMAs 1.62e-6; its pass 42 -> 45 us, the norms alone 37 -> 39;
-//                512^3, ranks 32, 186 -> 207 and 102 -> 122).  BF16 data, whose rounding is far larger, do not.
+//                1.72e-6 -> 1.62e-6 from 64 bits (FP32 FMAs 1.62e-6); 512^3, ranks 32, with dX 186 -> 201 us, the norms
+//                alone 102 -> 117.  BF16 data, whose rounding is far larger, do not.
 //   warps 2, 3   X's tiles: one thread by TMA, or, where X's columns have no 16-byte stride (`bulk`), two
 //                by one bulk copy per column, widened to 16-byte bounds (half of the columns each).
 //   warps 4-11   converters: W from global memory (any alignment; rows L*R numbered without regard to

@@ -513,8 +513,9 @@ void launch_ttm_tc(Ctx& c, const Tens& X, int j, const Mat& M, bool mtrans, int6
 }
 
 // Fused residuals of a contraction longer than the expansion kernel holds run on the plain kernel, whose epilogue then
-// compares instead of storing (512^3 FP32, K = 160: norms 668 us, with dX 753; stored and compared by kernels of their
-// own 671 and 1200 us, and Xhat's 512 MB of workspace).
+// compares instead of storing (512^3 FP32, K = 160: norms 573 us, with dX 653; stored and compared by kernels of their
+// own 672 and 1206 us, and Xhat's 512 MB of workspace.  BF16 1024 x 1024 x 512, K = 192, where the MMAs bound it: 2754
+// and 2586, with 2 GB).
 static bool residual_plain(int64_t nj) { return nj > tc::kExpandKResid; }
 
 bool ttm_tc_residual_eligible(const Tens& W, int j, int64_t m) {

@@ -18,10 +18,11 @@
 //   epilogue    (8 warps, up to 16 columns 4): each chunk's accumulator is added in FP32 registers, rounding to
 //               nearest (the tensor core's own additions round toward zero), rows written to global memory.
 // 64 steps a chunk rather than 32 because a chunk of FP8 is little to load: 176 cycles of the SM's share of HBM
-// at 32, less than a chunk takes.  Instruction issue still bounds it at 64 (ncu: 74% of the slots; a chunk takes
+// at 32, less than a chunk takes.  Instruction issue still bounds it at 64 (ncu: 68% of the slots; a chunk takes
 // 900 to 1400 cycles whether X is loaded or not, and its share of HBM is 350 for FP8, 700 for BF16).  SIMT and this
-// kernel: FP8 768^3 along the last mode, 9 columns 1541 -> 171 us (2.8 TB/s); 689 x 690 x 700, 10 columns, along the
-// last mode BF16 1064 -> 205, FP8 1147 -> 180; along the first BF16 3435 -> 176, FP8 3425 -> 168.
+// kernel: FP8 768^3 along the last mode, 9 columns 1541 -> 176 us (2.7 TB/s); 689 x 690 x 700, 10 columns, along the
+// last mode BF16 1064 -> 219, FP8 1147 -> 186; along the first BF16 3435 -> 178, FP8 3425 -> 168.  (Of these, the
+// search for infinite and NaN results takes up to 14 us.)
 //
 // Every mbarrier wait is bounded by a wall-clock limit; on expiry the CTA raises FLAG_TIMEOUT, stops
 // issuing work, drains what it issued and frees its TMEM.

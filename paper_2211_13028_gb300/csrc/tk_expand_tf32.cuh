@@ -35,13 +35,18 @@ inline int64_t expand_cols(int64_t nj) { return nj <= kExpandK ? 32 : 64; }
 // tile of W again, about as long as 1.2 blocks of output take from two buffers (K <= 32), 2.8 else; the parts whose waves
 // end first.  152 SMs, loss: 262144 x 512, K = 39 (1024 tiles, 16 blocks): one part 197 us, two 215, eight 385; 40000 x 512:
 // 85, 81, 107; 8800 x 391: two 60, four 57, one block each 69; 1600 x 4992 BF16, K = 39 (7 tiles, 156 blocks): one
-// block each 45 us, the 20 parts of a wave 18.
+// block each 45 us, the 21 parts of a wave 18.
 inline int64_t expand_parts(int64_t ntiles, int64_t nblk, int64_t nj, int64_t sms) {
     int64_t best = 1;
     double least = 1e300;
-    for (int64_t ncs = 1; ncs <= nblk && ncs <= 8 * sms; ++ncs) {
-        const int64_t blocks = (nblk + ncs - 1) / ncs, waves = (ntiles * ncs + sms - 1) / sms;
-        const double t = (double)waves * ((nj <= kChunk ? 1.2 : 2.8) + (double)blocks);
+    const double convert = nj <= kChunk ? 1.2 : 2.8;
+    const int64_t most = nblk < 8 * sms ? nblk : 8 * sms;
+    for (int64_t ncs = 1; ncs <= most; ++ncs) {
+        const int64_t waves = (ntiles * ncs + sms - 1) / sms;
+        if ((double)waves * (convert + 1.0) >= least) break;
+        const int64_t full = waves * sms / ntiles;  // the most parts that take no more waves
+        ncs = full < most ? full : most;
+        const double t = (double)waves * (convert + (double)((nblk + ncs - 1) / ncs));
         if (t < least) {
             least = t;
             best = ncs;

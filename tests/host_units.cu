@@ -69,7 +69,7 @@ static int per_device() {
 static int expand_parts() {
     struct {
         int64_t ntiles, nblk, nj, want;
-    } cases[] = {{7, 156, 39, 20},     // a wave: 8 blocks an item (156 items of one block: two waves)
+    } cases[] = {{7, 156, 39, 21},     // a wave: 8 blocks an item (156 items of one block: two waves)
                  {1, 30, 3, 30},       // few: every block its own item
                  {1024, 16, 39, 1},    // many waves: no part converts the tile again
                  {157, 16, 39, 2},     // three waves of half tiles, not two of whole ones
